@@ -235,3 +235,86 @@ def tolerance(case):
         return {"rel": 8e-6, "max": 1e-3}
     # probabilities and outputs are bf16 (seen: rel 2e-3, max 0.04); masks as above
     return {"rel": 1e-2, "max": 0.15, "differ": 1e-5}
+
+
+# ---- the same outputs in 64 bits, by plain torch
+
+def _sinkhorn64(scores):
+    """log-domain iteration over [batch, n, K] fp64"""
+    x = scores / TAU
+    for _ in range(ITERS):
+        x = x - torch.logsumexp(x, dim=1, keepdim=True)
+        x = x - torch.logsumexp(x, dim=2, keepdim=True)
+    return torch.exp(x)
+
+
+def _members64(x, centroids, topk):
+    """0/1 membership [batch, H, n, K] of the vectors x [batch, H, n, D]: the topk groups of largest cosine"""
+    c = centroids.double()
+    c = c / c.norm(dim=-1, keepdim=True)
+    out = torch.zeros(x.shape[:3] + (c.shape[1],), dtype=torch.float32, device=x.device)
+    group = x.shape[1] // c.shape[0]
+    for b in range(x.shape[0]):
+        for h in range(x.shape[1]):
+            v = x[b, h].double()
+            cos = (v @ c[h // group].T) / v.norm(dim=-1, keepdim=True)
+            out[b, h].scatter_(1, cos.topk(topk, dim=1).indices, 1.0)
+    return out
+
+
+def _attend64(q, k, v, first, cap, window, share=None, gate=None):
+    """O [n, D], lse [n] of the rows of q, at positions first.., over their causal keys; `share` = memberships of rows and keys
+    (a distant pair without a common group is left out), `gate` = soft assignments (a distant pair's logit is scaled)"""
+    o, lse = torch.empty(q.shape, dtype=torch.float64, device=q.device), torch.empty(q.shape[0], dtype=torch.float64, device=q.device)
+    k, v = k.double(), v.double()
+    for r in range(0, q.shape[0], 1024):
+        rows = slice(r, min(r + 1024, q.shape[0]))
+        i = torch.arange(first + rows.start, first + rows.stop, device=q.device)[:, None]
+        m = first + rows.stop
+        j = torch.arange(m, device=q.device)[None]
+        s = (q[rows].double() @ k[:m].T) / q.shape[-1] ** 0.5
+        if cap:
+            s = cap * torch.tanh(s / cap)
+        if gate is not None:
+            s = torch.where(i - j > window, s * torch.sigmoid(LAMBDA * (gate[0][rows] @ gate[1][:m].T)), s)
+        if share is not None:
+            s.masked_fill_((i - j > window) & ((share[0][rows] @ share[1][:m].T) < 0.5), -math.inf)
+        s.masked_fill_(j > i, -math.inf)
+        lse[rows] = torch.logsumexp(s, dim=1)
+        o[rows] = torch.exp(s - lse[rows, None]) @ v[:m]
+    return o, lse
+
+
+def exact(case, seed):
+    kind, n, K, B = case["kind"], case["n"], case["K"], case["batch"]
+    Hq = case.get("Hq", 1)
+    if kind in ("prefill", "train") and float(B) * Hq * n * n > 1.5e11:
+        return None                                # longer than a check should take
+    s = prepare(case, seed)
+    if kind == "sinkhorn":
+        x = s["scores"][..., :K].double().requires_grad_()
+        g = _sinkhorn64(x)
+        ds, = torch.autograd.grad(g, x, s["dg"][..., :K].double())
+        pad = (0, s["scores"].shape[-1] - K)
+        return {"g": torch.nn.functional.pad(g.detach(), pad), "ds": torch.nn.functional.pad(ds, pad)}
+    if kind == "route":
+        return {"mq": None, "mk": None, "folded": s["C"].double() @ s["Wg"].double().T}
+    G, w = Hq // case["Hkv"], case["window"]
+    q, k, v = s["q"], s["k"], s["v"]
+    o, lse = torch.empty(q.shape, dtype=torch.float64, device="cuda"), torch.empty(q.shape[:3], dtype=torch.float64, device="cuda")
+    if kind == "train":
+        folded = s["C"].double() @ s["Wg"].double().T
+        scores = torch.stack([torch.cat([part.double() @ folded.T for part in h.split(16384)]) for h in s["h"]])
+        g = _sinkhorn64(scores)
+    else:
+        mq, mk = _members64(q, s["centroids"], case["topk"]), _members64(k, s["centroids"], case["topk"])
+    for b in range(B):
+        for h in range(Hq):
+            pair = {"gate": (g[b], g[b])} if kind == "train" else {"share": (mq[b, h], mk[b, h // G])}
+            o[b, h], lse[b, h] = _attend64(q[b, h], k[b, h // G], v[b, h // G], n - q.shape[2], case["softcap"] if kind != "train" else 0.0, w, **pair)
+    if kind == "train":
+        pad = (0, s["g"].shape[-1] - K)
+        return {"o": o, "lse": lse.view(B * Hq, n), "g": torch.nn.functional.pad(g, pad), "scores": torch.nn.functional.pad(scores, pad), "status": None}
+    if kind == "decode":
+        return {"o": o[:, :, 0], "lse": lse.view(B * Hq), "mq_new": None, "mk": None}
+    return {"o": o, "lse": lse.view(B * Hq, n), "mq": None, "mk": None, "status": None}
