@@ -9,9 +9,12 @@
 // column offsets.  Offsets are kept as logarithms, so nothing overflows at a small temperature; the very first
 // column sum is taken relative to the column maximum.  Column sums are accumulated in fp64.
 //
-// The score matrix (n x K fp32, a few MB) stays in L2 between the passes; a pass is one small launch, and the
-// N + 2 launches, not bandwidth, set the time.
+// Two forms.  While a sequence's rows fit in the shared memory of the blocks that are resident at once, one cooperative
+// launch does the whole call (sinkhorn_team_kernel): every row is read once, and what separates two iterations is a
+// barrier between the blocks of a sequence.  Longer sequences take one launch per iteration over the matrix in L2.
 #include "common.cuh"
+
+#include <type_traits>
 
 namespace focus {
 
@@ -28,6 +31,7 @@ __device__ __forceinline__ float float_of_ordered(uint32_t o) {
 }
 
 // workspace of one sequence: double T[iters + 1][32] (column sums of pass 0, 1, ...), then uint32 M[32] (column maxima)
+// (then, for all sequences, the words of the one-launch form)
 __host__ __device__ inline size_t sk_seq_bytes(int iters) { return (size_t)(iters + 1) * 32 * sizeof(double) + 32 * sizeof(uint32_t); }
 
 template <int KMAX>
@@ -145,7 +149,395 @@ sinkhorn_pass_kernel(const float* __restrict__ S, int n, int K, int iters, int p
     }
 }
 
-size_t sinkhorn_workspace_bytes(const focus_shape* s, int iters) { return (size_t)s->batch * sk_seq_bytes(iters); }
+// ---- one launch for the whole call: the P blocks of a sequence (a "team") keep its rows in shared memory, `chunk`
+// tokens per block, and walk the iterations together.  Between two iterations stands one exchange: every block publishes
+// its K column sums and adds up the P x K numbers of its team.  A number travels with the exchange's ordinal in one 8-byte
+// word (the low 16 of a double's 52 mantissa bits give way to it), written and polled whole, so that neither a fence nor
+// a counter stands between writing and reading it (fp64 atomics into one sum, a fence and an arrival counter took 3.5 us
+// per exchange), and the order of every sum is fixed.  What bounds it is latency: of the ~2.6 us of an iteration a third
+// is the words' way through L2, the rest instruction issue and block barriers.  The launch is cooperative, so
+// that all blocks of a team run at once.
+constexpr int SKT_THREADS = 512;
+constexpr int SKT_TOKENS = 8 * SKT_THREADS;          // tokens per block at most: fp32 column sums of a thread over 8 rows
+constexpr int SKT_BLOCKS = 160;                      // blocks per team at most (the workspace has words for as many)
+constexpr size_t SKT_SMEM = 200 * 1024;
+constexpr unsigned long long SKT_TAG = 0xffffull;
+constexpr long long SKT_LEAD = 900;                  // cycles before the first poll
+
+// words of one sequence's exchanges: two sets, taken in turn.  A block writes set e mod 2 for exchange e + 2 after it has
+// read everybody's e + 1, which each of them wrote after reading everybody's e.
+static int skt_max_blocks(int n) { return cdiv(n, SKT_THREADS) < SKT_BLOCKS ? cdiv(n, SKT_THREADS) : SKT_BLOCKS; }
+// Every block has 128-byte lines of its own.
+__host__ __device__ constexpr size_t skt_stride(int ld) { return ld < 16 ? 128 : (size_t)ld * 8; }
+static size_t skt_words_bytes(const focus_shape* s) { return 2 * skt_max_blocks(s->n) * skt_stride(focus_soft_ld(s->K)); }
+
+__device__ __forceinline__ void put_word(void* p, double v, unsigned long long tag) {
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)__double_as_longlong(v) & ~SKT_TAG) | tag) : "memory");
+}
+__device__ __forceinline__ bool get_words(const void* p, unsigned long long tag, double& v0, double& v1) {
+    unsigned long long a, b;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    v0 = __longlong_as_double((long long)(a & ~SKT_TAG));
+    v1 = __longlong_as_double((long long)(b & ~SKT_TAG));
+    return (a & SKT_TAG) == tag && (b & SKT_TAG) == tag;
+}
+
+// log2 of a positive double to about 1e-11, in a quarter of the time of the library's (it stands between two iterations):
+// Tang's table method.  tab[k] = (c, -log2 c) with c a float near 1 / (1 + (k + 1/2) / 32); u = m c - 1 for the mantissa m
+// is below 1/60, and the terms of log1p(u) beyond the first are summed in fp32.
+__device__ __forceinline__ double2 log2_entry(int k) {
+    const float c = 1.f / (1.f + (k + 0.5f) / 32.f);
+    return make_double2((double)c, -log2((double)c));
+}
+__device__ __forceinline__ double log2_table(double x, const double2* tab) {
+    if (!(x >= 2.2250738585072014e-308 && x < INFINITY)) return log2(x);           // zero, denormal, infinity, NaN
+    const long long bits = __double_as_longlong(x);
+    const int e = (int)(bits >> 52) - 1023;
+    const double m = __longlong_as_double((bits & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
+    const double2 t = tab[(int)(bits >> 47) & 31];
+    const double u = fma(m, t.x, -1.0);
+    const float uf = (float)u;
+    const float tail = uf * uf * fmaf(uf, fmaf(uf, fmaf(uf, 0.2f, -0.25f), 0.333333333f), -0.5f);
+    return (double)e + t.y + 1.4426950408889634 * (u + (double)tail);
+}
+__device__ __forceinline__ float ex2f(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcpf(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// v[0..N) of the 32 lanes combined: lane l ends with the result of value l / (32 / N) in v[0]
+template <int N, bool MAX>
+__device__ __forceinline__ void reduce_lanes(float (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int w = N / 2; w >= 1; w /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const float r = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + w], off);
+            const float mine = up ? v[i + w] : v[i];
+            v[i] = MAX ? fmaxf(mine, r) : mine + r;
+        }
+    }
+    for (; off >= 1; off /= 2) {
+        const float r = __shfl_xor_sync(0xffffffffu, v[0], off);
+        v[0] = MAX ? fmaxf(v[0], r) : v[0] + r;
+    }
+}
+
+// BWD = false: out = the assignments.  BWD = true: the column sums again, then the derivative of the assignments
+// from d_in to out (the passes of sinkhorn_bwd_pass_kernel and sinkhorn_bwd_last_kernel below).
+template <int KMAX, bool BWD>
+__global__ void __launch_bounds__(SKT_THREADS, 1)
+sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float inv_tau, unsigned char* __restrict__ ws,
+                     unsigned char* __restrict__ words, size_t words_bytes, const float* d_in, float* out, int P, int chunk) {
+    extern __shared__ float4 rows_s[];               // [KMAX / 4][chunk] scores, then as many of the derivative
+    constexpr int NW = SKT_THREADS / 32, PIECES = KMAX / 4;
+    __shared__ float red[NW][KMAX];
+    __shared__ float colmax_s[KMAX], voff_s[KMAX], pend_sub_s[KMAX], pend_inv_s[KMAX], ct_s[KMAX];
+    __shared__ double team_s[NW][KMAX];
+    __shared__ int failed_s;
+    const int b = blockIdx.x / P, rank = blockIdx.x % P, tok0 = rank * chunk;
+    const int cnt = min(chunk, n - tok0);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double* const T = reinterpret_cast<double*>(ws + (size_t)b * sk_seq_bytes(iters));       // BWD: sums of pass 0 .. iters - 1
+    words += (size_t)b * words_bytes;
+    float4* const dcache = rows_s + (size_t)PIECES * chunk;
+    auto get = [&](const float4* c, int i, float (&x)[KMAX]) {
+#pragma unroll
+        for (int q = 0; q < PIECES; ++q) {
+            const float4 v = c[(size_t)q * chunk + i];
+            x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
+        }
+    };
+    auto put = [&](float4* c, int i, const float (&x)[KMAX]) {
+#pragma unroll
+        for (int q = 0; q < PIECES; ++q) c[(size_t)q * chunk + i] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+    };
+    __shared__ double2 tab_s[32];
+    if (threadIdx.x < 32) tab_s[threadIdx.x] = log2_entry(threadIdx.x);
+    if (threadIdx.x == 0) failed_s = 0;
+
+    // the exchange: the warps' values (red) become the block's, the blocks' the team's; collect(g, value) runs in lane g
+    // of the first warp.  Thread t polls the words of groups 2 (t mod KMAX / 2) and the next.
+    unsigned long long ordinal = 0;
+    auto exchange = [&](auto is_max, auto collect) {
+        constexpr bool MAX = decltype(is_max)::value;
+        constexpr int PARTS = 32 / KMAX, PAIRS = KMAX / 2;
+        auto combine = [](double x, double y) { return MAX ? fmax(x, y) : x + y; };
+        // lane l: value l mod KMAX of the warps, PARTS lanes a value
+        auto over_warps = [&](auto& vals) {
+            double v = (double)vals[lane / KMAX][lane % KMAX];
+#pragma unroll
+            for (int w = PARTS; w < NW; w += PARTS) v = combine(v, (double)vals[w + lane / KMAX][lane % KMAX]);
+#pragma unroll
+            for (int off = 16; off >= KMAX; off /= 2) v = combine(v, __shfl_xor_sync(0xffffffffu, v, off));
+            return v;
+        };
+        ++ordinal;
+        unsigned char* const set = words + (size_t)(ordinal & 1) * P * skt_stride(KMAX);
+        __syncthreads();                             // red holds the warps' values
+        if (warp == 0) {
+            const double v = over_warps(red);
+            if (lane < KMAX) put_word(set + (size_t)rank * skt_stride(KMAX) + lane * 8, v, ordinal);
+        }
+        double v0 = MAX ? -INFINITY : 0.0, v1 = v0;
+        if (!failed_s) {
+            constexpr int STEP = SKT_THREADS / PAIRS, PER = (SKT_BLOCKS + STEP - 1) / STEP;
+            double got[PER][2];
+            bool seen[PER];
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                got[j][0] = got[j][1] = v0;
+                seen[j] = threadIdx.x / PAIRS + j * STEP >= P;
+            }
+            // A poll that comes too early makes the next one take 1.4 us instead of 0.4, and a block that is late by that
+            // much makes the others' polls come too early in the next exchange; so wait out the words' way first (about
+            // 0.5 us): 31 + 60 us for forward and backward at 131072 x 8, 34 + 72 us without.
+            const long long t0 = clock64();
+            while (clock64() - t0 < SKT_LEAD) { }
+            for (bool all = false; !all;) {
+                all = true;
+#pragma unroll
+                for (int j = 0; j < PER; ++j) {
+                    const int q = threadIdx.x / PAIRS + j * STEP;
+                    if (!seen[j]) all &= seen[j] = get_words(set + (size_t)q * skt_stride(KMAX) + threadIdx.x % PAIRS * 16, ordinal, got[j][0], got[j][1]);
+                }
+                if (!all && clock64() - t0 > 4000000000ll) {          // two seconds
+                    failed_s = 1;
+                    break;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < PER; ++j) { v0 = combine(v0, got[j][0]); v1 = combine(v1, got[j][1]); }
+        }
+#pragma unroll
+        for (int off = 16; off >= PAIRS; off /= 2) {
+            v0 = combine(v0, __shfl_xor_sync(0xffffffffu, v0, off));
+            v1 = combine(v1, __shfl_xor_sync(0xffffffffu, v1, off));
+        }
+        if (lane < PAIRS) { team_s[warp][2 * lane] = v0; team_s[warp][2 * lane + 1] = v1; }
+        __syncthreads();
+        if (warp == 0) {
+            const double v = over_warps(team_s);
+            if (lane < KMAX) collect(lane, v);
+        }
+        __syncthreads();
+    };
+    auto store_warp = [&](float (&v)[KMAX]) {
+        if (lane % (32 / KMAX) == 0) red[warp][lane / (32 / KMAX)] = v[0];
+    };
+
+    // ---- rows to shared memory, column maxima
+    {
+        float mx[KMAX];
+#pragma unroll
+        for (int g = 0; g < KMAX; ++g) mx[g] = -INFINITY;
+        const float4* src = reinterpret_cast<const float4*>(S + ((size_t)b * n + tok0) * KMAX);
+        const float4* dsrc = BWD ? reinterpret_cast<const float4*>(d_in + ((size_t)b * n + tok0) * KMAX) : nullptr;
+        for (int i = threadIdx.x; i < cnt; i += SKT_THREADS)
+#pragma unroll
+            for (int q = 0; q < PIECES; ++q) {
+                const float4 v = src[(size_t)i * PIECES + q];
+                rows_s[(size_t)q * chunk + i] = v;
+                if (BWD) {
+                    const float4 d = dsrc[(size_t)i * PIECES + q];           // entries beyond K are ignored
+                    dcache[(size_t)q * chunk + i] = make_float4(4 * q < K ? d.x : 0.f, 4 * q + 1 < K ? d.y : 0.f,
+                                                                4 * q + 2 < K ? d.z : 0.f, 4 * q + 3 < K ? d.w : 0.f);
+                }
+                mx[4 * q] = fmaxf(mx[4 * q], v.x); mx[4 * q + 1] = fmaxf(mx[4 * q + 1], v.y);
+                mx[4 * q + 2] = fmaxf(mx[4 * q + 2], v.z); mx[4 * q + 3] = fmaxf(mx[4 * q + 3], v.w);
+            }
+        reduce_lanes<KMAX, true>(mx);
+        store_warp(mx);
+    }
+    exchange(std::true_type{}, [&](int g, double m) {
+        colmax_s[g] = m > -INFINITY ? (float)m : float_of_ordered(0u);         // (a word holds a float exactly); no maximum: NaN
+        voff_s[g] = g < K ? 0.f : -INFINITY;
+        ct_s[g] = pend_sub_s[g] = 0.f;
+        pend_inv_s[g] = g < K ? 1.f : 0.f;
+    });
+    // the cached scores become S - M, 0 beyond K (where the offsets of minus infinity leave nothing).  Log2 units are
+    // (S - M) * log2(e) / tau, the factor in two floats: a factor rounded once would shift every exponent alike
+    const double per_tau = 1.4426950408889634 / (double)tau;
+    const float c_hi = (float)per_tau, c_lo = (float)(per_tau - (double)c_hi);
+    for (int i = threadIdx.x; i < cnt; i += SKT_THREADS) {
+        float x[KMAX];
+        get(rows_s, i, x);
+#pragma unroll
+        for (int g = 0; g < KMAX; ++g) x[g] = g < K ? x[g] - colmax_s[g] : 0.f;
+        put(rows_s, i, x);
+    }
+    auto log2_units = [&](float x, float off) { return fmaf(x, c_hi, fmaf(x, c_lo, off)); };
+    // ---- column sums of pass 0 .. iters - 1.  Lane g of the first warp keeps column g's offset in double: minus the logs
+    // of the sums so far.
+    double acc = 0.0, sum = 1.0;                     // and the last sum collected
+    // Z = softmax over the groups of the scores plus offsets, as exponentials and the reciprocal of their sum
+    auto softmax_row = [&](float (&x)[KMAX]) {
+        float mx = -INFINITY;
+#pragma unroll
+        for (int g = 0; g < KMAX; ++g) {
+            x[g] = log2_units(x[g], voff_s[g]);
+            mx = fmaxf(mx, x[g]);
+        }
+        float se = 0.f;
+#pragma unroll
+        for (int g = 0; g < KMAX; ++g) {
+            x[g] = ex2f(x[g] - mx);
+            se += x[g];
+        }
+        return rcpf(se);
+    };
+    for (int pass = 0; pass < iters; ++pass) {
+        float tsum[KMAX];
+#pragma unroll
+        for (int g = 0; g < KMAX; ++g) tsum[g] = 0.f;
+        for (int i = threadIdx.x; i < cnt; i += SKT_THREADS) {
+            float x[KMAX];
+            get(rows_s, i, x);
+            if (pass == 0) {
+#pragma unroll
+                for (int g = 0; g < KMAX; ++g) tsum[g] += ex2f(log2_units(x[g], 0.f));
+            } else {
+                const float inv = softmax_row(x);
+#pragma unroll
+                for (int g = 0; g < KMAX; ++g) tsum[g] = fmaf(x[g], inv, tsum[g]);
+            }
+        }
+        reduce_lanes<KMAX, false>(tsum);
+        store_warp(tsum);
+        exchange(std::false_type{}, [&](int g, double total) {
+            if (g < K) {
+                sum = total;
+                acc -= log2_table(sum, tab_s);
+            }
+            // a row's softmax does not see what all offsets have in common (about log2(n / K) per pass): leave it out, so
+            // that a small number is rounded to fp32
+            const double common = __shfl_sync(KMAX == 32 ? 0xffffffffu : (1u << KMAX) - 1u, acc, 0);
+            if (g >= K) return;
+            voff_s[g] = (float)(BWD && iters == 1 ? acc : acc - common);      // (Y_0 below wants the offset itself)
+            if (BWD) {
+                T[(size_t)pass * 32 + g] = sum;      // the same value from every block; read back by this thread
+                ct_s[g] = (float)sum;                // for the first pass of the derivative, t = iters - 1
+            }
+        });
+    }
+    float4* const o = reinterpret_cast<float4*>(out + ((size_t)b * n + tok0) * KMAX);
+    if constexpr (!BWD) {
+        // ---- the last row division
+        for (int i = threadIdx.x; i < cnt; i += SKT_THREADS) {
+            float x[KMAX];
+            get(rows_s, i, x);
+            const float inv = softmax_row(x);
+#pragma unroll
+            for (int q = 0; q < PIECES; ++q)
+                o[(size_t)i * PIECES + q] = make_float4(x[4 * q] * inv, x[4 * q + 1] * inv, x[4 * q + 2] * inv, x[4 * q + 3] * inv);
+        }
+    } else {
+        // ---- the iterations in reverse
+        for (int t = iters - 1; t >= 0; --t) {
+            float tsum[KMAX];
+#pragma unroll
+            for (int g = 0; g < KMAX; ++g) tsum[g] = 0.f;
+            for (int i = threadIdx.x; i < cnt; i += SKT_THREADS) {
+                float x[KMAX], d[KMAX];
+                get(rows_s, i, x);
+                get(dcache, i, d);
+                const float inv = softmax_row(x);
+                float dot = 0.f, rinv = t >= 1 ? 0.f : 1.f;
+#pragma unroll
+                for (int g = 0; g < KMAX; ++g) {
+                    x[g] *= inv;                     // Z_t
+                    d[g] = (d[g] - pend_sub_s[g]) * pend_inv_s[g];
+                    dot = fmaf(d[g], x[g], dot);
+                    if (t >= 1) rinv = fmaf(x[g], ct_s[g], rinv);         // 1 / r_t (see sinkhorn_bwd_pass_kernel)
+                }
+#pragma unroll
+                for (int g = 0; g < KMAX; ++g) {
+                    const float e = d[g] - dot;
+                    tsum[g] = fmaf(e, x[g], tsum[g]);
+                    d[g] = e * rinv;
+                }
+                put(dcache, i, d);
+            }
+            reduce_lanes<KMAX, false>(tsum);
+            store_warp(tsum);
+            exchange(std::false_type{}, [&](int g, double total) {
+                if (g < K) {
+                    pend_sub_s[g] = (float)total;
+                    pend_inv_s[g] = (float)(1.0 / sum);              // sum = T[t]
+                    if (t >= 1) {
+                        acc += log2_table(sum, tab_s);
+                        sum = T[(size_t)(t - 1) * 32 + g];
+                        ct_s[g] = (float)sum;
+                    }
+                }
+                const double common = __shfl_sync(KMAX == 32 ? 0xffffffffu : (1u << KMAX) - 1u, acc, 0);
+                if (g < K && t >= 1) voff_s[g] = (float)(t == 1 ? acc : acc - common);
+            });
+        }
+        // dS = (e * Z_0 - B_0 * Y_0) / tau, e as pass 0 left it, B_0 in pend_sub_s
+        for (int i = threadIdx.x; i < cnt; i += SKT_THREADS) {
+            float x[KMAX], e[KMAX], y[KMAX];
+            get(rows_s, i, x);
+            get(dcache, i, e);
+#pragma unroll
+            for (int g = 0; g < KMAX; ++g) y[g] = ex2f(log2_units(x[g], voff_s[g]));            // Y_0 (may underflow to 0: then its term vanishes)
+            const float inv = softmax_row(x);
+#pragma unroll
+            for (int g = 0; g < KMAX; ++g) e[g] = g < K ? (e[g] * (x[g] * inv) - pend_sub_s[g] * y[g]) * inv_tau : 0.f;
+#pragma unroll
+            for (int q = 0; q < PIECES; ++q) o[(size_t)i * PIECES + q] = make_float4(e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3]);
+        }
+    }
+    if (failed_s) {                                  // a wait ran out: no number that looks like a result
+        const float bad = __int_as_float(0x7fffffff);
+        for (int i = threadIdx.x; i < cnt * PIECES; i += SKT_THREADS) o[i] = make_float4(bad, bad, bad, bad);
+    }
+}
+
+// Runs the call as one cooperative launch if the rows of every sequence fit in its team's shared memory; `done` says
+// whether it did.  A team has one block per 512 tokens, at most its share of the multiprocessors.
+template <int KMAX, bool BWD>
+static int launch_team(const focus_shape* s, const float* S, float tau, int iters, unsigned char* ws, const float* d_in, float* out,
+                       cudaStream_t st, bool& done) {
+    done = false;
+    int dev = 0, sms = 0, rc;
+    if ((rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
+    if ((rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute"))) return rc;
+    if (s->batch > sms) return 0;
+    int P = sms / s->batch;
+    if (P > skt_max_blocks(s->n)) P = skt_max_blocks(s->n);
+    const int chunk = cdiv(cdiv(s->n, P), SKT_THREADS) * SKT_THREADS;        // whole rounds of the threads
+    const size_t smem = (size_t)chunk * KMAX * sizeof(float) * (BWD ? 2 : 1);
+    if (chunk > SKT_TOKENS || smem > SKT_SMEM) return 0;
+    P = cdiv(s->n, chunk);                           // no block without tokens
+    auto kern = sinkhorn_team_kernel<KMAX, BWD>;
+    if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SKT_SMEM), "cudaFuncSetAttribute(sinkhorn)")))
+        return rc;
+    cudaLaunchAttribute coop;
+    coop.id = cudaLaunchAttributeCooperative;
+    coop.val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(P * s->batch);
+    cfg.blockDim = dim3(SKT_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &coop;
+    cfg.numAttrs = 1;
+    done = true;
+    return check_cuda(cudaLaunchKernelEx(&cfg, kern, S, s->n, s->K, iters, tau, 1.f / tau, ws, ws + s->batch * sk_seq_bytes(iters),
+                                         skt_words_bytes(s), d_in, out, P, chunk), "sinkhorn launch");
+}
+
+size_t sinkhorn_workspace_bytes(const focus_shape* s, int iters) { return (size_t)s->batch * (sk_seq_bytes(iters) + skt_words_bytes(s)); }
 
 template <int KMAX>
 static int launch_sk(const focus_shape* s, const float* S, float tau, int iters, unsigned char* ws, float* out, cudaStream_t st) {
@@ -155,7 +547,8 @@ static int launch_sk(const focus_shape* s, const float* S, float tau, int iters,
     const dim3 grid(nblk, s->batch);
     const float inv_tau = 1.f / tau;
     int rc = check_cuda(cudaMemsetAsync(ws, 0, sinkhorn_workspace_bytes(s, iters), st), "cudaMemsetAsync(sinkhorn workspace)");
-    if (rc) return rc;
+    bool done = false;
+    if (rc || (rc = launch_team<KMAX, false>(s, S, tau, iters, ws, nullptr, out, st, done)) || done) return rc;
     sinkhorn_colmax_kernel<KMAX><<<grid, SK_THREADS, 0, st>>>(S, n, K, iters, ws);
     sinkhorn_pass_kernel<KMAX, 0><<<grid, SK_THREADS, 0, st>>>(S, n, K, iters, 0, inv_tau, ws, nullptr);
     for (int pass = 1; pass < iters; ++pass)
@@ -323,7 +716,7 @@ sinkhorn_bwd_last_kernel(const float* __restrict__ S, int n, int K, int iters, f
 }
 
 size_t sinkhorn_bwd_workspace_bytes(const focus_shape* s, int iters) {
-    return (size_t)s->batch * (sk_seq_bytes(iters) + (size_t)iters * 32 * sizeof(double));
+    return sinkhorn_workspace_bytes(s, iters) + (size_t)s->batch * iters * 32 * sizeof(double);
 }
 
 template <int KMAX>
@@ -336,7 +729,9 @@ static int launch_sk_bwd(const focus_shape* s, const float* S, float tau, int it
     const float inv_tau = 1.f / tau;
     int rc = check_cuda(cudaMemsetAsync(ws, 0, sinkhorn_bwd_workspace_bytes(s, iters), st), "cudaMemsetAsync(sinkhorn workspace)");
     if (rc) return rc;
-    double* B = reinterpret_cast<double*>(ws + (size_t)s->batch * sk_seq_bytes(iters));
+    double* B = reinterpret_cast<double*>(ws + sinkhorn_workspace_bytes(s, iters));
+    bool done = false;
+    if ((rc = launch_team<KMAX, true>(s, S, tau, iters, ws, dG, dS, st, done)) || done) return rc;
     // the forward's column sums again (no assignments written)
     sinkhorn_colmax_kernel<KMAX><<<grid, SK_THREADS, 0, st>>>(S, n, K, iters, ws);
     sinkhorn_pass_kernel<KMAX, 0><<<grid, SK_THREADS, 0, st>>>(S, n, K, iters, 0, inv_tau, ws, nullptr);

@@ -66,6 +66,51 @@ def test_sinkhorn(n, K, tau, iters, batch, spread):
     assert torch.equal(S, out)
 
 
+@pytest.mark.parametrize("n,K,batch", [(511, 8, 1), (513, 8, 1), (4096 + 1, 3, 2), (148 * 1024, 8, 1), (700, 4, 150), (40000, 32, 2),
+                                       (148 * 4096 + 1, 4, 1)])
+def test_sinkhorn_one_launch_and_launch_per_iteration(n, K, batch):
+    """sizes around a block's 512 threads and the most tokens the one-launch form holds, batches above the multiprocessor count,
+    rows too long for its shared memory: forward and derivative, replayed from a graph over a changed input as well"""
+    tau, iters = 0.1, 4
+    g = torch.Generator(device="cuda"); g.manual_seed(n + K)
+    ld = fb.focus_soft_ld(K)
+    S = padded(0.3 * torch.randn((batch, n, K), generator=g, device="cuda"), ld)
+    dg = padded(torch.randn((batch, n, K), generator=g, device="cuda"), ld)
+    shape = fb.make_shape(4, 2, n, 128, K, 1, 16, batch=batch)
+    ws = torch.empty(fb.focus_sinkhorn_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+    wb = torch.empty(fb.focus_sinkhorn_bwd_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+    out, ds = torch.full_like(S, float("nan")), torch.full_like(S, float("nan"))
+
+    def both():
+        fb.focus_sinkhorn(shape, S, tau, iters, ws, out)
+        fb.focus_sinkhorn_bwd(shape, S, tau, iters, wb, dg, ds)
+
+    def check():
+        for b in {0, batch - 1}:
+            s64 = S[b, :, :K].double().requires_grad_()
+            x = s64 / tau
+            for _ in range(iters):
+                x = x - torch.logsumexp(x, dim=0, keepdim=True)
+                x = x - torch.logsumexp(x, dim=1, keepdim=True)
+            ref = x.exp()
+            ref_ds, = torch.autograd.grad(ref, s64, dg[b, :, :K].double())
+            torch.testing.assert_close(out[b, :, :K].double(), ref.detach(), rtol=5e-4, atol=1e-7)
+            assert (ds[b, :, :K].double() - ref_ds).abs().max() <= 2e-4 * ref_ds.abs().max()
+            assert (out[b, :, K:] == 0).all() and (ds[b, :, K:] == 0).all()
+
+    both()
+    check()
+    stream = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        both()
+    S.mul_(-1.0)
+    graph.replay(); graph.replay()
+    torch.cuda.synchronize()
+    check()
+
+
 def gate_case(Hq, Hkv, n, D, K, seed, batch=1):
     g = torch.Generator(device="cuda"); g.manual_seed(seed)
     Q = torch.randn((batch, Hq, n, D), generator=g, device="cuda").to(torch.bfloat16)
