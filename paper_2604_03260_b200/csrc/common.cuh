@@ -49,6 +49,30 @@ inline size_t sorted_scratch_bytes(const focus_shape* s) {
            align_up((size_t)s->batch * s->Hq * (size_t)(sorted_capacity(s->n) / 256) * 4, 256);
 }
 
+// Programmatic dependent launch: a kernel launched by launch_dependent may be set up while the kernel before it in the
+// stream still runs; before it touches memory that anything before it wrote or still reads, every thread of it executes
+// dep_wait(), which returns when all earlier work of the stream is complete and visible.  dep_trigger() lets the next
+// such kernel be set up from here on (it still waits for the end of this one).
+#ifdef __CUDACC__
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+inline cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+#endif
+
 // launchers implemented in the other translation units
 int launch_assign(const focus_shape* s, const focus_tensor& x, int H, const float* centroids, uint32_t* masks,
                   unsigned long long* near_ties, float eps, cudaStream_t st);

@@ -17,6 +17,20 @@ constexpr int DEC_NST = 3;           // stages of a warp's private K/V ring
 constexpr float DEC_LOG2E = 1.4426950408889634f;
 constexpr float DEC_LN2 = 0.6931471805599453f;
 
+constexpr int DEC_CTAS = 2 * 148;    // two CTAs per SM, all resident
+
+// How the work is cut: the steps of 16 keys of all KV heads in one list, dealt out as equal contiguous ranges, one per
+// CTA, whatever the number of heads (a whole number of splits per head left 64 heads x 5 splits = 320 CTAs on 296
+// places, a second wave for 24 of them: 173 us for 8 sequences of 16385 keys).  A CTA whose range enters another KV head
+// writes one partial result per head.
+struct DecPlan {
+    int groups;                      // steps per KV head
+    int ctas, slots;                 // CTAs, partial results per head at most
+    long long total, per;            // steps in all, steps per CTA
+    __host__ __device__ int first_cta(int bh) const { return (int)((long long)bh * groups / per); }
+    __host__ __device__ int last_cta(int bh) const { return (int)(((long long)(bh + 1) * groups - 1) / per); }
+};
+
 template <int D> struct DecCfg {
     static constexpr int WARPS = D == 256 ? 2 : 4;                 // warps per CTA: two CTAs fit an SM at every D
     static constexpr int ROWB = 2 * D + 16;                        // padded row: conflict-free ldmatrix rows
@@ -53,14 +67,12 @@ __global__ void __launch_bounds__(DecCfg<D>::WARPS * 32)
 decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t q_sh, const __nv_bfloat16* __restrict__ k,
                       int64_t k_sb, int64_t k_sh, int64_t k_sn, const __nv_bfloat16* __restrict__ v, int64_t v_sb,
                       int64_t v_sh, int64_t v_sn, const uint32_t* __restrict__ mq_new, const uint32_t* __restrict__ mk,
-                      int Hq, int Hkv, int G, int n, int w, float scale, float softcap, int nsplit, int groups_per_split,
-                      float* __restrict__ part) {
+                      int Hq, int Hkv, int G, int n, int w, float scale, float softcap, const DecPlan plan, float* __restrict__ part) {
     using C = DecCfg<D>;
     constexpr int VEC = D / 8;                                     // 16-byte pieces per row
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t kflag_s[C::WARPS][DEC_NST][DEC_GK];        // per staged key: bit g set when query head g attends it
-    const int split = blockIdx.x, bh = blockIdx.y;                 // bh = batch * Hkv + KV head
-    const int b = bh / Hkv, hk = bh % Hkv;
+    dep_trigger();                                                 // the merge may be set up now; it waits for this kernel's end
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, qd = lane & 3;                        // this thread's query head (MMA row) and column pair
     const int last = n - 1;                                        // position of the new token
@@ -69,9 +81,21 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
     unsigned char* ring = smem_raw + (size_t)warp * DEC_NST * C::STAGE;
     const uint32_t ring_u32 = (uint32_t)__cvta_generic_to_shared(ring);
 
+    // this CTA's steps of the list (KV head by KV head, 16 keys a step): one segment per KV head it touches
+    const long long f_end = min((long long)(blockIdx.x + 1) * plan.per, plan.total);
+    bool waited = false;
+    for (long long f = (long long)blockIdx.x * plan.per; f < f_end;) {
+    const int bh = (int)(f / plan.groups);                         // batch * Hkv + KV head
+    const int b = bh / Hkv, hk = bh % Hkv;
+    const int g_begin = (int)(f - (long long)bh * plan.groups);
+    const int g_end = (int)min((long long)plan.groups, g_begin + (f_end - f));
+    f += g_end - g_begin;
+
     // rows that are never copied still enter the MMAs (with probability 0): keep them finite
     for (int i = lane; i < DEC_NST * C::STAGE / 16; i += 32) reinterpret_cast<uint4*>(ring)[i] = make_uint4(0, 0, 0, 0);
     __syncwarp();
+    if (!waited) dep_wait();
+    waited = true;
 
     // Q as the row operand: rows >= G and rows 8..15 are zero
     uint32_t qa[D / 16][2];
@@ -92,9 +116,6 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
     const uint32_t* mkh = mk + (size_t)bh * n;
 
     // this warp's steps: groups g0 + warp, g0 + warp + WARPS, ... of 16 keys
-    const int total_groups = (n + DEC_GK - 1) / DEC_GK;
-    const int g_begin = split * groups_per_split;
-    const int g_end = min(g_begin + groups_per_split, total_groups);
     const int nsteps = g_begin + warp < g_end ? (g_end - g_begin - warp + C::WARPS - 1) / C::WARPS : 0;
     auto first_key = [&](int step) { return (g_begin + warp + step * C::WARPS) * DEC_GK; };
 
@@ -210,8 +231,8 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
         __syncwarp();                               // the stage may be refilled by the next issue
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    // ---- merge the warps of the CTA (through the ring, no longer needed), then one partial result per split:
-    //      [query head][split][2 + D] = (max, sum, O)
+    // ---- merge the warps of the CTA (through the ring, no longer needed), then one partial result per segment:
+    //      [query head][CTA, counted from the first that touches the head][2 + D] = (max, sum, O)
     __syncthreads();
     float* xw = reinterpret_cast<float*>(smem_raw);             // [WARPS][GMAX][D + 2]
     if (g < DEC_GMAX) {
@@ -235,33 +256,47 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
             L = fmaf(src[1], wgt, L);
             acc = fmaf(src[2 + d], wgt, acc);
         }
-        float* dst = part + (((size_t)b * Hq + hk * G + gg) * nsplit + split) * (D + 2);
+        float* dst = part + (((size_t)b * Hq + hk * G + gg) * plan.slots + (blockIdx.x - plan.first_cta(bh))) * (D + 2);
         if (d == 0) { dst[0] = M; dst[1] = L; }
         dst[2 + d] = acc;
     }
+    if (f < f_end) __syncthreads();                                // the next segment's ring
+    }
 }
 
-// one block per query head: merge the splits (weights of the splits once through shared memory, then every
-// thread one output dimension with independent loads)
+// One block per query head: the partial results of the CTAs that touched its KV head, joined by their maxima.  Latency is
+// all of it (a few KB per head): the threads form 256 / (D / 2) rows, row r taking partials r, r + rows, ...; a thread's first
+// eight loads of O are under way while the weights are worked out.
+template <int D>
 __global__ void __launch_bounds__(256)
-decode_merge_kernel(const float* __restrict__ part, int nsplit, int D, int Hq, __nv_bfloat16* __restrict__ o, int64_t o_sb,
+decode_merge_kernel(const float* __restrict__ part, const DecPlan plan, int Hq, int Hkv, __nv_bfloat16* __restrict__ o, int64_t o_sb,
                     int64_t o_sh, float* __restrict__ lse) {
-    __shared__ float wgt_s[512];
-    __shared__ float red_s[8];
-    const int hq = blockIdx.x, t = threadIdx.x;
-    const float* p = part + (size_t)hq * nsplit * (D + 2);
+    constexpr int LANES = D / 2, ROWS = 256 / LANES, AHEAD = 8;
+    __shared__ float wgt_s[DEC_CTAS + 1];
+    __shared__ float red_s[2][8];
+    __shared__ float2 acc_s[ROWS][LANES];
+    const int hq = blockIdx.x, t = threadIdx.x, row = t / LANES, col = t % LANES;
+    const int bh = hq / Hq * Hkv + hq % Hq / (Hq / Hkv);
+    const int first = plan.first_cta(bh), cnt = plan.last_cta(bh) - first + 1;
+    const float* p = part + (size_t)hq * plan.slots * (D + 2);
+    dep_wait();
+    float2 v[AHEAD];
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j) {
+        const int s = row + j * ROWS;
+        v[j] = s < cnt ? *reinterpret_cast<const float2*>(p + (size_t)s * (D + 2) + 2 + 2 * col) : make_float2(0.f, 0.f);
+    }
     float m = -INFINITY;
-    for (int s = t; s < nsplit; s += 256) m = fmaxf(m, p[(size_t)s * (D + 2)]);
+    for (int s = t; s < cnt; s += 256) m = fmaxf(m, p[(size_t)s * (D + 2)]);
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((t & 31) == 0) red_s[t >> 5] = m;
+    if ((t & 31) == 0) red_s[0][t >> 5] = m;
     __syncthreads();
-    float M = red_s[0];
+    float M = red_s[0][0];
 #pragma unroll
-    for (int i = 1; i < 8; ++i) M = fmaxf(M, red_s[i]);
-    __syncthreads();
+    for (int i = 1; i < 8; ++i) M = fmaxf(M, red_s[0][i]);
     float l = 0.f;
-    for (int s = t; s < nsplit; s += 256) {
+    for (int s = t; s < cnt; s += 256) {
         const float ms = p[(size_t)s * (D + 2)];
         const float wg = ms == -INFINITY ? 0.f : exp2f(ms - M);
         wgt_s[s] = wg;
@@ -269,35 +304,55 @@ decode_merge_kernel(const float* __restrict__ part, int nsplit, int D, int Hq, _
     }
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-    if ((t & 31) == 0) red_s[t >> 5] = l;
+    if ((t & 31) == 0) red_s[1][t >> 5] = l;
+    __syncthreads();
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j) {
+        const int s = row + j * ROWS;
+        const float wg = s < cnt ? wgt_s[s] : 0.f;
+        acc.x = fmaf(v[j].x, wg, acc.x);
+        acc.y = fmaf(v[j].y, wg, acc.y);
+    }
+#pragma unroll 4
+    for (int s = row + AHEAD * ROWS; s < cnt; s += ROWS) {
+        const float2 x = *reinterpret_cast<const float2*>(p + (size_t)s * (D + 2) + 2 + 2 * col);
+        const float wg = wgt_s[s];
+        acc.x = fmaf(x.x, wg, acc.x);
+        acc.y = fmaf(x.y, wg, acc.y);
+    }
+    acc_s[row][col] = acc;
     __syncthreads();
     float L = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) L += red_s[i];
-    for (int d = t; d < D; d += 256) {
-        float acc = 0.f;
-#pragma unroll 8
-        for (int s = 0; s < nsplit; ++s) acc = fmaf(p[(size_t)s * (D + 2) + 2 + d], wgt_s[s], acc);
-        o[(size_t)(hq / Hq) * o_sb + (size_t)(hq % Hq) * o_sh + d] = __float2bfloat16(acc / L);
+    for (int i = 0; i < 8; ++i) L += red_s[1][i];
+    if (row == 0) {
+#pragma unroll
+        for (int r = 1; r < ROWS; ++r) { acc.x += acc_s[r][col].x; acc.y += acc_s[r][col].y; }
+        __nv_bfloat16* dst = o + (size_t)(hq / Hq) * o_sb + (size_t)(hq % Hq) * o_sh + 2 * col;
+        dst[0] = __float2bfloat16(acc.x / L);
+        dst[1] = __float2bfloat16(acc.y / L);
     }
     if (t == 0) lse[hq] = (M + log2f(L)) * DEC_LN2;
 }
 
 static int decode_warps(int D) { return D == 256 ? 2 : 4; }
 
-static int decode_splits(const focus_shape* s) {
-    const int groups = cdiv(s->n, DEC_GK);
-    const int heads = s->batch * s->Hkv;
-    int want = cdiv(2 * 148, heads);                 // about two CTAs per SM in total
-    const int max_useful = cdiv(groups, 4 * decode_warps(s->D));     // at least four steps per warp
-    if (want > max_useful) want = max_useful;
-    if (want < 1) want = 1;
-    if (want > 512) want = 512;
-    return want;
+static DecPlan decode_plan(const focus_shape* s) {
+    DecPlan p;
+    p.groups = cdiv(s->n, DEC_GK);
+    p.total = (long long)s->batch * s->Hkv * p.groups;
+    long long ctas = p.total / (4 * decode_warps(s->D));            // at least four steps per warp
+    if (ctas > DEC_CTAS) ctas = DEC_CTAS;
+    if (ctas < 1) ctas = 1;
+    p.per = (p.total + ctas - 1) / ctas;
+    p.ctas = (int)((p.total + p.per - 1) / p.per);
+    p.slots = (int)((p.groups + p.per - 1) / p.per) + 1;
+    return p;
 }
 
 size_t decode_workspace_bytes(const focus_shape* s) {
-    return (size_t)s->batch * s->Hq * decode_splits(s) * (s->D + 2) * sizeof(float);
+    return (size_t)s->batch * s->Hq * decode_plan(s).slots * (s->D + 2) * sizeof(float);
 }
 
 template <int D>
@@ -305,21 +360,18 @@ static int launch_decode_d(const focus_shape* s, const focus_tensor& q, const fo
                            const uint32_t* mq_new, const uint32_t* mk, const focus_tensor& o, float* lse, float* part,
                            float scale, cudaStream_t st) {
     using C = DecCfg<D>;
-    const int nsplit = decode_splits(s);
-    const int groups = cdiv(s->n, DEC_GK);
-    const int gps = cdiv(groups, nsplit);
+    const DecPlan plan = decode_plan(s);
     auto kern = decode_partial_kernel<D>;
     int rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM),
                         "cudaFuncSetAttribute(decode)");
     if (rc) return rc;
-    kern<<<dim3(nsplit, s->batch * s->Hkv), C::WARPS * 32, C::SMEM, st>>>(
+    rc = check_cuda(launch_dependent(kern, dim3(plan.ctas), dim3(C::WARPS * 32), C::SMEM, st,
         reinterpret_cast<const __nv_bfloat16*>(q.ptr), q.stride_b, q.stride_h, reinterpret_cast<const __nv_bfloat16*>(k.ptr),
         k.stride_b, k.stride_h, k.stride_n, reinterpret_cast<const __nv_bfloat16*>(v.ptr), v.stride_b, v.stride_h, v.stride_n,
-        mq_new, mk, s->Hq, s->Hkv, s->Hq / s->Hkv, s->n, s->window, scale, s->softcap, nsplit, gps, part);
-    if ((rc = check_cuda(cudaGetLastError(), "decode kernel launch"))) return rc;
-    decode_merge_kernel<<<s->batch * s->Hq, 256, 0, st>>>(part, nsplit, D, s->Hq, reinterpret_cast<__nv_bfloat16*>(o.ptr),
-                                                          o.stride_b, o.stride_h, lse);
-    return check_cuda(cudaGetLastError(), "decode merge kernel launch");
+        mq_new, mk, s->Hq, s->Hkv, s->Hq / s->Hkv, s->n, s->window, scale, s->softcap, plan, part), "decode kernel launch");
+    if (rc) return rc;
+    return check_cuda(launch_dependent(decode_merge_kernel<D>, dim3(s->batch * s->Hq), dim3(256), 0, st, part, plan, s->Hq, s->Hkv,
+                                       reinterpret_cast<__nv_bfloat16*>(o.ptr), o.stride_b, o.stride_h, lse), "decode merge kernel launch");
 }
 
 int launch_decode(const focus_shape* s, const focus_tensor& q, const focus_tensor& k, const focus_tensor& v,

@@ -77,3 +77,30 @@ def test_decode_argument_checks():
     with pytest.raises(fb.FocusError) as e:        # workspace too small
         fb.focus_decode_step(shape, Q[:4, -1].contiguous(), K, V, m[:4, 0].contiguous(), m[:2], o[:4], lse[:4], ws[:16])
     assert e.value.status == -3
+
+
+@pytest.mark.parametrize("D,batch,Hq,Hkv,n", [(128, 40, 8, 8, 300), (64, 5, 4, 2, 1), (128, 8, 16, 4, 2049), (128, 1, 8, 1, 70000), (256, 150, 4, 4, 33),
+                                              (256, 3, 8, 2, 5001), (64, 2, 16, 2, 40000)])
+def test_decode_ranges_across_kv_heads(D, batch, Hq, Hkv, n):
+    """the list of steps cut into equal ranges: ranges that cover several KV heads, end inside one, hold less than a head"""
+    g = torch.Generator(device="cuda"); g.manual_seed(n + D)
+    K, topk, w = 4, 1, 20
+    q = torch.randn((batch, Hq, D), generator=g, device="cuda").to(torch.bfloat16)
+    k, v = (torch.randn((batch, Hkv, n, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    mq = (1 << torch.randint(0, K, (batch * Hq,), generator=g, device="cuda")).to(torch.int32)
+    mk = (1 << torch.randint(0, K, (batch * Hkv, n), generator=g, device="cuda")).to(torch.int32)
+    shape = fb.make_shape(Hq, Hkv, n, D, K, topk, w, batch=batch)
+    o = torch.full((batch, Hq, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((batch * Hq,), float("nan"), device="cuda")
+    ws = torch.empty(fb.focus_decode_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    fb.focus_decode_step(shape, q, k, v, mq, mk, o, lse, ws)
+    G = Hq // Hkv
+    kv = lambda x: x.double().repeat_interleave(G, 1)
+    s = (kv(k) @ q.double()[..., None])[..., 0] / D ** 0.5                        # [batch, Hq, n]
+    keep = (mk.view(batch, Hkv, n).repeat_interleave(G, 1) & mq.view(batch, Hq, 1)) != 0
+    keep |= torch.arange(n, device="cuda") >= n - 1 - w
+    s.masked_fill_(~keep, float("-inf"))
+    ref = (torch.softmax(s, -1)[:, :, None] @ kv(v))[:, :, 0]
+    err = (o.double() - ref).abs()
+    assert err.max() <= O_MAX_ABS and err.mean() <= O_MEAN_ABS
+    assert (lse.view(batch, Hq).double() - torch.logsumexp(s, -1)).abs().max() <= LSE_MAX_ABS
