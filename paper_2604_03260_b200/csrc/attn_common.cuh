@@ -20,9 +20,8 @@ constexpr float RESCALE_THRESHOLD = 8.0f;   // log2 units: the stale maximum may
 constexpr int EX2_POLY_PER_8 = 0;
 // Registers per thread after the warps have split into roles (setmaxnreg): the load/MMA warpgroup
 // gives most of its share to the softmax warpgroups.
-constexpr int REGS_CONTROL = 96;
-constexpr int REGS_SOFTMAX_2WG = 200;        // 128*96 + 256*200 = 63488 <= 65536
-constexpr int REGS_SOFTMAX_1WG = 232;        // 128*96 + 128*232 (unused while a single query tile is split over two warpgroups)
+constexpr int REGS_CONTROL = 88;
+constexpr int REGS_SOFTMAX_2WG = 208;        // 128*88 + 256*208 = 64512 = the 384 * 168 of the launch
 
 __device__ __forceinline__ float max3(float a, float b, float c) {
     float d;
@@ -53,10 +52,10 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
 }
 
 struct AttnParams {
-    int B, Hq, Hkv, G, n, w, K;
+    int B, Hq, Hkv, G, n, K;
+    int w;                   // window, at most n: positions and differences of positions stay within 32 bits
     int nqb;                 // items per head: 256-row query blocks (128-row tiles when D = 256)
     int nqt, nkt, nkw;
-    int dense;
     float scale, softcap;
     const uint32_t* mq;
     const uint32_t* gbits;
@@ -68,8 +67,8 @@ struct AttnParams {
     float* lse;
     int32_t* status;
     long long nitems;
+    int by_length;           // token order: items longest first over all heads (else KV head by KV head)
     // class-sorted layout: Q/K/V are the sorted copies, tiles are tiles of the sorted order
-    int sorted;
     int nqp, nkp, nqblk;
     int ipb;                 // items per block of 256 sorted queries (1, or 2 when an item is one query tile)
     const int32_t* perm_q;
@@ -94,75 +93,80 @@ struct AttnParams {
     long long stall_at;      // diagnostic: index of a K/V ring stage the producer leaves unfilled (-1 = none)
 };
 
+// What decides which tiles are visited and which pairs kept: every causal pair; masks of tokens in their own order (live far
+// tiles and the window, or the window alone: `local_only`); the class-sorted copies.  A template parameter of the kernel: the
+// softmax warps hold 128 scores a thread, and the state of a walk they do not take would go to local memory, every tile.
+enum : int { WALK_DENSE = 0, WALK_TOKEN = 1, WALK_SORTED = 2 };
+
 // Enumerates the key tiles a 256-row query block visits, in increasing order.  Every role of the
 // CTA runs the same walk over the same data, which keeps them in step without communication.
-struct TileWalk {
+template <int WALK> struct TileWalk;
+
+template <> struct TileWalk<WALK_DENSE> {
+    int b, b_last;
+    static constexpr int jk = 0;
+    // a0 = first 128-row query tile of the item, nq = number of query tiles of the item (1 or 2)
+    __device__ __forceinline__ void init(const AttnParams& p, int, int a0, int nq) {
+        b = 0;
+        b_last = (min(p.n, (a0 + nq) * 128) - 1) >> 7;
+    }
+    // next key tile, or -1
+    __device__ __forceinline__ int next() { return b <= b_last ? b++ : -1; }
+};
+
+template <> struct TileWalk<WALK_TOKEN> {
     const uint32_t* l0;
     int nl, nkw;                // live rows (query tiles) to OR, and their stride in words
-    int f0, b_last, b, wd;
+    int f0, b_last, b, wd;      // wd = current word of the live bitmap, past its end when the far tiles are through
     uint32_t bits;
-    bool far_phase;
-    // class-sorted layout: the ranges of sorted key tiles, key class by key class
-    const int32_t* qr;
-    int nck, jk, rend;
-    bool sorted;
-
-    // a0 = first 128-row query tile of the item, nq = number of query tiles of the item (1 or 2)
+    static constexpr int jk = 0;
     __device__ __forceinline__ void init(const AttnParams& p, int hq, int a0, int nq) {
-        sorted = p.sorted != 0;
-        if (sorted) {
-            const int hk = (hq / p.Hq) * p.Hkv + (hq % p.Hq) / p.G;
-            qr = p.qrange + ((size_t)hq * p.nqblk + (a0 >> 1)) * FOCUS_MAX_CLASSES * 2;
-            nck = __ldg(p.ncls_k + hk);
-            jk = -1;
-            b = rend = 0;
-            return;
-        }
-        const long long last_row = min((long long)p.n, (long long)(a0 + nq) * 128) - 1;
-        b_last = (int)(last_row / 128);
-        f0 = 0;
-        l0 = nullptr;
-        nl = 0;
+        b_last = (min(p.n, (a0 + nq) * 128) - 1) >> 7;
+        const int d = a0 * 128 - p.w;
+        f0 = d > 0 ? d >> 7 : 0;                          // tiles before f0 are far for every query tile of the item
         nkw = p.nkw;
-        if (!p.dense) {
-            const long long d = (long long)a0 * 128 - p.w;
-            f0 = d > 0 ? (int)(d / 128) : 0;              // tiles before f0 are far for every query tile of the item
-            l0 = p.live + ((size_t)hq * p.nqt + a0) * p.nkw;
-            nl = min(nq, p.nqt - a0);
-        }
-        far_phase = f0 > 0 && !p.local_only;
-        wd = -1;
+        l0 = p.live + ((size_t)hq * p.nqt + a0) * nkw;
+        nl = min(nq, p.nqt - a0);
+        wd = p.local_only ? nkw : -1;
         bits = 0;
         b = f0;
     }
-    // next key tile, or -1; in the sorted layout `jk` is then the class index of that tile
     __device__ __forceinline__ int next() {
-        if (sorted) {
-            while (b >= rend) {
-                if (++jk >= nck) return -1;
-                b = __ldg(qr + 2 * jk);
-                rend = __ldg(qr + 2 * jk + 1);
+        while (wd * 32 < f0) {
+            if (bits) {
+                const int c = __ffs(bits) - 1;
+                bits &= bits - 1;
+                return wd * 32 + c;
             }
-            return b++;
+            ++wd;
+            if (wd * 32 >= f0) break;
+            uint32_t x = 0;
+            for (int r = 0; r < nl; ++r) x |= __ldg(l0 + (size_t)r * nkw + wd);
+            const int rem = f0 - wd * 32;
+            bits = rem < 32 ? x & ((1u << rem) - 1u) : x;
         }
-        if (far_phase) {
-            for (;;) {
-                if (bits) {
-                    const int c = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    return wd * 32 + c;
-                }
-                ++wd;
-                if (wd * 32 >= f0) { far_phase = false; break; }
-                uint32_t x = 0;
-                for (int r = 0; r < nl; ++r) x |= __ldg(l0 + (size_t)r * nkw + wd);
-                const int rem = f0 - wd * 32;
-                if (rem < 32) x &= (1u << rem) - 1u;
-                bits = x;
-            }
+        return b <= b_last ? b++ : -1;
+    }
+};
+
+template <> struct TileWalk<WALK_SORTED> {
+    const int32_t* qr;          // the ranges of sorted key tiles, key class by key class
+    int nck, jk, b, rend;       // jk = class of the tile that next() returned
+    __device__ __forceinline__ void init(const AttnParams& p, int hq, int a0, int) {
+        const int hk = (hq / p.Hq) * p.Hkv + (hq % p.Hq) / p.G;
+        qr = p.qrange + ((size_t)hq * p.nqblk + (a0 >> 1)) * FOCUS_MAX_CLASSES * 2;
+        nck = __ldg(p.ncls_k + hk);
+        jk = -1;
+        b = rend = 0;
+    }
+    __device__ __forceinline__ int next() {
+        while (b >= rend) {
+            if (++jk >= nck) return -1;
+            const int2 r = __ldg(reinterpret_cast<const int2*>(qr) + jk);
+            b = r.x;
+            rend = r.y;
         }
-        if (b <= b_last) return b++;
-        return -1;
+        return b++;
     }
 };
 
@@ -173,14 +177,28 @@ struct TileMask {
     bool masked, all_masked;
 };
 
-__device__ __forceinline__ void build_tile_mask(TileMask& tm, const AttnParams& p, int a, int kb, long long i,
-                                                uint32_t mi, uint32_t aq, int f_x, int hk) {
-    const long long c0 = (long long)kb * 128;
-    const long long r_first = (long long)a * 128, r_last = r_first + 127;
+// every causal pair
+__device__ __forceinline__ void build_tile_mask_dense(TileMask& tm, const AttnParams& p, int a, int kb, int i) {
+    const int c0 = kb * 128;
+    tm.all_masked = kb > a || a * 128 >= p.n;
+    tm.masked = c0 + 127 > a * 128;
+    if (tm.masked && !tm.all_masked) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int nk = i - c0 + 1 - 32 * q;                          // columns < nk are causal
+            tm.kw[q] = nk >= 32 ? 0xffffffffu : (nk <= 0 ? 0u : ((1u << nk) - 1u));
+        }
+    }
+}
+
+__device__ __forceinline__ void build_tile_mask(TileMask& tm, const AttnParams& p, int a, int kb, int i, uint32_t mi, uint32_t aq,
+                                                int f_x, int hk) {
+    const int c0 = kb * 128;
+    const int r_first = a * 128, r_last = r_first + 127;
     tm.all_masked = c0 > r_last || r_first >= p.n;
     const bool need_causal = c0 + 127 > r_first;
     bool need_group = false, need_window = false;
-    if (!p.dense && !tm.all_masked) {
+    if (!tm.all_masked) {
         if (p.local_only) {
             need_group = need_window = true;
         } else if (kb < f_x) {
@@ -209,44 +227,45 @@ __device__ __forceinline__ void build_tile_mask(TileMask& tm, const AttnParams& 
             if (need_group) {
                 keep = sh[q];
                 if (need_window) {
-                    const long long lo = i - p.w - c0 - 32 * q;          // columns >= lo are inside the window
-                    const uint32_t win = lo <= 0 ? 0xffffffffu : (lo >= 32 ? 0u : ~((1u << (int)lo) - 1u));
+                    const int lo = i - p.w - c0 - 32 * q;                // columns >= lo are inside the window
+                    const uint32_t win = lo <= 0 ? 0xffffffffu : (lo >= 32 ? 0u : ~((1u << lo) - 1u));
                     keep = p.local_only ? (win & ~keep) : (keep | win);     // window pass: in the window and not sharing
                 }
             }
             if (need_causal) {
-                const long long nk = i - c0 + 1 - 32 * q;                // columns < nk are causal
-                keep &= nk >= 32 ? 0xffffffffu : (nk <= 0 ? 0u : ((1u << (int)nk) - 1u));
+                const int nk = i - c0 + 1 - 32 * q;                      // columns < nk are causal
+                keep &= nk >= 32 ? 0xffffffffu : (nk <= 0 ? 0u : ((1u << nk) - 1u));
             }
             tm.kw[q] = keep;
         }
     }
 }
 
-// Item order.  Items are laid out KV head by KV head, heaviest query block first inside a head
-// group, so that the CTAs running at the same time stream the K/V of one KV head through L2.  CTA c
-// takes position c of every even round of g items and position g-1-c of every odd round, which
-// cancels the cost gradient inside a round (g workers: CTAs, or CTA pairs).  Returns false past the last item.
-struct Item { int A, bb, h, hq; long long id; };
-__device__ __forceinline__ bool item_of(const AttnParams& p, int round, Item& t, int g, int c) {
-    t.id = (long long)round * g + ((round & 1) ? g - 1 - c : c);
-    if (t.id >= p.nitems) return false;
-    if (p.sorted) {
-        const long long e = t.id / p.ipb;
-        t.hq = __ldg(p.order + 2 * e);
-        t.A = __ldg(p.order + 2 * e + 1) * p.ipb + (int)(t.id % p.ipb);
-        t.bb = t.hq / p.Hq;
-        t.h = t.hq % p.Hq;
-        return true;
+// Item `id` of the list.  The grid has one block per item; blocks start in the order of the list and a running CTA takes
+// over the next one that has not started (cluster launch control), so the list is worked off like a queue and what counts
+// is that the expensive items come first.  Class-sorted: as build_tiles ordered them, KV head by KV head, most key tiles
+// first.  Token order: longest query blocks first, over all heads at once (`by_length`) while K and V of all heads stay in
+// L2, else KV head by KV head, so that the CTAs running at the same time stream the K/V of one head through L2.
+struct Item { int A, bb, h, hq; };
+template <int WALK>
+__device__ __forceinline__ void item_at(const AttnParams& p, int id, Item& t) {
+    if (WALK == WALK_SORTED) {
+        const int2 e = __ldg(reinterpret_cast<const int2*>(p.order) + id / p.ipb);
+        t.hq = e.x;
+        t.A = e.y * p.ipb + id % p.ipb;
+    } else if (p.by_length) {
+        const int heads = p.B * p.Hq;
+        t.A = p.nqb - 1 - id / heads;
+        t.hq = id % heads;
+    } else {
+        const int per_group = p.nqb * p.G;
+        const int grp = id / per_group;                   // batch * Hkv + KV head
+        const int rem = id % per_group;
+        t.A = p.nqb - 1 - rem / p.G;
+        t.hq = (grp / p.Hkv) * p.Hq + (grp % p.Hkv) * p.G + rem % p.G;
     }
-    const int per_group = p.nqb * p.G;
-    const int grp = (int)(t.id / per_group);              // batch * Hkv + KV head
-    const int rem = (int)(t.id % per_group);
-    t.A = p.nqb - 1 - rem / p.G;
-    t.bb = grp / p.Hkv;
-    t.h = (grp % p.Hkv) * p.G + rem % p.G;
-    t.hq = t.bb * p.Hq + t.h;
-    return true;
+    t.bb = t.hq / p.Hq;
+    t.h = t.hq % p.Hq;
 }
 
 // number of entries of the ascending 128-entry array `a` that are <= v (fixed-depth search)
@@ -273,13 +292,13 @@ __device__ __forceinline__ void build_tile_mask_sorted(TileMask& tm, int w, cons
     // (window_ok is the same for the whole grid, so the vote is skipped or taken by every lane alike)
     const bool any_none = !window_ok && __any_sync(0xffffffffu, none);
     const bool need_causal = k_last > wmin;
-    const bool need_window = !share && ((long long)wmax - k_first > w);
+    const bool need_window = !share && wmax - k_first > w;          // (wmax >= -1, k_first >= 0)
     tm.masked = need_causal || need_window || any_none;
     tm.kw[0] = tm.kw[1] = tm.kw[2] = tm.kw[3] = 0xffffffffu;
     if (tm.masked && !tm.all_masked) {
         const int hi = none ? 0 : (need_causal ? (pos < 0 ? 0 : count_le_128(kpos, pos)) : 128);          // columns < hi are causal
-        const long long edge = (long long)pos - w - 1;
-        const int lo = (need_window && pos >= 0 && edge >= 0) ? count_le_128(kpos, (int)edge) : 0;   // columns >= lo are in the window
+        const int edge = pos - w - 1;
+        const int lo = (need_window && pos >= 0 && edge >= 0) ? count_le_128(kpos, edge) : 0;   // columns >= lo are in the window
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int h = hi - 32 * q, l = lo - 32 * q;

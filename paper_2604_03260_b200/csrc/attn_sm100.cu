@@ -26,8 +26,10 @@
 //                   range of sorted key tiles listed for the query block; a row's kept columns of a
 //                   tile are a contiguous range found from the tile's ascending positions; O and lse
 //                   go straight to the rows' original positions
-// Items are laid out KV head by KV head (class-sorted: most key tiles first inside a group) and
-// dealt to the CTAs in alternating direction round by round.
+// The items are a queue, expensive ones first: the grid has one block per item, and a CTA that is through with its item
+// takes over the next block that has not started (cluster launch control; the TMA thread asks, every role reads the
+// answer from shared memory).  Dealing the items out beforehand, a fixed number per CTA, left the fullest CTA 18 % (one
+// sequence of 8192), 27 % (three of 3001) and 4.5 % (131072) above the average.
 #include "attn_common.cuh"
 #include "tma_host.cuh"
 
@@ -70,9 +72,12 @@ struct SharedCtl {
     uint64_t xchg[4];                 // split rows, per 32-row quadrant: both column halves have published a per-row value
     uint64_t gbar[2];                 // soft gate, per softmax warpgroup: the key assignments of the tile are in shared memory
     uint64_t kv_full[8], kv_empty[8];
+    uint64_t next_full[2], next_empty[2];         // the answers below: arrived, read by the MMA warp and every softmax warp
     unsigned long long limit_ns;      // how long a wait may last before the role gives up
     uint32_t tmem_base;
     int abort_flag;
+    uint32_t asked;                   // how many answers the TMA thread has asked for
+    uint4 next[2];                    // which item comes next, by the parity of its ordinal
 };
 
 // bounded wait that also gives up when another role of the CTA has already given up
@@ -98,14 +103,39 @@ __device__ __forceinline__ void report_timeout(const AttnParams& p, SharedCtl* c
     }
 }
 
-template <int D, bool SOFTCAP, int GATE>
+// The CTA's item number `ord` (0, 1, ...): the block it was launched as, then what the answers say; false after the last.
+// Called by every thread of a role's warp (`reader`: the warp reports that it has read), or by the TMA thread.
+template <int WALK>
+__device__ __forceinline__ bool next_item(const AttnParams& p, SharedCtl* ctl, uint32_t ord, bool reader, Item& t, bool& ok) {
+    uint32_t block = blockIdx.x;
+    if (ord > 0) {
+        const uint32_t slot = (ord - 1) & 1, use = (ord - 1) >> 1;
+        if (!ctl_wait(&ctl->next_full[slot], use & 1, ctl)) {
+            *(volatile int*)&ctl->abort_flag = 1;
+            if (p.status && atomicCAS(p.status, 0, 1) == 0) { p.status[1] = 50; p.status[2] = (int)ord; p.status[3] = (int)blockIdx.x; }
+            ok = false;
+            return false;
+        }
+        const bool more = clc_answer(smem_u32(&ctl->next[slot]), block);
+        if (reader) {
+            fence_proxy_async_smem();                   // the answer is read before the next one is written there
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) mbar_arrive(smem_u32(&ctl->next_empty[slot]));
+        }
+        if (!more) return false;
+    }
+    item_at<WALK>(p, (int)block, t);
+    return true;
+}
+
+template <int D, bool SOFTCAP, int GATE, int WALK>
 __global__ void __launch_bounds__(AttnCfg<D, GATE>::THREADS, 1)
 focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                   const __grid_constant__ CUtensorMap tm_v, const AttnParams p) {
     using C = AttnCfg<D, GATE>;
     constexpr int NQ = C::NQ;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) SharedCtl ctl;
+    __shared__ __align__(16) SharedCtl ctl;
     // split rows: [parity][column half][row] row maxima, at the end row sums (the other instantiations have no room to spare)
     // (bf16: a rounded row maximum serves as well as the exact one as long as both threads use the same value)
     __shared__ __nv_bfloat16 xval_s[C::NSPLIT == 2 ? 2 * 2 * 128 : 1];
@@ -116,7 +146,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     unsigned char* const gate_sm = smem_raw + (base - smem_u32(smem_raw)) + NQ * C::TILE_BYTES + C::NSTAGE * C::STAGE_BYTES;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    if (p.sorted && __ldg(p.counters + 4) != 0ull) {      // more mask values than the sorted layout holds: refuse
+    if (WALK == WALK_SORTED && __ldg(p.counters + 4) != 0ull) {      // more mask values than the sorted layout holds: refuse
         if (threadIdx.x == 0 && p.status && atomicCAS(p.status, 0, 2) == 0) {
             p.status[1] = 1; p.status[2] = 0; p.status[3] = (int)blockIdx.x;
         }
@@ -137,7 +167,12 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             mbar_init(smem_u32(&ctl.kv_full[s]), 1);
             mbar_init(smem_u32(&ctl.kv_empty[s]), 1);
         }
+        for (int x = 0; x < 2; ++x) {
+            mbar_init(smem_u32(&ctl.next_full[x]), 1);
+            mbar_init(smem_u32(&ctl.next_empty[x]), C::THREADS / 32 - 3);       // the MMA warp and the softmax warps
+        }
         ctl.abort_flag = 0;
+        ctl.asked = 0;
         ctl.limit_ns = p.wait_limit_ns;
         fence_mbar_init();
     }
@@ -158,19 +193,27 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             long long nload = 0;
             int it = 0;                     // items processed (items without key tiles are skipped by every role)
             bool ok = true;
+            // ask for the item after number `ord`, when all of that one's loads are on their way
+            auto ask_next = [&](uint32_t ord) {
+                const uint32_t slot = ord & 1, use = ord >> 1;
+                if (use > 0 && !ctl_wait(&ctl.next_empty[slot], (use - 1) & 1, &ctl)) { report_timeout(p, &ctl, 51, (int)ord); ok = false; return; }
+                mbar_arrive_expect_tx(smem_u32(&ctl.next_full[slot]), 16);
+                clc_try_cancel(smem_u32(&ctl.next[slot]), smem_u32(&ctl.next_full[slot]));
+                ctl.asked = ord + 1;
+            };
             Item t;
-            for (int round = 0; ok && item_of(p, round, t, (int)gridDim.x, (int)blockIdx.x); ++round) {
+            for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, false, t, ok); ++ord) {
                 const int A = t.A, hq = t.hq, b = t.bb, h = t.h, hk = h / p.G;
-                const long long item = t.id;
-                TileWalk walk;
+                const int item = t.A;
+                TileWalk<WALK> walk;
                 walk.init(p, hq, A * NQ, NQ);
                 int kb = walk.next();
-                if (kb < 0) continue;
-                if (it > 0 && !ctl_wait(&ctl.q_empty, (it - 1) & 1, &ctl)) { report_timeout(p, &ctl, 10, (int)item); break; }
+                if (kb < 0) { ask_next(ord); continue; }
+                if (it > 0 && !ctl_wait(&ctl.q_empty, (it - 1) & 1, &ctl)) { report_timeout(p, &ctl, 10, item); break; }
                 mbar_arrive_expect_tx(smem_u32(&ctl.q_full), NQ * C::TILE_BYTES);
                 // in the sorted layout the copies are indexed [head of the batch][sorted slot]
-                const int qh = p.sorted ? hq : h, qb = p.sorted ? 0 : b;
-                const int kh = p.sorted ? b * p.Hkv + hk : hk;
+                const int qh = WALK == WALK_SORTED ? hq : h, qb = WALK == WALK_SORTED ? 0 : b;
+                const int kh = WALK == WALK_SORTED ? b * p.Hkv + hk : hk;
                 for (int x = 0; x < NQ; ++x)
                     for (int c = 0; c < C::SUBT; ++c)
                         tma_load_4d(sq + x * C::TILE_BYTES + c * C::SUB_BYTES, &tm_q, smem_u32(&ctl.q_full), c * 64,
@@ -182,7 +225,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         const int slot = (int)(nload % C::NSTAGE);
                         const long long use = nload / C::NSTAGE;
                         if (use > 0 && !ctl_wait(&ctl.kv_empty[slot], (uint32_t)((use - 1) & 1), &ctl)) {
-                            report_timeout(p, &ctl, 11, (int)item);
+                            report_timeout(p, &ctl, 11, item);
                             ok = false;
                             return;
                         }
@@ -217,6 +260,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         if (ok) load_tile(true, kb);
                     }
                 }
+                if (ok) ask_next(ord);
                 ++it;
             }
         }
@@ -320,23 +364,23 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 return true;
             };
             Item t;
-            for (int round = 0; ok && item_of(p, round, t, (int)gridDim.x, (int)blockIdx.x); ++round) {
+            for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, true, t, ok); ++ord) {
                 const int A = t.A, hq = t.hq;
-                const long long item = t.id;
-                TileWalk walk;
+                const int item = t.A;
+                TileWalk<WALK> walk;
                 walk.init(p, hq, A * NQ, NQ);
                 int cur = walk.next();
                 if (cur < 0) continue;
-                if (!ctl_wait(&ctl.q_full, it & 1, &ctl)) { report_timeout(p, &ctl, 20, (int)item); break; }
+                if (!ctl_wait(&ctl.q_full, it & 1, &ctl)) { report_timeout(p, &ctl, 20, item); break; }
                 if constexpr (NQ == 2) {
                     int slot;
-                    if (!wait_kv(slot, 21, (int)item)) break;
+                    if (!wait_kv(slot, 21, item)) break;
                     tc_fence_after();
                     issue_s(0, 0, slot); commit(&ctl.s_full[0]);
                     issue_s(1, 1, slot); commit(&ctl.s_full[1]);
                     release_tile(slot);
                 } else {
-                    if (!s_tile(gs & 1, 21, (int)item)) break;
+                    if (!s_tile(gs & 1, 21, item)) break;
                     ++gs;
                 }
                 bool first = true;
@@ -345,22 +389,22 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     int vslot = 0, kslot = 0;
                     if constexpr (NQ == 2) {
                         // the ring carries V(current) ahead of K(next) here (see the producer)
-                        if (!wait_kv(vslot, 22, (int)item)) { ok = false; break; }
+                        if (!wait_kv(vslot, 22, item)) { ok = false; break; }
                         if (nxt >= 0) {
-                            if (!wait_kv(kslot, 23, (int)item)) { ok = false; break; }
+                            if (!wait_kv(kslot, 23, item)) { ok = false; break; }
                         }
                     }
                     if (nxt < 0) commit(&ctl.q_empty);     // every S of this item has been issued
                     if constexpr (NQ == 2) {
                         // query tile 0
-                        if (!ctl_wait(&ctl.p_full[0], np[0] & 1, &ctl)) { report_timeout(p, &ctl, 24, (int)item); ok = false; break; }
+                        if (!ctl_wait(&ctl.p_full[0], np[0] & 1, &ctl)) { report_timeout(p, &ctl, 24, item); ok = false; break; }
                         ++np[0];
                         tc_fence_after();
                         issue_o(0, 0, vslot, first);
                         if (nxt >= 0) { issue_s(0, 0, kslot); commit(&ctl.s_full[0]); }
                         else commit(&ctl.o_full[0]);
                         // query tile 1
-                        if (!ctl_wait(&ctl.p_full[1], np[1] & 1, &ctl)) { report_timeout(p, &ctl, 25, (int)item); ok = false; break; }
+                        if (!ctl_wait(&ctl.p_full[1], np[1] & 1, &ctl)) { report_timeout(p, &ctl, 25, item); ok = false; break; }
                         ++np[1];
                         tc_fence_after();
                         issue_o(1, 1, vslot, first);
@@ -374,14 +418,14 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     } else {
                         // S of the next tile goes to the other buffer before this tile's PV is issued
                         if (nxt >= 0) {
-                            if (!s_tile(gs & 1, 23, (int)item)) { ok = false; break; }
+                            if (!s_tile(gs & 1, 23, item)) { ok = false; break; }
                             ++gs;
                         }
                         const int buf = gp & 1;
-                        if (!ctl_wait(&ctl.p_full[buf], (gp >> 1) & 1, &ctl)) { report_timeout(p, &ctl, 26, (int)item); ok = false; break; }
+                        if (!ctl_wait(&ctl.p_full[buf], (gp >> 1) & 1, &ctl)) { report_timeout(p, &ctl, 26, item); ok = false; break; }
                         ++gp;
                         tc_fence_after();
-                        if (!o_tile(buf, first, 22, (int)item)) { ok = false; break; }
+                        if (!o_tile(buf, first, 22, item)) { ok = false; break; }
                         commit(&ctl.pv_done);
                         if (nxt < 0) commit(&ctl.o_full[0]);
                     }
@@ -411,28 +455,28 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         int it = 0;
         bool ok = true;
         Item t;
-        for (int round = 0; ok && item_of(p, round, t, (int)gridDim.x, (int)blockIdx.x); ++round) {
+        for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, true, t, ok); ++ord) {
             const int A = t.A, hq = t.hq, bb = t.bb, h = t.h;
-            const long long item = t.id;
+            const int item = t.A;
             const int hk = bb * p.Hkv + h / p.G;
             const int a = A * NQ + x;
-            TileWalk walk;
+            TileWalk<WALK> walk;
             walk.init(p, hq, A * NQ, NQ);
             int kb = walk.next();
             if (kb < 0) continue;
             // the row's position in the sequence: its index, or in the sorted layout the position its slot holds
-            long long i = (long long)a * 128 + row_in_tile;
+            int i = a * 128 + row_in_tile;
             int wmin = 0, wmax = 0;
-            if (p.sorted) {
+            if constexpr (WALK == WALK_SORTED) {
                 i = __ldg(p.perm_q + (size_t)hq * p.nqp + i);                       // -1 in the padding of a segment
-                wmin = __reduce_min_sync(0xffffffffu, i < 0 ? 0x7fffffff : (int)i);
-                wmax = __reduce_max_sync(0xffffffffu, (int)i);
+                wmin = __reduce_min_sync(0xffffffffu, i < 0 ? 0x7fffffff : i);
+                wmax = __reduce_max_sync(0xffffffffu, i);
             }
             const bool valid = i >= 0 && i < p.n;
-            const uint32_t mi = (valid && !p.dense) ? __ldg(p.mq + (size_t)hq * p.n + i) : 0u;
-            const uint32_t aq = (!p.dense && !p.sorted && a < p.nqt) ? __ldg(p.andq + (size_t)hq * p.nqt + a) : 0u;
-            const long long dfar = (long long)a * 128 - p.w;
-            const int f_x = (!p.dense && dfar > 0) ? (int)(dfar / 128) : 0;   // tiles b < f_x are far for this query tile
+            const uint32_t mi = (valid && WALK != WALK_DENSE) ? __ldg(p.mq + (size_t)hq * p.n + i) : 0u;
+            const uint32_t aq = (WALK == WALK_TOKEN && a < p.nqt) ? __ldg(p.andq + (size_t)hq * p.nqt + a) : 0u;
+            const int dfar = a * 128 - p.w;
+            const int f_x = (WALK == WALK_TOKEN && dfar > 0) ? dfar >> 7 : 0;   // tiles b < f_x are far for this query tile
             float m_used = -INFINITY, l = 0.f;
             bool first = true;
             // soft gate: this row's assignment times lambda / 2 (sigmoid(x) = 1/2 + 1/2 tanh(x / 2))
@@ -455,12 +499,14 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
             for (; kb >= 0; kb = walk.next()) {
                 TileMask tm;
-                if (p.sorted) {
+                if constexpr (WALK == WALK_SORTED) {
                     const bool share = (mi & __ldg(p.cls_k + (size_t)hk * FOCUS_MAX_CLASSES + walk.jk)) != 0u;
                     build_tile_mask_sorted(tm, p.w, p.perm_k + (size_t)hk * p.nkp + (size_t)kb * 128, share,
-                                           valid ? (int)i : -1, wmin, wmax, !p.share_only);
+                                           valid ? i : -1, wmin, wmax, !p.share_only);
                     if (p.gbits_s && !tm.all_masked)
                         exclude_lower_groups(tm, p.gbits_s + ((size_t)hk * (p.nkp / 128) + kb) * p.K * 4, mi & ((1u << walk.jk) - 1u), p.K);
+                } else if constexpr (WALK == WALK_DENSE) {
+                    build_tile_mask_dense(tm, p, a, kb, i);
                 } else {
                     build_tile_mask(tm, p, a, kb, i, mi, aq, f_x, hk);
                 }
@@ -469,16 +515,16 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 // thread then reads them with broadcast 16-byte loads, column by column.
                 const unsigned char* gb = nullptr;
                 bool gated = false;
-                const long long gj0 = (long long)kb * 128 + half * NC;    // first column of this thread's part of the tile
-                const long long ifar = i - p.w;                           // columns j < ifar are distant for this row
+                const int gj0 = kb * 128 + half * NC;    // first column of this thread's part of the tile
+                const int ifar = i - p.w;                           // columns j < ifar are distant for this row
                 if constexpr (GATE != 0) {
                     // the same decision in all four warps of the warpgroup: does the tile hold a distant pair at all
-                    const bool tile_gated = !tm.all_masked && ((long long)a * 128 + 127 - p.w > gj0);
+                    const bool tile_gated = !tm.all_masked && (a * 128 + 127 - p.w > gj0);
                     if (tile_gated) {
                         unsigned char* gw = gate_sm + (wg * 2 + (ng & 1)) * C::GATE_BUF_BYTES;
                         const int col = (warp & 3) * 32 + lane;
                         if (col < NC) {
-                            const long long j = gj0 + col;
+                            const int j = gj0 + col;
                             const float4* gp = reinterpret_cast<const float4*>(p.gate_g + ((size_t)bb * p.n + (size_t)(j < p.n ? j : p.n - 1)) * p.gate_ld);
 #pragma unroll
                             for (int f = 0; f < GQ; ++f)
@@ -486,7 +532,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctl.gbar[wg]));
-                        if (!ctl_wait(&ctl.gbar[wg], ng & 1, &ctl)) { report_timeout(p, &ctl, 37, (int)item); ok = false; break; }
+                        if (!ctl_wait(&ctl.gbar[wg], ng & 1, &ctl)) { report_timeout(p, &ctl, 37, item); ok = false; break; }
                         ++ng;
                         gb = gw;
                         gated = __any_sync(0xffffffffu, valid && ifar > gj0);
@@ -495,7 +541,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 // ---- wait for S
                 const int buf = NQ == 2 ? x : (int)(ns & 1);
                 const uint32_t par = NQ == 2 ? (ns & 1) : ((ns >> 1) & 1);
-                if (!ctl_wait(&ctl.s_full[buf], par, &ctl)) { report_timeout(p, &ctl, 30 + x, (int)item); ok = false; break; }
+                if (!ctl_wait(&ctl.s_full[buf], par, &ctl)) { report_timeout(p, &ctl, 30 + x, item); ok = false; break; }
                 // this thread's NC S columns; its packed P columns overwrite the first half of them
                 const uint32_t t_s = tmem + lane_base + (buf ? C::COL_S1 : C::COL_S0) + half * NC;
                 tc_fence_after();
@@ -512,7 +558,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             tmem_wait_ld();
                             if (gated) {
                                 const bool wide = p.gate_ld == 8;
-                                const int nfar = (int)(ifar - gj0 < 0 ? 0 : (ifar - gj0 > NC ? NC : ifar - gj0));   // columns < nfar are distant
+                                const int nfar = ifar - gj0 < 0 ? 0 : (ifar - gj0 > NC ? NC : ifar - gj0);   // columns < nfar are distant
 #pragma unroll
                                 for (int e0 = 0; e0 < 32; e0 += 4) {        // four columns in flight
                                     float arg[4];
@@ -592,7 +638,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         xval(par, half, row_in_tile) = mine;
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctl.xchg[warp & 3]));
-                        if (!ctl_wait(&ctl.xchg[warp & 3], (uint32_t)par, &ctl)) { report_timeout(p, &ctl, 36, (int)item); ok = false; }
+                        if (!ctl_wait(&ctl.xchg[warp & 3], (uint32_t)par, &ctl)) { report_timeout(p, &ctl, 36, item); ok = false; }
                         mraw = fmaxf(__bfloat162float(mine), __bfloat162float(xval(par, half ^ 1, row_in_tile)));
                         ++nx;
                     }
@@ -612,7 +658,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         // query tiles its commit precedes s_full; with double-buffered S it has its own barrier.
                         bool pv_ok = true;
                         if constexpr (NQ == 1) pv_ok = ctl_wait(&ctl.pv_done, (ns - 1) & 1, &ctl);
-                        if (!pv_ok) { report_timeout(p, &ctl, 35, (int)item); ok = false; }
+                        if (!pv_ok) { report_timeout(p, &ctl, 35, item); ok = false; }
                         tc_fence_after();
 #pragma unroll 1
                         for (int c = 0; c < D / 16 / NSPLIT; ++c) {      // this thread's part of the O row
@@ -676,10 +722,10 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     other += __bfloat162float(xval(par, half ^ 1, row_in_tile));
                     ++nx;
                 }
-                if (!xok) { report_timeout(p, &ctl, 38, (int)item); break; }
+                if (!xok) { report_timeout(p, &ctl, 38, item); break; }
                 l += other;
             }
-            if (!ctl_wait(&ctl.o_full[x], it & 1, &ctl)) { report_timeout(p, &ctl, 40 + x, (int)item); break; }
+            if (!ctl_wait(&ctl.o_full[x], it & 1, &ctl)) { report_timeout(p, &ctl, 40 + x, item); break; }
             tc_fence_after();
             const float inv_l = l > 0.f ? 1.f / l : 0.f;        // a row without any pair (possible in a partial pass): zeros, lse = -inf
             __nv_bfloat16* orow = p.o + (size_t)bb * p.o_sb + (size_t)h * p.o_sh + (size_t)(valid ? i : 0) * p.o_sn +
@@ -720,17 +766,34 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         // a role gave up: let copies that were already issued land before the CTA leaves
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 20000ull) { }
+        // ... and take the blocks that have not started out of the queue: each of them would wait as long
+        if (threadIdx.x == 0) {
+            uint32_t asked = ctl.asked, block;
+            for (;;) {
+                if (asked > 0) {
+                    const uint32_t slot = (asked - 1) & 1;
+                    if (!mbar_wait(smem_u32(&ctl.next_full[slot]), ((asked - 1) >> 1) & 1, 1000000ull)) break;
+                    if (!clc_answer(smem_u32(&ctl.next[slot]), block)) break;
+                    fence_proxy_async_smem();
+                }
+                const uint32_t slot = asked & 1;
+                mbar_arrive_expect_tx(smem_u32(&ctl.next_full[slot]), 16);
+                clc_try_cancel(smem_u32(&ctl.next[slot]), smem_u32(&ctl.next_full[slot]));
+                ++asked;
+            }
+        }
+        __syncthreads();
     }
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-template <int D, bool SOFTCAP, int GATE>
+template <int D, bool SOFTCAP, int GATE, int WALK>
 static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     using C = AttnCfg<D, GATE>;
     CUtensorMap tq, tk, tv;
     int rc;
-    const bool sorted = a.ws && !a.local_pass && layout_is_sorted(a.L.layout);
-    if (sorted) {
+    constexpr bool sorted = WALK == WALK_SORTED;
+    if constexpr (sorted) {
         // gather Q, K, V into the sorted order kept in the workspace; the kernel reads the copies
         char* ws = const_cast<char*>(a.ws);
         if ((rc = launch_gather_sorted(&a.s, a.q, a.s.Hq, true, a.L, a.ws, ws + a.L.qs, st))) return rc;
@@ -749,10 +812,9 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
         if ((rc = make_tmap_qkv(&tv, a.v, a.s.batch, a.s.Hkv, a.s.n, D, 128 / C::PARTS))) return rc;
     }
     AttnParams p;
-    p.B = a.s.batch; p.Hq = a.s.Hq; p.Hkv = a.s.Hkv; p.G = a.s.Hq / a.s.Hkv; p.n = a.s.n; p.w = a.s.window; p.K = a.s.K;
+    p.B = a.s.batch; p.Hq = a.s.Hq; p.Hkv = a.s.Hkv; p.G = a.s.Hq / a.s.Hkv; p.n = a.s.n; p.w = a.s.window < a.s.n ? a.s.window : a.s.n; p.K = a.s.K;
     p.nqb = cdiv(a.s.n, 128 * C::NQ);
     p.nqt = cdiv(a.s.n, 128); p.nkt = cdiv(a.s.n, 128); p.nkw = cdiv(p.nkt, 32);
-    p.dense = a.ws ? 0 : 1;
     p.scale = a.scale; p.softcap = a.s.softcap;
     p.mq = a.mq;
     p.gbits = a.ws ? reinterpret_cast<const uint32_t*>(a.ws + a.L.gbits) : nullptr;
@@ -764,7 +826,6 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.lse = a.lse;
     p.status = a.dev_status;
     p.nitems = (long long)a.s.batch * a.s.Hq * p.nqb;
-    p.sorted = sorted ? 1 : 0;
     p.nqp = a.L.nqp; p.nkp = a.L.nkp; p.nqblk = a.L.nqp / 256;
     p.ipb = 2 / C::NQ;
     p.perm_q = sorted ? reinterpret_cast<const int32_t*>(a.ws + a.L.perm_q) : nullptr;
@@ -782,15 +843,14 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.wait_limit_ns = a.wait_limit_ns;
     p.stall_at = a.stall_at;
     if (sorted) p.nitems = (long long)a.s.batch * a.s.Hq * p.nqblk * p.ipb;
-    int dev = 0, sms = 0;
-    if ((rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
-    if ((rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute"))) return rc;
-    auto kern = focus_attn_kernel<D, SOFTCAP, GATE>;
+    // K and V of all heads up to half of L2 (126 MB): the order of the items need not keep to one head at a time
+    p.by_length = (size_t)a.s.batch * a.s.Hkv * a.s.n * D * 4 <= ((size_t)64 << 20);
+    if (p.nitems > 0x7fffffffll) return fail(FOCUS_ERR_UNSUPPORTED, "attention: %lld query blocks exceed 2^31 - 1", p.nitems);
+    auto kern = focus_attn_kernel<D, SOFTCAP, GATE, WALK>;
     if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES),
                          "cudaFuncSetAttribute(attn)")))
         return rc;
-    const int grid = (int)(p.nitems < sms ? p.nitems : sms);
-    kern<<<grid, C::THREADS, C::SMEM_BYTES, st>>>(tq, tk, tv, p);
+    kern<<<(unsigned)p.nitems, C::THREADS, C::SMEM_BYTES, st>>>(tq, tk, tv, p);
     return check_cuda(cudaGetLastError(), "attention kernel launch");
 }
 
@@ -817,22 +877,27 @@ int launch_attn_sm100(const AttnArgs& a, cudaStream_t st) {
     return launch_attn_one(a, st);
 }
 
-static int launch_attn_one(const AttnArgs& a, cudaStream_t st) {
-    const bool cap = a.s.softcap > 0.f;
+template <int D>
+static int launch_attn_d(const AttnArgs& a, cudaStream_t st) {
     if (a.gate_g) {      // training-time gated forward: dense causal walk, no softcap
         const int chunks = a.gate_ld <= 8 ? 1 : a.gate_ld / 8;      // 8-float chunks of an assignment row
-        switch (a.s.D) {
-            case 64: return chunks == 1 ? launch_attn_t<64, false, 1>(a, st) : chunks == 2 ? launch_attn_t<64, false, 2>(a, st) : launch_attn_t<64, false, 4>(a, st);
-            case 128: return chunks == 1 ? launch_attn_t<128, false, 1>(a, st) : chunks == 2 ? launch_attn_t<128, false, 2>(a, st) : launch_attn_t<128, false, 4>(a, st);
-            case 256:
-                if (chunks == 4) return fail(FOCUS_ERR_UNSUPPORTED, "the gated forward at D = 256 supports K <= 16");
-                return chunks == 1 ? launch_attn_t<256, false, 1>(a, st) : launch_attn_t<256, false, 2>(a, st);
-        }
+        if (chunks == 1) return launch_attn_t<D, false, 1, WALK_DENSE>(a, st);
+        if (chunks == 2) return launch_attn_t<D, false, 2, WALK_DENSE>(a, st);
+        if constexpr (D != 256) return launch_attn_t<D, false, 4, WALK_DENSE>(a, st);
+        return fail(FOCUS_ERR_UNSUPPORTED, "the gated forward at D = 256 supports K <= 16");
     }
+    const bool cap = a.s.softcap > 0.f;
+    if (!a.ws) return cap ? launch_attn_t<D, true, 0, WALK_DENSE>(a, st) : launch_attn_t<D, false, 0, WALK_DENSE>(a, st);
+    if (a.local_pass || !layout_is_sorted(a.L.layout))
+        return cap ? launch_attn_t<D, true, 0, WALK_TOKEN>(a, st) : launch_attn_t<D, false, 0, WALK_TOKEN>(a, st);
+    return cap ? launch_attn_t<D, true, 0, WALK_SORTED>(a, st) : launch_attn_t<D, false, 0, WALK_SORTED>(a, st);
+}
+
+static int launch_attn_one(const AttnArgs& a, cudaStream_t st) {
     switch (a.s.D) {
-        case 64: return cap ? launch_attn_t<64, true, 0>(a, st) : launch_attn_t<64, false, 0>(a, st);
-        case 128: return cap ? launch_attn_t<128, true, 0>(a, st) : launch_attn_t<128, false, 0>(a, st);
-        case 256: return cap ? launch_attn_t<256, true, 0>(a, st) : launch_attn_t<256, false, 0>(a, st);
+        case 64: return launch_attn_d<64>(a, st);
+        case 128: return launch_attn_d<128>(a, st);
+        case 256: return launch_attn_d<256>(a, st);
     }
     return fail(FOCUS_ERR_UNSUPPORTED, "D (%d) must be 64, 128 or 256", a.s.D);
 }

@@ -55,6 +55,28 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
     }
 }
 
+// ---------------------------------------------------------------- cluster launch control
+// Ask for the grid's next block that has not started: a 16-byte answer lands in shared memory and completes 16 bytes on
+// the mbarrier.  Not to be asked again once an answer was "none".
+__device__ __forceinline__ void clc_try_cancel(uint32_t answer, uint32_t bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar) : "memory");
+}
+// blockIdx.x of the block the answer hands over; false when there is none left
+__device__ __forceinline__ bool clc_answer(uint32_t answer, uint32_t& block) {
+    uint32_t got;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+        "ld.shared.b128 r, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "selp.b32 %1, 1, 0, p;\n\t"
+        "mov.b32 %0, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}"
+        : "=r"(block), "=r"(got)
+        : "r"(answer)
+        : "memory");
+    return got != 0;
+}
+
 // ---------------------------------------------------------------- async-proxy fences
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
