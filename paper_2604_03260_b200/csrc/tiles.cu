@@ -9,24 +9,26 @@ namespace focus {
 constexpr int TM = FOCUS_TILE_M;
 constexpr int TN = FOCUS_TILE_N;
 
-// One block of 128 threads per (head, tile).  side = 0: query masks, 1: key masks (+ gbits).
+// One block of 128 threads per (head, tile): the heads of the query masks, then those of the key masks (+ gbits).  The first
+// block clears the counters of the passes that follow.
 __global__ void __launch_bounds__(128)
-summarise_kernel(const uint32_t* __restrict__ m, int n, int nt, int K, uint32_t* __restrict__ orv,
-                 uint32_t* __restrict__ andv, uint32_t* __restrict__ gbits) {
-    const int tile = blockIdx.x, head = blockIdx.y;
+summarise_kernel(const uint32_t* __restrict__ mq, const uint32_t* __restrict__ mk, int HQ, int n, int nt, int K, uint32_t* __restrict__ orq,
+                 uint32_t* __restrict__ andq, uint32_t* __restrict__ ork, uint32_t* __restrict__ andk, uint32_t* __restrict__ gbits,
+                 unsigned long long* __restrict__ counters) {
+    dep_trigger();
+    const int tile = blockIdx.x % nt, row = blockIdx.x / nt;
+    const bool key = row >= HQ;
+    const int head = key ? row - HQ : row;
     const int tok = tile * 128 + threadIdx.x;
     const bool in = tok < n;
-    const uint32_t v = in ? m[(size_t)head * n + tok] : 0u;
-    uint32_t o = v, a = in ? v : 0xffffffffu;
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-        o |= __shfl_xor_sync(0xffffffffu, o, off);
-        a &= __shfl_xor_sync(0xffffffffu, a, off);
-    }
+    dep_wait();
+    if (blockIdx.x == 0 && threadIdx.x < 8) counters[threadIdx.x] = 0ull;
+    const uint32_t v = in ? (key ? mk : mq)[(size_t)head * n + tok] : 0u;
+    const uint32_t o = __reduce_or_sync(0xffffffffu, v), a = __reduce_and_sync(0xffffffffu, in ? v : 0xffffffffu);
     __shared__ uint32_t so[4], sa[4];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) { so[warp] = o; sa[warp] = a; }
-    if (gbits) {
+    if (key) {
         uint32_t* gb = gbits + ((size_t)head * nt + tile) * K * 4;
         for (int g = 0; g < K; ++g) {
             const uint32_t word = __ballot_sync(0xffffffffu, (v >> g) & 1u);
@@ -35,78 +37,64 @@ summarise_kernel(const uint32_t* __restrict__ m, int n, int nt, int K, uint32_t*
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        orv[(size_t)head * nt + tile] = so[0] | so[1] | so[2] | so[3];
-        andv[(size_t)head * nt + tile] = sa[0] & sa[1] & sa[2] & sa[3];
-    }
-}
-
-// Per KV head and group g: which key tiles hold a member of g (from the OR summaries) and which key tiles
-// consist of members of g only (from the AND summaries), as bitmaps over the key tiles.  thread = (head, word).
-__global__ void __launch_bounds__(256)
-group_tiles_kernel(const uint32_t* __restrict__ ork, const uint32_t* __restrict__ andk, int HK, int nkt, int nkw, int K,
-                   uint32_t* __restrict__ kany, uint32_t* __restrict__ kall) {
-    const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= HK * nkw) return;
-    const int hk = gid / nkw, wd = gid % nkw;
-    uint32_t any_w[32], all_w[32];
-#pragma unroll
-    for (int g = 0; g < 32; ++g) any_w[g] = all_w[g] = 0u;
-    for (int c = 0; c < 32; ++c) {
-        const int b = wd * 32 + c;
-        if (b >= nkt) break;
-        const uint32_t o = ork[(size_t)hk * nkt + b], a = andk[(size_t)hk * nkt + b];
-#pragma unroll
-        for (int g = 0; g < 32; ++g) {
-            any_w[g] |= ((o >> g) & 1u) << c;
-            all_w[g] |= ((a >> g) & 1u) << c;
-        }
-    }
-    for (int g = 0; g < K; ++g) {
-        kany[((size_t)hk * K + g) * nkw + wd] = any_w[g];
-        kall[((size_t)hk * K + g) * nkw + wd] = all_w[g];
+        (key ? ork : orq)[(size_t)head * nt + tile] = so[0] | so[1] | so[2] | so[3];
+        (key ? andk : andq)[(size_t)head * nt + tile] = sa[0] & sa[1] & sa[2] & sa[3];
     }
 }
 
 // Live far-tile bitmap.  Key tile b is far for query tile a when every pair has i - j > w, i.e. b < (128 a - w) / 128;
-// a far tile is live when the query tile's OR summary meets the key tile's, full when the AND summaries meet.  A word
-// of the bitmap is the OR, over the groups present in the query tile, of the groups' key-tile bitmaps.
-// One block per (query tile, head); threads stride over the words of the row.
+// a far tile is live when the query tile's OR summary meets the key tile's, full when the AND summaries meet.  A warp makes
+// a word of the bitmap at a time, its lanes the 32 key tiles; the words past the far tiles are zero.
+// One block per (head, query tile).  The blocks past those of the HQ query heads, as many per KV head, write, per
+// group g, which key tiles hold a member of g and which consist of members of g only, as bitmaps over the key tiles, also a
+// word per warp; nothing in this launch waits for them.  (One thread per word in a launch of its own, before the live
+// bitmap, took 6 to 25 us for its 32 dependent loads.)
 __global__ void __launch_bounds__(128)
-live_kernel(const uint32_t* __restrict__ orq, const uint32_t* __restrict__ andq, const uint32_t* __restrict__ kany,
-            const uint32_t* __restrict__ kall, int G_heads, int Hq, int Hkv, int w, int K, int nqt, int nkw,
-            uint32_t* __restrict__ live, int32_t* __restrict__ live_cnt, unsigned long long* counters) {
-    const int a = blockIdx.x, hq = blockIdx.y;
-    const int b_idx = hq / Hq, h = hq % Hq;
-    const int hk = b_idx * Hkv + h / G_heads;
-    const uint32_t oq = orq[(size_t)hq * nqt + a], aq = andq[(size_t)hq * nqt + a];
-    const long long d = (long long)a * TM - w;
-    const int nfar_tiles = d > 0 ? (int)(d / TN) : 0;                 // far tiles are the first nfar_tiles key tiles
-    unsigned int nlive = 0, nfull = 0;
-    for (int wd = threadIdx.x; wd < nkw; wd += blockDim.x) {
-        const int rem = nfar_tiles - wd * 32;
-        const uint32_t far_mask = rem >= 32 ? 0xffffffffu : (rem <= 0 ? 0u : ((1u << rem) - 1u));
-        uint32_t lv = 0, fl = 0;
-        if (far_mask) {
-            for (uint32_t m = oq; m; m &= m - 1) {
-                const int g = __ffs(m) - 1;
-                if (g < K) lv |= kany[((size_t)hk * K + g) * nkw + wd];
-            }
-            for (uint32_t m = aq; m; m &= m - 1) {
-                const int g = __ffs(m) - 1;
-                if (g < K) fl |= kall[((size_t)hk * K + g) * nkw + wd];
-            }
-            lv &= far_mask;
-            fl &= far_mask;
-        }
-        live[((size_t)hq * nqt + a) * nkw + wd] = lv;
-        nlive += __popc(lv);
-        nfull += __popc(fl);
-    }
+live_kernel(const uint32_t* __restrict__ orq, const uint32_t* __restrict__ andq, const uint32_t* __restrict__ ork,
+            const uint32_t* __restrict__ andk, int G_heads, int Hq, int Hkv, int HQ, int w, int K, int nqt, int nkt, int nkw,
+            uint32_t* __restrict__ kany, uint32_t* __restrict__ kall, uint32_t* __restrict__ live, int32_t* __restrict__ live_cnt,
+            unsigned long long* counters) {
+    dep_trigger();
     __shared__ unsigned int s[2];
     if (threadIdx.x < 2) s[threadIdx.x] = 0;
     __syncthreads();
-    if (nlive) atomicAdd(&s[0], nlive);
-    if (nfull) atomicAdd(&s[1], nfull);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    dep_wait();
+    const int a = blockIdx.x % nqt, hq = blockIdx.x / nqt;
+    if (hq >= HQ) {
+        const int hk = hq - HQ;
+        for (int wd = a * 4 + warp; wd < nkw; wd += nqt * 4) {
+            const int b = wd * 32 + lane;
+            const uint32_t o = b < nkt ? ork[(size_t)hk * nkt + b] : 0u, all = b < nkt ? andk[(size_t)hk * nkt + b] : 0u;
+            for (int g = 0; g < K; ++g) {
+                const uint32_t any_w = __ballot_sync(0xffffffffu, (o >> g) & 1u), all_w = __ballot_sync(0xffffffffu, (all >> g) & 1u);
+                if (lane == 0) {
+                    kany[((size_t)hk * K + g) * nkw + wd] = any_w;
+                    kall[((size_t)hk * K + g) * nkw + wd] = all_w;
+                }
+            }
+        }
+        return;
+    }
+    const int b_idx = hq / Hq, h = hq % Hq;
+    const int hk = b_idx * Hkv + h / G_heads;
+    const uint32_t groups = K < 32 ? (1u << K) - 1u : 0xffffffffu;
+    const uint32_t oq = orq[(size_t)hq * nqt + a] & groups, aq = andq[(size_t)hq * nqt + a] & groups;
+    const long long d = (long long)a * TM - w;
+    const int nfar_tiles = d > 0 ? (int)(d / TN) : 0;                 // far tiles are the first nfar_tiles key tiles
+    unsigned int nlive = 0, nfull = 0;
+    uint32_t* row = live + ((size_t)hq * nqt + a) * nkw;
+    for (int wd = warp; wd < nkw; wd += 4) {
+        const int b = wd * 32 + lane;
+        const bool far = b < nfar_tiles;                              // (far tiles are all below nkt)
+        const uint32_t lv = __ballot_sync(0xffffffffu, far && (oq & ork[(size_t)hk * nkt + b]) != 0u);
+        const uint32_t fl = __ballot_sync(0xffffffffu, far && (aq & andk[(size_t)hk * nkt + b]) != 0u);
+        if (lane == 0) row[wd] = lv;
+        nlive += __popc(lv);
+        nfull += __popc(fl);
+    }
+    if (lane == 0 && nlive) atomicAdd(&s[0], nlive);
+    if (lane == 0 && nfull) atomicAdd(&s[1], nfull);
     __syncthreads();
     if (threadIdx.x == 0) {
         live_cnt[(size_t)hq * nqt + a] = (int32_t)s[0];
@@ -168,23 +156,18 @@ int launch_build_tiles_sorted(const focus_shape* s, const uint32_t* mq, const ui
 int launch_build_tiles(const focus_shape* s, const uint32_t* mq, const uint32_t* mk, int layout,
                        const focus_tiles_layout& L, char* ws, cudaStream_t st) {
     const int HQ = s->batch * s->Hq, HK = s->batch * s->Hkv;
-    int rc = check_cuda(cudaMemsetAsync(ws + L.counters, 0, 8 * sizeof(uint64_t), st), "cudaMemsetAsync(counters)");
+    if (HQ > 65535) return fail(FOCUS_ERR_CUDA, "build_tiles: batch*Hq (%d) must not exceed 65535", HQ);
+    const long long blocks = (long long)(HQ + HK) * L.nqt;
+    if (blocks > 0x7fffffffll) return fail(FOCUS_ERR_CUDA, "build_tiles: %lld tiles of 128 tokens exceed 2^31 - 1", blocks);
+    auto u32 = [&](size_t off) { return reinterpret_cast<uint32_t*>(ws + off); };
+    auto* counters = reinterpret_cast<unsigned long long*>(ws + L.counters);
+    int rc = check_cuda(launch_dependent(summarise_kernel, dim3((unsigned)blocks), dim3(128), 0, st, mq, mk, HQ, s->n, L.nqt, s->K, u32(L.orq),
+                                         u32(L.andq), u32(L.ork), u32(L.andk), u32(L.gbits), counters), "summarise kernel launch");
     if (rc) return rc;
-    auto* orq = reinterpret_cast<uint32_t*>(ws + L.orq);
-    auto* andq = reinterpret_cast<uint32_t*>(ws + L.andq);
-    auto* ork = reinterpret_cast<uint32_t*>(ws + L.ork);
-    auto* andk = reinterpret_cast<uint32_t*>(ws + L.andk);
-    auto* gb = reinterpret_cast<uint32_t*>(ws + L.gbits);
-    summarise_kernel<<<dim3(L.nqt, HQ), 128, 0, st>>>(mq, s->n, L.nqt, s->K, orq, andq, nullptr);
-    summarise_kernel<<<dim3(L.nkt, HK), 128, 0, st>>>(mk, s->n, L.nkt, s->K, ork, andk, gb);
-    auto* kany = reinterpret_cast<uint32_t*>(ws + L.kany);
-    auto* kall = reinterpret_cast<uint32_t*>(ws + L.kall);
-    group_tiles_kernel<<<cdiv(HK * L.nkw, 256), 256, 0, st>>>(ork, andk, HK, L.nkt, L.nkw, s->K, kany, kall);
-    live_kernel<<<dim3(L.nqt, HQ), 128, 0, st>>>(orq, andq, kany, kall, s->Hq / s->Hkv, s->Hq, s->Hkv, s->window, s->K, L.nqt,
-                                                 L.nkw, reinterpret_cast<uint32_t*>(ws + L.live),
-                                                 reinterpret_cast<int32_t*>(ws + L.live_cnt),
-                                                 reinterpret_cast<unsigned long long*>(ws + L.counters));
-    if ((rc = check_cuda(cudaGetLastError(), "build_tiles kernels"))) return rc;
+    rc = check_cuda(launch_dependent(live_kernel, dim3((unsigned)blocks), dim3(128), 0, st, u32(L.orq), u32(L.andq), u32(L.ork), u32(L.andk),
+                                     s->Hq / s->Hkv, s->Hq, s->Hkv, HQ, s->window, s->K, L.nqt, L.nkt, L.nkw, u32(L.kany), u32(L.kall),
+                                     u32(L.live), reinterpret_cast<int32_t*>(ws + L.live_cnt), counters), "live tiles kernel launch");
+    if (rc) return rc;
     if (layout_is_sorted(layout))
         return launch_build_tiles_sorted(s, mq, mk, L, ws, st);
     return FOCUS_OK;
