@@ -53,7 +53,12 @@ struct AttnCfg {
     static constexpr uint32_t GATE_ROW_BYTES = 32 * (GATE ? GATE : 1);
     static constexpr uint32_t GATE_BUF_BYTES = 128 * GATE_ROW_BYTES;
     static_assert(!(D == 256 && GATE == 4), "no room for the K/V ring beside 64 KB of gate buffers at D = 256");
-    static constexpr uint32_t SMEM_BYTES = 1024 + NQ * TILE_BYTES + NSTAGE * STAGE_BYTES + (GATE ? 4 * GATE_BUF_BYTES : 0);
+    static constexpr int NINFO = (D == 256) ? 3 : 4;         // tiles handed on ahead (what fits beside the K/V ring)
+    // shared memory: Q | K/V ring | gate buffers | tile ring | row exchange | barriers
+    static constexpr uint32_t OFF_GATE = NQ * TILE_BYTES + NSTAGE * STAGE_BYTES;
+    static constexpr uint32_t OFF_INFO = OFF_GATE + (GATE ? 4 * GATE_BUF_BYTES : 0);
+    static constexpr uint32_t OFF_XVAL = OFF_INFO + (GATE ? 0 : NINFO * (uint32_t)sizeof(TileInfo));
+    static constexpr uint32_t OFF_CTL = OFF_XVAL + (NQ == 1 ? 2 * 2 * 128 * 2 : 0);
     // Ring order of the tiles.  With one query tile the S of the next key tile is issued before the current P V, so
     // K(next) travels ahead of V(current); with two query tiles V(current) is consumed and released first.
     static constexpr bool K_AHEAD = NQ == 1;
@@ -72,6 +77,7 @@ struct SharedCtl {
     uint64_t xchg[4];                 // split rows, per 32-row quadrant: both column halves have published a per-row value
     uint64_t gbar[2];                 // soft gate, per softmax warpgroup: the key assignments of the tile are in shared memory
     uint64_t kv_full[8], kv_empty[8];
+    uint64_t info_full[4], info_empty[4];         // tile ring: handed on, read by the MMA warp and every softmax warp
     uint64_t next_full[2], next_empty[2];         // the answers below: arrived, read by the MMA warp and every softmax warp
     unsigned long long limit_ns;      // how long a wait may last before the role gives up
     uint32_t tmem_base;
@@ -134,21 +140,28 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                   const __grid_constant__ CUtensorMap tm_v, const AttnParams p) {
     using C = AttnCfg<D, GATE>;
     constexpr int NQ = C::NQ;
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(16) SharedCtl ctl;
-    // split rows: [parity][column half][row] row maxima, at the end row sums (the other instantiations have no room to spare)
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    SharedCtl& ctl = *reinterpret_cast<SharedCtl*>(smem_raw + C::OFF_CTL);
+    // split rows: [parity][column half][row] row maxima, at the end row sums
     // (bf16: a rounded row maximum serves as well as the exact one as long as both threads use the same value)
-    __shared__ __nv_bfloat16 xval_s[C::NSPLIT == 2 ? 2 * 2 * 128 : 1];
-    auto xval = [&](int par, int hf, int row) -> __nv_bfloat16& { return xval_s[C::NSPLIT == 2 ? (par * 2 + hf) * 128 + row : 0]; };
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    __nv_bfloat16* const xval_s = reinterpret_cast<__nv_bfloat16*>(smem_raw + C::OFF_XVAL);
+    auto xval = [&](int par, int hf, int row) -> __nv_bfloat16& { return xval_s[(par * 2 + hf) * 128 + row]; };
+    TileInfo* const info = reinterpret_cast<TileInfo*>(smem_raw + C::OFF_INFO);
+    const uint32_t base = smem_u32(smem_raw);
     const uint32_t sq = base;                                 // NQ query tiles
     const uint32_t skv = base + NQ * C::TILE_BYTES;            // ring of K / V tiles
-    unsigned char* const gate_sm = smem_raw + (base - smem_u32(smem_raw)) + NQ * C::TILE_BYTES + C::NSTAGE * C::STAGE_BYTES;
+    unsigned char* const gate_sm = smem_raw + C::OFF_GATE;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (WALK == WALK_SORTED && __ldg(p.counters + 4) != 0ull) {      // more mask values than the sorted layout holds: refuse
         if (threadIdx.x == 0 && p.status && atomicCAS(p.status, 0, 2) == 0) {
             p.status[1] = 1; p.status[2] = 0; p.status[3] = (int)blockIdx.x;
+        }
+        return;
+    }
+    if (base & 1023u) {                                   // the operands' swizzle is a function of the address
+        if (threadIdx.x == 0 && p.status && atomicCAS(p.status, 0, 1) == 0) {
+            p.status[1] = 2; p.status[2] = 0; p.status[3] = (int)blockIdx.x;
         }
         return;
     }
@@ -166,6 +179,10 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         for (int s = 0; s < C::NSTAGE; ++s) {
             mbar_init(smem_u32(&ctl.kv_full[s]), 1);
             mbar_init(smem_u32(&ctl.kv_empty[s]), 1);
+        }
+        for (int x = 0; x < C::NINFO; ++x) {
+            mbar_init(smem_u32(&ctl.info_full[x]), 1);
+            mbar_init(smem_u32(&ctl.info_empty[x]), C::THREADS / 32 - 3);
         }
         for (int x = 0; x < 2; ++x) {
             mbar_init(smem_u32(&ctl.next_full[x]), 1);
@@ -191,6 +208,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         if (lane == 0) {
             prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
             long long nload = 0;
+            uint32_t ninfo = 0;             // tiles handed on
             int it = 0;                     // items processed (items without key tiles are skipped by every role)
             bool ok = true;
             // ask for the item after number `ord`, when all of that one's loads are on their way
@@ -207,7 +225,41 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 const int item = t.A;
                 TileWalk<WALK> walk;
                 walk.init(p, hq, A * NQ, NQ);
-                int kb = walk.next();
+                int cls_at = -1;
+                uint32_t cls = 0;
+                // the next tile of the walk, handed on to the other roles
+                auto next_tile = [&]() -> int {
+                    const int kb = walk.next();
+                    if constexpr (WALK != WALK_DENSE) {
+                        const uint32_t slot = ninfo % C::NINFO, use = ninfo / C::NINFO;
+                        if (use > 0 && !ctl_wait(&ctl.info_empty[slot], (use - 1) & 1, &ctl)) { report_timeout(p, &ctl, 12, item); ok = false; return -1; }
+                        ++ninfo;
+                        const uint32_t bar = smem_u32(&ctl.info_full[slot]);
+                        info[slot].kb = kb;
+                        if (kb < 0) {
+                            mbar_arrive(bar);
+                        } else {
+                            const int khead = b * p.Hkv + hk;
+                            const void* src;
+                            uint32_t bytes;
+                            if constexpr (WALK == WALK_SORTED) {
+                                if (walk.jk != cls_at) cls = __ldg(p.cls_k + (size_t)khead * FOCUS_MAX_CLASSES + (cls_at = walk.jk));
+                                info[slot].cls = cls;
+                                info[slot].pad[0] = (uint32_t)walk.jk;
+                                src = p.perm_k + (size_t)khead * p.nkp + (size_t)kb * 128;
+                                bytes = 512;
+                            } else {
+                                src = p.gbits + ((size_t)khead * p.nkt + kb) * p.K * 4;
+                                bytes = (uint32_t)p.K * 16;
+                            }
+                            mbar_arrive_expect_tx(bar, bytes);
+                            bulk_load(smem_u32(info[slot].data), src, bytes, bar);
+                        }
+                    }
+                    return kb;
+                };
+                int kb = next_tile();
+                if (!ok) break;
                 if (kb < 0) { ask_next(ord); continue; }
                 if (it > 0 && !ctl_wait(&ctl.q_empty, (it - 1) & 1, &ctl)) { report_timeout(p, &ctl, 10, item); break; }
                 mbar_arrive_expect_tx(smem_u32(&ctl.q_full), NQ * C::TILE_BYTES);
@@ -248,14 +300,14 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     // S is issued before the current P V) and so travels ahead of the V it shares the ring with
                     load_tile(false, kb);
                     while (ok && kb >= 0) {
-                        const int nxt = walk.next();
+                        const int nxt = next_tile();
                         if (nxt >= 0) load_tile(false, nxt);
                         if (ok) load_tile(true, kb);
                         kb = nxt;
                     }
                 } else {
                     // two query tiles: V(current) is consumed and released before K(next), so it goes first
-                    for (; ok && kb >= 0; kb = walk.next()) {
+                    for (; ok && kb >= 0; kb = next_tile()) {
                         load_tile(false, kb);
                         if (ok) load_tile(true, kb);
                     }
@@ -274,6 +326,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
             long long nuse = 0;             // K/V stages consumed so far
             uint32_t np[2] = {0, 0};        // P tiles consumed per S/P buffer
+            uint32_t ninfo = 0;             // tiles taken from the ring
             uint32_t gs = 0, gp = 0;        // NQ == 1: S tiles issued / P tiles consumed (buffer = count & 1)
             int it = 0;
             bool ok = true;
@@ -368,8 +421,22 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 const int A = t.A, hq = t.hq;
                 const int item = t.A;
                 TileWalk<WALK> walk;
-                walk.init(p, hq, A * NQ, NQ);
-                int cur = walk.next();
+                if constexpr (WALK == WALK_DENSE) walk.init(p, hq, A * NQ, NQ);
+                auto next_tile = [&]() -> int {
+                    if constexpr (WALK == WALK_DENSE) {
+                        return walk.next();
+                    } else {
+                        const uint32_t slot = ninfo % C::NINFO;
+                        if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, &ctl)) { report_timeout(p, &ctl, 27, item); ok = false; return -1; }
+                        const int kb = info[slot].kb;
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctl.info_empty[slot]));
+                        ++ninfo;
+                        return kb;
+                    }
+                };
+                int cur = next_tile();
+                if (!ok) break;
                 if (cur < 0) continue;
                 if (!ctl_wait(&ctl.q_full, it & 1, &ctl)) { report_timeout(p, &ctl, 20, item); break; }
                 if constexpr (NQ == 2) {
@@ -385,7 +452,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 }
                 bool first = true;
                 while (cur >= 0) {
-                    const int nxt = walk.next();
+                    const int nxt = next_tile();
+                    if (!ok) break;
                     int vslot = 0, kslot = 0;
                     if constexpr (NQ == 2) {
                         // the ring carries V(current) ahead of K(next) here (see the producer)
@@ -451,6 +519,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         const float sl2 = SOFTCAP ? p.softcap * LOG2E : p.scale * LOG2E;
         const float cap_in = SOFTCAP ? p.scale / p.softcap : 0.f;
         uint32_t ns = 0;                                     // S tiles consumed by this warpgroup
+        uint32_t ninfo = 0;                                  // tiles taken from the ring
         uint32_t ng = 0;                                     // soft gate: tiles whose key assignments this warpgroup has staged
         int it = 0;
         bool ok = true;
@@ -461,9 +530,28 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             const int hk = bb * p.Hkv + h / p.G;
             const int a = A * NQ + x;
             TileWalk<WALK> walk;
-            walk.init(p, hq, A * NQ, NQ);
-            int kb = walk.next();
-            if (kb < 0) continue;
+            if constexpr (WALK == WALK_DENSE) walk.init(p, hq, A * NQ, NQ);
+            const TileInfo* tile = nullptr;
+            auto next_tile = [&]() -> int {
+                if constexpr (WALK == WALK_DENSE) {
+                    return walk.next();
+                } else {
+                    const uint32_t slot = ninfo % C::NINFO;
+                    if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, &ctl)) { report_timeout(p, &ctl, 39, item); ok = false; return -1; }
+                    tile = info + slot;
+                    return tile->kb;
+                }
+            };
+            auto tile_read = [&]() {                     // the warp is through with what the ring says of the tile
+                if constexpr (WALK != WALK_DENSE) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl.info_empty[ninfo % C::NINFO]));
+                    ++ninfo;
+                }
+            };
+            int kb = next_tile();
+            if (!ok) break;
+            if (kb < 0) { tile_read(); continue; }
             // the row's position in the sequence: its index, or in the sorted layout the position its slot holds
             int i = a * 128 + row_in_tile;
             int wmin = 0, wmax = 0;
@@ -473,8 +561,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 wmax = __reduce_max_sync(0xffffffffu, i);
             }
             const bool valid = i >= 0 && i < p.n;
-            const uint32_t mi = (valid && WALK != WALK_DENSE) ? __ldg(p.mq + (size_t)hq * p.n + i) : 0u;
-            const uint32_t aq = (WALK == WALK_TOKEN && a < p.nqt) ? __ldg(p.andq + (size_t)hq * p.nqt + a) : 0u;
+            uint32_t mi = (valid && WALK != WALK_DENSE) ? __ldg(p.mq + (size_t)hq * p.n + i) : 0u;
+            if (WALK == WALK_TOKEN) mi &= 0xffffffffu >> (32 - p.K);
             const int dfar = a * 128 - p.w;
             const int f_x = (WALK == WALK_TOKEN && dfar > 0) ? dfar >> 7 : 0;   // tiles b < f_x are far for this query tile
             float m_used = -INFINITY, l = 0.f;
@@ -497,19 +585,19 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     }
                 }
             }
-            for (; kb >= 0; kb = walk.next()) {
+            for (; kb >= 0; kb = next_tile()) {
                 TileMask tm;
                 if constexpr (WALK == WALK_SORTED) {
-                    const bool share = (mi & __ldg(p.cls_k + (size_t)hk * FOCUS_MAX_CLASSES + walk.jk)) != 0u;
-                    build_tile_mask_sorted(tm, p.w, p.perm_k + (size_t)hk * p.nkp + (size_t)kb * 128, share,
-                                           valid ? i : -1, wmin, wmax, !p.share_only);
+                    const bool share = (mi & tile->cls) != 0u;
+                    build_tile_mask_sorted(tm, p.w, reinterpret_cast<const int32_t*>(tile->data), share, valid ? i : -1, wmin, wmax, !p.share_only);
                     if (p.gbits_s && !tm.all_masked)
-                        exclude_lower_groups(tm, p.gbits_s + ((size_t)hk * (p.nkp / 128) + kb) * p.K * 4, mi & ((1u << walk.jk) - 1u), p.K);
+                        exclude_lower_groups(tm, p.gbits_s + ((size_t)hk * (p.nkp / 128) + kb) * p.K * 4, mi & ((1u << tile->pad[0]) - 1u), p.K);
                 } else if constexpr (WALK == WALK_DENSE) {
                     build_tile_mask_dense(tm, p, a, kb, i);
                 } else {
-                    build_tile_mask(tm, p, a, kb, i, mi, aq, f_x, hk);
+                    build_tile_mask(tm, p, a, kb, i, mi, f_x, tile->data);
                 }
+                tile_read();
                 // ---- soft gate (Eq. 2): the score of a distant pair (i - j > w) is multiplied by sigmoid(lambda g_i . g_j).
                 // The warpgroup stages the key assignments of its columns in shared memory before S is needed; every
                 // thread then reads them with broadcast 16-byte loads, column by column.
@@ -706,6 +794,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if (!ok) break;
             }
             if (!ok) break;
+            tile_read();                                 // the end of the item
             // ---- epilogue: O / l -> bf16 -> global, lse
             if constexpr (NSPLIT == 2) {
                 // the two halves add their row sums: two exchanges, the leading bf16 part of the sum and its remainder
@@ -819,8 +908,6 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.mq = a.mq;
     p.gbits = a.ws ? reinterpret_cast<const uint32_t*>(a.ws + a.L.gbits) : nullptr;
     p.live = a.ws ? reinterpret_cast<const uint32_t*>(a.ws + a.L.live) : nullptr;
-    p.andq = a.ws ? reinterpret_cast<const uint32_t*>(a.ws + a.L.andq) : nullptr;
-    p.andk = a.ws ? reinterpret_cast<const uint32_t*>(a.ws + a.L.andk) : nullptr;
     p.o = reinterpret_cast<__nv_bfloat16*>(a.o.ptr);
     p.o_sb = a.o.stride_b; p.o_sh = a.o.stride_h; p.o_sn = a.o.stride_n;
     p.lse = a.lse;
@@ -847,10 +934,12 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.by_length = (size_t)a.s.batch * a.s.Hkv * a.s.n * D * 4 <= ((size_t)64 << 20);
     if (p.nitems > 0x7fffffffll) return fail(FOCUS_ERR_UNSUPPORTED, "attention: %lld query blocks exceed 2^31 - 1", p.nitems);
     auto kern = focus_attn_kernel<D, SOFTCAP, GATE, WALK>;
-    if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES),
+    constexpr uint32_t smem = C::OFF_CTL + (uint32_t)sizeof(SharedCtl);
+    static_assert(smem <= 227 * 1024, "shared memory of one block");
+    if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                          "cudaFuncSetAttribute(attn)")))
         return rc;
-    kern<<<(unsigned)p.nitems, C::THREADS, C::SMEM_BYTES, st>>>(tq, tk, tv, p);
+    kern<<<(unsigned)p.nitems, C::THREADS, smem, st>>>(tq, tk, tv, p);
     return check_cuda(cudaGetLastError(), "attention kernel launch");
 }
 
