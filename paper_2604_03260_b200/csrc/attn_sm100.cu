@@ -18,6 +18,14 @@
 // there an item is a single 128-row query tile, S is double-buffered over consecutive key tiles
 // and one warpgroup does the softmax while the MMAs of the neighbouring tiles run.
 //
+// Training-time soft gate, two query tiles: the factor of a distant pair is a function of g_i . g_j, and those products are
+// an MMA as well.  For a pair of tiles that holds distant pairs G_x = g_q g_k^T goes to the place of S_x first, the softmax
+// warps take it into registers and work out the 128 factors while S_x = Q_x K^T is computed over it; warps 2 and 3 write
+// the operands (assignments split into bf16 terms).  Per key tile that leaves the softmax warps a tanh, a fused
+// multiply-add and half a packed multiplication per pair, in place of K / 2 packed multiply-adds on 2 K / 4 shared-memory
+// reads: 8192 tokens, K = 8, 32/8 heads: 1290 -> 862 us; 32768: 20.7 -> 13.5 ms.  At D = 256 tensor memory and the ring
+// leave one query tile, whose softmax warps evaluate the products themselves.
+//
 // Which key tiles are visited, and in which order of items:
 //   dense mode      every tile up to the diagonal
 //   original layout far tiles (every pair beyond the window) only when the live bitmap says the OR
@@ -48,15 +56,27 @@ struct AttnCfg {
     // all 256 dimensions.  Five half stages fit, and a half goes back to the producer as soon as its own MMAs are done.
     static constexpr int PARTS = (D == 256) ? 2 : 1;         // ring stages per tile
     static constexpr uint32_t STAGE_BYTES = TILE_BYTES / PARTS;
-    static constexpr int NSTAGE = (D == 256) ? (GATE ? 4 : 5) : ((D == 128) ? (GATE == 4 ? 3 : (GATE ? 4 : 5)) : 8);
-    // soft gate: per softmax warpgroup two buffers of 128 key assignments, 8 GATE floats each (after the ring)
+    static constexpr int NSTAGE = (D == 256) ? (GATE ? 4 : 5)
+                                             : ((D == 128) ? (GATE == 4 ? 2 : GATE == 2 ? 3 : GATE == 1 ? 4 : 5) : (GATE == 4 ? 6 : 8));
+    // Soft gate, one query tile: per softmax warpgroup two buffers of 128 key assignments, 8 GATE floats each.
     static constexpr uint32_t GATE_ROW_BYTES = 32 * (GATE ? GATE : 1);
     static constexpr uint32_t GATE_BUF_BYTES = 128 * GATE_ROW_BYTES;
     static_assert(!(D == 256 && GATE == 4), "no room for the K/V ring beside 64 KB of gate buffers at D = 256");
+    // Soft gate, two query tiles: the inner products of the assignments are an MMA of their own, G = g_q g_k^T.  Every
+    // assignment is split into three bf16 terms (24 mantissa bits) and six of the nine products of terms are taken, those
+    // above 2^-24.  An operand holds its terms side by side in column blocks of 8, 128 rows x 16 bytes each, no swizzle
+    // (so that a 16-deep MMA can pair any two blocks); with 8 values per assignment the key side repeats its first term
+    // as the fourth block, see gate_step.
+    static constexpr bool GATE_MMA = GATE != 0 && NQ == 2;
+    static constexpr int GATE_CH = GATE ? GATE : 1;                              // column blocks per term
+    static constexpr uint32_t GBLK_BYTES = 128 * 16;
+    static constexpr uint32_t GQ_BYTES = 3 * GATE_CH * GBLK_BYTES;               // one query tile
+    static constexpr uint32_t GK_BYTES = (GATE == 1 ? 4 : 3 * GATE_CH) * GBLK_BYTES;     // one key tile, two buffers
+    static constexpr uint32_t GATE_SMEM = GATE == 0 ? 0 : (NQ == 2 ? 2 * GQ_BYTES + 2 * GK_BYTES : 4 * GATE_BUF_BYTES);
     static constexpr int NINFO = (D == 256) ? 3 : 4;         // tiles handed on ahead (what fits beside the K/V ring)
     // shared memory: Q | K/V ring | gate buffers | tile ring | row exchange | barriers
     static constexpr uint32_t OFF_GATE = NQ * TILE_BYTES + NSTAGE * STAGE_BYTES;
-    static constexpr uint32_t OFF_INFO = OFF_GATE + (GATE ? 4 * GATE_BUF_BYTES : 0);
+    static constexpr uint32_t OFF_INFO = OFF_GATE + GATE_SMEM;
     static constexpr uint32_t OFF_XVAL = OFF_INFO + (GATE ? 0 : NINFO * (uint32_t)sizeof(TileInfo));
     static constexpr uint32_t OFF_CTL = OFF_XVAL + (NQ == 1 ? 2 * 2 * 128 * 2 : 0);
     // Ring order of the tiles.  With one query tile the S of the next key tile is issued before the current P V, so
@@ -68,6 +88,7 @@ struct AttnCfg {
     static constexpr int NSPLIT = NQ == 1 ? 2 : 1;
     static constexpr int NC = 128 / NSPLIT;                  // S columns per softmax thread
     static constexpr int THREADS = 128 + 128 * NQ * NSPLIT;
+    static constexpr int READERS = THREADS / 32 - 3 + (GATE_MMA ? 2 : 0);     // warps that read the queue: MMA, softmax, gate operands
 };
 
 struct SharedCtl {
@@ -75,7 +96,7 @@ struct SharedCtl {
     uint64_t s_full[2], p_full[2], o_full[2];
     uint64_t pv_done;
     uint64_t xchg[4];                 // split rows, per 32-row quadrant: both column halves have published a per-row value
-    uint64_t gbar[2];                 // soft gate, per softmax warpgroup: the key assignments of the tile are in shared memory
+    uint64_t gbar[2];                 // soft gate, one query tile, per softmax warpgroup: the key assignments are in shared memory
     uint64_t kv_full[8], kv_empty[8];
     uint64_t info_full[4], info_empty[4];         // tile ring: handed on, read by the MMA warp and every softmax warp
     uint64_t next_full[2], next_empty[2];         // the answers below: arrived, read by the MMA warp and every softmax warp
@@ -84,6 +105,12 @@ struct SharedCtl {
     int abort_flag;
     uint32_t asked;                   // how many answers the TMA thread has asked for
     uint4 next[2];                    // which item comes next, by the parity of its ordinal
+};
+
+// soft gate, two query tiles (behind SharedCtl)
+struct GateCtl {
+    uint64_t gq_full, gq_empty, gk_full[2], gk_empty[2];      // operands of G written / read
+    uint64_t g_full[2], g_taken[2];   // G of a query tile is in tensor memory / in the softmax warps' registers
 };
 
 // bounded wait that also gives up when another role of the CTA has already given up
@@ -108,6 +135,56 @@ __device__ __forceinline__ void report_timeout(const AttnParams& p, SharedCtl* c
         p.status[3] = (int)blockIdx.x;
     }
 }
+
+// soft gate: does the pair of query tile a and key tile kb hold a distant pair
+__device__ __forceinline__ bool gate_tile(const AttnParams& p, int a, int kb) {
+    return kb <= a && a * 128 < p.n && a * 128 + 127 - p.w > kb * 128;
+}
+
+// One assignment row (8 CH floats, times `scale`) as three bf16 terms into row r of an operand of G: term t, columns 8 c .. at
+// block t CH + c; with `again` the first term once more behind the third (CH = 1).
+template <int CH>
+__device__ __forceinline__ void put_gate_row(unsigned char* op, int r, const float* row, int ld, bool in, float scale, bool again) {
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+        float v[8];
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const bool have = in && 8 * c + 4 * f < ld;
+            const float4 x = have ? __ldg(reinterpret_cast<const float4*>(row) + 2 * c + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[4 * f] = x.x * scale; v[4 * f + 1] = x.y * scale; v[4 * f + 2] = x.z * scale; v[4 * f + 3] = x.w * scale;
+        }
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                w[e] = pack_bf16x2(v[2 * e], v[2 * e + 1]);
+                v[2 * e] -= __uint_as_float(w[e] << 16);
+                v[2 * e + 1] -= __uint_as_float(w[e] & 0xffff0000u);
+            }
+            const uint4 x = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4*>(op + (t * CH + c) * 2048 + r * 16) = x;
+            if (again && t == 0) *reinterpret_cast<uint4*>(op + (3 * CH + c) * 2048 + r * 16) = x;
+        }
+    }
+}
+
+// Step s of the MMA chain of G, the small products first: byte offset of the first column block of 8 and distance to the
+// second, of each side.  CH = 1: a step takes two products at once (terms h, m, l; the key side h, m, l, h):
+// (h l + l h), (h m + m h), (h h + m m).  CH > 1: one product of terms, 16 columns of it.
+template <int CH> struct GateSteps {
+    static constexpr int N = CH == 1 ? 3 : 6 * (CH / 2);
+    struct Step { uint32_t a, a_lbo, b, b_lbo; };
+    static __device__ __forceinline__ constexpr Step at(int s) {
+        constexpr uint32_t B = 2048;
+        if (CH == 1) return s == 0 ? Step{0, 2 * B, 2 * B, B} : s == 1 ? Step{0, B, B, 2 * B} : Step{0, B, 0, B};
+        constexpr int H = CH > 1 ? CH / 2 : 1;              // steps per product
+        const int pr = s / H, c = 2 * (s % H);
+        const uint32_t ta = pr == 1 ? 2 : (pr == 2 || pr == 4) ? 1 : 0, tb = pr == 0 ? 2 : (pr == 2 || pr == 3) ? 1 : 0;
+        return Step{(ta * CH + c) * B, B, (tb * CH + c) * B, B};
+    }
+};
 
 // The CTA's item number `ord` (0, 1, ...): the block it was launched as, then what the answers say; false after the last.
 // Called by every thread of a role's warp (`reader`: the warp reports that it has read), or by the TMA thread.
@@ -142,6 +219,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     constexpr int NQ = C::NQ;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     SharedCtl& ctl = *reinterpret_cast<SharedCtl*>(smem_raw + C::OFF_CTL);
+    GateCtl& gctl = *reinterpret_cast<GateCtl*>(smem_raw + C::OFF_CTL + sizeof(SharedCtl));
     // split rows: [parity][column half][row] row maxima, at the end row sums
     // (bf16: a rounded row maximum serves as well as the exact one as long as both threads use the same value)
     __nv_bfloat16* const xval_s = reinterpret_cast<__nv_bfloat16*>(smem_raw + C::OFF_XVAL);
@@ -169,6 +247,10 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         mbar_init(smem_u32(&ctl.q_full), 1);
         mbar_init(smem_u32(&ctl.q_empty), 1);
         mbar_init(smem_u32(&ctl.pv_done), 1);
+        if constexpr (C::GATE_MMA) {
+            mbar_init(smem_u32(&gctl.gq_full), 2);
+            mbar_init(smem_u32(&gctl.gq_empty), 1);
+        }
         for (int qd = 0; qd < 4; ++qd) mbar_init(smem_u32(&ctl.xchg[qd]), 2);
         for (int g = 0; g < 2; ++g) mbar_init(smem_u32(&ctl.gbar[g]), 4);
         for (int x = 0; x < 2; ++x) {
@@ -186,7 +268,13 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         for (int x = 0; x < 2; ++x) {
             mbar_init(smem_u32(&ctl.next_full[x]), 1);
-            mbar_init(smem_u32(&ctl.next_empty[x]), C::THREADS / 32 - 3);       // the MMA warp and the softmax warps
+            mbar_init(smem_u32(&ctl.next_empty[x]), C::READERS);
+            if constexpr (C::GATE_MMA) {
+                mbar_init(smem_u32(&gctl.gk_full[x]), 2);
+                mbar_init(smem_u32(&gctl.gk_empty[x]), 1);
+                mbar_init(smem_u32(&gctl.g_full[x]), 1);
+                mbar_init(smem_u32(&gctl.g_taken[x]), 4);
+            }
         }
         ctl.abort_flag = 0;
         ctl.asked = 0;
@@ -345,6 +433,35 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     }
                 }
             };
+            // two query tiles, soft gate: G_x = g_q g_k^T into the place of S_x, if the pair of tiles holds a distant pair; returns
+            // when the softmax warps have it in registers
+            uint32_t ngt[2] = {0, 0};       // G tiles per query tile
+            uint32_t ngk = 0;               // key operands taken
+            auto issue_gate = [&](int x, int a0, int kb, int item) -> bool {
+                if constexpr (C::GATE_MMA) {
+                    const bool g0 = gate_tile(p, a0, kb), g1 = gate_tile(p, a0 + 1, kb);
+                    if (!(x ? g1 : g0)) return true;       // (a gated tile 0 without a gated tile 1 gives the key operand back itself)
+                    const uint32_t buf = ngk & 1;
+                    if (!ctl_wait(&gctl.gk_full[buf], (ngk >> 1) & 1, &ctl)) { report_timeout(p, &ctl, 53, item); return false; }
+                    tc_fence_after();
+                    if (elect_one()) {
+                        using Steps = GateSteps<C::GATE_CH>;
+                        const uint32_t qa = sq + C::OFF_GATE + x * C::GQ_BYTES, ka = sq + C::OFF_GATE + 2 * C::GQ_BYTES + buf * C::GK_BYTES;
+#pragma unroll
+                        for (int st = 0; st < Steps::N; ++st)
+                            umma_ss(tmem + (x ? C::COL_S1 : C::COL_S0), smem_desc_plain(qa + Steps::at(st).a, Steps::at(st).a_lbo, 128),
+                                    smem_desc_plain(ka + Steps::at(st).b, Steps::at(st).b_lbo, 128), IDESC_S, st > 0);
+                        umma_commit(smem_u32(&gctl.g_full[x]));
+                        if (x == 1 || !g1) umma_commit(smem_u32(&gctl.gk_empty[buf]));
+                    }
+                    __syncwarp();
+                    if (x == 1 || !g1) ++ngk;
+                    if (!ctl_wait(&gctl.g_taken[x], ngt[x] & 1, &ctl)) { report_timeout(p, &ctl, 54, item); return false; }
+                    ++ngt[x];
+                    tc_fence_after();
+                }
+                return true;
+            };
             // O_x (+)= P[buf] V
             auto issue_o = [&](int x, int buf, int vslot, bool first) {
                 if (elect_one()) {
@@ -439,11 +556,16 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if (!ok) break;
                 if (cur < 0) continue;
                 if (!ctl_wait(&ctl.q_full, it & 1, &ctl)) { report_timeout(p, &ctl, 20, item); break; }
+                if constexpr (C::GATE_MMA) {
+                    if (!ctl_wait(&gctl.gq_full, it & 1, &ctl)) { report_timeout(p, &ctl, 29, item); break; }
+                }
                 if constexpr (NQ == 2) {
                     int slot;
                     if (!wait_kv(slot, 21, item)) break;
                     tc_fence_after();
+                    if (!issue_gate(0, A * NQ, cur, item)) break;
                     issue_s(0, 0, slot); commit(&ctl.s_full[0]);
+                    if (!issue_gate(1, A * NQ, cur, item)) break;
                     issue_s(1, 1, slot); commit(&ctl.s_full[1]);
                     release_tile(slot);
                 } else {
@@ -462,15 +584,22 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             if (!wait_kv(kslot, 23, item)) { ok = false; break; }
                         }
                     }
-                    if (nxt < 0) commit(&ctl.q_empty);     // every S of this item has been issued
+                    if (nxt < 0) {                         // every S (and G) of this item has been issued
+                        commit(&ctl.q_empty);
+                        if constexpr (C::GATE_MMA) commit(&gctl.gq_empty);
+                    }
                     if constexpr (NQ == 2) {
                         // query tile 0
                         if (!ctl_wait(&ctl.p_full[0], np[0] & 1, &ctl)) { report_timeout(p, &ctl, 24, item); ok = false; break; }
                         ++np[0];
                         tc_fence_after();
                         issue_o(0, 0, vslot, first);
-                        if (nxt >= 0) { issue_s(0, 0, kslot); commit(&ctl.s_full[0]); }
-                        else commit(&ctl.o_full[0]);
+                        if (nxt >= 0) {
+                            if (!issue_gate(0, A * NQ, nxt, item)) { ok = false; break; }
+                            issue_s(0, 0, kslot); commit(&ctl.s_full[0]);
+                        } else {
+                            commit(&ctl.o_full[0]);
+                        }
                         // query tile 1
                         if (!ctl_wait(&ctl.p_full[1], np[1] & 1, &ctl)) { report_timeout(p, &ctl, 25, item); ok = false; break; }
                         ++np[1];
@@ -478,6 +607,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         issue_o(1, 1, vslot, first);
                         release_tile(vslot);
                         if (nxt >= 0) {
+                            if (!issue_gate(1, A * NQ, nxt, item)) { ok = false; break; }
                             issue_s(1, 1, kslot); commit(&ctl.s_full[1]);
                             release_tile(kslot);
                         } else {
@@ -502,6 +632,48 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 }
                 ++it;
             }
+        }
+        __syncwarp();
+    } else if (C::GATE_MMA && warp < 4) {
+        // ------------------------------------------------------------------ soft gate: operands of G
+        const int t64 = threadIdx.x - 64;
+        unsigned char* const gq = smem_raw + C::OFF_GATE;
+        unsigned char* const gk = gq + 2 * C::GQ_BYTES;
+        uint32_t ngk = 0;
+        int it = 0;
+        bool ok = true;
+        Item t;
+        for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, true, t, ok); ++ord) {
+            const int a0 = t.A * NQ, item = t.A;
+            TileWalk<WALK_DENSE> walk;
+            walk.init(p, t.hq, a0, NQ);
+            int kb = walk.next();
+            if (kb < 0) continue;
+            const float* gseq = p.gate_g + (size_t)t.bb * p.n * p.gate_ld;
+            if (it > 0 && !ctl_wait(&gctl.gq_empty, (it - 1) & 1, &ctl)) { report_timeout(p, &ctl, 55, item); break; }
+#pragma unroll 1
+            for (int r = t64; r < 256; r += 64) {
+                const int i = a0 * 128 + r;
+                put_gate_row<C::GATE_CH>(gq + (r >> 7) * C::GQ_BYTES, r & 127, gseq + (size_t)min(i, p.n - 1) * p.gate_ld, p.gate_ld, i < p.n, p.gate_hl, false);
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&gctl.gq_full));
+            for (; kb >= 0; kb = walk.next()) {
+                if (!gate_tile(p, a0, kb) && !gate_tile(p, a0 + 1, kb)) continue;
+                const uint32_t buf = ngk & 1, use = ngk >> 1;
+                if (use > 0 && !ctl_wait(&gctl.gk_empty[buf], (use - 1) & 1, &ctl)) { report_timeout(p, &ctl, 56, item); ok = false; break; }
+                ++ngk;
+#pragma unroll 1
+                for (int r = t64; r < 128; r += 64) {
+                    const int j = kb * 128 + r;
+                    put_gate_row<C::GATE_CH>(gk + buf * C::GK_BYTES, r, gseq + (size_t)min(j, p.n - 1) * p.gate_ld, p.gate_ld, j < p.n, 1.f, C::GATE_CH == 1);
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&gctl.gk_full[buf]));
+            }
+            ++it;
         }
         __syncwarp();
     } else if (warp >= 4) {
@@ -568,11 +740,12 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             float m_used = -INFINITY, l = 0.f;
             bool first = true;
             // soft gate: this row's assignment times lambda / 2 (sigmoid(x) = 1/2 + 1/2 tanh(x / 2))
-            constexpr int GQ = GATE ? 2 * GATE : 2;               // 16-byte pieces of an assignment row held per token
+            constexpr bool GATE_ALU = GATE != 0 && !C::GATE_MMA;  // one query tile: the inner products are taken here
+            constexpr int GQ = GATE_ALU ? 2 * GATE : 2;           // 16-byte pieces of an assignment row held per token
             float gi[4 * GQ];
 #pragma unroll
             for (int e = 0; e < 4 * GQ; ++e) gi[e] = 0.f;
-            if constexpr (GATE != 0) {
+            if constexpr (GATE_ALU) {
                 if (valid) {
                     const float4* gp = reinterpret_cast<const float4*>(p.gate_g + ((size_t)bb * p.n + (size_t)i) * p.gate_ld);
 #pragma unroll
@@ -605,7 +778,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 bool gated = false;
                 const int gj0 = kb * 128 + half * NC;    // first column of this thread's part of the tile
                 const int ifar = i - p.w;                           // columns j < ifar are distant for this row
-                if constexpr (GATE != 0) {
+                const bool tile_gated = C::GATE_MMA && gate_tile(p, a, kb);
+                if constexpr (GATE_ALU) {
                     // the same decision in all four warps of the warpgroup: does the tile hold a distant pair at all
                     const bool tile_gated = !tm.all_masked && (a * 128 + 127 - p.w > gj0);
                     if (tile_gated) {
@@ -626,6 +800,29 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         gated = __any_sync(0xffffffffu, valid && ifar > gj0);
                     }
                 }
+                // ---- two query tiles: G first, its factors computed while S is
+                uint32_t sr[NC];
+                if constexpr (C::GATE_MMA) {
+                    if (tile_gated) {
+                        if (!ctl_wait(&gctl.g_full[x], ng & 1, &ctl)) { report_timeout(p, &ctl, 37, item); ok = false; break; }
+                        ++ng;
+                        tc_fence_after();
+                        const uint32_t t_g = tmem + lane_base + (x ? C::COL_S1 : C::COL_S0);
+#pragma unroll
+                        for (int c = 0; c < NC / 32; ++c) tmem_ld32(t_g + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
+                        tmem_wait_ld();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&gctl.g_taken[x]));
+                        const int nfar = ifar - gj0;                    // columns < nfar are distant
+                        if (__any_sync(0xffffffffu, nfar < NC)) {
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) sr[c] = c < nfar ? sr[c] : 0x7f800000u;        // tanh(inf) = 1: factor 1
+                        }
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) sr[c] = __float_as_uint(fmaf(tanh_approx(__uint_as_float(sr[c])), 0.5f, 0.5f));
+                    }
+                }
                 // ---- wait for S
                 const int buf = NQ == 2 ? x : (int)(ns & 1);
                 const uint32_t par = NQ == 2 ? (ns & 1) : ((ns >> 1) & 1);
@@ -638,11 +835,25 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
                     for (int c = 0; c < NC / 2; ++c) pk[c] = 0u;
                 } else {
-                    uint32_t sr[NC];
+                    if (tile_gated) {                    // the factors are in place of the scores
+#pragma unroll
+                        for (int c = 0; c < NC / 16; ++c) {      // 16 at a time: with 32 more scores beside the factors the loop spills
+                            uint32_t sv[16];
+                            tmem_ld16(t_s + c * 16, sv);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 16; e += 2) {
+                                const float2 f = __fmul2_rn(make_float2(__uint_as_float(sr[c * 16 + e]), __uint_as_float(sr[c * 16 + e + 1])),
+                                                            make_float2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])));
+                                sr[c * 16 + e] = __float_as_uint(f.x);
+                                sr[c * 16 + e + 1] = __float_as_uint(f.y);
+                            }
+                        }
+                    } else
 #pragma unroll
                     for (int c = 0; c < NC / 32; ++c) {
                         tmem_ld32(t_s + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
-                        if constexpr (GATE != 0) {       // chunk by chunk: 32 scores, then their factors
+                        if constexpr (GATE_ALU) {        // chunk by chunk: 32 scores, then their factors
                             tmem_wait_ld();
                             if (gated) {
                                 const bool wide = p.gate_ld == 8;
@@ -934,7 +1145,7 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.by_length = (size_t)a.s.batch * a.s.Hkv * a.s.n * D * 4 <= ((size_t)64 << 20);
     if (p.nitems > 0x7fffffffll) return fail(FOCUS_ERR_UNSUPPORTED, "attention: %lld query blocks exceed 2^31 - 1", p.nitems);
     auto kern = focus_attn_kernel<D, SOFTCAP, GATE, WALK>;
-    constexpr uint32_t smem = C::OFF_CTL + (uint32_t)sizeof(SharedCtl);
+    constexpr uint32_t smem = C::OFF_CTL + (uint32_t)sizeof(SharedCtl) + (C::GATE_MMA ? (uint32_t)sizeof(GateCtl) : 0);
     static_assert(smem <= 227 * 1024, "shared memory of one block");
     if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                          "cudaFuncSetAttribute(attn)")))

@@ -72,7 +72,6 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
     constexpr int VEC = D / 8;                                     // 16-byte pieces per row
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint32_t kflag_s[C::WARPS][DEC_NST][DEC_GK];        // per staged key: bit g set when query head g attends it
-    dep_trigger();                                                 // the merge may be set up now; it waits for this kernel's end
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, qd = lane & 3;                        // this thread's query head (MMA row) and column pair
     const int last = n - 1;                                        // position of the new token
@@ -94,8 +93,11 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
     // rows that are never copied still enter the MMAs (with probability 0): keep them finite
     for (int i = lane; i < DEC_NST * C::STAGE / 16; i += 32) reinterpret_cast<uint4*>(ring)[i] = make_uint4(0, 0, 0, 0);
     __syncwarp();
-    if (!waited) dep_wait();
-    waited = true;
+    if (!waited) {
+        dep_wait();
+        dep_trigger();                                             // the merge may be set up now; it waits for this kernel's end
+        waited = true;
+    }
 
     // Q as the row operand: rows >= G and rows 8..15 are zero
     uint32_t qa[D / 16][2];

@@ -284,6 +284,11 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo
     d |= (uint64_t)2 << 61;
     return d;
 }
+// The same without swizzle, K-major: 8-row x 16-byte core matrices, `lbo` bytes from one to the next along K, `sbo` along M / N.
+__device__ __forceinline__ uint64_t smem_desc_plain(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
+    return (uint64_t)((saddr >> 4) & 0x3fffu) | (uint64_t)((lbo_bytes >> 4) & 0x3fffu) << 16 | (uint64_t)((sbo_bytes >> 4) & 0x3fffu) << 32 |
+           (uint64_t)1 << 46;
+}
 // Instruction descriptor for kind::f16 with bf16 operands and fp32 accumulation:
 //   [4,6) D format (1 = f32), [7,10) A format (1 = bf16), [10,13) B format, bit 15 A major (1 = MN),
 //   bit 16 B major, [17,23) N >> 3, [24,29) M >> 4.

@@ -15,13 +15,13 @@ __global__ void __launch_bounds__(128)
 summarise_kernel(const uint32_t* __restrict__ mq, const uint32_t* __restrict__ mk, int HQ, int n, int nt, int K, uint32_t* __restrict__ orq,
                  uint32_t* __restrict__ andq, uint32_t* __restrict__ ork, uint32_t* __restrict__ andk, uint32_t* __restrict__ gbits,
                  unsigned long long* __restrict__ counters) {
-    dep_trigger();
     const int tile = blockIdx.x % nt, row = blockIdx.x / nt;
     const bool key = row >= HQ;
     const int head = key ? row - HQ : row;
     const int tok = tile * 128 + threadIdx.x;
     const bool in = tok < n;
     dep_wait();
+    dep_trigger();
     if (blockIdx.x == 0 && threadIdx.x < 8) counters[threadIdx.x] = 0ull;
     const uint32_t v = in ? (key ? mk : mq)[(size_t)head * n + tok] : 0u;
     const uint32_t o = __reduce_or_sync(0xffffffffu, v), a = __reduce_and_sync(0xffffffffu, in ? v : 0xffffffffu);
@@ -54,12 +54,12 @@ live_kernel(const uint32_t* __restrict__ orq, const uint32_t* __restrict__ andq,
             const uint32_t* __restrict__ andk, int G_heads, int Hq, int Hkv, int HQ, int w, int K, int nqt, int nkt, int nkw,
             uint32_t* __restrict__ kany, uint32_t* __restrict__ kall, uint32_t* __restrict__ live, int32_t* __restrict__ live_cnt,
             unsigned long long* counters) {
-    dep_trigger();
     __shared__ unsigned int s[2];
     if (threadIdx.x < 2) s[threadIdx.x] = 0;
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     dep_wait();
+    dep_trigger();
     const int a = blockIdx.x % nqt, hq = blockIdx.x / nqt;
     if (hq >= HQ) {
         const int hk = hq - HQ;
