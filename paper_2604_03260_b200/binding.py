@@ -119,14 +119,22 @@ def _check(rc):
         raise FocusError(rc, lib().focus_last_error().decode())
 
 
+# A short call (a decode step, a prompt of a thousand tokens) takes the GPU no longer than Python takes to marshal its
+# arguments, so these stay plain: addresses and stream handles as integers, one look at a tensor's strides, the current
+# stream's handle without a Stream object around it (3.2 us per call of a step whose GPU work is 17).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _p(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def make_shape(Hq, Hkv, n, D, K, topk, window, scale=0.0, softcap=0.0, batch=1) -> focus_shape:
@@ -140,11 +148,12 @@ def shape_of(wl) -> focus_shape:
 
 def tensor_arg(t: torch.Tensor) -> focus_tensor:
     """[H, n, D] or [batch, H, n, D] bf16 CUDA tensor with D contiguous"""
-    assert t.is_cuda and t.dtype == torch.bfloat16 and t.stride(-1) == 1
-    if t.dim() == 3:
-        return focus_tensor(t.data_ptr(), t.stride(0) * t.shape[0], t.stride(0), t.stride(1))
-    assert t.dim() == 4
-    return focus_tensor(t.data_ptr(), t.stride(0), t.stride(1), t.stride(2))
+    st = t.stride()
+    assert t.is_cuda and t.dtype is torch.bfloat16 and st[-1] == 1
+    if len(st) == 3:
+        return focus_tensor(t.data_ptr(), st[0] * t.shape[0], st[0], st[1])
+    assert len(st) == 4
+    return focus_tensor(t.data_ptr(), st[0], st[1], st[2])
 
 
 def focus_version() -> int:
@@ -191,10 +200,11 @@ def focus_decode_workspace_bytes(shape) -> int:
 def focus_decode_step(shape, q, k, v, mq_new, mk, o, lse, ws, stream=None):
     """q, o bf16 [Hq, D] (or [batch, Hq, D]); k, v bf16 caches [Hkv, n, D]; mq_new int32 [batch*Hq]; mk int32 [batch*Hkv, n]"""
     def vec_arg(t):
-        assert t.is_cuda and t.dtype == torch.bfloat16 and t.stride(-1) == 1
-        if t.dim() == 2:
-            return focus_tensor(t.data_ptr(), t.stride(0) * t.shape[0], t.stride(0), t.shape[-1])
-        return focus_tensor(t.data_ptr(), t.stride(0), t.stride(1), t.shape[-1])
+        st = t.stride()
+        assert t.is_cuda and t.dtype is torch.bfloat16 and st[-1] == 1
+        if len(st) == 2:
+            return focus_tensor(t.data_ptr(), st[0] * t.shape[0], st[0], t.shape[-1])
+        return focus_tensor(t.data_ptr(), st[0], st[1], t.shape[-1])
     _check(lib().focus_decode_step(C.byref(shape), vec_arg(q), tensor_arg(k), tensor_arg(v), _p(mq_new), _p(mk), vec_arg(o),
                                    _p(lse), _p(ws), ws.numel() * ws.element_size(), _stream(stream)))
 

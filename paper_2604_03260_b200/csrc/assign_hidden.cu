@@ -51,6 +51,8 @@ __global__ void __launch_bounds__(256)
 fold_router_kernel(const float* __restrict__ Wg, const float* __restrict__ C, int d, int dg, int K, float* __restrict__ folded) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     const int g = blockIdx.y;
+    dep_wait();
+    dep_trigger();
     if (e >= d) return;
     float s = 0.f;
     for (int j = 0; j < dg; ++j) s = fmaf(Wg[(size_t)e * dg + j], C[(size_t)g * dg + j], s);
@@ -98,7 +100,6 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
             fv[i] = (g < K && e < d) ? __ldg(folded + (size_t)g * d + e) : 0.f;
         }
     };
-    load_folded();
     auto stage_chunk = [&](int j) {
         if (j < total) {
             const int item = item0 + it_next;
@@ -152,8 +153,6 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
             }
         }
     }
-#pragma unroll
-    for (int j = 0; j < AH_NS - 1; ++j) stage_chunk(j);
     if (warp == 0) {
         tmem_alloc(smem_u32(&ctl->tmem_base), Cfg::TMEM_COLS);
         tmem_relinquish();
@@ -163,6 +162,11 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
         fence_mbar_init();
         ctl->fault = 0;
     }
+    dep_wait();
+    dep_trigger();
+    load_folded();
+#pragma unroll
+    for (int j = 0; j < AH_NS - 1; ++j) stage_chunk(j);
 
     bool ok = aligned;
     unsigned int near_votes = 0;
@@ -266,11 +270,8 @@ static int launch_k(const focus_shape* s, const void* h, int64_t sb, int64_t sn,
                     uint32_t* mq, uint32_t* mk, unsigned long long* near_ties, float eps, float* scores, cudaStream_t st) {
     using Cfg = HiddenCfg<KMAX>;
     auto kern = assign_hidden_kernel<KMAX>;
-    int rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM_BYTES),
-                        "cudaFuncSetAttribute(assign_hidden)");
+    int rc = check_cuda(allow_smem<assign_hidden_kernel<KMAX>>(Cfg::SMEM_BYTES, true), "cudaFuncSetAttribute(assign_hidden)");
     if (rc) return rc;
-    if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100),
-                         "cudaFuncSetAttribute(assign_hidden)"))) return rc;
     // one resident wave: as many blocks as fit on the device at once (fewer when there are fewer tiles).  Blocks of
     // 128 threads per SM: by shared memory (227 KB, 1 KB reserved per block), by the 512 columns of tensor memory, at most 3
     int dev = 0, sms = 0;
@@ -288,16 +289,15 @@ static int launch_k(const focus_shape* s, const void* h, int64_t sb, int64_t sn,
         return fail(FOCUS_ERR_UNSUPPORTED, "focus_assign_hidden: too many chunks of 128 x 128 elements for one launch");
     const int nblocks = (int)(nitems < resident ? nitems : resident);
     const int share = (int)(nitems / nblocks), extra = (int)(nitems % nblocks);
-    kern<<<nblocks, AH_THREADS, Cfg::SMEM_BYTES, st>>>(reinterpret_cast<const __nv_bfloat16*>(h), sb, sn, s->n, d, s->K, s->topk, folded,
-                                                       bias, s->Hq, s->Hkv, mq, mk, near_ties, eps, scores, ntile, share, extra);
-    return check_cuda(cudaGetLastError(), "assign_hidden kernel launch");
+    return check_cuda(launch_dependent(kern, dim3(nblocks), dim3(AH_THREADS), Cfg::SMEM_BYTES, st, reinterpret_cast<const __nv_bfloat16*>(h), sb, sn,
+                                       s->n, d, s->K, s->topk, folded, bias, s->Hq, s->Hkv, mq, mk, near_ties, eps, scores, ntile, share, extra),
+                      "assign_hidden kernel launch");
 }
 
 int launch_assign_hidden(const focus_shape* s, const void* h, int64_t sb, int64_t sn, int d, int dg, const float* Wg,
                          const float* C, const float* bias, float* folded, uint32_t* mq, uint32_t* mk,
                          unsigned long long* near_ties, float eps, float* scores, cudaStream_t st) {
-    fold_router_kernel<<<dim3(cdiv(d, 256), s->K), 256, 0, st>>>(Wg, C, d, dg, s->K, folded);
-    int rc = check_cuda(cudaGetLastError(), "fold_router kernel launch");
+    int rc = check_cuda(launch_dependent(fold_router_kernel, dim3(cdiv(d, 256), s->K), dim3(256), 0, st, Wg, C, d, dg, s->K, folded), "fold_router kernel launch");
     if (rc) return rc;
     if (s->K <= 4) return launch_k<4>(s, h, sb, sn, d, folded, bias, mq, mk, near_ties, eps, scores, st);
     if (s->K <= 8) return launch_k<8>(s, h, sb, sn, d, folded, bias, mq, mk, near_ties, eps, scores, st);

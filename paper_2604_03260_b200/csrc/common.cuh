@@ -7,6 +7,8 @@
 #include <stdio.h>
 #include <stdarg.h>
 
+#include <atomic>
+
 #include "focus.h"
 
 namespace focus {
@@ -71,6 +73,23 @@ inline cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 blo
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+
+// Lets KERN use `bytes` of dynamic shared memory on the current device (and, `carveout`, all of the SM's storage as shared
+// memory).  The driver is asked once per kernel and device: the attributes stay with the kernel, and asking costs about as
+// much as a launch.
+template <auto KERN>
+inline cudaError_t allow_smem(size_t bytes, bool carveout = false) {
+    static std::atomic<unsigned long long> devices{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (devices.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    if ((e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if (carveout && (e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess) return e;
+    devices.fetch_or(bit, std::memory_order_release);
+    return cudaSuccess;
 }
 #endif
 

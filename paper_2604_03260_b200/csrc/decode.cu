@@ -364,8 +364,7 @@ static int launch_decode_d(const focus_shape* s, const focus_tensor& q, const fo
     using C = DecCfg<D>;
     const DecPlan plan = decode_plan(s);
     auto kern = decode_partial_kernel<D>;
-    int rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM),
-                        "cudaFuncSetAttribute(decode)");
+    int rc = check_cuda(allow_smem<decode_partial_kernel<D>>(C::SMEM), "cudaFuncSetAttribute(decode)");
     if (rc) return rc;
     rc = check_cuda(launch_dependent(kern, dim3(plan.ctas), dim3(C::WARPS * 32), C::SMEM, st,
         reinterpret_cast<const __nv_bfloat16*>(q.ptr), q.stride_b, q.stride_h, reinterpret_cast<const __nv_bfloat16*>(k.ptr),

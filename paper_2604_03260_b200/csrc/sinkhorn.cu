@@ -520,8 +520,7 @@ static int launch_team(const focus_shape* s, const float* S, float tau, int iter
     if (chunk > SKT_TOKENS || smem > SKT_SMEM) return 0;
     P = cdiv(s->n, chunk);                           // no block without tokens
     auto kern = sinkhorn_team_kernel<KMAX, BWD>;
-    if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SKT_SMEM), "cudaFuncSetAttribute(sinkhorn)")))
-        return rc;
+    if ((rc = check_cuda(allow_smem<sinkhorn_team_kernel<KMAX, BWD>>(SKT_SMEM), "cudaFuncSetAttribute(sinkhorn)"))) return rc;
     cudaLaunchAttribute coop;
     coop.id = cudaLaunchAttributeCooperative;
     coop.val.cooperative = 1;
