@@ -140,8 +140,8 @@ typedef struct {
     /* FOCUS_LAYOUT_SORTED_LOCAL and FOCUS_LAYOUT_GROUP_MAJOR only (0 otherwise): the two partial results, kept in fp32
        until they are joined */
     size_t o_sorted;         /* fp32 [B*Hq][n][D]: class-sorted pass (its logsumexp goes to the caller's lse) */
-    size_t o_local;          /* fp32 [B*Hq][n][D]: window pass */
-    size_t lse_local;        /* fp32 [B*Hq][n] */
+    size_t o_local;          /* fp32 [B*Hq][n][D]: reserved (the window pass joins its result in registers) */
+    size_t lse_local;        /* fp32 [B*Hq][n]: reserved */
 } focus_tiles_layout;
 
 /* Library version (major*10000 + minor*100 + patch). */

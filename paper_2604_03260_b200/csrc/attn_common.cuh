@@ -62,6 +62,7 @@ struct AttnParams {
     const uint32_t* live;
     __nv_bfloat16* o;
     int64_t o_sb, o_sh, o_sn;
+    bool o_wide;             // its base and strides allow 32-byte stores
     float* lse;
     int32_t* status;
     long long nitems;
@@ -86,6 +87,7 @@ struct AttnParams {
     // group-major keys: bitmaps of the list entries per group, [B*Hkv][nkp/128][K][4] (nullptr in the other layouts)
     const uint32_t* gbits_s;
     int local_only;
+    const float* join;       // partial O (fp32, rows as in o32; its logsumexps in `lse`) to join with this pass's, or nullptr
     float* o32;              // partial passes: O in fp32, rows [B*Hq][n][D], instead of bf16 to `o`
     unsigned long long wait_limit_ns;   // bound of every wait inside the kernel
     long long stall_at;      // diagnostic: index of a K/V ring stage the producer leaves unfilled (-1 = none)

@@ -231,6 +231,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     unsigned char* const gate_sm = smem_raw + C::OFF_GATE;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+    if (WALK == WALK_SORTED) dep_wait();
     if (WALK == WALK_SORTED && __ldg(p.counters + 4) != 0ull) {      // more mask values than the sorted layout holds: refuse
         if (threadIdx.x == 0 && p.status && atomicCAS(p.status, 0, 2) == 0) {
             p.status[1] = 1; p.status[2] = 0; p.status[3] = (int)blockIdx.x;
@@ -289,6 +290,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ctl.tmem_base;
+    if (WALK != WALK_SORTED) dep_wait();
+    dep_trigger();
 
     if (warp < 4) reg_dec<REGS_CONTROL>();
     if (warp == 0) {
@@ -695,8 +698,24 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         uint32_t ng = 0;                                     // soft gate: tiles whose key assignments this warpgroup has staged
         int it = 0;
         bool ok = true;
-        Item t;
-        for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, true, t, ok); ++ord) {
+        // An item's row position and mask are loaded while the item before it ends, so that its first tile need not wait for
+        // them (three dependent reads of L2 in the sorted order): its order entry before the wait for the last P V, the mask
+        // word before the output is written.
+        Item t = {};
+        int i_row = -1;
+        uint32_t m_row = 0;
+        auto load_row = [&]() {
+            const int r = (t.A * NQ + x) * 128 + row_in_tile;
+            i_row = r;
+            // the row's position in the sequence: its index, or in the sorted layout the position its slot holds (-1: padding)
+            if constexpr (WALK == WALK_SORTED) i_row = __ldg(p.perm_q + (size_t)t.hq * p.nqp + r);
+        };
+        auto load_mask = [&]() {
+            if constexpr (WALK != WALK_DENSE) m_row = (i_row >= 0 && i_row < p.n) ? __ldg(p.mq + (size_t)t.hq * p.n + i_row) : 0u;
+        };
+        bool have = next_item<WALK>(p, &ctl, 0, true, t, ok);
+        if (have) { load_row(); load_mask(); }
+        for (uint32_t ord = 0; ok && have; ++ord) {
             const int A = t.A, hq = t.hq, bb = t.bb, h = t.h;
             const int item = t.A;
             const int hk = bb * p.Hkv + h / p.G;
@@ -723,17 +742,20 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             };
             int kb = next_tile();
             if (!ok) break;
-            if (kb < 0) { tile_read(); continue; }
-            // the row's position in the sequence: its index, or in the sorted layout the position its slot holds
-            int i = a * 128 + row_in_tile;
+            if (kb < 0) {
+                tile_read();
+                have = next_item<WALK>(p, &ctl, ord + 1, true, t, ok);
+                if (have) { load_row(); load_mask(); }
+                continue;
+            }
+            const int i = i_row;
             int wmin = 0, wmax = 0;
             if constexpr (WALK == WALK_SORTED) {
-                i = __ldg(p.perm_q + (size_t)hq * p.nqp + i);                       // -1 in the padding of a segment
                 wmin = __reduce_min_sync(0xffffffffu, i < 0 ? 0x7fffffff : i);
                 wmax = __reduce_max_sync(0xffffffffu, i);
             }
             const bool valid = i >= 0 && i < p.n;
-            uint32_t mi = (valid && WALK != WALK_DENSE) ? __ldg(p.mq + (size_t)hq * p.n + i) : 0u;
+            uint32_t mi = m_row;
             if (WALK == WALK_TOKEN) mi &= 0xffffffffu >> (32 - p.K);
             const int dfar = a * 128 - p.w;
             const int f_x = (WALK == WALK_TOKEN && dfar > 0) ? dfar >> 7 : 0;   // tiles b < f_x are far for this query tile
@@ -1006,7 +1028,13 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
             if (!ok) break;
             tile_read();                                 // the end of the item
-            // ---- epilogue: O / l -> bf16 -> global, lse
+            have = next_item<WALK>(p, &ctl, ord + 1, true, t, ok);
+            if (!ok) break;
+            if (have) load_row();
+            // ---- epilogue: O / l -> bf16 -> global, lse.  With a partial result to join (window pass of the split layout) the
+            // row's logsumexp there is read now, before a thread that shares the row can write the joint one.
+            float lse_other = -INFINITY;
+            if (WALK == WALK_TOKEN && p.join && valid) lse_other = p.lse[(size_t)hq * p.n + i];
             if constexpr (NSPLIT == 2) {
                 // the two halves add their row sums: two exchanges, the leading bf16 part of the sum and its remainder
                 float other = 0.f, rest = l;
@@ -1027,7 +1055,18 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
             if (!ctl_wait(&ctl.o_full[x], it & 1, &ctl)) { report_timeout(p, &ctl, 40 + x, item); break; }
             tc_fence_after();
+            if (have) load_mask();
             const float inv_l = l > 0.f ? 1.f / l : 0.f;        // a row without any pair (possible in a partial pass): zeros, lse = -inf
+            float own = inv_l, w_other = 0.f, lse_row = (m_used + lg2_approx(l)) * LN2;
+            if (WALK == WALK_TOKEN && p.join) {
+                // the two partial results cover disjoint sets of pairs and join through their logsumexps (Appendix D)
+                const float m = fmaxf(lse_other, lse_row);
+                const float wo = m == -INFINITY ? 0.f : __expf(lse_other - m), wl = m == -INFINITY ? 0.f : __expf(lse_row - m);
+                const float tot = wo + wl, inv = tot > 0.f ? 1.f / tot : 0.f;
+                own = inv_l * wl * inv;
+                w_other = wo * inv;
+                lse_row = tot > 0.f ? m + __logf(tot) : -INFINITY;
+            }
             __nv_bfloat16* orow = p.o + (size_t)bb * p.o_sb + (size_t)h * p.o_sh + (size_t)(valid ? i : 0) * p.o_sn +
                                   half * (D / 2);
 #pragma unroll 1
@@ -1035,26 +1074,49 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 uint32_t ov[32];
                 tmem_ld32(t_o + c * 32, ov);
                 tmem_wait_ld();
+                float add[32];
+                if constexpr (WALK == WALK_TOKEN) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) add[e] = 0.f;
+                    if (w_other > 0.f) {               // (a partial result without any pair has unspecified contents)
+                        const float* jrow = p.join + ((size_t)hq * p.n + (size_t)i) * D + half * (D / 2) + c * 32;
+#pragma unroll
+                        for (int e = 0; e < 32; e += 4) {
+                            const float4 v4 = *reinterpret_cast<const float4*>(jrow + e);
+                            add[e] = v4.x * w_other; add[e + 1] = v4.y * w_other; add[e + 2] = v4.z * w_other; add[e + 3] = v4.w * w_other;
+                        }
+                    }
+                }
+                auto out = [&](int e) {
+                    const float v = __uint_as_float(ov[e]);
+                    if constexpr (WALK == WALK_TOKEN) return fmaf(v, own, add[e]);
+                    else return v * own;
+                };
                 if (valid && p.o32) {
                     float* o32row = p.o32 + ((size_t)hq * p.n + (size_t)i) * D + half * (D / 2) + c * 32;
 #pragma unroll
-                    for (int e = 0; e < 32; e += 4)
-                        *reinterpret_cast<float4*>(o32row + e) =
-                            make_float4(__uint_as_float(ov[e]) * inv_l, __uint_as_float(ov[e + 1]) * inv_l,
-                                        __uint_as_float(ov[e + 2]) * inv_l, __uint_as_float(ov[e + 3]) * inv_l);
+                    for (int e = 0; e < 32; e += 8) {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) w[j] = __float_as_uint(out(e + j));
+                        st_global_v8(o32row + e, w);
+                    }
                 } else if (valid) {
 #pragma unroll
-                    for (int e = 0; e < 32; e += 8) {
-                        uint4 w4;
-                        w4.x = pack_bf16x2(__uint_as_float(ov[e]) * inv_l, __uint_as_float(ov[e + 1]) * inv_l);
-                        w4.y = pack_bf16x2(__uint_as_float(ov[e + 2]) * inv_l, __uint_as_float(ov[e + 3]) * inv_l);
-                        w4.z = pack_bf16x2(__uint_as_float(ov[e + 4]) * inv_l, __uint_as_float(ov[e + 5]) * inv_l);
-                        w4.w = pack_bf16x2(__uint_as_float(ov[e + 6]) * inv_l, __uint_as_float(ov[e + 7]) * inv_l);
-                        *reinterpret_cast<uint4*>(orow + c * 32 + e) = w4;
+                    for (int e = 0; e < 32; e += 16) {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) w[j] = pack_bf16x2(out(e + 2 * j), out(e + 2 * j + 1));
+                        if (p.o_wide) {
+                            st_global_v8(orow + c * 32 + e, w);
+                        } else {
+                            *reinterpret_cast<uint4*>(orow + c * 32 + e) = make_uint4(w[0], w[1], w[2], w[3]);
+                            *reinterpret_cast<uint4*>(orow + c * 32 + e + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+                        }
                     }
                 }
             }
-            if (valid && half == 0) p.lse[(size_t)hq * p.n + i] = (m_used + lg2_approx(l)) * LN2;
+            if (valid && half == 0) p.lse[(size_t)hq * p.n + i] = lse_row;
             tc_fence_before();
             ++it;
         }
@@ -1096,9 +1158,7 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     if constexpr (sorted) {
         // gather Q, K, V into the sorted order kept in the workspace; the kernel reads the copies
         char* ws = const_cast<char*>(a.ws);
-        if ((rc = launch_gather_sorted(&a.s, a.q, a.s.Hq, true, a.L, a.ws, ws + a.L.qs, st))) return rc;
-        if ((rc = launch_gather_sorted(&a.s, a.k, a.s.Hkv, false, a.L, a.ws, ws + a.L.ks, st))) return rc;
-        if ((rc = launch_gather_sorted(&a.s, a.v, a.s.Hkv, false, a.L, a.ws, ws + a.L.vs, st))) return rc;
+        if ((rc = launch_gather_sorted(&a.s, a.q, a.k, a.v, a.L, ws, st))) return rc;
         const int HQ = a.s.batch * a.s.Hq, HK = a.s.batch * a.s.Hkv;
         const focus_tensor sq_t{ws + a.L.qs, (int64_t)HQ * a.L.nqp * D, (int64_t)a.L.nqp * D, D};
         const focus_tensor sk_t{ws + a.L.ks, (int64_t)HK * a.L.nkp * D, (int64_t)a.L.nkp * D, D};
@@ -1121,6 +1181,8 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.live = a.ws ? reinterpret_cast<const uint32_t*>(a.ws + a.L.live) : nullptr;
     p.o = reinterpret_cast<__nv_bfloat16*>(a.o.ptr);
     p.o_sb = a.o.stride_b; p.o_sh = a.o.stride_h; p.o_sn = a.o.stride_n;
+    // rows of O on the 32-byte grid: whole sectors per store (a warp's stores go to 32 rows at a time)
+    p.o_wide = (uintptr_t)a.o.ptr % 32 == 0 && (a.o.stride_b | a.o.stride_h | a.o.stride_n) % 16 == 0;
     p.lse = a.lse;
     p.status = a.dev_status;
     p.nitems = (long long)a.s.batch * a.s.Hq * p.nqb;
@@ -1138,6 +1200,7 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.share_only = (sorted && layout_has_window_pass(a.L.layout)) ? 1 : 0;
     p.gbits_s = (sorted && a.L.layout == FOCUS_LAYOUT_GROUP_MAJOR) ? reinterpret_cast<const uint32_t*>(a.ws + a.L.gbits_s) : nullptr;
     p.o32 = a.o32;
+    p.join = a.join;
     p.wait_limit_ns = a.wait_limit_ns;
     p.stall_at = a.stall_at;
     if (sorted) p.nitems = (long long)a.s.batch * a.s.Hq * p.nqblk * p.ipb;
@@ -1147,11 +1210,8 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     auto kern = focus_attn_kernel<D, SOFTCAP, GATE, WALK>;
     constexpr uint32_t smem = C::OFF_CTL + (uint32_t)sizeof(SharedCtl) + (C::GATE_MMA ? (uint32_t)sizeof(GateCtl) : 0);
     static_assert(smem <= 227 * 1024, "shared memory of one block");
-    if ((rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                         "cudaFuncSetAttribute(attn)")))
-        return rc;
-    kern<<<(unsigned)p.nitems, C::THREADS, smem, st>>>(tq, tk, tv, p);
-    return check_cuda(cudaGetLastError(), "attention kernel launch");
+    if ((rc = check_cuda(allow_smem<focus_attn_kernel<D, SOFTCAP, GATE, WALK>>(smem), "cudaFuncSetAttribute(attn)"))) return rc;
+    return check_cuda(launch_dependent(kern, dim3((unsigned)p.nitems), dim3(C::THREADS), smem, st, tq, tk, tv, p), "attention kernel launch");
 }
 
 static int launch_attn_one(const AttnArgs& a, cudaStream_t st);
@@ -1159,7 +1219,8 @@ static int launch_attn_one(const AttnArgs& a, cudaStream_t st);
 int launch_attn_sm100(const AttnArgs& a, cudaStream_t st) {
     if (a.ws && layout_has_window_pass(a.L.layout) && !a.local_pass) {
         // (1) sharing pairs in the class-sorted order -> o, lse; rows of blocks without key tiles keep lse = -inf
-        // (2) window-only pairs in token order -> workspace; (3) join through the logsumexps
+        // (2) window-only pairs in token order, each row joined with what (1) left (a pass of its own for that read and wrote
+        // another 1.3 GB at 32 heads x 32768 tokens x 128: 202 us)
         char* ws = const_cast<char*>(a.ws);
         const size_t rows = (size_t)a.s.batch * a.s.Hq * a.s.n;
         int rc = launch_fill_f32(a.lse, rows, -INFINITY, st);
@@ -1169,10 +1230,8 @@ int launch_attn_sm100(const AttnArgs& a, cudaStream_t st) {
         if ((rc = launch_attn_one(s1, st))) return rc;
         AttnArgs s2 = a;
         s2.local_pass = true;
-        s2.o32 = reinterpret_cast<float*>(ws + a.L.o_local);
-        s2.lse = reinterpret_cast<float*>(ws + a.L.lse_local);
-        if ((rc = launch_attn_one(s2, st))) return rc;
-        return launch_merge_partials(&a.s, a.o, a.lse, s1.o32, s2.o32, s2.lse, st);
+        s2.join = s1.o32;
+        return launch_attn_one(s2, st);
     }
     return launch_attn_one(a, st);
 }

@@ -20,16 +20,34 @@ constexpr unsigned long long HASH_EMPTY = 0ull;
 
 __device__ __forceinline__ unsigned int hash_slot(uint32_t v) { return (v * 2654435761u) >> 24; }   // 0..255
 
+// Query and key heads go through the same steps, in the same launches: row r of a grid is head r of the query side, then
+// of the key side.
+struct SortSide {
+    const uint32_t* m;
+    unsigned long long* table;
+    uint32_t* cls;
+    int32_t *ncls, *hist, *cnt, *seg, *perm;
+    int heads, npad, pad, fill;          // pad = slots a class segment is rounded up to; fill = what perm holds in the padding
+};
+struct SortSides { SortSide s[2]; };
+__device__ __forceinline__ const SortSide& side_of(const SortSides& sides, int row, int& head) {
+    const bool second = row >= sides.s[0].heads;
+    head = second ? row - sides.s[0].heads : row;
+    return sides.s[second ? 1 : 0];
+}
+
 // ---------------------------------------------------------------------------------------------
 // 1. distinct mask values per head: block-local hash set, merged into a global one per head
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-collect_classes_kernel(const uint32_t* __restrict__ m, int n, unsigned long long* __restrict__ table) {
+collect_classes_kernel(const SortSides sides, int n, int nchunk) {
     __shared__ unsigned long long loc[SORT_HASH];
-    const int head = blockIdx.y;
+    int head;
+    const SortSide& sd = side_of(sides, blockIdx.x / nchunk, head);
+    const uint32_t* __restrict__ m = sd.m;
     for (int s = threadIdx.x; s < SORT_HASH; s += blockDim.x) loc[s] = HASH_EMPTY;
     __syncthreads();
-    const int t0 = blockIdx.x * SORT_CHUNK;
+    const int t0 = (blockIdx.x % nchunk) * SORT_CHUNK;
     for (int t = t0 + threadIdx.x; t < min(n, t0 + SORT_CHUNK); t += blockDim.x) {
         const uint32_t v = m[(size_t)head * n + t];
         const unsigned long long key = (1ull << 32) | v;
@@ -41,7 +59,7 @@ collect_classes_kernel(const uint32_t* __restrict__ m, int n, unsigned long long
         }
     }
     __syncthreads();
-    unsigned long long* glob = table + (size_t)head * SORT_HASH;
+    unsigned long long* glob = sd.table + (size_t)head * SORT_HASH;
     for (int i = threadIdx.x; i < SORT_HASH; i += blockDim.x) {
         const unsigned long long key = loc[i];
         if (key == HASH_EMPTY) continue;
@@ -56,14 +74,15 @@ collect_classes_kernel(const uint32_t* __restrict__ m, int n, unsigned long long
 
 // one block per head: compact the hash set, sort ascending, flag more than MAXC values
 __global__ void __launch_bounds__(SORT_HASH)
-finalize_classes_kernel(const unsigned long long* __restrict__ table, uint32_t* __restrict__ cls,
-                        int32_t* __restrict__ ncls, unsigned long long* counters) {
+finalize_classes_kernel(const SortSides sides, unsigned long long* counters) {
     __shared__ uint32_t vals[SORT_HASH];
     __shared__ int cnt;
-    const int head = blockIdx.x;
+    int head;
+    const SortSide& sd = side_of(sides, blockIdx.x, head);
+    uint32_t* __restrict__ cls = sd.cls;
     if (threadIdx.x == 0) cnt = 0;
     __syncthreads();
-    const unsigned long long key = table[(size_t)head * SORT_HASH + threadIdx.x];
+    const unsigned long long key = sd.table[(size_t)head * SORT_HASH + threadIdx.x];
     if (key != HASH_EMPTY) vals[atomicAdd(&cnt, 1)] = (uint32_t)key;
     __syncthreads();
     const int c = cnt;
@@ -73,8 +92,9 @@ finalize_classes_kernel(const unsigned long long* __restrict__ table, uint32_t* 
         for (int j = 0; j < c; ++j) rank += vals[j] < v;
         if (rank < MAXC) cls[(size_t)head * MAXC + rank] = v;
     }
+    if ((int)threadIdx.x >= c && threadIdx.x < MAXC) cls[(size_t)head * MAXC + threadIdx.x] = 0u;
     if (threadIdx.x == 0) {
-        ncls[head] = min(c, MAXC);
+        sd.ncls[head] = min(c, MAXC);
         if (c > MAXC) atomicAdd(&counters[4], 1ull);
     }
 }
@@ -94,45 +114,55 @@ __device__ __forceinline__ int class_index(const uint32_t* tab, int c, uint32_t 
 // 2. counting sort: per-chunk histograms, scan over chunks, stable scatter
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(SORT_CHUNK)
-chunk_hist_kernel(const uint32_t* __restrict__ m, int n, const uint32_t* __restrict__ cls,
-                  const int32_t* __restrict__ ncls, int nchunk, int32_t* __restrict__ hist) {
+chunk_hist_kernel(const SortSides sides, int n, int nchunk) {
     __shared__ uint32_t tab[MAXC];
     __shared__ int h[MAXC];
-    const int head = blockIdx.y, chunk = blockIdx.x;
-    if (threadIdx.x < MAXC) { tab[threadIdx.x] = cls[(size_t)head * MAXC + threadIdx.x]; h[threadIdx.x] = 0; }
+    int head;
+    const SortSide& sd = side_of(sides, blockIdx.x / nchunk, head);
+    const int chunk = blockIdx.x % nchunk;
+    if (threadIdx.x < MAXC) { tab[threadIdx.x] = sd.cls[(size_t)head * MAXC + threadIdx.x]; h[threadIdx.x] = 0; }
     __syncthreads();
-    const int c = ncls[head];
+    const int c = sd.ncls[head];
     const int t = chunk * SORT_CHUNK + threadIdx.x;
-    if (t < n) atomicAdd(&h[class_index(tab, c, m[(size_t)head * n + t])], 1);
+    const int ci = t < n ? class_index(tab, c, sd.m[(size_t)head * n + t]) : -1;
+    const unsigned int same = __match_any_sync(0xffffffffu, ci);
+    if (ci >= 0 && (threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&h[ci], __popc(same));        // one per warp and class
     __syncthreads();
-    if (threadIdx.x < MAXC) hist[((size_t)head * nchunk + chunk) * MAXC + threadIdx.x] = h[threadIdx.x];
+    if (threadIdx.x < MAXC) sd.hist[((size_t)head * nchunk + chunk) * MAXC + threadIdx.x] = h[threadIdx.x];
 }
 
 // one block of MAXC threads per head (thread = class): running offsets over the chunks, class
 // totals and padded segment starts
 __global__ void __launch_bounds__(MAXC)
-scan_chunks_kernel(int32_t* __restrict__ hist, int nchunk, const int32_t* __restrict__ ncls, int pad,
-                   int32_t* __restrict__ cnt, int32_t* __restrict__ seg, int npad, unsigned long long* counters) {
+scan_chunks_kernel(const SortSides sides, int nchunk, unsigned long long* counters) {
     __shared__ int tot[MAXC];
-    const int head = blockIdx.x, c = threadIdx.x;
+    int head;
+    const SortSide& sd = side_of(sides, blockIdx.x, head);
+    const int c = threadIdx.x;
     int run = 0;
-    for (int k = 0; k < nchunk; ++k) {
-        int32_t* p = hist + ((size_t)head * nchunk + k) * MAXC + c;
-        const int v = *p;
-        *p = run;                   // tokens of class c in earlier chunks
-        run += v;
+    constexpr int AHEAD = 16;       // loads under way at a time
+    for (int k0 = 0; k0 < nchunk; k0 += AHEAD) {
+        int32_t* p = sd.hist + ((size_t)head * nchunk + k0) * MAXC + c;
+        int v[AHEAD];
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) v[k] = k0 + k < nchunk ? p[(size_t)k * MAXC] : 0;
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) {
+            if (k0 + k < nchunk) p[(size_t)k * MAXC] = run;           // tokens of class c in earlier chunks
+            run += v[k];
+        }
     }
     tot[c] = run;
-    cnt[(size_t)head * MAXC + c] = run;
+    sd.cnt[(size_t)head * MAXC + c] = run;
     __syncthreads();
     if (c == 0) {
-        const int nc = ncls[head];
+        const int nc = sd.ncls[head];
         int s = 0;
         for (int j = 0; j <= MAXC; ++j) {
-            seg[(size_t)head * (MAXC + 1) + j] = s;
-            if (j < nc) s += (tot[j] + pad - 1) / pad * pad;
+            sd.seg[(size_t)head * (MAXC + 1) + j] = s;
+            if (j < nc) s += (tot[j] + sd.pad - 1) / sd.pad * sd.pad;
         }
-        if (s > npad) atomicAdd(&counters[4], 1ull);      // more entries than the sorted arrays hold (group-major lists of
+        if (s > sd.npad) atomicAdd(&counters[4], 1ull);      // more entries than the sorted arrays hold (group-major lists of
                                                           // masks with more than topk bits): the attention kernel refuses
     }
 }
@@ -143,22 +173,27 @@ __global__ void fill_kernel(int32_t* __restrict__ p, size_t count, int32_t value
 }
 
 // stable scatter: slot = segment start + tokens of the class in earlier chunks + earlier warps of
-// this chunk + earlier lanes of this warp
+// this chunk + earlier lanes of this warp.  Every block also fills its share of the padding slots.
 __global__ void __launch_bounds__(SORT_CHUNK)
-scatter_kernel(const uint32_t* __restrict__ m, int n, const uint32_t* __restrict__ cls, const int32_t* __restrict__ ncls,
-               int nchunk, const int32_t* __restrict__ base, const int32_t* __restrict__ seg, int npad,
-               int32_t* __restrict__ perm) {
+scatter_kernel(const SortSides sides, int n, int nchunk) {
     __shared__ uint32_t tab[MAXC];
     __shared__ int wcnt[SORT_CHUNK / 32][MAXC];
-    const int head = blockIdx.y, chunk = blockIdx.x;
+    __shared__ int seg[MAXC + 1], end[MAXC];
+    int head;
+    const SortSide& sd = side_of(sides, blockIdx.x / nchunk, head);
+    const int chunk = blockIdx.x % nchunk, npad = sd.npad;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x < MAXC) tab[threadIdx.x] = cls[(size_t)head * MAXC + threadIdx.x];
+    if (threadIdx.x < MAXC) tab[threadIdx.x] = sd.cls[(size_t)head * MAXC + threadIdx.x];
+    if (threadIdx.x <= MAXC) {
+        seg[threadIdx.x] = sd.seg[(size_t)head * (MAXC + 1) + threadIdx.x];
+        if (threadIdx.x < MAXC) end[threadIdx.x] = seg[threadIdx.x] + sd.cnt[(size_t)head * MAXC + threadIdx.x];
+    }
     for (int i = threadIdx.x; i < (SORT_CHUNK / 32) * MAXC; i += blockDim.x) (&wcnt[0][0])[i] = 0;
     __syncthreads();
-    const int c = ncls[head];
+    const int c = sd.ncls[head];
     const int t = chunk * SORT_CHUNK + threadIdx.x;
     const bool in = t < n;
-    const int ci = in ? class_index(tab, c, m[(size_t)head * n + t]) : -1;
+    const int ci = in ? class_index(tab, c, sd.m[(size_t)head * n + t]) : -1;
     const unsigned int same = __match_any_sync(0xffffffffu, ci);
     const int rank = __popc(same & ((1u << lane) - 1u));
     if (in && rank == 0) wcnt[warp][ci] = __popc(same);
@@ -172,10 +207,20 @@ scatter_kernel(const uint32_t* __restrict__ m, int n, const uint32_t* __restrict
         }
     }
     __syncthreads();
+    int32_t* __restrict__ perm = sd.perm + (size_t)head * npad;
     if (in) {
-        const int slot = seg[(size_t)head * (MAXC + 1) + ci] + base[((size_t)head * nchunk + chunk) * MAXC + ci] +
-                         wcnt[warp][ci] + rank;
-        if (slot < npad) perm[(size_t)head * npad + slot] = t;
+        const int slot = seg[ci] + sd.hist[((size_t)head * nchunk + chunk) * MAXC + ci] + wcnt[warp][ci] + rank;
+        if (slot < npad) perm[slot] = t;
+    }
+    // the padding: slots past the tokens of their class, and past the last class
+    const int share = (npad + nchunk - 1) / nchunk;
+    for (int slot = chunk * share + threadIdx.x; slot < min(npad, (chunk + 1) * share); slot += SORT_CHUNK) {
+        int lo = 0, hi = c - 1;             // last class that starts at or before the slot
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (seg[mid] <= slot) lo = mid; else hi = mid - 1;
+        }
+        if (slot >= end[lo]) perm[slot] = sd.fill;
     }
 }
 
@@ -276,18 +321,21 @@ qrange_kernel(int HQ, int Hq, int Hkv, int G_heads, int w, int nqp, int nkp, con
               const int32_t* __restrict__ cnt_q, const int32_t* __restrict__ cnt_k, const int32_t* __restrict__ seg_q,
               const int32_t* __restrict__ seg_k, const int32_t* __restrict__ perm_q, const int32_t* __restrict__ perm_k,
               int32_t* __restrict__ qrange, int32_t* __restrict__ cost, unsigned long long* counters, int sharing_only) {
+    // a block of 256 threads holds the classes of four query blocks: their costs are summed here (an atomic per thread on
+    // the one counter of all tiles made this launch 50 us long at 32 heads x 32768 tokens, 81 us at 131072)
+    __shared__ int sum_s[8];
     const int nqblk = nqp / 256;
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= (long long)HQ * nqblk * MAXC) return;
+    const bool in = gid < (long long)HQ * nqblk * MAXC;
     const int jk = (int)(gid % MAXC);
     const int blk = (int)((gid / MAXC) % nqblk);
-    const int hq = (int)(gid / ((long long)MAXC * nqblk));
+    const int hq = in ? (int)(gid / ((long long)MAXC * nqblk)) : 0;
     const int hk = (hq / Hq) * Hkv + (hq % Hq) / G_heads;
     int first = 0, last = 0;
     const int32_t* sq = seg_q + (size_t)hq * (MAXC + 1);
     const int ncq = ncls_q[hq], nck = ncls_k[hk];
     const int start = blk * 256;
-    if (jk < nck && start < sq[ncq]) {
+    if (in && jk < nck && start < sq[ncq]) {
         int jq = 0;
         while (jq + 1 < ncq && sq[jq + 1] <= start) ++jq;          // class of this query block
         const int valid_end = sq[jq] + cnt_q[(size_t)hq * MAXC + jq];    // one past the last real row of the class
@@ -304,11 +352,16 @@ qrange_kernel(int HQ, int Hq, int Hkv, int G_heads, int w, int nqp, int nkp, con
             last = (ks0 + hi + 127) / 128;
         }
     }
-    qrange[gid * 2] = first;
-    qrange[gid * 2 + 1] = last;
-    if (last > first) {
-        atomicAdd(&cost[(size_t)hq * nqblk + blk], last - first);
-        atomicAdd(&counters[3], (unsigned long long)(last - first));
+    if (in) reinterpret_cast<int2*>(qrange)[gid] = make_int2(first, last);
+    const int tiles = __reduce_add_sync(0xffffffffu, last - first);
+    if ((threadIdx.x & 31) == 0) sum_s[threadIdx.x >> 5] = tiles;
+    __syncthreads();
+    static_assert(MAXC == 64, "two warps per query block");
+    if (in && jk == 0) cost[(size_t)hq * nqblk + blk] = sum_s[threadIdx.x >> 5] + sum_s[(threadIdx.x >> 5) + 1];
+    if (threadIdx.x == 0) {
+        int all = 0;
+        for (int w = 0; w < 8; ++w) all += sum_s[w];
+        if (all) atomicAdd(&counters[3], (unsigned long long)all);
     }
 }
 
@@ -373,37 +426,71 @@ order_kernel(int Hq, int Hkv, int G_heads, int nqblk, int max_cost, const int32_
 }
 
 // ---------------------------------------------------------------------------------------------
-// 4. gather of Q / K / V rows into the sorted order (run by focus_attn_fwd), 16 bytes per thread
+// 4. gather of Q / K / V rows into the sorted order (run by focus_attn_fwd), one launch
 // ---------------------------------------------------------------------------------------------
+// Four rows per thread, all their loads under way at once (one row per thread: 4.5 TB/s read and written at 32 x 131072 x 128).
+constexpr int GATHER_ROWS = 4;
+struct GatherSide {
+    const __nv_bfloat16* src;
+    int64_t sb, sh, sn;
+    const int32_t* perm;
+    const int32_t* seg;
+    __nv_bfloat16* dst;
+    int H, npad, blocks;             // heads per sequence, slots per head, thread blocks per head
+};
+struct GatherSides { GatherSide s[3]; int first[3]; };       // first[k] = first block of side k
+
+template <int D>
 __global__ void __launch_bounds__(256)
-gather_rows_kernel(const __nv_bfloat16* __restrict__ src, int64_t sb, int64_t sh, int64_t sn, int H, int D,
-                   const int32_t* __restrict__ perm, const int32_t* __restrict__ seg, int npad, int n,
-                   __nv_bfloat16* __restrict__ dst) {
-    const int vec = D / 8;                               // 16-byte vectors per row
-    const int head = blockIdx.y;
-    const int used = seg[(size_t)head * (MAXC + 1) + MAXC];
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int slot = (int)(gid / vec), v = (int)(gid % vec);
-    if (slot >= used) return;
-    const int pos = perm[(size_t)head * npad + slot];
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);              // padding rows are zero
-    if (pos >= 0 && pos < n) {
-        const __nv_bfloat16* row = src + (size_t)(head / H) * sb + (size_t)(head % H) * sh + (size_t)pos * sn;
-        val = *reinterpret_cast<const uint4*>(row + v * 8);
+gather_rows_kernel(const GatherSides sides, int n) {
+    constexpr int VEC = D / 8, RPB = 256 / VEC;          // 16-byte pieces per row, rows a block covers at a time
+    const int k = (int)blockIdx.x >= sides.first[2] ? 2 : (int)blockIdx.x >= sides.first[1] ? 1 : 0;
+    const GatherSide& g = sides.s[k];
+    const int head = (blockIdx.x - sides.first[k]) / g.blocks, blk = (blockIdx.x - sides.first[k]) % g.blocks;
+    const int used = g.seg[(size_t)head * (MAXC + 1) + MAXC];
+    const int slot0 = blk * RPB * GATHER_ROWS + threadIdx.x / VEC, v = threadIdx.x % VEC;
+    if (slot0 >= used) return;
+    const __nv_bfloat16* src = g.src + (size_t)(head / g.H) * g.sb + (size_t)(head % g.H) * g.sh + v * 8;
+    int pos[GATHER_ROWS];
+    uint4 val[GATHER_ROWS];
+#pragma unroll
+    for (int r = 0; r < GATHER_ROWS; ++r) {
+        const int slot = slot0 + r * RPB;
+        pos[r] = slot < used ? g.perm[(size_t)head * g.npad + slot] : -1;
     }
-    *reinterpret_cast<uint4*>(dst + ((size_t)head * npad + slot) * D + v * 8) = val;
+#pragma unroll
+    for (int r = 0; r < GATHER_ROWS; ++r) {
+        val[r] = make_uint4(0u, 0u, 0u, 0u);             // padding rows are zero
+        if (pos[r] >= 0 && pos[r] < n) val[r] = *reinterpret_cast<const uint4*>(src + (size_t)pos[r] * g.sn);
+    }
+#pragma unroll
+    for (int r = 0; r < GATHER_ROWS; ++r) {
+        const int slot = slot0 + r * RPB;
+        if (slot < used) *reinterpret_cast<uint4*>(g.dst + ((size_t)head * g.npad + slot) * D + v * 8) = val[r];
+    }
 }
 
-int launch_gather_sorted(const focus_shape* s, const focus_tensor& t, int H, bool query, const focus_tiles_layout& L,
-                         const char* ws, char* dst, cudaStream_t st) {
-    const int heads = s->batch * H;
-    const int npad = query ? L.nqp : L.nkp;
-    const long long threads = (long long)npad * (s->D / 8);
-    gather_rows_kernel<<<dim3((unsigned)((threads + 255) / 256), heads), 256, 0, st>>>(
-        reinterpret_cast<const __nv_bfloat16*>(t.ptr), t.stride_b, t.stride_h, t.stride_n, H, s->D,
-        reinterpret_cast<const int32_t*>(ws + (query ? L.perm_q : L.perm_k)),
-        reinterpret_cast<const int32_t*>(ws + (query ? L.seg_q : L.seg_k)), npad, s->n,
-        reinterpret_cast<__nv_bfloat16*>(dst));
+int launch_gather_sorted(const focus_shape* s, const focus_tensor& q, const focus_tensor& k, const focus_tensor& v, const focus_tiles_layout& L,
+                         char* ws, cudaStream_t st) {
+    const int per_block = 256 / (s->D / 8) * GATHER_ROWS;
+    GatherSides sides;
+    long long blocks = 0;
+    for (int i = 0; i < 3; ++i) {
+        const focus_tensor& t = i == 0 ? q : i == 1 ? k : v;
+        const int npad = i == 0 ? L.nqp : L.nkp, H = i == 0 ? s->Hq : s->Hkv;
+        sides.s[i] = {reinterpret_cast<const __nv_bfloat16*>(t.ptr), t.stride_b, t.stride_h, t.stride_n,
+                      reinterpret_cast<const int32_t*>(ws + (i == 0 ? L.perm_q : L.perm_k)), reinterpret_cast<const int32_t*>(ws + (i == 0 ? L.seg_q : L.seg_k)),
+                      reinterpret_cast<__nv_bfloat16*>(ws + (i == 0 ? L.qs : i == 1 ? L.ks : L.vs)), H, npad, cdiv(npad, per_block)};
+        sides.first[i] = (int)blocks;
+        blocks += (long long)s->batch * H * sides.s[i].blocks;
+    }
+    if (blocks > 0x7fffffffll) return fail(FOCUS_ERR_CUDA, "gather: too many rows for one launch");
+    switch (s->D) {
+        case 64: gather_rows_kernel<64><<<(unsigned)blocks, 256, 0, st>>>(sides, s->n); break;
+        case 128: gather_rows_kernel<128><<<(unsigned)blocks, 256, 0, st>>>(sides, s->n); break;
+        case 256: gather_rows_kernel<256><<<(unsigned)blocks, 256, 0, st>>>(sides, s->n); break;
+        default: return fail(FOCUS_ERR_UNSUPPORTED, "D (%d) must be 64, 128 or 256", s->D);
+    }
     return check_cuda(cudaGetLastError(), "gather kernel");
 }
 
@@ -420,41 +507,35 @@ int launch_build_tiles_sorted(const focus_shape* s, const uint32_t* mq, const ui
     auto* hist = reinterpret_cast<int32_t*>(scr + table_bytes);
     const size_t hist_bytes = align_up((size_t)(HQ + HK) * nchunk * MAXC * 4, 256);
     auto* cost = reinterpret_cast<int32_t*>(scr + table_bytes + hist_bytes);
-    const size_t cost_bytes = (size_t)HQ * nqblk * 4;
     auto* counters = reinterpret_cast<unsigned long long*>(ws + L.counters);
     int rc;
     if ((rc = check_cuda(cudaMemsetAsync(table, 0, table_bytes, st), "cudaMemsetAsync(class tables)"))) return rc;
-    if ((rc = check_cuda(cudaMemsetAsync(cost, 0, cost_bytes, st), "cudaMemsetAsync(block costs)"))) return rc;
-    if ((rc = check_cuda(cudaMemsetAsync(ws + L.cls_q, 0, (size_t)HQ * MAXC * 4, st), "cudaMemsetAsync(cls_q)"))) return rc;
-    if ((rc = check_cuda(cudaMemsetAsync(ws + L.cls_k, 0, (size_t)HK * MAXC * 4, st), "cudaMemsetAsync(cls_k)"))) return rc;
-
-    for (int side = 0; side < 2; ++side) {
-        const int heads = side ? HK : HQ;
-        const uint32_t* m = side ? mk : mq;
-        unsigned long long* tab = table + (side ? (size_t)HQ * SORT_HASH : 0);
-        int32_t* hs = hist + (side ? (size_t)HQ * nchunk * MAXC : 0);
-        auto* cls = reinterpret_cast<uint32_t*>(ws + (side ? L.cls_k : L.cls_q));
-        auto* ncls = reinterpret_cast<int32_t*>(ws + (side ? L.ncls_k : L.ncls_q));
-        auto* cnt = reinterpret_cast<int32_t*>(ws + (side ? L.cnt_k : L.cnt_q));
-        auto* seg = reinterpret_cast<int32_t*>(ws + (side ? L.seg_k : L.seg_q));
-        auto* perm = reinterpret_cast<int32_t*>(ws + (side ? L.perm_k : L.perm_q));
-        const int npad = side ? L.nkp : L.nqp;
-        if (side && L.layout == FOCUS_LAYOUT_GROUP_MAJOR) {
-            group_classes_kernel<<<cdiv(heads * MAXC, 256), 256, 0, st>>>(heads, s->K, cls, ncls);
-            group_hist_kernel<<<dim3(nchunk, heads), SORT_CHUNK, 0, st>>>(m, s->n, s->K, nchunk, hs);
-            scan_chunks_kernel<<<heads, MAXC, 0, st>>>(hs, nchunk, ncls, 128, cnt, seg, npad, counters);
-            fill_kernel<<<1184, 256, 0, st>>>(perm, (size_t)heads * npad, INT_MAX);
-            group_scatter_kernel<<<dim3(nchunk, heads), SORT_CHUNK, 0, st>>>(m, s->n, s->K, nchunk, hs, seg, npad, perm);
-            gbits_sorted_kernel<<<dim3(npad / 128, heads), 128, 0, st>>>(m, s->n, s->K, perm, npad,
-                                                                         reinterpret_cast<uint32_t*>(ws + L.gbits_s));
-            continue;
-        }
-        collect_classes_kernel<<<dim3(nchunk, heads), 256, 0, st>>>(m, s->n, tab);
-        finalize_classes_kernel<<<heads, SORT_HASH, 0, st>>>(tab, cls, ncls, counters);
-        chunk_hist_kernel<<<dim3(nchunk, heads), SORT_CHUNK, 0, st>>>(m, s->n, cls, ncls, nchunk, hs);
-        scan_chunks_kernel<<<heads, MAXC, 0, st>>>(hs, nchunk, ncls, side ? 128 : 256, cnt, seg, npad, counters);
-        fill_kernel<<<1184, 256, 0, st>>>(perm, (size_t)heads * npad, side ? INT_MAX : -1);
-        scatter_kernel<<<dim3(nchunk, heads), SORT_CHUNK, 0, st>>>(m, s->n, cls, ncls, nchunk, hs, seg, npad, perm);
+    SortSides sides;
+    for (int k = 0; k < 2; ++k)
+        sides.s[k] = {k ? mk : mq, table + (k ? (size_t)HQ * SORT_HASH : 0), reinterpret_cast<uint32_t*>(ws + (k ? L.cls_k : L.cls_q)),
+                      reinterpret_cast<int32_t*>(ws + (k ? L.ncls_k : L.ncls_q)), hist + (k ? (size_t)HQ * nchunk * MAXC : 0),
+                      reinterpret_cast<int32_t*>(ws + (k ? L.cnt_k : L.cnt_q)), reinterpret_cast<int32_t*>(ws + (k ? L.seg_k : L.seg_q)),
+                      reinterpret_cast<int32_t*>(ws + (k ? L.perm_k : L.perm_q)), k ? HK : HQ, k ? L.nkp : L.nqp, k ? 128 : 256, k ? INT_MAX : -1};
+    // group-major keys have lists of their own: only the query side is sorted by class
+    const bool lists = L.layout == FOCUS_LAYOUT_GROUP_MAJOR;
+    const int rows = lists ? HQ : HQ + HK;
+    if ((long long)rows * nchunk > 0x7fffffffll) return fail(FOCUS_ERR_CUDA, "build_tiles: too many chunks of %d tokens for one launch", SORT_CHUNK);
+    const unsigned grid = (unsigned)rows * (unsigned)nchunk;
+    collect_classes_kernel<<<grid, 256, 0, st>>>(sides, s->n, nchunk);
+    finalize_classes_kernel<<<rows, SORT_HASH, 0, st>>>(sides, counters);
+    chunk_hist_kernel<<<grid, SORT_CHUNK, 0, st>>>(sides, s->n, nchunk);
+    scan_chunks_kernel<<<rows, MAXC, 0, st>>>(sides, nchunk, counters);
+    scatter_kernel<<<grid, SORT_CHUNK, 0, st>>>(sides, s->n, nchunk);
+    if (lists) {
+        SortSides keys;
+        keys.s[0] = keys.s[1] = sides.s[1];
+        const SortSide& k = keys.s[0];
+        group_classes_kernel<<<cdiv(HK * MAXC, 256), 256, 0, st>>>(HK, s->K, k.cls, k.ncls);
+        group_hist_kernel<<<dim3(nchunk, HK), SORT_CHUNK, 0, st>>>(mk, s->n, s->K, nchunk, k.hist);
+        scan_chunks_kernel<<<HK, MAXC, 0, st>>>(keys, nchunk, counters);
+        fill_kernel<<<1184, 256, 0, st>>>(k.perm, (size_t)HK * k.npad, INT_MAX);
+        group_scatter_kernel<<<dim3(nchunk, HK), SORT_CHUNK, 0, st>>>(mk, s->n, s->K, nchunk, k.hist, k.seg, k.npad, k.perm);
+        gbits_sorted_kernel<<<dim3(k.npad / 128, HK), 128, 0, st>>>(mk, s->n, s->K, k.perm, k.npad, reinterpret_cast<uint32_t*>(ws + L.gbits_s));
     }
     const long long nthreads = (long long)HQ * nqblk * MAXC;
     qrange_kernel<<<(unsigned)((nthreads + 255) / 256), 256, 0, st>>>(
@@ -470,9 +551,6 @@ int launch_build_tiles_sorted(const focus_shape* s, const uint32_t* mq, const ui
     return check_cuda(cudaGetLastError(), "build_tiles (class-sorted) kernels");
 }
 
-// ---- FOCUS_LAYOUT_SORTED_LOCAL: the two partial results (sharing pairs from the class-sorted pass, window-only pairs
-// from the pass in token order) cover disjoint sets of pairs and join through their logsumexps (paper Appendix D).
-
 __global__ void __launch_bounds__(256) fill_f32_kernel(float* __restrict__ x, size_t count, float v) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) x[i] = v;
@@ -481,73 +559,6 @@ __global__ void __launch_bounds__(256) fill_f32_kernel(float* __restrict__ x, si
 int launch_fill_f32(float* x, size_t count, float v, cudaStream_t st) {
     fill_f32_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(x, count, v);
     return check_cuda(cudaGetLastError(), "fill kernel launch");
-}
-
-// thread = 8 consecutive elements of a row; the D/8 threads of a row sit in one warp, so that all of them have read the
-// row's two logsumexps before the first of them overwrites one
-template <int D>
-__global__ void __launch_bounds__(256)
-merge_partials_kernel(__nv_bfloat16* __restrict__ o, int64_t o_sb, int64_t o_sh, int64_t o_sn, float* __restrict__ lse,
-                      const float* __restrict__ o_sorted, const float* __restrict__ o_local, const float* __restrict__ lse_local,
-                      int Hq, int n) {
-    constexpr int TPR = D / 8;
-    const int hq = blockIdx.y;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long i = t / TPR;
-    const int c = (int)(t % TPR);
-    const bool in = i < n;
-    float ls = -INFINITY, ll = -INFINITY;
-    if (in) {
-        ls = lse[(size_t)hq * n + i];
-        ll = lse_local[(size_t)hq * n + i];
-    }
-    __syncwarp();
-    if (!in) return;
-    const float m = fmaxf(ls, ll);
-    const float ws = m == -INFINITY ? 0.f : __expf(ls - m), wl = m == -INFINITY ? 0.f : __expf(ll - m);
-    const float tot = ws + wl;
-    const float inv = tot > 0.f ? 1.f / tot : 0.f;
-    const size_t src = ((size_t)hq * n + i) * D + c * 8;
-    float r[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) r[e] = 0.f;
-    // a partial result without any pair has weight 0 and unspecified contents: it is not read
-    if (ws > 0.f) {
-        const float4 a0 = *reinterpret_cast<const float4*>(o_sorted + src), a1 = *reinterpret_cast<const float4*>(o_sorted + src + 4);
-        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) r[e] = av[e] * ws;
-    }
-    if (wl > 0.f) {
-        const float4 b0 = *reinterpret_cast<const float4*>(o_local + src), b1 = *reinterpret_cast<const float4*>(o_local + src + 4);
-        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) r[e] = fmaf(bv[e], wl, r[e]);
-    }
-    uint32_t rw[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const __nv_bfloat162 h2 = __floats2bfloat162_rn(r[2 * e] * inv, r[2 * e + 1] * inv);
-        rw[e] = *reinterpret_cast<const uint32_t*>(&h2);
-    }
-    __nv_bfloat16* orow = o + (size_t)(hq / Hq) * o_sb + (size_t)(hq % Hq) * o_sh + (size_t)i * o_sn + c * 8;
-    *reinterpret_cast<uint4*>(orow) = make_uint4(rw[0], rw[1], rw[2], rw[3]);
-    if (c == 0) lse[(size_t)hq * n + i] = tot > 0.f ? m + __logf(tot) : -INFINITY;
-}
-
-int launch_merge_partials(const focus_shape* s, const focus_tensor& o, float* lse, const float* o_sorted, const float* o_local,
-                          const float* lse_local, cudaStream_t st) {
-    const int HQ = s->batch * s->Hq;
-    const long long threads = (long long)s->n * (s->D / 8);
-    const dim3 grid((unsigned)((threads + 255) / 256), HQ);
-    auto* op = reinterpret_cast<__nv_bfloat16*>(o.ptr);
-    switch (s->D) {
-        case 64: merge_partials_kernel<64><<<grid, 256, 0, st>>>(op, o.stride_b, o.stride_h, o.stride_n, lse, o_sorted, o_local, lse_local, s->Hq, s->n); break;
-        case 128: merge_partials_kernel<128><<<grid, 256, 0, st>>>(op, o.stride_b, o.stride_h, o.stride_n, lse, o_sorted, o_local, lse_local, s->Hq, s->n); break;
-        case 256: merge_partials_kernel<256><<<grid, 256, 0, st>>>(op, o.stride_b, o.stride_h, o.stride_n, lse, o_sorted, o_local, lse_local, s->Hq, s->n); break;
-        default: return fail(FOCUS_ERR_UNSUPPORTED, "D (%d) must be 64, 128 or 256", s->D);
-    }
-    return check_cuda(cudaGetLastError(), "merge kernel launch");
 }
 
 }  // namespace focus
