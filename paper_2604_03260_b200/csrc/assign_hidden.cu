@@ -16,6 +16,10 @@
 // states sum to the fp32 dot product) as the second operand.  One thread issues the MMAs of the chunk, which
 // accumulate S = H F'^T (128 x 3K, fp32) in tensor memory over the chunks of the tile; after the last chunk every
 // thread reads its row of S, adds the three terms per group and the bias, and selects (or stores the scores).
+//
+// Few tokens: a tile is one block's work for d / 128 chunks in series, whatever the rest of the chip does.  While the tiles
+// leave places free, a cluster of 2, 4 or 8 blocks takes a tile, each a range of d, and the first block adds the others'
+// partial scores (fp32, through distributed shared memory).
 #include "assign_common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -64,7 +68,7 @@ __global__ void __launch_bounds__(AH_THREADS)
 assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int64_t stride_n, int n, int d, int K, int topk,
                      const float* __restrict__ folded, const float* __restrict__ bias, int Hq, int Hkv,
                      uint32_t* __restrict__ mq, uint32_t* __restrict__ mk, unsigned long long* near_ties, float eps,
-                     float* __restrict__ scores, int ntile, int share, int extra) {
+                     float* __restrict__ scores, int ntile, int share, int extra, int split) {
     using Cfg = HiddenCfg<KMAX>;
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t base = smem_u32(sm);
@@ -74,10 +78,13 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
 
     // block i takes `share` tiles, the first `extra` blocks one more: tiles item0 .. item0 + T - 1 of the list
     // (batch, tile); its work is the T * nchunk chunks of those tiles, walked in order
-    const int item0 = blockIdx.x * share + min((int)blockIdx.x, extra);
-    const int T = share + ((int)blockIdx.x < extra ? 1 : 0);
+    // (split > 1: one tile per cluster of `split` blocks, block r of it chunks c_begin .. c_end - 1)
+    const int rank = split > 1 ? (int)cluster_ctarank() : 0;
+    const int item0 = split > 1 ? (int)blockIdx.x / split : blockIdx.x * share + min((int)blockIdx.x, extra);
+    const int T = split > 1 ? 1 : share + ((int)blockIdx.x < extra ? 1 : 0);
     const int nchunk = (d + AH_CHUNK - 1) / AH_CHUNK;
-    const int total = T * nchunk;
+    const int c_begin = nchunk * rank / split, c_end = nchunk * (rank + 1) / split;
+    const int total = T * (c_end - c_begin);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the swizzle is a function of the shared-memory address: a base off the 1024-byte grid would scramble both
     // operands, so such a block reports a fault and computes nothing
@@ -88,7 +95,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
     // written or counted; pieces past d are zero), folded vectors split on the way in (thread = column).  Every
     // call commits one group, empty when the chunk does not exist.  (it, ic) = tile and chunk of the next call.
     const int r0 = threadIdx.x / CPR, cc = threadIdx.x % CPR;
-    int it_next = 0, ic_next = 0;
+    int it_next = 0, ic_next = c_begin;
     constexpr int FPT = KMAX * AH_CHUNK / AH_THREADS;          // folded values per thread and chunk
     float fv[FPT];                                             // those of the chunk the next call stages, loaded one call ahead
     auto load_folded = [&]() {
@@ -134,7 +141,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
                 *reinterpret_cast<__nv_bfloat16*>(fp + sw128_offset(KMAX + g, col, Cfg::NCOLS)) = mid;
                 *reinterpret_cast<__nv_bfloat16*>(fp + sw128_offset(2 * KMAX + g, col, Cfg::NCOLS)) = lo;
             }
-            if (++ic_next == nchunk) { ic_next = 0; ++it_next; }
+            if (++ic_next == c_end) { ic_next = c_begin; ++it_next; }
             if (j + 1 < total) load_folded();
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -170,7 +177,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
 
     bool ok = aligned;
     unsigned int near_votes = 0;
-    int it = 0, ic = 0;                                        // tile and chunk of iteration j
+    int it = 0, ic = c_begin;                                  // tile and chunk of iteration j
     for (int j = 0; j < total; ++j) {
         const int buf = j % AH_NS;
         asm volatile("cp.async.wait_group %0;" ::"n"(AH_NS - 2) : "memory");   // this thread's copies of chunk j have landed
@@ -187,7 +194,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
 #pragma unroll
                 for (int ks = 0; ks < AH_CHUNK / 16; ++ks)
                     umma_ss(tmem, ad + (uint64_t)(((ks / 4) * Cfg::SUB_BYTES + (ks % 4) * 32) >> 4),
-                            fd + (uint64_t)(((ks / 4) * Cfg::FSUB_BYTES + (ks % 4) * 32) >> 4), IDESC, (ic > 0 || ks > 0) ? 1u : 0u);
+                            fd + (uint64_t)(((ks / 4) * Cfg::FSUB_BYTES + (ks % 4) * 32) >> 4), IDESC, (ic > c_begin || ks > 0) ? 1u : 0u);
                 umma_commit(smem_u32(&ctl->mma_done[buf]));
             }
             __syncwarp();
@@ -199,7 +206,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
             ctl->fault = 1;
         }
         stage_chunk(j + AH_NS - 1);
-        const bool last_chunk = ic == nchunk - 1;
+        const bool last_chunk = ic == c_end - 1;
         float sc3[Cfg::NCOLS];
         if (last_chunk) {
             if (ok && !mbar_wait(smem_u32(&ctl->mma_done[buf]), (uint32_t)((j / AH_NS) & 1))) {
@@ -230,9 +237,31 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
             float score[KMAX];
 #pragma unroll
             for (int g = 0; g < KMAX; ++g)
-                score[g] = ((sc3[2 * KMAX + g] + sc3[KMAX + g]) + sc3[g]) + ((bias && g < K) ? __ldg(bias + g) : 0.f);
+                score[g] = (sc3[2 * KMAX + g] + sc3[KMAX + g]) + sc3[g];
+            if (split > 1) {
+                // the stages are free: every MMA of this block has completed and no copy is on its way
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncthreads();
+                float* const mine = reinterpret_cast<float*>(sm) + threadIdx.x;
+#pragma unroll
+                for (int g = 0; g < KMAX; ++g) mine[g * AH_THREADS] = score[g];
+                mine[KMAX * AH_THREADS] = ok ? 1.f : 0.f;
+                cluster_sync_all();
+                if (rank == 0) {
+                    for (int r = 1; r < split; ++r) {
+                        const uint32_t theirs = mapa_shared(smem_u32(mine), r);
+#pragma unroll
+                        for (int g = 0; g < KMAX; ++g) score[g] += ld_shared_cluster_f32(theirs + g * AH_THREADS * 4);
+                        ok = ld_shared_cluster_f32(theirs + KMAX * AH_THREADS * 4) != 0.f && ok;
+                    }
+                }
+                cluster_sync_all();                            // the others' shared memory has been read
+            }
+            const bool own = rank == 0;
+#pragma unroll
+            for (int g = 0; g < KMAX; ++g) score[g] += (bias && g < K) ? __ldg(bias + g) : 0.f;
             if (scores) {   // the scores themselves (training-time soft assignment), rows of KMAX floats, zero beyond K
-                if (in && ok) {
+                if (in && ok && own) {
                     float4* o = reinterpret_cast<float4*>(scores + ((size_t)b * n + tok) * KMAX);
 #pragma unroll
                     for (int c = 0; c < KMAX / 4; ++c)
@@ -242,14 +271,14 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
             } else {
                 float last, next;
                 const uint32_t taken = select_topk<KMAX>(score, K, topk, last, next);
-                if (in && ok) {   // every head of the layer shares the token's mask
+                if (in && ok && own) {   // every head of the layer shares the token's mask
                     if (mq) for (int hh = 0; hh < Hq; ++hh) mq[((size_t)b * Hq + hh) * n + tok] = taken;
                     if (mk) for (int hh = 0; hh < Hkv; ++hh) mk[((size_t)b * Hkv + hh) * n + tok] = taken;
                 }
-                if (near_ties) near_votes += __popc(__ballot_sync(0xffffffffu, ok && in && topk < K && (last - next) < eps));
+                if (near_ties) near_votes += __popc(__ballot_sync(0xffffffffu, ok && own && in && topk < K && (last - next) < eps));
             }
         }
-        if (++ic == nchunk) { ic = 0; ++it; }
+        if (++ic == c_end) { ic = c_begin; ++it; }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (near_ties && lane == 0 && near_votes) atomicAdd(near_ties, (unsigned long long)near_votes);
@@ -287,10 +316,29 @@ static int launch_k(const focus_shape* s, const void* h, int64_t sb, int64_t sn,
     if (nitems == 0) return 0;
     if (nitems > 0x7fffffffll || (long long)(nitems / (nitems < resident ? nitems : resident) + 1) * cdiv(d, AH_CHUNK) > 0x7fffffffll)
         return fail(FOCUS_ERR_UNSUPPORTED, "focus_assign_hidden: too many chunks of 128 x 128 elements for one launch");
+    // blocks per tile: as many as there are places for, with two chunks each at least
+    int split = 1;
+    while (split < 8 && nitems * split * 2 <= (long long)sms * (per_sm < 2 ? per_sm : 2) && cdiv(d, AH_CHUNK) >= 4 * split) split *= 2;
     const int nblocks = (int)(nitems < resident ? nitems : resident);
     const int share = (int)(nitems / nblocks), extra = (int)(nitems % nblocks);
+    if (split > 1) {
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(nitems * split));
+        cfg.blockDim = dim3(AH_THREADS);
+        cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
+        cfg.stream = st;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        return check_cuda(cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<const __nv_bfloat16*>(h), sb, sn, s->n, d, s->K, s->topk, folded, bias, s->Hq,
+                                             s->Hkv, mq, mk, near_ties, eps, scores, ntile, 1, 0, split), "assign_hidden kernel launch");
+    }
     return check_cuda(launch_dependent(kern, dim3(nblocks), dim3(AH_THREADS), Cfg::SMEM_BYTES, st, reinterpret_cast<const __nv_bfloat16*>(h), sb, sn,
-                                       s->n, d, s->K, s->topk, folded, bias, s->Hq, s->Hkv, mq, mk, near_ties, eps, scores, ntile, share, extra),
+                                       s->n, d, s->K, s->topk, folded, bias, s->Hq, s->Hkv, mq, mk, near_ties, eps, scores, ntile, share, extra, 1),
                       "assign_hidden kernel launch");
 }
 
