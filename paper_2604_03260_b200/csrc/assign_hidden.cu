@@ -9,7 +9,7 @@
 // Scoring runs on the tensor cores.  The tiles of 128 tokens are dealt out as one contiguous range per block,
 // one resident wave of small blocks.  A block walks its tiles in chunks of 128 elements of d: the chunk of the
 // 128 rows goes to shared memory with coalesced asynchronous 16-byte copies, laid out as the K-major,
-// 128-byte-swizzled operand of a tcgen05 MMA, in a ring of three stages (a stage is refilled as soon as the
+// 128-byte-swizzled operand of a tcgen05 MMA, in a ring of stages (with three, a stage is refilled as soon as the
 // MMAs of the chunk before the current one are done, so two chunks are in flight while a third is multiplied);
 // the same chunk of the K folded vectors (loaded into registers one chunk ahead) is
 // split into three bf16 terms each (hi + mid + lo carries 24 mantissa bits, so the products with the bf16 hidden
@@ -28,24 +28,26 @@ namespace focus {
 using namespace ptx;
 
 constexpr int AH_THREADS = 128;      // one thread per token of the tile = one lane of tensor memory
-constexpr int AH_CHUNK = 128;        // elements of d per stage: two 64-column sub-tiles
-constexpr int AH_NS = 3;             // stages of the chunk ring: one being read by the MMAs, two being filled
 
 template <int KMAX>
 struct HiddenCfg {
+    static constexpr int CHUNK = 128;                                    // elements of d per stage: two 64-column sub-tiles
+    // Stages of the chunk ring: one being read by the MMAs, the others being filled.  Three where two blocks still fit an SM
+    // (K <= 4: 36 KB a stage), else two (K = 8: one block of three stages 72.4 us for 32768 x 4096, two of two 61.4).
+    static constexpr int NS = KMAX <= 4 ? 3 : 2;
     static constexpr int NCOLS = (3 * KMAX + 15) / 16 * 16;             // rows of F' = columns of S
     static constexpr uint32_t SUB_BYTES = 128 * 128;                     // 128 tokens x 64 elements
-    static constexpr uint32_t A_BYTES = (AH_CHUNK / 64) * SUB_BYTES;
+    static constexpr uint32_t A_BYTES = (CHUNK / 64) * SUB_BYTES;
     static constexpr uint32_t FSUB_BYTES = NCOLS * 128;                  // NCOLS rows x 64 elements
-    static constexpr uint32_t F_BYTES = (AH_CHUNK / 64) * FSUB_BYTES;
+    static constexpr uint32_t F_BYTES = (CHUNK / 64) * FSUB_BYTES;
     static constexpr uint32_t STAGE_BYTES = A_BYTES + F_BYTES;
     static constexpr uint32_t TMEM_COLS = NCOLS <= 32 ? 32 : (NCOLS <= 64 ? 64 : 128);
-    static constexpr uint32_t SMEM_BYTES = AH_NS * STAGE_BYTES + 256;
+    static constexpr uint32_t SMEM_BYTES = NS * STAGE_BYTES + 256;
     static_assert(STAGE_BYTES % 1024 == 0, "every operand starts on a swizzle atom");
 };
 
 struct HiddenCtl {
-    uint64_t mma_done[AH_NS];         // the MMAs that read the stage have completed
+    uint64_t mma_done[3];         // the MMAs that read the stage have completed
     uint32_t tmem_base;
     int fault;
 };
@@ -72,8 +74,8 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
     using Cfg = HiddenCfg<KMAX>;
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t base = smem_u32(sm);
-    HiddenCtl* const ctl = reinterpret_cast<HiddenCtl*>(sm + AH_NS * Cfg::STAGE_BYTES);
-    constexpr int CPR = AH_CHUNK / 8;                          // 16-byte pieces per row of a chunk
+    HiddenCtl* const ctl = reinterpret_cast<HiddenCtl*>(sm + Cfg::NS * Cfg::STAGE_BYTES);
+    constexpr int CPR = Cfg::CHUNK / 8;                          // 16-byte pieces per row of a chunk
     constexpr int RSTEP = AH_THREADS / CPR;                    // rows covered by one copy per thread (8)
 
     // block i takes `share` tiles, the first `extra` blocks one more: tiles item0 .. item0 + T - 1 of the list
@@ -82,7 +84,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
     const int rank = split > 1 ? (int)cluster_ctarank() : 0;
     const int item0 = split > 1 ? (int)blockIdx.x / split : blockIdx.x * share + min((int)blockIdx.x, extra);
     const int T = split > 1 ? 1 : share + ((int)blockIdx.x < extra ? 1 : 0);
-    const int nchunk = (d + AH_CHUNK - 1) / AH_CHUNK;
+    const int nchunk = (d + Cfg::CHUNK - 1) / Cfg::CHUNK;
     const int c_begin = nchunk * rank / split, c_end = nchunk * (rank + 1) / split;
     const int total = T * (c_end - c_begin);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -96,14 +98,14 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
     // call commits one group, empty when the chunk does not exist.  (it, ic) = tile and chunk of the next call.
     const int r0 = threadIdx.x / CPR, cc = threadIdx.x % CPR;
     int it_next = 0, ic_next = c_begin;
-    constexpr int FPT = KMAX * AH_CHUNK / AH_THREADS;          // folded values per thread and chunk
+    constexpr int FPT = KMAX * Cfg::CHUNK / AH_THREADS;          // folded values per thread and chunk
     float fv[FPT];                                             // those of the chunk the next call stages, loaded one call ahead
     auto load_folded = [&]() {
-        const int e0 = ic_next * AH_CHUNK;
+        const int e0 = ic_next * Cfg::CHUNK;
 #pragma unroll
         for (int i = 0; i < FPT; ++i) {
             const int q = i * AH_THREADS + threadIdx.x;
-            const int g = q / AH_CHUNK, e = e0 + q % AH_CHUNK;
+            const int g = q / Cfg::CHUNK, e = e0 + q % Cfg::CHUNK;
             fv[i] = (g < K && e < d) ? __ldg(folded + (size_t)g * d + e) : 0.f;
         }
     };
@@ -111,9 +113,9 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
         if (j < total) {
             const int item = item0 + it_next;
             const int b = item / ntile, tok0 = (item % ntile) * 128;
-            const int e0 = ic_next * AH_CHUNK;
-            unsigned char* const st = sm + (j % AH_NS) * Cfg::STAGE_BYTES;
-            const uint32_t dstb = base + (j % AH_NS) * Cfg::STAGE_BYTES + (cc >> 3) * Cfg::SUB_BYTES + r0 * 128 +
+            const int e0 = ic_next * Cfg::CHUNK;
+            unsigned char* const st = sm + (j % Cfg::NS) * Cfg::STAGE_BYTES;
+            const uint32_t dstb = base + (j % Cfg::NS) * Cfg::STAGE_BYTES + (cc >> 3) * Cfg::SUB_BYTES + r0 * 128 +
                                   ((((uint32_t)cc & 7u) ^ ((uint32_t)r0 & 7u)) << 4);
             if (e0 + cc * 8 < d) {
                 const __nv_bfloat16* src = h + (size_t)b * stride_b + (size_t)(tok0 + r0) * stride_n + e0 + cc * 8;
@@ -134,7 +136,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
 #pragma unroll
             for (int i = 0; i < FPT; ++i) {
                 const int q = i * AH_THREADS + threadIdx.x;
-                const int g = q / AH_CHUNK, col = q % AH_CHUNK;
+                const int g = q / Cfg::CHUNK, col = q % Cfg::CHUNK;
                 __nv_bfloat16 hi, mid, lo;
                 split3_bf16(fv[i], hi, mid, lo);
                 *reinterpret_cast<__nv_bfloat16*>(fp + sw128_offset(g, col, Cfg::NCOLS)) = hi;
@@ -151,8 +153,8 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
     {
         constexpr int ZROWS = Cfg::NCOLS - 3 * KMAX;
         if constexpr (ZROWS > 0) {
-            constexpr int NSUB = AH_CHUNK / 64;
-            for (int i = threadIdx.x; i < AH_NS * NSUB * ZROWS * 8; i += AH_THREADS) {
+            constexpr int NSUB = Cfg::CHUNK / 64;
+            for (int i = threadIdx.x; i < Cfg::NS * NSUB * ZROWS * 8; i += AH_THREADS) {
                 const int stg = i / (NSUB * ZROWS * 8), rem = i % (NSUB * ZROWS * 8);
                 const int sub = rem / (ZROWS * 8), q = rem % (ZROWS * 8);
                 *reinterpret_cast<uint4*>(sm + stg * Cfg::STAGE_BYTES + Cfg::A_BYTES + sub * Cfg::FSUB_BYTES + (3 * KMAX) * 128 + q * 16) =
@@ -165,7 +167,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
         tmem_relinquish();
     }
     if (threadIdx.x == 32) {
-        for (int i = 0; i < AH_NS; ++i) mbar_init(smem_u32(&ctl->mma_done[i]), 1);
+        for (int i = 0; i < Cfg::NS; ++i) mbar_init(smem_u32(&ctl->mma_done[i]), 1);
         fence_mbar_init();
         ctl->fault = 0;
     }
@@ -173,14 +175,14 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
     dep_trigger();
     load_folded();
 #pragma unroll
-    for (int j = 0; j < AH_NS - 1; ++j) stage_chunk(j);
+    for (int j = 0; j < Cfg::NS - 1; ++j) stage_chunk(j);
 
     bool ok = aligned;
     unsigned int near_votes = 0;
     int it = 0, ic = c_begin;                                  // tile and chunk of iteration j
     for (int j = 0; j < total; ++j) {
-        const int buf = j % AH_NS;
-        asm volatile("cp.async.wait_group %0;" ::"n"(AH_NS - 2) : "memory");   // this thread's copies of chunk j have landed
+        const int buf = j % Cfg::NS;
+        asm volatile("cp.async.wait_group %0;" ::"n"(Cfg::NS - 2) : "memory");   // this thread's copies of chunk j have landed
         fence_proxy_async_smem();                              // generic-proxy writes before the MMA's async-proxy reads
         tc_fence_before();
         __syncthreads();
@@ -192,7 +194,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
                 const uint64_t ad = smem_desc_sw128(base + buf * Cfg::STAGE_BYTES, 16, 1024);
                 const uint64_t fd = smem_desc_sw128(base + buf * Cfg::STAGE_BYTES + Cfg::A_BYTES, 16, 1024);
 #pragma unroll
-                for (int ks = 0; ks < AH_CHUNK / 16; ++ks)
+                for (int ks = 0; ks < Cfg::CHUNK / 16; ++ks)
                     umma_ss(tmem, ad + (uint64_t)(((ks / 4) * Cfg::SUB_BYTES + (ks % 4) * 32) >> 4),
                             fd + (uint64_t)(((ks / 4) * Cfg::FSUB_BYTES + (ks % 4) * 32) >> 4), IDESC, (ic > c_begin || ks > 0) ? 1u : 0u);
                 umma_commit(smem_u32(&ctl->mma_done[buf]));
@@ -201,15 +203,15 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
         }
         // the stage chunk j - 1 was read from is free once its MMAs are done (long ago, as a rule): refill it while
         // the MMAs of chunk j run
-        if (ok && j > 0 && !mbar_wait(smem_u32(&ctl->mma_done[(j - 1) % AH_NS]), (uint32_t)(((j - 1) / AH_NS) & 1))) {
+        if (ok && j > 0 && !mbar_wait(smem_u32(&ctl->mma_done[(j - 1) % Cfg::NS]), (uint32_t)(((j - 1) / Cfg::NS) & 1))) {
             ok = false;
             ctl->fault = 1;
         }
-        stage_chunk(j + AH_NS - 1);
+        stage_chunk(j + Cfg::NS - 1);
         const bool last_chunk = ic == c_end - 1;
         float sc3[Cfg::NCOLS];
         if (last_chunk) {
-            if (ok && !mbar_wait(smem_u32(&ctl->mma_done[buf]), (uint32_t)((j / AH_NS) & 1))) {
+            if (ok && !mbar_wait(smem_u32(&ctl->mma_done[buf]), (uint32_t)((j / Cfg::NS) & 1))) {
                 ok = false;
                 ctl->fault = 1;
             }
@@ -314,11 +316,11 @@ static int launch_k(const focus_shape* s, const void* h, int64_t sb, int64_t sn,
     const int ntile = cdiv(s->n, 128);
     const long long nitems = (long long)s->batch * ntile;
     if (nitems == 0) return 0;
-    if (nitems > 0x7fffffffll || (long long)(nitems / (nitems < resident ? nitems : resident) + 1) * cdiv(d, AH_CHUNK) > 0x7fffffffll)
+    if (nitems > 0x7fffffffll || (long long)(nitems / (nitems < resident ? nitems : resident) + 1) * cdiv(d, Cfg::CHUNK) > 0x7fffffffll)
         return fail(FOCUS_ERR_UNSUPPORTED, "focus_assign_hidden: too many chunks of 128 x 128 elements for one launch");
     // blocks per tile: as many as there are places for, with two chunks each at least
     int split = 1;
-    while (split < 8 && nitems * split * 2 <= (long long)sms * (per_sm < 2 ? per_sm : 2) && cdiv(d, AH_CHUNK) >= 4 * split) split *= 2;
+    while (split < 8 && nitems * split * 2 <= (long long)sms * (per_sm < 2 ? per_sm : 2) && cdiv(d, Cfg::CHUNK) >= 4 * split) split *= 2;
     const int nblocks = (int)(nitems < resident ? nitems : resident);
     const int share = (int)(nitems / nblocks), extra = (int)(nitems % nblocks);
     if (split > 1) {
