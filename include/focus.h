@@ -232,7 +232,7 @@ FOCUS_API int focus_build_tiles(const focus_shape* shape, const uint32_t* mq, co
  *   tiles_ws    workspace written by focus_build_tiles for the same shape and masks.  NULL = dense
  *               causal mode (every causal pair attended; masks and layout ignored).
  *   layout      the layout the workspace was built with (FOCUS_LAYOUT_SORTED_LOCAL: the class-sorted pass over
- *               sharing pairs, the window pass in token order, then a merge kernel): FOCUS_LAYOUT_ORIGINAL walks tiles in token
+ *               sharing pairs, then the window pass in token order, which joins the two): FOCUS_LAYOUT_ORIGINAL walks tiles in token
  *               order and skips dead far tiles; FOCUS_LAYOUT_CLASS_SORTED gathers Q/K/V into the
  *               class-sorted order kept in the workspace, walks only sharing class pairs plus the
  *               window, and scatters O/lse back to token order.

@@ -34,6 +34,8 @@
 //                   range of sorted key tiles listed for the query block; a row's kept columns of a
 //                   tile are a contiguous range found from the tile's ascending positions; O and lse
 //                   go straight to the rows' original positions
+// In the last two the TMA thread alone walks; the other roles get the tiles, with what their masks are made from, through a
+// ring in shared memory (TileInfo).
 // The items are a queue, expensive ones first: the grid has one block per item, and a CTA that is through with its item
 // takes over the next block that has not started (cluster launch control; the TMA thread asks, every role reads the
 // answer from shared memory).  Dealing the items out beforehand, a fixed number per CTA, left the fullest CTA 18 % (one
