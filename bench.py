@@ -261,9 +261,9 @@ def main():
     O = torch.empty_like(Q)
     lse = torch.empty((wl.Hq, wl.n), dtype=torch.float32, device="cuda")
     status = torch.zeros(4, dtype=torch.int32, device="cuda")
-    # assign x2, build_tiles (4 kernels; class-sorted: + 6 per side + ranges + order), attention (+ 3 gathers)
-    # layout 3: + fill, second attention launch, merge
-    launches_per_step = 2 + 4 + 1 + (14 + 3 if layout in (1, 3, 4) else 0) + (3 if layout in (3, 4) else 0)
+    # assign x2, build_tiles (2 kernels; class-sorted: + 5 of the sort + ranges + order; group-major keys: + 6 for their lists),
+    # attention (+ gather); with a window pass: + fill, second attention launch
+    launches_per_step = 2 + 2 + 1 + (7 + 1 if layout in (1, 3, 4) else 0) + (2 if layout in (3, 4) else 0) + (6 if layout == 4 else 0)
 
     ev = lambda: torch.cuda.Event(enable_timing=True)
     marks = []
@@ -385,8 +385,8 @@ def main():
         ms_skb = timed_alone(lambda: fb.focus_sinkhorn_bwd(shape, scores, 0.1, 10, ws_skb, dsoft, dscores))
         del scores, dsoft, dscores
         tr = dict(router_scores_ms=ms_sc, sinkhorn_ms=ms_sk, sinkhorn_bwd_ms=ms_skb,
-                  note="tau = 0.1, 10 Sinkhorn iterations (12 small launches on an L2-resident score matrix; the backward "
-                       "repeats the column sums and adds 11 launches), lambda = 10")
+                  note="tau = 0.1, 10 Sinkhorn iterations (one cooperative launch each for the forward and the "
+                       "derivative, which repeats the column sums), lambda = 10")
         if wl.softcap == 0 and (wl.K <= 16 or wl.D < 256):
             O_g, lse_g = torch.empty_like(Q), torch.empty_like(lse)
             ms_g = timed_alone(lambda: fb.focus_gate_attn_fwd(shape, Q, K, V, soft, 10.0, O_g, lse_g, status), reps=2)

@@ -154,7 +154,7 @@ sinkhorn_pass_kernel(const float* __restrict__ S, int n, int K, int iters, int p
 // its K column sums and adds up the P x K numbers of its team.  A number travels with the exchange's ordinal in one 8-byte
 // word (the low 16 of a double's 52 mantissa bits give way to it), written and polled whole, so that neither a fence nor
 // a counter stands between writing and reading it (fp64 atomics into one sum, a fence and an arrival counter took 3.5 us
-// per exchange), and the order of every sum is fixed.  What bounds it is latency: of the ~2.6 us of an iteration a third
+// per exchange), and the order of every sum is fixed.  What bounds it is latency: of the ~2.3 us of an iteration a third
 // is the words' way through L2, the rest instruction issue and block barriers.  The launch is cooperative, so
 // that all blocks of a team run at once.
 constexpr int SKT_THREADS = 512;
@@ -162,7 +162,7 @@ constexpr int SKT_TOKENS = 8 * SKT_THREADS;          // tokens per block at most
 constexpr int SKT_BLOCKS = 160;                      // blocks per team at most (the workspace has words for as many)
 constexpr size_t SKT_SMEM = 200 * 1024;
 constexpr unsigned long long SKT_TAG = 0xffffull;
-constexpr long long SKT_LEAD = 900;                  // cycles before the first poll
+constexpr long long SKT_LEAD = 500;                  // cycles before the first poll
 
 // words of one sequence's exchanges: two sets, taken in turn.  A block writes set e mod 2 for exchange e + 2 after it has
 // read everybody's e + 1, which each of them wrote after reading everybody's e.
@@ -299,10 +299,11 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
                 seen[j] = threadIdx.x / PAIRS + j * STEP >= P;
             }
             // A poll that comes too early makes the next one take 1.4 us instead of 0.4, and a block that is late by that
-            // much makes the others' polls come too early in the next exchange; so wait out the words' way first (about
-            // 0.5 us): 31 + 60 us for forward and backward at 131072 x 8, 34 + 72 us without.
+            // much makes the others' polls come too early in the next exchange; so wait out most of the words' way first.
+            // Forward and derivative, 500 cycles against none: 131072 x 8 83 and 87 us, 30000 x 8 70 and 105, 8192 x 8 70
+            // and 98; 900 cycles cost another 5 us each.
             const long long t0 = clock64();
-            while (clock64() - t0 < SKT_LEAD) { }
+            while (P > 1 && clock64() - t0 < SKT_LEAD) { }
             for (bool all = false; !all;) {
                 all = true;
 #pragma unroll
