@@ -369,11 +369,24 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
     // (S - M) * log2(e) / tau, the factor in two floats: a factor rounded once would shift every exponent alike
     const double per_tau = 1.4426950408889634 / (double)tau;
     const float c_hi = (float)per_tau, c_lo = (float)(per_tau - (double)c_hi);
+    // A difference whose exponent overflows (minus infinity among them) has weight 0.  It is kept at the lowest value whose
+    // exponent is finite: c_lo may be negative, and times minus infinity it would add plus infinity to the exponent.  A row
+    // with no other entry has no assignment and becomes NaN, as (-inf) - (-inf) makes it in the passes below; NaN stays NaN.
+    const float lowest = -3.4e38f / fmaxf(c_hi, 1.f);
     for (int i = threadIdx.x; i < cnt; i += SKT_THREADS) {
         float x[KMAX];
         get(rows_s, i, x);
+        bool closed = true;
 #pragma unroll
-        for (int g = 0; g < KMAX; ++g) x[g] = g < K ? x[g] - colmax_s[g] : 0.f;
+        for (int g = 0; g < KMAX; ++g) {
+            x[g] = g < K ? x[g] - colmax_s[g] : 0.f;
+            if (g < K) closed &= x[g] < lowest;
+        }
+#pragma unroll
+        for (int g = 0; g < KMAX; ++g) {
+            if (x[g] < lowest) x[g] = lowest;
+            if (g < K && closed) x[g] = __int_as_float(0x7fffffff);
+        }
         put(rows_s, i, x);
     }
     auto log2_units = [&](float x, float off) { return fmaf(x, c_hi, fmaf(x, c_lo, off)); };
@@ -513,7 +526,8 @@ static int launch_team(const focus_shape* s, const float* S, float tau, int iter
     int dev = 0, sms = 0, rc;
     if ((rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
     if ((rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute"))) return rc;
-    if (s->batch > sms) return 0;
+    // (from about 1e36 on the lowest finite exponent of a row no longer stands for weight 0)
+    if (s->batch > sms || tau > 1e30f) return 0;
     int P = sms / s->batch;
     if (P > skt_max_blocks(s->n)) P = skt_max_blocks(s->n);
     const int chunk = cdiv(cdiv(s->n, P), SKT_THREADS) * SKT_THREADS;        // whole rounds of the threads

@@ -111,6 +111,48 @@ def test_sinkhorn_one_launch_and_launch_per_iteration(n, K, batch):
     check()
 
 
+@pytest.mark.parametrize("tau", [0.05, 0.1, 0.5, 3.0])
+@pytest.mark.parametrize("n,K", [(600, 4), (5000, 7), (148 * 4096 + 1, 4)])
+def test_sinkhorn_closed_groups(n, K, tau):
+    """scores of minus infinity (a group closed to a token) and differences to the column maximum that overflow: weight 0 and
+    derivative 0 there, every other number as in 64 bits, in the one-launch form (the first two sizes) and the other one"""
+    iters = 5
+    g = torch.Generator(device="cuda"); g.manual_seed(n + K)
+    ld = fb.focus_soft_ld(K)
+    S = padded(0.3 * torch.randn((1, n, K), generator=g, device="cuda"), ld)
+    shut = torch.rand((1, n, K), generator=g, device="cuda") < 0.2
+    shut[..., 0] = False                                     # every token keeps a group
+    S[..., :K][shut] = float("-inf")
+    S[0, 1, 1], S[0, 2, 1] = -3.4e38, -3.0e38
+    shut[0, 1:3, 1] = True
+    dg = padded(torch.randn((1, n, K), generator=g, device="cuda"), ld)
+    shape = fb.make_shape(4, 2, n, 128, K, 1, 16)
+    ws = torch.empty(fb.focus_sinkhorn_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+    wb = torch.empty(fb.focus_sinkhorn_bwd_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+    out, ds = torch.full_like(S, float("nan")), torch.full_like(S, float("nan"))
+
+    def both():
+        fb.focus_sinkhorn(shape, S, tau, iters, ws, out)
+        fb.focus_sinkhorn_bwd(shape, S, tau, iters, wb, dg, ds)
+
+    both()
+    s64 = S[0, :, :K].double().requires_grad_()
+    x = s64 / tau
+    for _ in range(iters):
+        x = x - torch.logsumexp(x, dim=0, keepdim=True)
+        x = x - torch.logsumexp(x, dim=1, keepdim=True)
+    ref = x.exp()
+    ref_ds, = torch.autograd.grad(ref, s64, dg[0, :, :K].double())
+    assert (out[..., :K][shut] == 0).all() and (ds[..., :K][shut] == 0).all()
+    torch.testing.assert_close(out[0, :, :K].double(), ref.detach(), rtol=5e-4, atol=1e-7)
+    assert (ds[0, :, :K].double() - ref_ds).abs().max() <= 2e-4 * ref_ds.abs().max()
+    # a score that is not a number, and a token closed to every group, have no normalisation: NaN everywhere
+    for bad in (float("nan"), float("-inf")):
+        S[0, n // 2, :K] = bad
+        both()
+        assert out[..., :K].isnan().all() and ds[..., :K].isnan().all()
+
+
 def gate_case(Hq, Hkv, n, D, K, seed, batch=1):
     g = torch.Generator(device="cuda"); g.manual_seed(seed)
     Q = torch.randn((batch, Hq, n, D), generator=g, device="cuda").to(torch.bfloat16)
