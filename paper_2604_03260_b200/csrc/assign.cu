@@ -310,7 +310,8 @@ static int launch_one(const focus_shape* s, const focus_tensor& x, int H, const 
                       unsigned long long* near_ties, float eps, cudaStream_t st) {
     using Cfg = AssignCfg<D, KMAX>;
     const long long vectors = (long long)s->batch * H * s->n;
-    if (KMAX <= 8 && vectors * KMAX <= FEW_SCORES) {
+    // (it reads the centroids in pairs; the tile kernel one by one, at any float's address)
+    if (KMAX <= 8 && vectors * KMAX <= FEW_SCORES && (uintptr_t)C % 8 == 0) {
         if constexpr (KMAX <= 8)
             return check_cuda(launch_dependent(assign_few_kernel<D, KMAX>, dim3((unsigned)((vectors + FEW_WARPS - 1) / FEW_WARPS)), dim3(FEW_WARPS * 32), 0,
                                                st, reinterpret_cast<const __nv_bfloat16*>(x.ptr), x.stride_b, x.stride_h, x.stride_n, H, H / s->Hkv,

@@ -28,3 +28,19 @@ def test_few_vectors(D, H, Hkv, n, K, topk, batch):
     margin[0, 0, 0] = 1.0                                   # all scores of the zero vector tie: the first groups
     sure = (margin >= 1e-5).reshape(batch * H, n)
     assert (m == ref)[sure].all() and near.item() <= (~sure).sum().item() + (1 if topk < K else 0) and (~sure).sum().item() < 3 + 1e-3 * m.numel()
+
+
+@pytest.mark.parametrize("D,n", [(64, 3), (128, 1), (256, 40)])
+def test_centroids_at_an_odd_float(D, n):
+    """a contiguous set of centroids that starts on the 4-byte grid only, as a slice of a parameter buffer can"""
+    H, Hkv, K = 8, 4, 5
+    g = torch.Generator(device="cuda"); g.manual_seed(n + D)
+    x = torch.randn((1, H, n, D), generator=g, device="cuda").to(torch.bfloat16)
+    buf = torch.randn(Hkv * K * D + 1, generator=g, device="cuda")
+    odd = buf[1:].view(Hkv, K, D)
+    assert odd.data_ptr() % 8 == 4
+    shape = fb.make_shape(H, Hkv, n, D, K, 2, 16)
+    got, want = (torch.full((H, n), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+    fb.focus_assign(shape, x, H, odd, got)
+    fb.focus_assign(shape, x, H, odd.clone(), want)
+    assert torch.equal(got, want) and (want > 0).all()
