@@ -29,6 +29,7 @@ constexpr int DEC_MAX_CTAS = 4 * DEC_SMS;
 struct DecPlan {
     int groups, stride;              // steps per KV head, and the distance of two heads in the list
     int ctas, slots;                 // CTAs, partial results per head at most
+    int cap;                         // CTAs the length allows: does not fall as n or batch grow
     long long total, per;            // length of the list, steps per CTA
     __host__ __device__ int first_cta(int bh) const { return (int)((long long)bh * stride / per); }
     __host__ __device__ int last_cta(int bh) const { return (int)(((long long)bh * stride + groups - 1) / per); }
@@ -355,6 +356,7 @@ static DecPlan decode_plan(const focus_shape* s) {
     long long ctas = p.total / (2 * warps);                         // at least two steps per warp (2049 keys: 11 us, with four 13)
     if (ctas > places) ctas = places;
     if (ctas < 1) ctas = 1;
+    p.cap = (int)ctas;
     // a CTA's range in whole rounds of its warps: the last round takes as long half full
     p.per = ((p.total + ctas - 1) / ctas + warps - 1) / warps * warps;
     if (ctas >= heads) {
@@ -370,8 +372,11 @@ static DecPlan decode_plan(const focus_shape* s) {
     return p;
 }
 
+// Scratch for the longest cache serves every shorter one: `slots` itself falls where `per` steps up to the next round of the
+// warps, but heads * slots <= cap + 2 * heads always (a range holds at least total / cap steps).
 size_t decode_workspace_bytes(const focus_shape* s) {
-    return (size_t)s->batch * s->Hq * decode_plan(s).slots * (s->D + 2) * sizeof(float);
+    const size_t heads = (size_t)s->batch * s->Hkv;
+    return (decode_plan(s).cap + 2 * heads) * (s->Hq / s->Hkv) * (s->D + 2) * sizeof(float);
 }
 
 template <int D>

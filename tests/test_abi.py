@@ -123,6 +123,17 @@ def test_auto_layout_is_resolved_from_the_shape():
     assert L4.vs - L4.ks >= 8 * L4.nkp * 128 * 2
 
 
+@pytest.mark.parametrize("D", [64, 128, 256])
+def test_decode_scratch_never_shrinks_as_the_cache_or_the_batch_grows(D):
+    for batch, Hq, Hkv in ((1, 32, 8), (1, 12, 12), (8, 32, 8), (1, 8, 1), (3, 16, 2), (40, 8, 8), (700, 4, 4)):
+        sizes = [fb.focus_decode_workspace_bytes(fb.make_shape(Hq, Hkv, n, D, 4, 2, 16, batch=batch))
+                 for n in list(range(1, 6000, 8)) + list(range(6000, 140000, 112)) + [1 << 20, 1 << 30]]
+        assert sizes == sorted(sizes) and sizes[0] > 0
+    for n in (1, 497, 4721, 131072):
+        sizes = [fb.focus_decode_workspace_bytes(fb.make_shape(32, 8, n, D, 4, 2, 16, batch=b)) for b in range(1, 200)]
+        assert sizes == sorted(sizes)
+
+
 def test_training_forward_host_checks():
     """row length of the soft assignments, Sinkhorn workspace size, and argument checks that precede any launch"""
     L = fb.lib()
