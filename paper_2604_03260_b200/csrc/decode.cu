@@ -355,7 +355,9 @@ static DecPlan decode_plan(const focus_shape* s) {
     p.total = (long long)heads * p.groups;
     long long ctas = p.total / (2 * warps);                         // at least two steps per warp (2049 keys: 11 us, with four 13)
     if (ctas > places) ctas = places;
-    if (ctas < 1) ctas = 1;
+    // but no range over several short heads while places are free: each further head costs a CTA 3 us (a call with
+    // 1 cached key: 8 heads in one CTA 27 us, 128 heads at 8 a CTA 28; a CTA per head 10.6 both)
+    if (ctas < heads) ctas = heads < places ? heads : places;
     p.cap = (int)ctas;
     // a CTA's range in whole rounds of its warps: the last round takes as long half full
     p.per = ((p.total + ctas - 1) / ctas + warps - 1) / warps * warps;

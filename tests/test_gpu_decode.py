@@ -80,7 +80,7 @@ def test_decode_argument_checks():
 
 
 @pytest.mark.parametrize("D,batch,Hq,Hkv,n", [(128, 40, 8, 8, 300), (64, 5, 4, 2, 1), (128, 8, 16, 4, 2049), (128, 1, 8, 1, 70000), (256, 150, 4, 4, 33),
-                                              (256, 3, 8, 2, 5001), (64, 2, 16, 2, 40000)])
+                                              (256, 3, 8, 2, 5001), (64, 2, 16, 2, 40000), (128, 16, 8, 8, 1), (64, 200, 4, 4, 17), (256, 1, 8, 8, 31)])
 def test_decode_ranges_across_kv_heads(D, batch, Hq, Hkv, n):
     """the list of steps cut into equal ranges: ranges that cover several KV heads, end inside one, hold less than a head"""
     g = torch.Generator(device="cuda"); g.manual_seed(n + D)
