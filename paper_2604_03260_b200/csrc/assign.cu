@@ -100,7 +100,6 @@ assign_kernel(const __nv_bfloat16* __restrict__ x, int64_t stride_b, int64_t str
         ctl->fault = 0;
     }
     dep_wait();
-    dep_trigger();
     copy_tile(0);
     copy_tile(1);
     __syncthreads();
@@ -229,6 +228,10 @@ assign_kernel(const __nv_bfloat16* __restrict__ x, int64_t stride_b, int64_t str
         if (in && ok) masks[(size_t)bh * n + tok] = taken;
         if (near_ties) near_votes += __popc(__ballot_sync(0xffffffffu, ok && in && topk < K && (last - next) < eps));
     }
+    // Only now: the next kernel's blocks may need tensor memory, which every block of this one has by here, and a next
+    // focus_assign set up any earlier fills the gaps this one leaves on the SMs and so starts unevenly (back to back, 32 heads x
+    // 32768 x 64: K = 8 41 us, triggered at the start 53; K = 4 31 and 41).
+    dep_trigger();
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (near_ties && lane == 0 && near_votes) atomicAdd(near_ties, (unsigned long long)near_votes);
     __syncthreads();

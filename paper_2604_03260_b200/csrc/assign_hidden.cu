@@ -172,7 +172,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
         ctl->fault = 0;
     }
     dep_wait();
-    dep_trigger();
+    if (warp == 0) dep_trigger();            // this warp has the block's tensor memory: the next kernel's blocks may want some
     load_folded();
 #pragma unroll
     for (int j = 0; j < Cfg::NS - 1; ++j) stage_chunk(j);

@@ -54,8 +54,10 @@ inline size_t sorted_scratch_bytes(const focus_shape* s) {
 // Programmatic dependent launch: a kernel launched by launch_dependent may be set up while the kernel before it in the
 // stream still runs; before it touches memory that anything before it wrote or still reads, every thread of it executes
 // dep_wait(), which returns when all earlier work of the stream is complete and visible.  dep_trigger() lets the next
-// such kernel be set up from here on (it still waits for the end of this one); it comes after dep_wait(), so that a kernel is
-// set up only when everything before its direct predecessor is complete.
+// such kernel be set up from here on (it still waits for the end of this one), once one thread of every block has called it.
+// It comes after dep_wait(), so that a kernel is set up only when everything before its direct predecessor is complete, and
+// after the block's last tcgen05.alloc: the next kernel allocates before its own dep_wait(), keeps that until this one has
+// ended, and a block of this one waiting for tensor memory behind it would never end.
 #ifdef __CUDACC__
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

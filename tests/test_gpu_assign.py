@@ -5,6 +5,7 @@ import pytest
 import torch
 
 from oracle import focus_oracle as fo
+from paper_2604_03260_b200 import binding as fb
 from paper_2604_03260_b200 import inputs as fi
 from tests.gpu_util import as_u32, gpu_assign
 
@@ -92,3 +93,26 @@ def test_assign_strided_input():
     a, _ = gpu_assign(wl, Q, C, wl.Hq)
     b, _ = gpu_assign(wl, Qs, C, wl.Hq)
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("D,K,n", [(64, 32, 3001), (128, 17, 1000), (64, 8, 9000)])
+def test_calls_back_to_back_that_fill_tensor_memory(D, K, n):
+    """queries, keys, queries, ... without a wait in between: blocks of one call are set up while those of the one before still
+    run and share the SM's tensor memory with them (K > 16: 256 of its 512 columns each)"""
+    Hq, Hkv = 32, 8
+    g = torch.Generator(device="cuda"); g.manual_seed(n + K)
+    q, k = (torch.randn((1, H, n, D), generator=g, device="cuda").to(torch.bfloat16) for H in (Hq, Hkv))
+    C = torch.randn((Hkv, K, D), generator=g, device="cuda")
+    shape = fb.make_shape(Hq, Hkv, n, D, K, 2, 16)
+    want = []
+    for x, H in ((q, Hq), (k, Hkv)):
+        want.append(torch.empty((H, n), dtype=torch.int32, device="cuda"))
+        fb.focus_assign(shape, x, H, C, want[-1])
+        torch.cuda.synchronize()
+    got = [torch.full_like(want[i % 2], -1) for i in range(12)]
+    for i, m in enumerate(got):
+        fb.focus_assign(shape, (q, k)[i % 2], (Hq, Hkv)[i % 2], C, m)
+    torch.cuda.synchronize()
+    for i, m in enumerate(got):
+        # (|c|^2 is added up by several warps in no fixed order: an exact tie may fall either way)
+        assert (m != want[i % 2]).sum() <= 2
