@@ -43,9 +43,9 @@ struct AssignCtl {
 
 template <int D, int KMAX>
 __global__ void __launch_bounds__(ASSIGN_THREADS)
-assign_kernel(const __nv_bfloat16* __restrict__ x, int64_t stride_b, int64_t stride_h, int64_t stride_n,
-              int H, int G, int n, int K, int topk, int ntile, int share, int extra, const float* __restrict__ C,
-              uint32_t* __restrict__ masks, unsigned long long* near_ties, float eps) {
+assign_kernel(const __nv_bfloat16* x, int64_t stride_b, int64_t stride_h, int64_t stride_n,
+              int H, int G, int n, int K, int topk, int ntile, int share, int extra, const float* C,
+              uint32_t* masks, unsigned long long* near_ties, float eps) {
     using Cfg = AssignCfg<D, KMAX>;
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t base = smem_u32(sm);
@@ -116,7 +116,7 @@ assign_kernel(const __nv_bfloat16* __restrict__ x, int64_t stride_b, int64_t str
         for (int j = 0; j < KMAX * D / ASSIGN_THREADS; ++j) {
             const int e = j * ASSIGN_THREADS + threadIdx.x;
             const int g = e / D, d = e % D;                     // g is the same for the 32 lanes of a warp (D >= 64)
-            float v = g < K ? __ldg(Ch + e) : 0.f;
+            float v = g < K ? dep_load(Ch + e) : 0.f;
             float s = v * v;
             __nv_bfloat16 hi, mid, lo;
             split3_bf16(v, hi, mid, lo);
@@ -255,8 +255,8 @@ constexpr long long FEW_SCORES = 16384;              // vectors x groups (4 or 8
 
 template <int D, int KMAX>
 __global__ void __launch_bounds__(FEW_WARPS * 32)
-assign_few_kernel(const __nv_bfloat16* __restrict__ x, int64_t stride_b, int64_t stride_h, int64_t stride_n, int H, int G, int n, int total,
-                  int K, int topk, const float* __restrict__ C, uint32_t* __restrict__ masks, unsigned long long* near_ties, float eps) {
+assign_few_kernel(const __nv_bfloat16* x, int64_t stride_b, int64_t stride_h, int64_t stride_n, int H, int G, int n, int total,
+                  int K, int topk, const float* C, uint32_t* masks, unsigned long long* near_ties, float eps) {
     constexpr int DPL = D / 32;
     const int id = blockIdx.x * FEW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (id >= total) return;
@@ -269,7 +269,7 @@ assign_few_kernel(const __nv_bfloat16* __restrict__ x, int64_t stride_b, int64_t
     float v[DPL];
 #pragma unroll
     for (int e = 0; e < DPL; e += 2) {
-        const uint32_t w = __ldg(reinterpret_cast<const unsigned int*>(src + e));
+        const uint32_t w = dep_load(reinterpret_cast<const unsigned int*>(src + e));
         v[e] = __uint_as_float(w << 16);
         v[e + 1] = __uint_as_float(w & 0xffff0000u);
     }
@@ -282,7 +282,7 @@ assign_few_kernel(const __nv_bfloat16* __restrict__ x, int64_t stride_b, int64_t
         if (g < K) {
 #pragma unroll
             for (int e = 0; e < DPL; e += 2) {
-                const float2 c = __ldg(reinterpret_cast<const float2*>(Ch + (size_t)g * D + e));
+                const float2 c = dep_load(reinterpret_cast<const float2*>(Ch + (size_t)g * D + e));
                 dot[g] = fmaf(v[e], c.x, dot[g]); dot[g] = fmaf(v[e + 1], c.y, dot[g]);
                 cc[g] = fmaf(c.x, c.x, cc[g]); cc[g] = fmaf(c.y, c.y, cc[g]);
             }

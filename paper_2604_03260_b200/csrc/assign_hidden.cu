@@ -54,7 +54,7 @@ struct HiddenCtl {
 
 // folded[g][e] = sum_j Wg[e][j] * C[g][j]
 __global__ void __launch_bounds__(256)
-fold_router_kernel(const float* __restrict__ Wg, const float* __restrict__ C, int d, int dg, int K, float* __restrict__ folded) {
+fold_router_kernel(const float* Wg, const float* C, int d, int dg, int K, float* folded) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     const int g = blockIdx.y;
     dep_wait();
@@ -67,10 +67,10 @@ fold_router_kernel(const float* __restrict__ Wg, const float* __restrict__ C, in
 
 template <int KMAX>
 __global__ void __launch_bounds__(AH_THREADS)
-assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int64_t stride_n, int n, int d, int K, int topk,
-                     const float* __restrict__ folded, const float* __restrict__ bias, int Hq, int Hkv,
-                     uint32_t* __restrict__ mq, uint32_t* __restrict__ mk, unsigned long long* near_ties, float eps,
-                     float* __restrict__ scores, int ntile, int share, int extra, int split) {
+assign_hidden_kernel(const __nv_bfloat16* h, int64_t stride_b, int64_t stride_n, int n, int d, int K, int topk,
+                     const float* folded, const float* bias, int Hq, int Hkv,
+                     uint32_t* mq, uint32_t* mk, unsigned long long* near_ties, float eps,
+                     float* scores, int ntile, int share, int extra, int split) {
     using Cfg = HiddenCfg<KMAX>;
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t base = smem_u32(sm);
@@ -106,7 +106,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
         for (int i = 0; i < FPT; ++i) {
             const int q = i * AH_THREADS + threadIdx.x;
             const int g = q / Cfg::CHUNK, e = e0 + q % Cfg::CHUNK;
-            fv[i] = (g < K && e < d) ? __ldg(folded + (size_t)g * d + e) : 0.f;
+            fv[i] = (g < K && e < d) ? dep_load(folded + (size_t)g * d + e) : 0.f;
         }
     };
     auto stage_chunk = [&](int j) {
@@ -261,7 +261,7 @@ assign_hidden_kernel(const __nv_bfloat16* __restrict__ h, int64_t stride_b, int6
             }
             const bool own = rank == 0;
 #pragma unroll
-            for (int g = 0; g < KMAX; ++g) score[g] += (bias && g < K) ? __ldg(bias + g) : 0.f;
+            for (int g = 0; g < KMAX; ++g) score[g] += (bias && g < K) ? dep_load(bias + g) : 0.f;
             if (scores) {   // the scores themselves (training-time soft assignment), rows of KMAX floats, zero beyond K
                 if (in && ok && own) {
                     float4* o = reinterpret_cast<float4*>(scores + ((size_t)b * n + tok) * KMAX);

@@ -153,7 +153,7 @@ template <> struct TileWalk<WALK_TOKEN> {
             ++wd;
             if (wd * 32 >= f0) break;
             uint32_t x = 0;
-            for (int r = 0; r < nl; ++r) x |= __ldg(l0 + (size_t)r * nkw + wd);
+            for (int r = 0; r < nl; ++r) x |= dep_load(l0 + (size_t)r * nkw + wd);
             const int rem = f0 - wd * 32;
             bits = rem < 32 ? x & ((1u << rem) - 1u) : x;
         }
@@ -167,14 +167,14 @@ template <> struct TileWalk<WALK_SORTED> {
     __device__ __forceinline__ void init(const AttnParams& p, int hq, int a0, int) {
         const int hk = (hq / p.Hq) * p.Hkv + (hq % p.Hq) / p.G;
         qr = p.qrange + ((size_t)hq * p.nqblk + (a0 >> 1)) * FOCUS_MAX_CLASSES * 2;
-        nck = __ldg(p.ncls_k + hk);
+        nck = dep_load(p.ncls_k + hk);
         jk = -1;
         b = rend = 0;
     }
     __device__ __forceinline__ int next() {
         while (b >= rend) {
             if (++jk >= nck) return -1;
-            const int2 r = __ldg(reinterpret_cast<const int2*>(qr) + jk);
+            const int2 r = dep_load(reinterpret_cast<const int2*>(qr) + jk);
             b = r.x;
             rend = r.y;
         }
@@ -252,7 +252,7 @@ struct Item { int A, bb, h, hq; };
 template <int WALK>
 __device__ __forceinline__ void item_at(const AttnParams& p, int id, Item& t) {
     if (WALK == WALK_SORTED) {
-        const int2 e = __ldg(reinterpret_cast<const int2*>(p.order) + id / p.ipb);
+        const int2 e = dep_load(reinterpret_cast<const int2*>(p.order) + id / p.ipb);
         t.hq = e.x;
         t.A = e.y * p.ipb + id % p.ipb;
     } else if (p.by_length) {
@@ -314,12 +314,12 @@ __device__ __forceinline__ void build_tile_mask_sorted(TileMask& tm, int w, cons
 // Group-major keys: the tile belongs to the list of group g.  A key that shares a LOWER group with the row is attended
 // under that lower group's list, so here it is masked out: `lower` = the row's groups below g, `gb` = the tile's
 // per-group bitmaps.  Every sharing pair is then computed exactly once.
-__device__ __forceinline__ void exclude_lower_groups(TileMask& tm, const uint32_t* __restrict__ gb, uint32_t lower, int K) {
+__device__ __forceinline__ void exclude_lower_groups(TileMask& tm, const uint32_t* gb, uint32_t lower, int K) {
     uint32_t ex[4] = {0u, 0u, 0u, 0u};
     for (uint32_t rem = lower; rem; rem &= rem - 1) {
         const int a = __ffs(rem) - 1;
         if (a < K) {
-            const uint4 t = __ldg(reinterpret_cast<const uint4*>(gb + a * 4));
+            const uint4 t = dep_load(reinterpret_cast<const uint4*>(gb + a * 4));
             ex[0] |= t.x; ex[1] |= t.y; ex[2] |= t.z; ex[3] |= t.w;
         }
     }

@@ -153,7 +153,7 @@ __device__ __forceinline__ void put_gate_row(unsigned char* op, int r, const flo
 #pragma unroll
         for (int f = 0; f < 2; ++f) {
             const bool have = in && 8 * c + 4 * f < ld;
-            const float4 x = have ? __ldg(reinterpret_cast<const float4*>(row) + 2 * c + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 x = have ? dep_load(reinterpret_cast<const float4*>(row) + 2 * c + f) : make_float4(0.f, 0.f, 0.f, 0.f);
             v[4 * f] = x.x * scale; v[4 * f + 1] = x.y * scale; v[4 * f + 2] = x.z * scale; v[4 * f + 3] = x.w * scale;
         }
 #pragma unroll
@@ -234,7 +234,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (WALK == WALK_SORTED) dep_wait();
-    if (WALK == WALK_SORTED && __ldg(p.counters + 4) != 0ull) {      // more mask values than the sorted layout holds: refuse
+    if (WALK == WALK_SORTED && dep_load(p.counters + 4) != 0ull) {      // more mask values than the sorted layout holds: refuse
         if (threadIdx.x == 0 && p.status && atomicCAS(p.status, 0, 2) == 0) {
             p.status[1] = 1; p.status[2] = 0; p.status[3] = (int)blockIdx.x;
         }
@@ -336,7 +336,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             const void* src;
                             uint32_t bytes;
                             if constexpr (WALK == WALK_SORTED) {
-                                if (walk.jk != cls_at) cls = __ldg(p.cls_k + (size_t)khead * FOCUS_MAX_CLASSES + (cls_at = walk.jk));
+                                if (walk.jk != cls_at) cls = dep_load(p.cls_k + (size_t)khead * FOCUS_MAX_CLASSES + (cls_at = walk.jk));
                                 info[slot].cls = cls;
                                 info[slot].pad[0] = (uint32_t)walk.jk;
                                 src = p.perm_k + (size_t)khead * p.nkp + (size_t)kb * 128;
@@ -710,10 +710,10 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             const int r = (t.A * NQ + x) * 128 + row_in_tile;
             i_row = r;
             // the row's position in the sequence: its index, or in the sorted layout the position its slot holds (-1: padding)
-            if constexpr (WALK == WALK_SORTED) i_row = __ldg(p.perm_q + (size_t)t.hq * p.nqp + r);
+            if constexpr (WALK == WALK_SORTED) i_row = dep_load(p.perm_q + (size_t)t.hq * p.nqp + r);
         };
         auto load_mask = [&]() {
-            if constexpr (WALK != WALK_DENSE) m_row = (i_row >= 0 && i_row < p.n) ? __ldg(p.mq + (size_t)t.hq * p.n + i_row) : 0u;
+            if constexpr (WALK != WALK_DENSE) m_row = (i_row >= 0 && i_row < p.n) ? dep_load(p.mq + (size_t)t.hq * p.n + i_row) : 0u;
         };
         bool have = next_item<WALK>(p, &ctl, 0, true, t, ok);
         if (have) { load_row(); load_mask(); }
@@ -775,7 +775,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
                     for (int f = 0; f < GQ; ++f) {
                         if (4 * f < p.gate_ld) {
-                            const float4 g0 = __ldg(gp + f);
+                            const float4 g0 = dep_load(gp + f);
                             gi[4 * f] = g0.x * p.gate_hl; gi[4 * f + 1] = g0.y * p.gate_hl;
                             gi[4 * f + 2] = g0.z * p.gate_hl; gi[4 * f + 3] = g0.w * p.gate_hl;
                         }
@@ -814,7 +814,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             const float4* gp = reinterpret_cast<const float4*>(p.gate_g + ((size_t)bb * p.n + (size_t)(j < p.n ? j : p.n - 1)) * p.gate_ld);
 #pragma unroll
                             for (int f = 0; f < GQ; ++f)
-                                reinterpret_cast<float4*>(gw + col * C::GATE_ROW_BYTES)[f] = 4 * f < p.gate_ld ? __ldg(gp + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+                                reinterpret_cast<float4*>(gw + col * C::GATE_ROW_BYTES)[f] = 4 * f < p.gate_ld ? dep_load(gp + f) : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctl.gbar[wg]));

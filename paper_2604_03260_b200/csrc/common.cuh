@@ -62,6 +62,12 @@ inline size_t sorted_scratch_bytes(const focus_shape* s) {
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A read in a kernel that may have been set up before its predecessor's end: a plain load, which stays behind dep_wait().  The
+// non-coherent path (__ldg, or a pointer to const declared __restrict__) is for data that is constant for the kernel's whole
+// lifetime, and that starts before the writer is through; so these kernels use neither.
+template <class T>
+__device__ __forceinline__ T dep_load(const T* p) { return *p; }
+
 template <class... Params, class... Args>
 inline cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchAttribute attr;

@@ -70,10 +70,10 @@ __device__ __forceinline__ uint32_t dec_pack_bf16(float lo, float hi) {
 // Each warp keeps its own running maximum, sum and O and writes its own partial result.
 template <int D>
 __global__ void __launch_bounds__(DecCfg<D>::WARPS * 32)
-decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t q_sh, const __nv_bfloat16* __restrict__ k,
-                      int64_t k_sb, int64_t k_sh, int64_t k_sn, const __nv_bfloat16* __restrict__ v, int64_t v_sb,
-                      int64_t v_sh, int64_t v_sn, const uint32_t* __restrict__ mq_new, const uint32_t* __restrict__ mk,
-                      int Hq, int Hkv, int G, int n, int w, float scale, float softcap, const DecPlan plan, float* __restrict__ part) {
+decode_partial_kernel(const __nv_bfloat16* q, int64_t q_sb, int64_t q_sh, const __nv_bfloat16* k,
+                      int64_t k_sb, int64_t k_sh, int64_t k_sn, const __nv_bfloat16* v, int64_t v_sb,
+                      int64_t v_sh, int64_t v_sn, const uint32_t* mq_new, const uint32_t* mk,
+                      int Hq, int Hkv, int G, int n, int w, float scale, float softcap, const DecPlan plan, float* part) {
     using C = DecCfg<D>;
     constexpr int VEC = D / 8;                                     // 16-byte pieces per row
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -118,7 +118,7 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
         }
         uint32_t mq_all[DEC_GMAX];                                     // every lane needs all heads' masks to flag its key
 #pragma unroll
-        for (int gg = 0; gg < DEC_GMAX; ++gg) mq_all[gg] = gg < G ? __ldg(mq_new + (size_t)b * Hq + hk * G + gg) : 0u;
+        for (int gg = 0; gg < DEC_GMAX; ++gg) mq_all[gg] = gg < G ? dep_load(mq_new + (size_t)b * Hq + hk * G + gg) : 0u;
 
         const __nv_bfloat16* kb = k + (size_t)b * k_sb + (size_t)hk * k_sh;
         const __nv_bfloat16* vb = v + (size_t)b * v_sb + (size_t)hk * v_sh;
@@ -131,7 +131,7 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
         // mask word of the key lane % 16 of a step (0 when it is local or past the end: not needed then)
         auto load_mask = [&](int step) {
             const int j = first_key(step) + (lane & 15);
-            return (step < nsteps && j <= last && last - j > w) ? __ldg(mkh + j) : 0u;
+            return (step < nsteps && j <= last && last - j > w) ? dep_load(mkh + j) : 0u;
         };
         // flag the 16 keys of a step and start copying the attended rows into ring stage `st` (16-byte asynchronous
         // copies, 16 consecutive lanes per row); one commit group per call, also when nothing is copied
@@ -278,8 +278,8 @@ decode_partial_kernel(const __nv_bfloat16* __restrict__ q, int64_t q_sb, int64_t
 // eight loads of O are under way while the weights are worked out.
 template <int D>
 __global__ void __launch_bounds__(256)
-decode_merge_kernel(const float* __restrict__ part, const DecPlan plan, int Hq, int Hkv, __nv_bfloat16* __restrict__ o, int64_t o_sb,
-                    int64_t o_sh, float* __restrict__ lse) {
+decode_merge_kernel(const float* part, const DecPlan plan, int Hq, int Hkv, __nv_bfloat16* o, int64_t o_sb,
+                    int64_t o_sh, float* lse) {
     constexpr int LANES = D / 2, ROWS = 256 / LANES, AHEAD = 8;
     __shared__ float wgt_s[DEC_MAX_CTAS + 1];
     __shared__ float red_s[2][8];

@@ -12,9 +12,9 @@ constexpr int TN = FOCUS_TILE_N;
 // One block of 128 threads per (head, tile): the heads of the query masks, then those of the key masks (+ gbits).  The first
 // block clears the counters of the passes that follow.
 __global__ void __launch_bounds__(128)
-summarise_kernel(const uint32_t* __restrict__ mq, const uint32_t* __restrict__ mk, int HQ, int n, int nt, int K, uint32_t* __restrict__ orq,
-                 uint32_t* __restrict__ andq, uint32_t* __restrict__ ork, uint32_t* __restrict__ andk, uint32_t* __restrict__ gbits,
-                 unsigned long long* __restrict__ counters) {
+summarise_kernel(const uint32_t* mq, const uint32_t* mk, int HQ, int n, int nt, int K, uint32_t* orq,
+                 uint32_t* andq, uint32_t* ork, uint32_t* andk, uint32_t* gbits,
+                 unsigned long long* counters) {
     const int tile = blockIdx.x % nt, row = blockIdx.x / nt;
     const bool key = row >= HQ;
     const int head = key ? row - HQ : row;
@@ -50,9 +50,9 @@ summarise_kernel(const uint32_t* __restrict__ mq, const uint32_t* __restrict__ m
 // word per warp; nothing in this launch waits for them.  (One thread per word in a launch of its own, before the live
 // bitmap, took 6 to 25 us for its 32 dependent loads.)
 __global__ void __launch_bounds__(128)
-live_kernel(const uint32_t* __restrict__ orq, const uint32_t* __restrict__ andq, const uint32_t* __restrict__ ork,
-            const uint32_t* __restrict__ andk, int G_heads, int Hq, int Hkv, int HQ, int w, int K, int nqt, int nkt, int nkw,
-            uint32_t* __restrict__ kany, uint32_t* __restrict__ kall, uint32_t* __restrict__ live, int32_t* __restrict__ live_cnt,
+live_kernel(const uint32_t* orq, const uint32_t* andq, const uint32_t* ork,
+            const uint32_t* andk, int G_heads, int Hq, int Hkv, int HQ, int w, int K, int nqt, int nkt, int nkw,
+            uint32_t* kany, uint32_t* kall, uint32_t* live, int32_t* live_cnt,
             unsigned long long* counters) {
     __shared__ unsigned int s[2];
     if (threadIdx.x < 2) s[threadIdx.x] = 0;
