@@ -82,3 +82,47 @@ def test_count_kept_on_cfg2_masks():
     assert cnt.cpu().tolist() == ref.tolist()
     frac = cnt.sum().item() / wl.dense_pairs()
     assert 0.80 < frac < 0.90          # 5/6 of far pairs + the window (0.854 for uniform memberships)
+
+
+@pytest.mark.parametrize("n,K,w", [(65536, 4, 300), (65537, 4, 300), (70000, 8, 100000), (90001, 1, 0), (131072, 9, 2048), (131073, 32, 2048)])
+def test_long_live_bitmaps(n, K, w):
+    """both sides of the length from which the live bitmap is made from the groups' bitmaps, with masks that hold bits past K"""
+    Hq, Hkv, batch = 2, 1, 2
+    g = torch.Generator(device="cuda"); g.manual_seed(n + K)
+    pos = torch.arange(n, device="cuda")
+
+    def draw(H):         # long runs of one group with a few other members, so that far tiles of every kind occur
+        run = (pos[None] // 700 + torch.arange(batch * H, device="cuda")[:, None]) % K
+        other = torch.randint(0, K, (batch * H, n), generator=g, device="cuda")
+        m = 1 << torch.where(torch.rand((batch * H, n), generator=g, device="cuda") < 0.002, other, run)
+        return torch.where(m >= 1 << 31, m - (1 << 32), m).to(torch.int32)
+    mq, mk = draw(Hq), draw(Hkv)
+    if K < 32:
+        mq |= 1 << K
+        mk |= 1 << K
+    shape = fb.make_shape(Hq, Hkv, n, 64, K, 1, w, batch=batch)
+    L = fb.focus_tiles_layout_of(shape, 0)
+    ws = torch.full((L.total_bytes,), 0xff, dtype=torch.uint8, device="cuda")
+    fb.focus_build_tiles(shape, mq, mk, 0, ws)
+    bits = lambda t, c: ((t.long()[..., None] >> torch.arange(c, device="cuda")) & 1).bool()
+    view = lambda off, *s: fb.ws_view(ws, off, int(np.prod(s)), torch.int32).view(s)
+
+    def member(m):       # [heads, tiles, 128, K], and which tokens exist
+        pad = torch.zeros((m.shape[0], L.nqt * 128 - n), dtype=torch.int32, device="cuda")
+        return bits(torch.cat([m, pad], 1), K).view(m.shape[0], L.nqt, 128, K)
+    exists = (torch.arange(L.nqt * 128, device="cuda") < n).view(1, L.nqt, 128, 1)
+    some = {k: member(m).any(2) for k, m in (("q", mq), ("k", mk))}
+    every = {k: (member(m) | ~exists).all(2) for k, m in (("q", mq), ("k", mk))}
+    of = torch.arange(batch * Hq, device="cuda") // Hq * Hkv
+    far = torch.arange(L.nkt, device="cuda")[None] < ((torch.arange(L.nqt, device="cuda") * 128 - w) // 128).clamp_min(0)[:, None]
+    meets = lambda t: (t["q"].float() @ t["k"][of].float().transpose(1, 2) > 0) & far
+    live = bits(view(L.live, batch * Hq, L.nqt, L.nkw), 32).flatten(2)
+    assert torch.equal(live[..., :L.nkt], meets(some)) and not live[..., L.nkt:].any()
+    assert torch.equal(view(L.live_cnt, batch * Hq, L.nqt).long(), meets(some).sum(-1))
+    counters = fb.ws_view(ws, L.counters, 3, torch.int64).tolist()
+    assert counters == [int(far.sum()) * batch * Hq, int(meets(some).sum()), int(meets(every).sum())]
+    for off, t in ((L.kany, some), (L.kall, every)):
+        got = bits(view(off, batch * Hkv, K, L.nkw), 32).flatten(2)
+        assert torch.equal(got[..., :L.nkt], t["k"].transpose(1, 2)) and not got[..., L.nkt:].any()
+    gb = bits(view(L.gbits, batch * Hkv, L.nkt, K, 4), 32).flatten(3)
+    assert torch.equal(gb, member(mk).transpose(2, 3))
