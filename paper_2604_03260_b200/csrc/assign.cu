@@ -38,7 +38,7 @@ struct AssignCtl {
     uint64_t s_full[2];               // the MMAs that read the piece in buffer 0 / 1 have completed
     uint32_t tmem_base;
     int fault;
-    float cn2[32];                    // |c_g|^2, then 1/|c_g|
+    float cn2[32];                    // 1/|c_g|
 };
 
 template <int D, int KMAX>
@@ -109,23 +109,30 @@ assign_kernel(const __nv_bfloat16* x, int64_t stride_b, int64_t stride_h, int64_
     // barrier keeps the previous norms until every thread has used them.
     auto build_centroids = [&](int hk) {
         __syncthreads();
-        if (threadIdx.x < 32) ctl->cn2[threadIdx.x] = 0.f;
-        __syncthreads();
         const float* Ch = C + (size_t)hk * K * D;
+        // A warp per centroid; |c_g|^2 as the sums of 32 squares, added in the order of the dimensions (in whatever order the
+        // warps came, a near-tie of two groups could fall either way from one call to the next).  Its loads come first: with a
+        // load, its split and an atomic addition in turn a set of 32 centroids of 256 took 15 us longer (24.5 us for 8 vectors,
+        // 9.5 so; 32 heads x 32768 x 256, K = 8 128 -> 99 us, 32 heads x 32768 x 128, K = 4 49 -> 45).
+#pragma unroll 2
+        for (int g = warp; g < KMAX; g += ASSIGN_THREADS / 32) {
+            float v[D / 32], norm2 = 0.f;
 #pragma unroll
-        for (int j = 0; j < KMAX * D / ASSIGN_THREADS; ++j) {
-            const int e = j * ASSIGN_THREADS + threadIdx.x;
-            const int g = e / D, d = e % D;                     // g is the same for the 32 lanes of a warp (D >= 64)
-            float v = g < K ? dep_load(Ch + e) : 0.f;
-            float s = v * v;
-            __nv_bfloat16 hi, mid, lo;
-            split3_bf16(v, hi, mid, lo);
-            *reinterpret_cast<__nv_bfloat16*>(cprime + sw128_offset(g, d, Cfg::NCOLS)) = hi;
-            *reinterpret_cast<__nv_bfloat16*>(cprime + sw128_offset(KMAX + g, d, Cfg::NCOLS)) = mid;
-            *reinterpret_cast<__nv_bfloat16*>(cprime + sw128_offset(2 * KMAX + g, d, Cfg::NCOLS)) = lo;
+            for (int c = 0; c < D / 32; ++c) v[c] = g < K ? dep_load(Ch + (size_t)g * D + c * 32 + lane) : 0.f;
 #pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            if (lane == 0) atomicAdd(&ctl->cn2[g], s);
+            for (int c = 0; c < D / 32; ++c) {
+                const int d = c * 32 + lane;
+                float s = v[c] * v[c];
+                __nv_bfloat16 hi, mid, lo;
+                split3_bf16(v[c], hi, mid, lo);
+                *reinterpret_cast<__nv_bfloat16*>(cprime + sw128_offset(g, d, Cfg::NCOLS)) = hi;
+                *reinterpret_cast<__nv_bfloat16*>(cprime + sw128_offset(KMAX + g, d, Cfg::NCOLS)) = mid;
+                *reinterpret_cast<__nv_bfloat16*>(cprime + sw128_offset(2 * KMAX + g, d, Cfg::NCOLS)) = lo;
+#pragma unroll
+                for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+                norm2 += s;
+            }
+            if (lane == 0) ctl->cn2[g] = norm2 > 0.f ? rsqrtf(norm2) : 0.f;     // read by everyone after the tile's first barrier
         }
         constexpr int ZROWS = Cfg::NCOLS - 3 * KMAX;           // whole rows, so the swizzle does not matter for them
         if constexpr (ZROWS > 0) {
@@ -133,11 +140,6 @@ assign_kernel(const __nv_bfloat16* x, int64_t stride_b, int64_t stride_h, int64_
                 const int sub = i / (ZROWS * 8), rem = i % (ZROWS * 8);
                 *reinterpret_cast<uint4*>(cprime + sub * Cfg::CSUB_BYTES + (3 * KMAX) * 128 + rem * 16) = make_uint4(0, 0, 0, 0);
             }
-        }
-        __syncthreads();
-        if (threadIdx.x < KMAX) {
-            const float s = ctl->cn2[threadIdx.x];
-            ctl->cn2[threadIdx.x] = s > 0.f ? rsqrtf(s) : 0.f;  // read by everyone after the tile's first barrier
         }
     };
 
