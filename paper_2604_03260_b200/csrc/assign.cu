@@ -11,6 +11,9 @@
 // memory); while it runs every thread sums the squares of its own row from shared memory; then it reads its
 // row of S, adds the three terms per group, scales by 1/(|x| |c_g|), selects the top-k groups and writes its
 // mask word, while the copies of the tile after next are already under way.
+// One kernel for every number of vectors: the mask of a vector must not depend on the call it is in, and another order of the
+// sums decides near-ties otherwise.  (A warp per vector without tensor cores, 32 vectors x 128 in 1.5 us instead of 2.9, did; with
+// its near-ties done over by this code it was behind from about 64 vectors on.)
 #include "assign_common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -247,81 +250,10 @@ assign_kernel(const __nv_bfloat16* x, int64_t stride_b, int64_t stride_h, int64_
     }
 }
 
-// Few vectors (a token's queries and keys in generation, short prompts): a warp per vector, lane l the dimensions from
-// l D / 32 on; the K inner products, |x|^2 and the |c_g|^2 in fp32, summed over the lanes.  Latency is all of it: the tile kernel above
-// takes as long for one tile as for a wave of them (centroid operand, tensor memory, one MMA chain).  Back to back, D = 128,
-// K = 4: 32 vectors 4.8 us there and 1.4 here, 4096 5.0 and 3.0, 8192 5.1 and 4.9, 16384 5.2 and 8.1; K = 8: 1024 6.4 and
-// 2.5, 4096 6.4 and 4.7, 8192 6.5 and 8.6; D = 64 and 256 cross between 4000 and 8000 vectors too.
-constexpr int FEW_WARPS = 4;
-constexpr long long FEW_SCORES = 16384;              // vectors x groups (4 or 8) up to here
-
-template <int D, int KMAX>
-__global__ void __launch_bounds__(FEW_WARPS * 32)
-assign_few_kernel(const __nv_bfloat16* x, int64_t stride_b, int64_t stride_h, int64_t stride_n, int H, int G, int n, int total,
-                  int K, int topk, const float* C, uint32_t* masks, unsigned long long* near_ties, float eps) {
-    constexpr int DPL = D / 32;
-    const int id = blockIdx.x * FEW_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (id >= total) return;
-    const int bh = id / n, tok = id % n;
-    const int hk = bh % H / G;
-    const __nv_bfloat16* src = x + (size_t)(bh / H) * stride_b + (size_t)(bh % H) * stride_h + (size_t)tok * stride_n + lane * DPL;
-    const float* Ch = C + (size_t)hk * K * D + lane * DPL;
-    dep_wait();
-    dep_trigger();
-    float v[DPL];
-#pragma unroll
-    for (int e = 0; e < DPL; e += 2) {
-        const uint32_t w = dep_load(reinterpret_cast<const unsigned int*>(src + e));
-        v[e] = __uint_as_float(w << 16);
-        v[e + 1] = __uint_as_float(w & 0xffff0000u);
-    }
-    float dot[KMAX], cc[KMAX], xx = 0.f;
-#pragma unroll
-    for (int e = 0; e < DPL; ++e) xx = fmaf(v[e], v[e], xx);
-#pragma unroll
-    for (int g = 0; g < KMAX; ++g) {
-        dot[g] = cc[g] = 0.f;
-        if (g < K) {
-#pragma unroll
-            for (int e = 0; e < DPL; e += 2) {
-                const float2 c = dep_load(reinterpret_cast<const float2*>(Ch + (size_t)g * D + e));
-                dot[g] = fmaf(v[e], c.x, dot[g]); dot[g] = fmaf(v[e + 1], c.y, dot[g]);
-                cc[g] = fmaf(c.x, c.x, cc[g]); cc[g] = fmaf(c.y, c.y, cc[g]);
-            }
-        }
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-        xx += __shfl_xor_sync(0xffffffffu, xx, off);
-#pragma unroll
-        for (int g = 0; g < KMAX; ++g) {
-            dot[g] += __shfl_xor_sync(0xffffffffu, dot[g], off);
-            cc[g] += __shfl_xor_sync(0xffffffffu, cc[g], off);
-        }
-    }
-    const float xinv = xx > 0.f ? rsqrtf(xx) : 0.f;
-#pragma unroll
-    for (int g = 0; g < KMAX; ++g) dot[g] = dot[g] * (cc[g] > 0.f ? rsqrtf(cc[g]) : 0.f) * xinv;
-    float last, next;
-    const uint32_t taken = select_topk<KMAX>(dot, K, topk, last, next);
-    if (lane == 0) {
-        masks[(size_t)bh * n + tok] = taken;
-        if (near_ties && topk < K && (last - next) < eps) atomicAdd(near_ties, 1ull);
-    }
-}
-
 template <int D, int KMAX>
 static int launch_one(const focus_shape* s, const focus_tensor& x, int H, const float* C, uint32_t* masks,
                       unsigned long long* near_ties, float eps, cudaStream_t st) {
     using Cfg = AssignCfg<D, KMAX>;
-    const long long vectors = (long long)s->batch * H * s->n;
-    // (it reads the centroids in pairs; the tile kernel one by one, at any float's address)
-    if (KMAX <= 8 && vectors * KMAX <= FEW_SCORES && (uintptr_t)C % 8 == 0) {
-        if constexpr (KMAX <= 8)
-            return check_cuda(launch_dependent(assign_few_kernel<D, KMAX>, dim3((unsigned)((vectors + FEW_WARPS - 1) / FEW_WARPS)), dim3(FEW_WARPS * 32), 0,
-                                               st, reinterpret_cast<const __nv_bfloat16*>(x.ptr), x.stride_b, x.stride_h, x.stride_n, H, H / s->Hkv,
-                                               s->n, (int)vectors, s->K, s->topk, C, masks, near_ties, eps), "assign kernel launch");
-    }
     auto kern = assign_kernel<D, KMAX>;
     int rc = check_cuda(allow_smem<assign_kernel<D, KMAX>>(Cfg::SMEM_BYTES, true), "cudaFuncSetAttribute(assign)");
     if (rc) return rc;

@@ -1,4 +1,4 @@
-"""focus_assign's warp-per-vector form against the tile form and fp64: the sizes on both sides of the line between them."""
+"""focus_assign of few vectors (generation, short prompts) against fp64, and against the same vectors in a long call."""
 import pytest
 import torch
 
@@ -44,3 +44,35 @@ def test_centroids_at_an_odd_float(D, n):
     fb.focus_assign(shape, x, H, odd, got)
     fb.focus_assign(shape, x, H, odd.clone(), want)
     assert torch.equal(got, want) and (want > 0).all()
+
+
+@pytest.mark.parametrize("D,K,topk", [(64, 4, 2), (128, 4, 1), (128, 8, 2), (256, 7, 3), (256, 4, 2), (64, 3, 3)])
+def test_masks_do_not_depend_on_the_size_of_the_call(D, K, topk):
+    """the vectors of one long call in short calls of every size: the same masks and near-ties, bit for bit, with pairs of
+    centroids a rounding apart, a zero one, one with a vanishing norm, and vectors that are zero, huge, tiny, infinite or not numbers"""
+    H, Hkv, n = 8, 4, 3000
+    g = torch.Generator(device="cuda"); g.manual_seed(D + K)
+    x = torch.randn((1, H, n, D), generator=g, device="cuda").to(torch.bfloat16)
+    x[:, :, 5], x[:, :, 6], x[:, :, 7], x[:, :, 8] = 0, x[:, :, 6] * 1e30, x[:, :, 7] * 1e-25, x[:, :, 8] * 1e18
+    x[:, :, 9, 3], x[:, :, 10, 0] = float("inf"), float("nan")
+    C = torch.randn((Hkv, K, D), generator=g, device="cuda")
+    C[:, 1] = C[:, 0] * (1 + 2e-7 * torch.randn((Hkv, D), generator=g, device="cuda"))
+    C[1, K - 1], C[2, K - 1] = 0, 1e-24 * C[2, K - 1]
+    C[3] *= 1e-6
+
+    def assign(x):
+        m = torch.full((H, x.shape[2]), -1, dtype=torch.int32, device="cuda")
+        near = torch.zeros(1, dtype=torch.int64, device="cuda")
+        fb.focus_assign(fb.make_shape(H, Hkv, x.shape[2], D, K, topk, 16), x, H, C, m, near)
+        return m, near.item()
+    want, near = assign(x)
+    assert topk == K or 0.02 < ((want ^ (want >> 1)) & 1).float().mean()          # some vectors take one of the pair alone
+    for sizes in ((1, 2, 3, 127), (128, 129, 200), (256,)):
+        at, i, total, parts = 0, 0, 0, []
+        while at < n:
+            c = min(sizes[i % len(sizes)], n - at)
+            if sizes[0] == 1 and at >= 700:                  # the shortest calls over the first part only
+                c = min(256, n - at)
+            m, t = assign(x[:, :, at:at + c])
+            parts.append(m); total += t; at += c; i += 1
+        assert torch.equal(torch.cat(parts, 1), want) and total == near
