@@ -151,8 +151,8 @@ sinkhorn_pass_kernel(const float* __restrict__ S, int n, int K, int iters, int p
 
 // ---- one launch for the whole call: the P blocks of a sequence (a "team") keep its rows in shared memory, `chunk`
 // tokens per block, and walk the iterations together.  Between two iterations stands one exchange: every block publishes
-// its K column sums and adds up the P x K numbers of its team.  A number travels with the exchange's ordinal in one 8-byte
-// word (the low 16 of a double's 52 mantissa bits give way to it), written and polled whole, so that neither a fence nor
+// its K column sums and adds up the P x K numbers of its team.  A number, a double whole, travels as two 8-byte words, each half
+// of its bits and the exchange's ordinal, written and polled whole, so that neither a fence nor
 // a counter stands between writing and reading it (fp64 atomics into one sum, a fence and an arrival counter took 3.5 us
 // per exchange), and the order of every sum is fixed.  What bounds it is latency: of the ~2.3 us of an iteration a third
 // is the words' way through L2, the rest instruction issue and block barriers.  The launch is cooperative, so
@@ -161,30 +161,29 @@ constexpr int SKT_THREADS = 512;
 constexpr int SKT_TOKENS = 8 * SKT_THREADS;          // tokens per block at most: fp32 column sums of a thread over 8 rows
 constexpr int SKT_BLOCKS = 160;                      // blocks per team at most (the workspace has words for as many)
 constexpr size_t SKT_SMEM = 200 * 1024;
-constexpr unsigned long long SKT_TAG = 0xffffull;
 constexpr long long SKT_LEAD = 500;                  // cycles before the first poll
 
 // words of one sequence's exchanges: two sets, taken in turn.  A block writes set e mod 2 for exchange e + 2 after it has
 // read everybody's e + 1, which each of them wrote after reading everybody's e.
 static int skt_max_blocks(int n) { return cdiv(n, SKT_THREADS) < SKT_BLOCKS ? cdiv(n, SKT_THREADS) : SKT_BLOCKS; }
 // Every block has 128-byte lines of its own.
-__host__ __device__ constexpr size_t skt_stride(int ld) { return ld < 16 ? 128 : (size_t)ld * 8; }
+__host__ __device__ constexpr size_t skt_stride(int ld) { return ld < 8 ? 128 : (size_t)ld * 16; }
 static size_t skt_words_bytes(const focus_shape* s) { return 2 * skt_max_blocks(s->n) * skt_stride(focus_soft_ld(s->K)); }
 
-__device__ __forceinline__ void put_word(void* p, double v, unsigned long long tag) {
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)__double_as_longlong(v) & ~SKT_TAG) | tag) : "memory");
+__device__ __forceinline__ void put_word(void* p, double v, unsigned int tag) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"((bits & 0xffffffff00000000ull) | tag), "l"(bits << 32 | tag) : "memory");
 }
-__device__ __forceinline__ bool get_words(const void* p, unsigned long long tag, double& v0, double& v1) {
+__device__ __forceinline__ bool get_word(const void* p, unsigned int tag, double& v) {
     unsigned long long a, b;
     asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-    v0 = __longlong_as_double((long long)(a & ~SKT_TAG));
-    v1 = __longlong_as_double((long long)(b & ~SKT_TAG));
-    return (a & SKT_TAG) == tag && (b & SKT_TAG) == tag;
+    v = __longlong_as_double((long long)((a & 0xffffffff00000000ull) | b >> 32));
+    return (unsigned int)a == tag && (unsigned int)b == tag;
 }
 
-// log2 of a positive double to about 1e-11, in a quarter of the time of the library's (it stands between two iterations):
-// Tang's table method.  tab[k] = (c, -log2 c) with c a float near 1 / (1 + (k + 1/2) / 32); u = m c - 1 for the mantissa m
-// is below 1/60, and the terms of log1p(u) beyond the first are summed in fp32.
+// log2 of a positive double to 1e-15, in less time than the library's (it stands between two iterations): Tang's table
+// method.  tab[k] = (c, -log2 c) with c a float near 1 / (1 + (k + 1/2) / 32); u = m c - 1 for the mantissa m is below 1/60, exact
+// but for one rounding, and log1p(u) is summed to its eighth term (the ninth is below 1e-17).
 __device__ __forceinline__ double2 log2_entry(int k) {
     const float c = 1.f / (1.f + (k + 0.5f) / 32.f);
     return make_double2((double)c, -log2((double)c));
@@ -195,10 +194,11 @@ __device__ __forceinline__ double log2_table(double x, const double2* tab) {
     const int e = (int)(bits >> 52) - 1023;
     const double m = __longlong_as_double((bits & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
     const double2 t = tab[(int)(bits >> 47) & 31];
-    const double u = fma(m, t.x, -1.0);
-    const float uf = (float)u;
-    const float tail = uf * uf * fmaf(uf, fmaf(uf, fmaf(uf, 0.2f, -0.25f), 0.333333333f), -0.5f);
-    return (double)e + t.y + 1.4426950408889634 * (u + (double)tail);
+    const double u = fma(m, t.x, -1.0), u2 = u * u;
+    // -1/2 + u/3 - u^2/4 + ... - u^6/8, in pairs so that the chain is short
+    const double p01 = fma(u, 1.0 / 3, -0.5), p23 = fma(u, 1.0 / 5, -0.25), p45 = fma(u, 1.0 / 7, -1.0 / 6);
+    const double tail = u2 * fma(u2, fma(u2, fma(u2, -0.125, p45), p23), p01);
+    return ((double)e + t.y) + 1.4426950408889634 * (u + tail);
 }
 __device__ __forceinline__ float ex2f(float x) {
     float y;
@@ -266,11 +266,11 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
     if (threadIdx.x == 0) failed_s = 0;
 
     // the exchange: the warps' values (red) become the block's, the blocks' the team's; collect(g, value) runs in lane g
-    // of the first warp.  Thread t polls the words of groups 2 (t mod KMAX / 2) and the next.
-    unsigned long long ordinal = 0;
+    // of the first warp.  Thread t polls the words of group t mod KMAX.
+    unsigned int ordinal = 0;
     auto exchange = [&](auto is_max, auto collect) {
         constexpr bool MAX = decltype(is_max)::value;
-        constexpr int PARTS = 32 / KMAX, PAIRS = KMAX / 2;
+        constexpr int PARTS = 32 / KMAX;
         auto combine = [](double x, double y) { return MAX ? fmax(x, y) : x + y; };
         // lane l: value l mod KMAX of the warps, PARTS lanes a value
         auto over_warps = [&](auto& vals) {
@@ -286,17 +286,17 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
         __syncthreads();                             // red holds the warps' values
         if (warp == 0) {
             const double v = over_warps(red);
-            if (lane < KMAX) put_word(set + (size_t)rank * skt_stride(KMAX) + lane * 8, v, ordinal);
+            if (lane < KMAX) put_word(set + (size_t)rank * skt_stride(KMAX) + lane * 16, v, ordinal);
         }
-        double v0 = MAX ? -INFINITY : 0.0, v1 = v0;
+        double v = MAX ? -INFINITY : 0.0;
         if (!failed_s) {
-            constexpr int STEP = SKT_THREADS / PAIRS, PER = (SKT_BLOCKS + STEP - 1) / STEP;
-            double got[PER][2];
+            constexpr int STEP = SKT_THREADS / KMAX, PER = (SKT_BLOCKS + STEP - 1) / STEP;
+            double got[PER];
             bool seen[PER];
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
-                got[j][0] = got[j][1] = v0;
-                seen[j] = threadIdx.x / PAIRS + j * STEP >= P;
+                got[j] = v;
+                seen[j] = threadIdx.x / KMAX + j * STEP >= P;
             }
             // A poll that comes too early makes the next one take 1.4 us instead of 0.4, and a block that is late by that
             // much makes the others' polls come too early in the next exchange; so wait out most of the words' way first.
@@ -308,8 +308,8 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
                 all = true;
 #pragma unroll
                 for (int j = 0; j < PER; ++j) {
-                    const int q = threadIdx.x / PAIRS + j * STEP;
-                    if (!seen[j]) all &= seen[j] = get_words(set + (size_t)q * skt_stride(KMAX) + threadIdx.x % PAIRS * 16, ordinal, got[j][0], got[j][1]);
+                    const int q = threadIdx.x / KMAX + j * STEP;
+                    if (!seen[j]) all &= seen[j] = get_word(set + (size_t)q * skt_stride(KMAX) + threadIdx.x % KMAX * 16, ordinal, got[j]);
                 }
                 if (!all && clock64() - t0 > 4000000000ll) {          // two seconds
                     failed_s = 1;
@@ -317,14 +317,11 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
                 }
             }
 #pragma unroll
-            for (int j = 0; j < PER; ++j) { v0 = combine(v0, got[j][0]); v1 = combine(v1, got[j][1]); }
+            for (int j = 0; j < PER; ++j) v = combine(v, got[j]);
         }
 #pragma unroll
-        for (int off = 16; off >= PAIRS; off /= 2) {
-            v0 = combine(v0, __shfl_xor_sync(0xffffffffu, v0, off));
-            v1 = combine(v1, __shfl_xor_sync(0xffffffffu, v1, off));
-        }
-        if (lane < PAIRS) { team_s[warp][2 * lane] = v0; team_s[warp][2 * lane + 1] = v1; }
+        for (int off = 16; off >= KMAX; off /= 2) v = combine(v, __shfl_xor_sync(0xffffffffu, v, off));
+        if (lane < KMAX) team_s[warp][lane] = v;
         __syncthreads();
         if (warp == 0) {
             const double v = over_warps(team_s);

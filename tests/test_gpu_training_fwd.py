@@ -153,6 +153,20 @@ def test_sinkhorn_closed_groups(n, K, tau):
         assert out[..., :K].isnan().all() and ds[..., :K].isnan().all()
 
 
+def test_sinkhorn_column_sums_keep_all_bits():
+    """the column sums that the derivative leaves at the start of its workspace are sums in fp64: 1 from one warp's token plus exp(-14)
+    in fp32 from another's needs 44 bits"""
+    n, K, tau, iters = 512, 1, 0.1, 1
+    S = torch.full((1, n, 4), -60.0, device="cuda")              # exp(-600): 0 in fp32
+    S[0, 0, 0], S[0, 170, 0] = 0.0, -1.4
+    shape = fb.make_shape(4, 2, n, 128, K, 1, 16)
+    ws = torch.zeros(fb.focus_sinkhorn_bwd_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+    fb.focus_sinkhorn_bwd(shape, S, tau, iters, ws, torch.ones_like(S), torch.empty_like(S))
+    small = ws[:8].view(torch.float64).item() - 1.0
+    assert abs(small / np.exp(-14.0) - 1) < 1e-5 and np.float32(small) == small
+    assert small * 2.0 ** 36 != round(small * 2.0 ** 36)
+
+
 def gate_case(Hq, Hkv, n, D, K, seed, batch=1):
     g = torch.Generator(device="cuda"); g.manual_seed(seed)
     Q = torch.randn((batch, Hq, n, D), generator=g, device="cuda").to(torch.bfloat16)
