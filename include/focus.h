@@ -326,6 +326,8 @@ FOCUS_API int focus_count_kept_noalloc(const focus_shape* shape, const uint32_t*
  *   tau > 0, iters >= 1 (the paper uses tau = 0.1, iters = 10)
  *   ws          device scratch, focus_sinkhorn_workspace_bytes(shape, iters) bytes, 16-byte aligned
  *   g_out       device fp32 [batch, n, ld]; entries g >= K are written as 0; may be the scores buffer itself
+ * A score of minus infinity closes a group to a token (weight 0); a token closed to every group, or a score that is not a number, makes
+ * the sequence NaN.  So does a wait between the blocks of the one-launch form that runs out after two seconds.
  *
  * focus_gate_attn_fwd -- Eq. 2: for j <= i
  *        s_ij = scale * q_i.k_j * ( 1 if i - j <= window, else sigmoid(lambda * g_i.g_j) ),
@@ -393,6 +395,15 @@ FOCUS_API int focus_selftest_umma(int32_t D, const void* a, const void* b, const
 FOCUS_API int focus_selftest_stalled_wait(const focus_shape* shape, focus_tensor q, focus_tensor k, focus_tensor v,
                                           focus_tensor o, float* lse, unsigned long long wait_limit_ns,
                                           int32_t* dev_status, void* stream);
+
+/*
+ * focus_selftest_stalled_exchange -- diagnostic, not on the hot path: focus_sinkhorn in its one-launch form (K <= 4, a sequence whose
+ * rows fit the blocks' shared memory) with waits of wait_limit_cycles, in which the first block of every sequence is late by four of
+ * them at exchange stall_at (1 = column maxima, 2 = first column sums, ... iters + 1; 0 = never).  Where a block's wait runs out
+ * before the last exchange, g_out holds NaN throughout.
+ */
+FOCUS_API int focus_selftest_stalled_exchange(const focus_shape* shape, const float* scores, float tau, int32_t iters, void* ws,
+                                              size_t ws_bytes, int64_t wait_limit_cycles, int32_t stall_at, float* g_out, void* stream);
 
 /*
  * focus_selftest_umma_pair -- diagnostic (the paper has no counterpart): the same two tiles with D = 128 through one

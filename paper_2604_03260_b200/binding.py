@@ -110,6 +110,8 @@ def lib():
         L.focus_selftest_mma_rate.argtypes = [i32, i32, i32, i32, i32, vp, vp]
         L.focus_selftest_stalled_wait.restype = C.c_int
         L.focus_selftest_stalled_wait.argtypes = [SP, focus_tensor, focus_tensor, focus_tensor, focus_tensor, vp, C.c_uint64, vp, vp]
+        L.focus_selftest_stalled_exchange.restype = C.c_int
+        L.focus_selftest_stalled_exchange.argtypes = [SP, vp, f32, i32, vp, sz, C.c_int64, i32, vp, vp]
         _lib = L
     return _lib
 
@@ -274,6 +276,11 @@ def focus_selftest_mma_rate(pair, N, ts, pattern, rounds, result, stream=None):
 def focus_selftest_stalled_wait(shape, q, k, v, o, lse, wait_limit_ns, dev_status, stream=None):
     _check(lib().focus_selftest_stalled_wait(C.byref(shape), tensor_arg(q), tensor_arg(k), tensor_arg(v), tensor_arg(o), _p(lse),
                                              wait_limit_ns, _p(dev_status), _stream(stream)))
+
+
+def focus_selftest_stalled_exchange(shape, scores, tau, iters, ws, wait_limit_cycles, stall_at, g_out, stream=None):
+    _check(lib().focus_selftest_stalled_exchange(C.byref(shape), _p(scores), tau, iters, _p(ws), ws.numel() * ws.element_size(),
+                                                 wait_limit_cycles, stall_at, _p(g_out), _stream(stream)))
 
 
 def alloc_workspace(shape, layout, device="cuda") -> torch.Tensor:

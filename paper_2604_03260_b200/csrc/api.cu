@@ -258,6 +258,21 @@ int focus_sinkhorn(const focus_shape* shape, const float* scores, float tau, int
     return launch_sinkhorn(shape, scores, tau, iters, ws, g_out, (cudaStream_t)stream);
 }
 
+int focus_selftest_stalled_exchange(const focus_shape* shape, const float* scores, float tau, int32_t iters, void* ws, size_t ws_bytes,
+                                    int64_t wait_limit_cycles, int32_t stall_at, float* g_out, void* stream) {
+    int rc = validate_shape(shape);
+    if (rc) return rc;
+    if (!scores || !ws || !g_out) return fail(FOCUS_ERR_INVALID_ARG, "scores, ws or g_out is NULL");
+    if (!(tau > 0.f) || iters < 1 || iters > 1000) return fail(FOCUS_ERR_INVALID_ARG, "tau must be positive and iters in [1, 1000]");
+    if ((uintptr_t)scores % 16 || (uintptr_t)g_out % 16 || (uintptr_t)ws % 16)
+        return fail(FOCUS_ERR_INVALID_ARG, "scores, g_out and ws must be 16-byte aligned");
+    if (ws_bytes < sinkhorn_workspace_bytes(shape, iters)) return fail(FOCUS_ERR_CAPACITY, "sinkhorn workspace is too small");
+    if (wait_limit_cycles < 1000 || wait_limit_cycles > 4000000000ll || stall_at < 0 || stall_at > iters + 1)
+        return fail(FOCUS_ERR_INVALID_ARG, "wait_limit_cycles must lie in [1e3, 4e9] and stall_at in [0, iters + 1]");
+    if ((rc = require_sm100())) return rc;
+    return launch_sinkhorn_stalled(shape, scores, tau, iters, ws, g_out, wait_limit_cycles, stall_at, (cudaStream_t)stream);
+}
+
 size_t focus_sinkhorn_bwd_workspace_bytes(const focus_shape* shape, int32_t iters) {
     if (validate_shape(shape) || iters < 1) return 0;
     return sinkhorn_bwd_workspace_bytes(shape, iters);

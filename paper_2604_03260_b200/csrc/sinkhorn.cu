@@ -162,6 +162,7 @@ constexpr int SKT_TOKENS = 8 * SKT_THREADS;          // tokens per block at most
 constexpr int SKT_BLOCKS = 160;                      // blocks per team at most (the workspace has words for as many)
 constexpr size_t SKT_SMEM = 200 * 1024;
 constexpr long long SKT_LEAD = 500;                  // cycles before the first poll
+constexpr long long SKT_LIMIT = 4000000000ll;        // cycles of a wait: two seconds
 
 // words of one sequence's exchanges: two sets, taken in turn.  A block writes set e mod 2 for exchange e + 2 after it has
 // read everybody's e + 1, which each of them wrote after reading everybody's e.
@@ -234,10 +235,12 @@ __device__ __forceinline__ void reduce_lanes(float (&v)[N]) {
 
 // BWD = false: out = the assignments.  BWD = true: the column sums again, then the derivative of the assignments
 // from d_in to out (the passes of sinkhorn_bwd_pass_kernel and sinkhorn_bwd_last_kernel below).
-template <int KMAX, bool BWD>
+// LATE: diagnostic, waits of late_limit cycles, and the first block of a sequence comes late by four of them to exchange late_at.
+template <int KMAX, bool BWD, bool LATE>
 __global__ void __launch_bounds__(SKT_THREADS, 1)
 sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float inv_tau, unsigned char* __restrict__ ws,
-                     unsigned char* __restrict__ words, size_t words_bytes, const float* d_in, float* out, int P, int chunk) {
+                     unsigned char* __restrict__ words, size_t words_bytes, const float* d_in, float* out, int P, int chunk,
+                     long long late_limit, unsigned int late_at) {
     extern __shared__ float4 rows_s[];               // [KMAX / 4][chunk] scores, then as many of the derivative
     constexpr int NW = SKT_THREADS / 32, PIECES = KMAX / 4;
     __shared__ float red[NW][KMAX];
@@ -281,8 +284,13 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
             for (int off = 16; off >= KMAX; off /= 2) v = combine(v, __shfl_xor_sync(0xffffffffu, v, off));
             return v;
         };
+        // A wait that runs out leaves the block with sums that are not numbers, hence with such offsets and such sums to publish from
+        // then on: nobody goes on with sums that lack somebody's.  (A maximum passes over what is not a number; see there.)
+        const double none = __longlong_as_double(0x7fffffffffffffffll);
         ++ordinal;
         unsigned char* const set = words + (size_t)(ordinal & 1) * P * skt_stride(KMAX);
+        if (LATE && ordinal == late_at && rank == 0 && threadIdx.x == 0)
+            for (const long long t0 = clock64(); clock64() - t0 < 4 * late_limit;) { }
         __syncthreads();                             // red holds the warps' values
         if (warp == 0) {
             const double v = over_warps(red);
@@ -311,13 +319,16 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
                     const int q = threadIdx.x / KMAX + j * STEP;
                     if (!seen[j]) all &= seen[j] = get_word(set + (size_t)q * skt_stride(KMAX) + threadIdx.x % KMAX * 16, ordinal, got[j]);
                 }
-                if (!all && clock64() - t0 > 4000000000ll) {          // two seconds
+                if (!all && clock64() - t0 > (LATE ? late_limit : SKT_LIMIT)) {
                     failed_s = 1;
+                    got[0] = none;
                     break;
                 }
             }
 #pragma unroll
             for (int j = 0; j < PER; ++j) v = combine(v, got[j]);
+        } else {
+            v = none;
         }
 #pragma unroll
         for (int off = 16; off >= KMAX; off /= 2) v = combine(v, __shfl_xor_sync(0xffffffffu, v, off));
@@ -357,7 +368,7 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
         store_warp(mx);
     }
     exchange(std::true_type{}, [&](int g, double m) {
-        colmax_s[g] = m > -INFINITY ? (float)m : float_of_ordered(0u);         // (a word holds a float exactly); no maximum: NaN
+        colmax_s[g] = m > -INFINITY && !failed_s ? (float)m : float_of_ordered(0u);         // no maximum: NaN
         voff_s[g] = g < K ? 0.f : -INFINITY;
         ct_s[g] = pend_sub_s[g] = 0.f;
         pend_inv_s[g] = g < K ? 1.f : 0.f;
@@ -516,9 +527,9 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
 
 // Runs the call as one cooperative launch if the rows of every sequence fit in its team's shared memory; `done` says
 // whether it did.  A team has one block per 512 tokens, at most its share of the multiprocessors.
-template <int KMAX, bool BWD>
+template <int KMAX, bool BWD, bool LATE = false>
 static int launch_team(const focus_shape* s, const float* S, float tau, int iters, unsigned char* ws, const float* d_in, float* out,
-                       cudaStream_t st, bool& done) {
+                       cudaStream_t st, bool& done, long long late_limit = 0, unsigned int late_at = 0) {
     done = false;
     int dev = 0, sms = 0, rc;
     if ((rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
@@ -531,8 +542,8 @@ static int launch_team(const focus_shape* s, const float* S, float tau, int iter
     const size_t smem = (size_t)chunk * KMAX * sizeof(float) * (BWD ? 2 : 1);
     if (chunk > SKT_TOKENS || smem > SKT_SMEM) return 0;
     P = cdiv(s->n, chunk);                           // no block without tokens
-    auto kern = sinkhorn_team_kernel<KMAX, BWD>;
-    if ((rc = check_cuda(allow_smem<sinkhorn_team_kernel<KMAX, BWD>>(SKT_SMEM), "cudaFuncSetAttribute(sinkhorn)"))) return rc;
+    auto kern = sinkhorn_team_kernel<KMAX, BWD, LATE>;
+    if ((rc = check_cuda(allow_smem<sinkhorn_team_kernel<KMAX, BWD, LATE>>(SKT_SMEM), "cudaFuncSetAttribute(sinkhorn)"))) return rc;
     cudaLaunchAttribute coop;
     coop.id = cudaLaunchAttributeCooperative;
     coop.val.cooperative = 1;
@@ -545,7 +556,7 @@ static int launch_team(const focus_shape* s, const float* S, float tau, int iter
     cfg.numAttrs = 1;
     done = true;
     return check_cuda(cudaLaunchKernelEx(&cfg, kern, S, s->n, s->K, iters, tau, 1.f / tau, ws, ws + s->batch * sk_seq_bytes(iters),
-                                         skt_words_bytes(s), d_in, out, P, chunk), "sinkhorn launch");
+                                         skt_words_bytes(s), d_in, out, P, chunk, late_limit, late_at), "sinkhorn launch");
 }
 
 size_t sinkhorn_workspace_bytes(const focus_shape* s, int iters) { return (size_t)s->batch * (sk_seq_bytes(iters) + skt_words_bytes(s)); }
@@ -566,6 +577,16 @@ static int launch_sk(const focus_shape* s, const float* S, float tau, int iters,
         sinkhorn_pass_kernel<KMAX, 1><<<grid, SK_THREADS, 0, st>>>(S, n, K, iters, pass, inv_tau, ws, nullptr);
     sinkhorn_pass_kernel<KMAX, 2><<<grid, SK_THREADS, 0, st>>>(S, n, K, iters, iters, inv_tau, ws, out);
     return check_cuda(cudaGetLastError(), "sinkhorn kernel launch");
+}
+
+int launch_sinkhorn_stalled(const focus_shape* s, const float* S, float tau, int iters, void* ws, float* out, long long limit, int stall_at,
+                            cudaStream_t st) {
+    if (s->K > 4) return fail(FOCUS_ERR_UNSUPPORTED, "the stalled exchange takes K <= 4");
+    unsigned char* w = reinterpret_cast<unsigned char*>(ws);
+    int rc = check_cuda(cudaMemsetAsync(w, 0, sinkhorn_workspace_bytes(s, iters), st), "cudaMemsetAsync(sinkhorn workspace)");
+    bool done = false;
+    if (rc || (rc = launch_team<4, false, true>(s, S, tau, iters, w, nullptr, out, st, done, limit, (unsigned int)stall_at))) return rc;
+    return done ? FOCUS_OK : fail(FOCUS_ERR_UNSUPPORTED, "the sequence does not fit the one-launch form");
 }
 
 int launch_sinkhorn(const focus_shape* s, const float* S, float tau, int iters, void* ws, float* out, cudaStream_t st) {

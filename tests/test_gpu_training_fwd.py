@@ -167,6 +167,28 @@ def test_sinkhorn_column_sums_keep_all_bits():
     assert small * 2.0 ** 36 != round(small * 2.0 ** 36)
 
 
+@pytest.mark.parametrize("n,batch", [(5000, 1), (1500, 3), (20000, 1)])
+def test_sinkhorn_wait_that_runs_out(n, batch):
+    """one block of a sequence is late by four times the limit of a wait (half a millisecond): wherever that is, nothing that looks like
+    a result is left, not even in the late block's rows, and the next call is right again"""
+    K, tau, iters = 4, 0.1, 6
+    g = torch.Generator(device="cuda"); g.manual_seed(n)
+    S = 0.3 * torch.randn((batch, n, K), generator=g, device="cuda")
+    shape = fb.make_shape(4, 2, n, 128, K, 1, 16, batch=batch)
+    ws = torch.empty(fb.focus_sinkhorn_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+    want, got = torch.empty_like(S), torch.empty_like(S)
+    fb.focus_sinkhorn(shape, S, tau, iters, ws, want)
+    assert want.isfinite().all()
+    for stall_at in (1, 2, 4, iters - 1, iters):
+        fb.focus_selftest_stalled_exchange(shape, S, tau, iters, ws, 1000000, stall_at, got)
+        assert got.isnan().all(), stall_at
+    fb.focus_selftest_stalled_exchange(shape, S, tau, iters, ws, 1000000, iters + 1, got)
+    late = got.isnan()                             # the last exchange: the late block has everybody's sums and is right
+    assert late.any() and torch.equal(got[~late], want[~late])
+    fb.focus_selftest_stalled_exchange(shape, S, tau, iters, ws, 1000000, 0, got)
+    assert torch.equal(got, want)
+
+
 def gate_case(Hq, Hkv, n, D, K, seed, batch=1):
     g = torch.Generator(device="cuda"); g.manual_seed(seed)
     Q = torch.randn((batch, Hq, n, D), generator=g, device="cuda").to(torch.bfloat16)
