@@ -62,6 +62,9 @@ inline size_t sorted_scratch_bytes(const focus_shape* s) {
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The driver's number of the calling thread's context, never used twice in a process; 0 = none yet, or not told
+unsigned long long current_context();
+
 // A read in a kernel that may have been set up before its predecessor's end: a plain load, which stays behind dep_wait().  The
 // non-coherent path (__ldg, or a pointer to const declared __restrict__) is for data that is constant for the kernel's whole
 // lifetime, and that starts before the writer is through; so these kernels use neither.
@@ -83,20 +86,20 @@ inline cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 blo
     return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
 }
 
-// Lets KERN use `bytes` of dynamic shared memory on the current device (and, `carveout`, all of the SM's storage as shared
-// memory).  The driver is asked once per kernel and device: the attributes stay with the kernel, and asking costs about as
-// much as a launch.
+// Lets KERN use `bytes` of dynamic shared memory in the current context (and, `carveout`, all of the SM's storage as shared
+// memory).  The driver is asked once per kernel and context, as long as the calls on a device stay in one context: the attributes
+// belong to the context, and asking costs about as much as a launch.
 template <auto KERN>
 inline cudaError_t allow_smem(size_t bytes, bool carveout = false) {
-    static std::atomic<unsigned long long> devices{0};
+    static std::atomic<unsigned long long> set_in[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-    if (devices.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const unsigned long long ctx = dev < 64 ? current_context() : 0ull;
+    if (ctx && set_in[dev].load(std::memory_order_acquire) == ctx) return cudaSuccess;
     if ((e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
     if (carveout && (e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess) return e;
-    devices.fetch_or(bit, std::memory_order_release);
+    if (ctx) set_in[dev].store(ctx, std::memory_order_release);
     return cudaSuccess;
 }
 #endif

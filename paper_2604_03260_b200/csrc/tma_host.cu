@@ -16,6 +16,17 @@ static PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
     return fn;
 }
 
+unsigned long long current_context() {
+    static const PFN_cuCtxGetId_v12000 fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool found = cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
+        return found ? reinterpret_cast<PFN_cuCtxGetId_v12000>(p) : nullptr;
+    }();
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0ull;
+}
+
 int make_tmap_bf16_4d(CUtensorMap* out, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3,
                       uint64_t s1_bytes, uint64_t s2_bytes, uint64_t s3_bytes, uint32_t box0, uint32_t box1) {
     auto enc = get_encoder();
