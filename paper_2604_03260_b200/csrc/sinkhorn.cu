@@ -525,8 +525,8 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
     }
 }
 
-// Runs the call as one cooperative launch if the rows of every sequence fit in its team's shared memory; `done` says
-// whether it did.  A team has one block per 512 tokens, at most its share of the multiprocessors.
+// Runs the call as one cooperative launch if the rows of every sequence fit in its team's shared memory and the context has the
+// multiprocessors for all teams at once; `done` says whether it did.  A team has one block per 512 tokens, at most its share of the multiprocessors.
 template <int KMAX, bool BWD, bool LATE = false>
 static int launch_team(const focus_shape* s, const float* S, float tau, int iters, unsigned char* ws, const float* d_in, float* out,
                        cudaStream_t st, bool& done, long long late_limit = 0, unsigned int late_at = 0) {
@@ -554,9 +554,14 @@ static int launch_team(const focus_shape* s, const float* S, float tau, int iter
     cfg.stream = st;
     cfg.attrs = &coop;
     cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, S, s->n, s->K, iters, tau, 1.f / tau, ws, ws + s->batch * sk_seq_bytes(iters),
+                                         skt_words_bytes(s), d_in, out, P, chunk, late_limit, late_at);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {   // a partition of the multiprocessors that does not hold the teams at once
+        cudaGetLastError();                          // (not an error of the caller's)
+        return 0;
+    }
     done = true;
-    return check_cuda(cudaLaunchKernelEx(&cfg, kern, S, s->n, s->K, iters, tau, 1.f / tau, ws, ws + s->batch * sk_seq_bytes(iters),
-                                         skt_words_bytes(s), d_in, out, P, chunk, late_limit, late_at), "sinkhorn launch");
+    return check_cuda(e, "sinkhorn launch");
 }
 
 size_t sinkhorn_workspace_bytes(const focus_shape* s, int iters) { return (size_t)s->batch * (sk_seq_bytes(iters) + skt_words_bytes(s)); }

@@ -1,4 +1,4 @@
-"""The entry points in a context other than the device's primary one, in a process of its own."""
+"""The entry points in contexts other than the device's primary one, in processes of their own."""
 import os
 import subprocess
 import sys
@@ -50,6 +50,34 @@ print("done")
 """
 
 
+PARTITION = r"""
+import torch
+from paper_2604_03260_b200 import binding as fb
+from torch.cuda import green_contexts
+n, K, iters = 131072, 8, 5
+S, dg = 0.3 * torch.randn((1, n, K), device="cuda"), torch.randn((1, n, K), device="cuda")
+shape = fb.make_shape(4, 2, n, 128, K, 1, 16)
+ws = torch.empty(fb.focus_sinkhorn_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+wb = torch.empty(fb.focus_sinkhorn_bwd_workspace_bytes(shape, iters), dtype=torch.uint8, device="cuda")
+def both():
+    g, ds = torch.empty_like(S), torch.empty_like(S)
+    fb.focus_sinkhorn(shape, S, 0.1, iters, ws, g)
+    fb.focus_sinkhorn_bwd(shape, S, 0.1, iters, wb, dg, ds)
+    torch.cuda.synchronize()
+    return g, ds
+want = both()
+part = green_contexts.GreenContext.create(num_sms=24, device_id=0)
+part.set_context()
+got = both()
+part.pop_context()
+for a, b in zip(got, want):
+    assert (a - b).abs().max() <= 2e-4 * b.abs().max(), (a - b).abs().max()
+again = both()                                         # no error is left behind
+assert torch.equal(again[0], want[0]) and torch.equal(again[1], want[1])
+print("done")
+"""
+
+
 def run(code):
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=240)
     assert r.returncode == 0 and "done" in r.stdout, r.stdout[-1000:] + r.stderr[-2000:]
@@ -57,3 +85,9 @@ def run(code):
 
 def test_second_context_on_the_device():
     run(SECOND_CONTEXT)
+
+
+def test_partition_of_the_multiprocessors():
+    """24 multiprocessors do not hold the blocks of a long Sinkhorn call at once: a launch per iteration instead"""
+    pytest.importorskip("torch.cuda.green_contexts")
+    run(PARTITION)
