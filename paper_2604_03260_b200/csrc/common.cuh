@@ -65,6 +65,10 @@ __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.lau
 // The driver's number of the calling thread's context, never used twice in a process; 0 = none yet, or not told
 unsigned long long current_context();
 
+// Multiprocessors that a launch of the calling thread into `st` runs on: the device's, or the part that the current context or
+// the stream's green context has; 0 when the driver does not say
+int launch_multiprocessors(cudaStream_t st);
+
 // A read in a kernel that may have been set up before its predecessor's end: a plain load, which stays behind dep_wait().  The
 // non-coherent path (__ldg, or a pointer to const declared __restrict__) is for data that is constant for the kernel's whole
 // lifetime, and that starts before the writer is through; so these kernels use neither.

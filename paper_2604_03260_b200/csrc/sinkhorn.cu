@@ -526,14 +526,14 @@ sinkhorn_team_kernel(const float* S, int n, int K, int iters, float tau, float i
 }
 
 // Runs the call as one cooperative launch if the rows of every sequence fit in its team's shared memory and the context has the
-// multiprocessors for all teams at once; `done` says whether it did.  A team has one block per 512 tokens, at most its share of the multiprocessors.
+// multiprocessors for all teams at once; `done` says whether it did.  A team has one block per 512 tokens, at most its share of
+// the multiprocessors.
 template <int KMAX, bool BWD, bool LATE = false>
 static int launch_team(const focus_shape* s, const float* S, float tau, int iters, unsigned char* ws, const float* d_in, float* out,
                        cudaStream_t st, bool& done, long long late_limit = 0, unsigned int late_at = 0) {
     done = false;
-    int dev = 0, sms = 0, rc;
-    if ((rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice"))) return rc;
-    if ((rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute"))) return rc;
+    int rc;
+    const int sms = launch_multiprocessors(st);      // (a capture takes a cooperative launch without asking whether its blocks fit)
     // (from about 1e36 on the lowest finite exponent of a row no longer stands for weight 0)
     if (s->batch > sms || tau > 1e30f) return 0;
     int P = sms / s->batch;

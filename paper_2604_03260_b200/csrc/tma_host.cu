@@ -16,15 +16,39 @@ static PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
     return fn;
 }
 
+template <class Fn>
+static Fn driver_entry(const char* name) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool found = cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
+    return found ? reinterpret_cast<Fn>(p) : nullptr;
+}
+
 unsigned long long current_context() {
-    static const PFN_cuCtxGetId_v12000 fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const bool found = cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
-        return found ? reinterpret_cast<PFN_cuCtxGetId_v12000>(p) : nullptr;
-    }();
+    static const auto id_of = driver_entry<PFN_cuCtxGetId_v12000>("cuCtxGetId");
     unsigned long long id = 0;
-    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0ull;
+    return id_of && id_of(nullptr, &id) == CUDA_SUCCESS ? id : 0ull;
+}
+
+int launch_multiprocessors(cudaStream_t st) {
+    static const auto current = driver_entry<PFN_cuCtxGetCurrent_v4000>("cuCtxGetCurrent");
+    static const auto of_context = driver_entry<PFN_cuCtxGetDevResource_v12040>("cuCtxGetDevResource");
+    static const auto green_of = driver_entry<PFN_cuStreamGetGreenCtx_v12040>("cuStreamGetGreenCtx");
+    static const auto of_green = driver_entry<PFN_cuGreenCtxGetDevResource_v12040>("cuGreenCtxGetDevResource");
+    if (!current || !of_context || !green_of || !of_green) return 0;
+    CUcontext ctx = nullptr;
+    CUdevResource res;
+    if (current(&ctx) != CUDA_SUCCESS || !ctx || of_context(ctx, &res, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return 0;
+    unsigned int sms = res.sm.smCount;
+    if (st && st != cudaStreamLegacy && st != cudaStreamPerThread) {         // (those are the current context's)
+        CUgreenCtx green = nullptr;
+        if (green_of((CUstream)st, &green) != CUDA_SUCCESS) return 0;
+        if (green) {
+            if (of_green(green, &res, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return 0;
+            if (res.sm.smCount < sms) sms = res.sm.smCount;
+        }
+    }
+    return (int)sms;
 }
 
 int make_tmap_bf16_4d(CUtensorMap* out, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3,
