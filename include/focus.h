@@ -140,7 +140,7 @@ typedef struct {
     /* FOCUS_LAYOUT_SORTED_LOCAL and FOCUS_LAYOUT_GROUP_MAJOR only (0 otherwise): the two partial results, kept in fp32
        until they are joined */
     size_t o_sorted;         /* fp32 [B*Hq][n][D]: class-sorted pass (its logsumexp goes to the caller's lse) */
-    size_t o_local;          /* fp32 [B*Hq][n][D]: reserved (the window pass joins its result in registers) */
+    size_t o_local;          /* empty (the window pass joins its result in registers) */
     size_t lse_local;        /* fp32 [B*Hq][n]: reserved */
 } focus_tiles_layout;
 

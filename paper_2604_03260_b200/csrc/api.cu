@@ -153,7 +153,7 @@ static int layout_of(const focus_shape* s, int layout, focus_tiles_layout* L) {
     }
     if (layout_has_window_pass(layout)) {
         L->o_sorted = take(HQ * (size_t)s->n * s->D * 4);
-        L->o_local = take(HQ * (size_t)s->n * s->D * 4);
+        L->o_local = take(1);                   // (the window pass keeps its result in registers)
         L->lse_local = take(HQ * (size_t)s->n * 4);
     }
     L->total_bytes = off;
