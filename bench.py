@@ -263,7 +263,10 @@ def main():
     status = torch.zeros(4, dtype=torch.int32, device="cuda")
     # assign x2, build_tiles (2 kernels; class-sorted: + 5 of the sort + ranges + order; group-major keys: + 6 for their lists),
     # attention (+ gather); with a window pass: + fill, second attention launch
-    launches_per_step = 2 + 2 + 1 + (7 + 1 if layout in (1, 3, 4) else 0) + (2 if layout in (3, 4) else 0) + (6 if layout == 4 else 0)
+    # (summaries, live bitmap; the groups' bitmaps are a launch of their own when a bitmap row has more than 16 (K > 8: 32) words)
+    words = -(-wl.n // (128 * 32))
+    launches_per_step = (2 + 2 + (1 if words > (16 if wl.K <= 8 else 32) else 0) + 1 + (7 + 1 if layout in (1, 3, 4) else 0) +
+                         (2 if layout in (3, 4) else 0) + (6 if layout == 4 else 0))
 
     ev = lambda: torch.cuda.Event(enable_timing=True)
     marks = []
@@ -392,9 +395,10 @@ def main():
             ms_g = timed_alone(lambda: fb.focus_gate_attn_fwd(shape, Q, K, V, soft, 10.0, O_g, lse_g, status), reps=2)
             del O_g, lse_g
             gtf = dense_flop / (ms_g * 1e-3) / 1e12
-            tr.update(gate_attn_ms=ms_g, gate_attn_tflops=gtf, bound="alu",
-                      gate_note="every causal pair; 4 D flop per pair on the tensor cores, limited by the per-pair gate "
-                                "(K-term dot product, tanh, two multiplies) on the softmax warps")
+            tr.update(gate_attn_ms=ms_g, gate_attn_tflops=gtf, bound="special-function unit",
+                      gate_note="every causal pair; 4 D flop per pair on the tensor cores, limited by a tanh and an exponential per "
+                                "pair and the chain products -> factors -> scores -> softmax of a tile (at D = 256 the softmax "
+                                "warps also take the K-term dot products)")
         extra["focus_training_fwd"] = tr
         del hid, flush
 

@@ -319,9 +319,9 @@ FOCUS_API int focus_count_kept_noalloc(const focus_shape* shape, const uint32_t*
  *
  * focus_sinkhorn -- the Sinkhorn normalisation of Sec. 2: Q = exp(S / tau); `iters` times divide every column
  * by its sum over the tokens of the sequence, then every row by its sum over the groups.  Each sequence of the
- * batch is normalised on its own.  Computed in the log domain (offsets per token and per group, fp32, column
- * sums accumulated in fp64), which is the same arithmetic without overflow; after the first row division every
- * entry lies in (0, 1].
+ * batch is normalised on its own.  Computed in the log domain (offsets per token and per group, fp32; column
+ * sums and their logarithms in fp64 from the warps' fp32 sums on), which is the same arithmetic without overflow; after the
+ * first row division every entry lies in (0, 1].
  *   shape       batch, n, K are read             scores   device fp32 [batch, n, ld] (ld as above)
  *   tau > 0, iters >= 1 (the paper uses tau = 0.1, iters = 10)
  *   ws          device scratch, focus_sinkhorn_workspace_bytes(shape, iters) bytes, 16-byte aligned
@@ -334,7 +334,9 @@ FOCUS_API int focus_count_kept_noalloc(const focus_shape* shape, const uint32_t*
  * then exact row softmax over all j <= i, o_i = sum_j p_ij v_j, lse_i = log sum_j exp(s_ij).  The equation is
  * followed as printed: two orthogonal assignments give the gate sigmoid(0) = 1/2.  Same kernel, operand
  * precision and accumulation as focus_attn_fwd in dense causal mode; the gate is evaluated in fp32 as
- * 1/2 + 1/2 tanh(lambda/2 g_i.g_j) with the hardware tanh approximation.
+ * 1/2 + 1/2 tanh(lambda/2 g_i.g_j) with the hardware tanh approximation.  The products g_i.g_j are fp32 multiply-adds at D = 256;
+ * up to D = 128 they run on the tensor cores, each assignment split into three bf16 terms (24 mantissa bits) and the six
+ * products of terms above 2^-24 accumulated in fp32.
  *   shape       softcap must be 0; K <= 32, and K <= 16 at D = 256 (FOCUS_ERR_UNSUPPORTED otherwise); masks and topk
  *               are not used
  *   q, k, v, o, lse, dev_status   as for focus_attn_fwd

@@ -88,7 +88,8 @@ static int choose_layout(const focus_shape* s) {
     // rows span about 256 * classes positions, so the window of the block covers (256 * classes + w) / classes keys of
     // every class that shares no group with it.  The separate window pass in token order reads w + 256 keys once per
     // 256 rows, plus what a second pass costs per block whatever its length (query load, pipeline fill, fp32 partial
-    // results, merge): about six key tiles' worth, measured.  The pass is taken when it saves a quarter or more.
+    // results): about six key tiles' worth, measured while a kernel of its own still joined the two results; the crossovers have
+    // not been measured again since the second pass joins them.  The pass is taken when it saves a quarter or more.
     const double apart = binom(s->K - s->topk, s->topk);                 // classes without a shared group
     const double in_sorted = apart * ((256.0 * classes + s->window) / classes / 128.0 + 1.0);
     const double in_order = (s->window + 256.0) / 128.0 + 7.0;

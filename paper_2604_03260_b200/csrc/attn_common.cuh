@@ -182,8 +182,8 @@ template <> struct TileWalk<WALK_SORTED> {
     }
 };
 
-// Per-row 128-bit keep bitmap of one (query tile, key tile) pair.  Returns false when the tile needs
-// no mask at all; `all_masked` is set when no pair of the tile can be attended.
+// Per-row 128-bit keep bitmap of one (query tile, key tile) pair: `masked` when it has to be applied at all, `all_masked` when no
+// pair of the tile can be attended.
 struct TileMask {
     uint32_t kw[4];
     bool masked, all_masked;
