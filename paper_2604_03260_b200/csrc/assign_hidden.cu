@@ -261,7 +261,7 @@ assign_hidden_kernel(const __nv_bfloat16* h, int64_t stride_b, int64_t stride_n,
             }
             const bool own = rank == 0;
 #pragma unroll
-            for (int g = 0; g < KMAX; ++g) score[g] += (bias && g < K) ? dep_load(bias + g) : 0.f;
+            for (int g = 0; g < KMAX; ++g) score[g] += (bias && g < K) ? __ldg(bias + g) : 0.f;      // (not the fold kernel's: constant)
             if (scores) {   // the scores themselves (training-time soft assignment), rows of KMAX floats, zero beyond K
                 if (in && ok && own) {
                     float4* o = reinterpret_cast<float4*>(scores + ((size_t)b * n + tok) * KMAX);

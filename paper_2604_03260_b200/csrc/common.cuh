@@ -71,7 +71,8 @@ int launch_multiprocessors(cudaStream_t st);
 
 // A read in a kernel that may have been set up before its predecessor's end: a plain load, which stays behind dep_wait().  The
 // non-coherent path (__ldg, or a pointer to const declared __restrict__) is for data that is constant for the kernel's whole
-// lifetime, and that starts before the writer is through; so these kernels use neither.
+// lifetime, and that starts before the writer is through; so these kernels use neither on what their direct predecessor may
+// have written.  (What is older is complete before they are set up.)
 template <class T>
 __device__ __forceinline__ T dep_load(const T* p) { return *p; }
 

@@ -46,7 +46,8 @@ def test_dependent_kernels_use_plain_loads():
                 continue
             seen.add(name)
             assert not re.search(r"const[^,]*__restrict__", funcs[name][0]), (f, name)
-            assert not any("__ldg" in body for _, body in parts), (f, name)
+            # (the bias is older than the fold kernel that precedes the one place where it is read)
+            assert not any("__ldg" in body.replace("__ldg(bias + g)", "") for _, body in parts), (f, name)
     assert seen >= {"assign_kernel", "assign_hidden_kernel", "fold_router_kernel", "decode_partial_kernel",
                     "decode_merge_kernel", "summarise_kernel", "group_tiles_kernel", "live_kernel", "focus_attn_kernel"}, seen
 
