@@ -51,11 +51,33 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
     return r;
 }
 
+// Division of 0 <= n < 2^31 by d >= 1 as a multiplication: q = n (2^(31 + l) / d + 1) / 2^(31 + l) with 2^l >= d.  (The compiler's
+// own, for a divisor it does not know, is some 20 instructions.)
+struct Divisor {
+    uint32_t d, m;
+    int s;
+    Divisor() = default;
+    explicit Divisor(int by) : d((uint32_t)by), m(0), s(0) {
+        int l = 0;
+        while ((1ll << l) < by) ++l;
+        if (l > 0) { m = (uint32_t)((1ull << (31 + l)) / d + 1); s = l - 1; }
+    }
+    __host__ __device__ int div(int n) const {
+        if (d == 1) return n;
+#ifdef __CUDA_ARCH__
+        return (int)(__umulhi((uint32_t)n, m) >> s);
+#else
+        return (int)((uint64_t)(uint32_t)n * m >> 32 >> s);
+#endif
+    }
+};
+
 struct AttnParams {
     int B, Hq, Hkv, G, n, K;
     int w;                   // window, at most n: positions and differences of positions stay within 32 bits
     int nqb;                 // items per head: 256-row query blocks (128-row tiles when D = 256)
     int nqt, nkt, nkw;
+    Divisor by_heads, by_group, by_G, by_Hkv, by_Hq;      // by batch * Hq, nqb * G, G, Hkv, Hq
     float scale, softcap;
     const uint32_t* mq;
     const uint32_t* gbits;
@@ -144,6 +166,7 @@ template <> struct TileWalk<WALK_TOKEN> {
         b = f0;
     }
     __device__ __forceinline__ int next() {
+#pragma unroll 1
         while (wd * 32 < f0) {
             if (bits) {
                 const int c = __ffs(bits) - 1;
@@ -153,6 +176,7 @@ template <> struct TileWalk<WALK_TOKEN> {
             ++wd;
             if (wd * 32 >= f0) break;
             uint32_t x = 0;
+#pragma unroll 1
             for (int r = 0; r < nl; ++r) x |= dep_load(l0 + (size_t)r * nkw + wd);
             const int rem = f0 - wd * 32;
             bits = rem < 32 ? x & ((1u << rem) - 1u) : x;
@@ -165,13 +189,14 @@ template <> struct TileWalk<WALK_SORTED> {
     const int32_t* qr;          // the ranges of sorted key tiles, key class by key class
     int nck, jk, b, rend;       // jk = class of the tile that next() returned
     __device__ __forceinline__ void init(const AttnParams& p, int hq, int a0, int) {
-        const int hk = (hq / p.Hq) * p.Hkv + (hq % p.Hq) / p.G;
+        const int bb = p.by_Hq.div(hq), hk = bb * p.Hkv + p.by_G.div(hq - bb * p.Hq);
         qr = p.qrange + ((size_t)hq * p.nqblk + (a0 >> 1)) * FOCUS_MAX_CLASSES * 2;
         nck = dep_load(p.ncls_k + hk);
         jk = -1;
         b = rend = 0;
     }
     __device__ __forceinline__ int next() {
+#pragma unroll 1
         while (b >= rend) {
             if (++jk >= nck) return -1;
             const int2 r = dep_load(reinterpret_cast<const int2*>(qr) + jk);
@@ -182,24 +207,20 @@ template <> struct TileWalk<WALK_SORTED> {
     }
 };
 
-// Per-row 128-bit keep bitmap of one (query tile, key tile) pair: `masked` when it has to be applied at all, `all_masked` when no
-// pair of the tile can be attended.
+// Per-row 128-bit keep bitmap of one (query tile, key tile) pair; `masked` when it has to be applied at all.
 struct TileMask {
     uint32_t kw[4];
-    bool masked, all_masked;
+    bool masked;
 };
 
+__device__ __forceinline__ uint32_t low_bits(int n) { return n >= 32 ? 0xffffffffu : (n <= 0 ? 0u : ((1u << n) - 1u)); }
+
 // every causal pair
-__device__ __forceinline__ void build_tile_mask_dense(TileMask& tm, const AttnParams& p, int a, int kb, int i) {
-    const int c0 = kb * 128;
-    tm.all_masked = kb > a || a * 128 >= p.n;
-    tm.masked = c0 + 127 > a * 128;
-    if (tm.masked && !tm.all_masked) {
+__device__ __forceinline__ void build_tile_mask_dense(TileMask& tm, int a, int kb, int i) {
+    tm.masked = kb >= a;
+    if (tm.masked) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int nk = i - c0 + 1 - 32 * q;                          // columns < nk are causal
-            tm.kw[q] = nk >= 32 ? 0xffffffffu : (nk <= 0 ? 0u : ((1u << nk) - 1u));
-        }
+        for (int q = 0; q < 4; ++q) tm.kw[q] = low_bits(i - kb * 128 + 1 - 32 * q);       // columns < that are causal
     }
 }
 
@@ -207,15 +228,14 @@ __device__ __forceinline__ void build_tile_mask_dense(TileMask& tm, const AttnPa
 __device__ __forceinline__ void build_tile_mask(TileMask& tm, const AttnParams& p, int a, int kb, int i, uint32_t mi, int f_x,
                                                 const uint32_t* gbits) {
     const int c0 = kb * 128;
-    const int r_first = a * 128, r_last = r_first + 127;
-    tm.all_masked = c0 > r_last || r_first >= p.n;
-    const bool need_causal = c0 + 127 > r_first;
-    const bool need_window = p.local_only || (kb >= f_x && r_last - c0 > p.w);
+    const bool need_causal = kb >= a;
+    const bool need_window = p.local_only || (kb >= f_x && a * 128 + 127 - c0 > p.w);
     const bool need_group = need_window || kb < f_x;
     tm.masked = need_causal || need_group;
-    if (tm.masked && !tm.all_masked) {
+    if (tm.masked) {
         uint32_t sh[4] = {0, 0, 0, 0};
         if (need_group) {
+#pragma unroll 1
             for (uint32_t rem = mi; rem; rem &= rem - 1) {
                 const uint4 t = *reinterpret_cast<const uint4*>(gbits + (__ffs(rem) - 1) * 4);
                 sh[0] |= t.x; sh[1] |= t.y; sh[2] |= t.z; sh[3] |= t.w;
@@ -227,15 +247,11 @@ __device__ __forceinline__ void build_tile_mask(TileMask& tm, const AttnParams& 
             if (need_group) {
                 keep = sh[q];
                 if (need_window) {
-                    const int lo = i - p.w - c0 - 32 * q;                // columns >= lo are inside the window
-                    const uint32_t win = lo <= 0 ? 0xffffffffu : (lo >= 32 ? 0u : ~((1u << lo) - 1u));
+                    const uint32_t win = ~low_bits(i - p.w - c0 - 32 * q);      // columns from there on are inside the window
                     keep = p.local_only ? (win & ~keep) : (keep | win);     // window pass: in the window and not sharing
                 }
             }
-            if (need_causal) {
-                const int nk = i - c0 + 1 - 32 * q;                      // columns < nk are causal
-                keep &= nk >= 32 ? 0xffffffffu : (nk <= 0 ? 0u : ((1u << nk) - 1u));
-            }
+            if (need_causal) keep &= low_bits(i - c0 + 1 - 32 * q);
             tm.kw[q] = keep;
         }
         // a tile that every row of the warp keeps whole needs no mask after all (rows past the end keep nothing: not asked)
@@ -252,22 +268,21 @@ struct Item { int A, bb, h, hq; };
 template <int WALK>
 __device__ __forceinline__ void item_at(const AttnParams& p, int id, Item& t) {
     if (WALK == WALK_SORTED) {
-        const int2 e = dep_load(reinterpret_cast<const int2*>(p.order) + id / p.ipb);
+        const int2 e = dep_load(reinterpret_cast<const int2*>(p.order) + (id >> (p.ipb - 1)));      // (ipb is 1 or 2)
         t.hq = e.x;
-        t.A = e.y * p.ipb + id % p.ipb;
+        t.A = e.y * p.ipb + (id & (p.ipb - 1));
     } else if (p.by_length) {
-        const int heads = p.B * p.Hq;
-        t.A = p.nqb - 1 - id / heads;
-        t.hq = id % heads;
+        const int q = p.by_heads.div(id);
+        t.A = p.nqb - 1 - q;
+        t.hq = id - q * p.B * p.Hq;
     } else {
-        const int per_group = p.nqb * p.G;
-        const int grp = id / per_group;                   // batch * Hkv + KV head
-        const int rem = id % per_group;
-        t.A = p.nqb - 1 - rem / p.G;
-        t.hq = (grp / p.Hkv) * p.Hq + (grp % p.Hkv) * p.G + rem % p.G;
+        const int grp = p.by_group.div(id);               // batch * Hkv + KV head
+        const int rem = id - grp * p.nqb * p.G, q = p.by_G.div(rem), b = p.by_Hkv.div(grp);
+        t.A = p.nqb - 1 - q;
+        t.hq = b * p.Hq + (grp - b * p.Hkv) * p.G + rem - q * p.G;
     }
-    t.bb = t.hq / p.Hq;
-    t.h = t.hq % p.Hq;
+    t.bb = p.by_Hq.div(t.hq);
+    t.h = t.hq - t.bb * p.Hq;
 }
 
 // number of entries of the ascending 128-entry array `a` that are <= v (fixed-depth search)
@@ -289,25 +304,17 @@ __device__ __forceinline__ int count_le_128(const int32_t* __restrict__ a, int v
 __device__ __forceinline__ void build_tile_mask_sorted(TileMask& tm, int w, const int32_t* __restrict__ kpos, bool share,
                                                        int pos, int wmin, int wmax, bool window_ok) {
     const int k_first = kpos[0], k_last = kpos[127];
-    tm.all_masked = wmax < 0 || k_first > wmax;
-    const bool none = !share && !window_ok;
-    // (window_ok is the same for the whole grid, so the vote is skipped or taken by every lane alike)
-    const bool any_none = !window_ok && __any_sync(0xffffffffu, none);
+    const bool none = wmax < 0 || k_first > wmax || (!share && !window_ok);
     const bool need_causal = k_last > wmin;
     const bool need_window = !share && wmax - k_first > w;          // (wmax >= -1, k_first >= 0)
-    tm.masked = need_causal || need_window || any_none;
+    tm.masked = __any_sync(0xffffffffu, need_causal || need_window || none);        // (rows of one warp may differ: padding)
     tm.kw[0] = tm.kw[1] = tm.kw[2] = tm.kw[3] = 0xffffffffu;
-    if (tm.masked && !tm.all_masked) {
+    if (tm.masked) {
         const int hi = none ? 0 : (need_causal ? (pos < 0 ? 0 : count_le_128(kpos, pos)) : 128);          // columns < hi are causal
         const int edge = pos - w - 1;
         const int lo = (need_window && pos >= 0 && edge >= 0) ? count_le_128(kpos, edge) : 0;   // columns >= lo are in the window
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int h = hi - 32 * q, l = lo - 32 * q;
-            const uint32_t below_hi = h >= 32 ? 0xffffffffu : (h <= 0 ? 0u : ((1u << h) - 1u));
-            const uint32_t below_lo = l >= 32 ? 0xffffffffu : (l <= 0 ? 0u : ((1u << l) - 1u));
-            tm.kw[q] = below_hi & ~below_lo;
-        }
+        for (int q = 0; q < 4; ++q) tm.kw[q] = low_bits(hi - 32 * q) & ~low_bits(lo - 32 * q);
     }
 }
 
@@ -316,6 +323,7 @@ __device__ __forceinline__ void build_tile_mask_sorted(TileMask& tm, int w, cons
 // per-group bitmaps.  Every sharing pair is then computed exactly once.
 __device__ __forceinline__ void exclude_lower_groups(TileMask& tm, const uint32_t* gb, uint32_t lower, int K) {
     uint32_t ex[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
     for (uint32_t rem = lower; rem; rem &= rem - 1) {
         const int a = __ffs(rem) - 1;
         if (a < K) {
@@ -323,11 +331,8 @@ __device__ __forceinline__ void exclude_lower_groups(TileMask& tm, const uint32_
             ex[0] |= t.x; ex[1] |= t.y; ex[2] |= t.z; ex[3] |= t.w;
         }
     }
-    if (ex[0] | ex[1] | ex[2] | ex[3]) {
-        tm.masked = true;
-        tm.kw[0] &= ~ex[0]; tm.kw[1] &= ~ex[1]; tm.kw[2] &= ~ex[2]; tm.kw[3] &= ~ex[3];
-    }
+    tm.kw[0] &= ~ex[0]; tm.kw[1] &= ~ex[1]; tm.kw[2] &= ~ex[2]; tm.kw[3] &= ~ex[3];
+    tm.masked = __any_sync(0xffffffffu, tm.masked || (ex[0] | ex[1] | ex[2] | ex[3]) != 0u);
 }
-
 
 }  // namespace focus

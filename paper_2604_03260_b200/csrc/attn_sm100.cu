@@ -26,6 +26,14 @@
 // reads: 8192 tokens, K = 8, 32/8 heads: 1290 -> 862 us; 32768: 20.7 -> 13.5 ms.  At D = 256 tensor memory and the ring
 // leave one query tile, whose softmax warps evaluate the products themselves.
 //
+// Code size: 45 to 82 KB a kernel, from 65 to 118.  The roles run side by side and each streams through its own code once per
+// tile, so what is executed per tile should fit the instruction caches, and code that is rarely executed should not lie in
+// between: waits and their reports inlined at full length, loops the compiler unrolled by itself and divisions by launch
+// parameters were half of it.  Loops with short trip counts therefore say `unroll 1`, except the issue of a tile's MMAs, whose
+// descriptors must be there when the tensor pipe is (rolled up: 1228 -> 1714 cycles from P to the next S).  12 heads x 16384
+// tokens at D = 64 in dense mode: 614 -> 547 us; 65536 tokens at D = 256 class-sorted: 13.1 -> 12.0 ms; 32 heads x 8192 in token
+// order: 551 -> 530 us, gated: 794 -> 707.
+//
 // Which key tiles are visited, and in which order of items:
 //   dense mode      every tile up to the diagonal
 //   original layout far tiles (every pair beyond the window) only when the live bitmap says the OR
@@ -76,7 +84,7 @@ struct AttnCfg {
     static constexpr uint32_t GK_BYTES = (GATE == 1 ? 4 : 3 * GATE_CH) * GBLK_BYTES;     // one key tile, two buffers
     static constexpr uint32_t GATE_SMEM = GATE == 0 ? 0 : (NQ == 2 ? 2 * GQ_BYTES + 2 * GK_BYTES : 4 * GATE_BUF_BYTES);
     static constexpr int NINFO = (D == 256) ? 3 : 4;         // tiles handed on ahead (what fits beside the K/V ring)
-    // shared memory: Q | K/V ring | gate buffers | tile ring | row exchange | barriers
+    // shared memory: Q | K/V ring | gate operands | tile ring | row exchange | barriers
     static constexpr uint32_t OFF_GATE = NQ * TILE_BYTES + NSTAGE * STAGE_BYTES;
     static constexpr uint32_t OFF_INFO = OFF_GATE + GATE_SMEM;
     static constexpr uint32_t OFF_XVAL = OFF_INFO + (GATE ? 0 : NINFO * (uint32_t)sizeof(TileInfo));
@@ -91,6 +99,7 @@ struct AttnCfg {
     static constexpr int NC = 128 / NSPLIT;                  // S columns per softmax thread
     static constexpr int THREADS = 128 + 128 * NQ * NSPLIT;
     static constexpr int READERS = THREADS / 32 - 3 + (GATE_MMA ? 2 : 0);     // warps that read the queue: MMA, softmax, gate operands
+    static constexpr int TILE_READERS = THREADS / 32 - 3;     // warps that read the tile ring: MMA, softmax
 };
 
 struct SharedCtl {
@@ -100,9 +109,9 @@ struct SharedCtl {
     uint64_t xchg[4];                 // split rows, per 32-row quadrant: both column halves have published a per-row value
     uint64_t gbar[2];                 // soft gate, one query tile, per softmax warpgroup: the key assignments are in shared memory
     uint64_t kv_full[8], kv_empty[8];
-    uint64_t info_full[4], info_empty[4];         // tile ring: handed on, read by the MMA warp and every softmax warp
+    uint64_t info_full[4], info_empty[4];         // tile ring: handed on, read by TILE_READERS warps
     uint64_t next_full[2], next_empty[2];         // the answers below: arrived, read by the MMA warp and every softmax warp
-    unsigned long long limit_ns;      // how long a wait may last before the role gives up
+    uint32_t limit_ns;                // how long a wait may last before the role gives up
     uint32_t tmem_base;
     int abort_flag;
     uint32_t asked;                   // how many answers the TMA thread has asked for
@@ -115,21 +124,24 @@ struct GateCtl {
     uint64_t g_full[2], g_taken[2];   // G of a query tile is in tensor memory / in the softmax warps' registers
 };
 
-// bounded wait that also gives up when another role of the CTA has already given up
-__device__ __forceinline__ bool ctl_wait(uint64_t* bar, uint32_t parity, SharedCtl* ctl) {
-    const uint32_t a = smem_u32(bar);
-    if (mbar_try_wait(a, parity)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    for (;;) {
+// Bounded wait that also gives up when another role of the CTA has given up.  `gave_up` becomes `where`; the role reports it once, at
+// its end (give_up).  Few instructions, for there are some thirty places (the note on code size above); the try in front of the loop is
+// worth its own (D = 256, 16384 tokens dense: 1580 us without it, 1537 so).
+__device__ __forceinline__ bool ctl_wait(uint64_t* bar, uint32_t parity, SharedCtl& ctl, int& gave_up, int where) {
+    if (mbar_try_wait(smem_u32(bar), parity)) return true;          // (a try lasts until the phase completes, or about a millisecond)
+    uint32_t t0 = 0;
 #pragma unroll 1
-        for (int it = 0; it < 128; ++it)
-            if (mbar_try_wait(a, parity)) return true;
-        if (*(volatile int*)&ctl->abort_flag) return false;
-        if (globaltimer_ns() - t0 > ctl->limit_ns) return false;
+    for (;;) {
+        if (mbar_try_wait(smem_u32(bar), parity)) return true;
+        const uint32_t now = globaltimer_lo() | 1u;
+        if (t0 == 0) t0 = now;
+        if (*(volatile int*)&ctl.abort_flag || now - t0 > ctl.limit_ns) break;
     }
+    gave_up = where;
+    return false;
 }
 
-__device__ __forceinline__ void report_timeout(const AttnParams& p, SharedCtl* ctl, int where, int item) {
+__device__ __forceinline__ void give_up(const AttnParams& p, SharedCtl* ctl, int where, int item) {
     *(volatile int*)&ctl->abort_flag = 1;
     if (p.status && atomicCAS(p.status, 0, 1) == 0) {
         p.status[1] = where;
@@ -191,21 +203,16 @@ template <int CH> struct GateSteps {
 // The CTA's item number `ord` (0, 1, ...): the block it was launched as, then what the answers say; false after the last.
 // Called by every thread of a role's warp (`reader`: the warp reports that it has read), or by the TMA thread.
 template <int WALK>
-__device__ __forceinline__ bool next_item(const AttnParams& p, SharedCtl* ctl, uint32_t ord, bool reader, Item& t, bool& ok) {
+__device__ __forceinline__ bool next_item(const AttnParams& p, SharedCtl& ctl, uint32_t ord, bool reader, Item& t, int& gave_up) {
     uint32_t block = blockIdx.x;
     if (ord > 0) {
         const uint32_t slot = (ord - 1) & 1, use = (ord - 1) >> 1;
-        if (!ctl_wait(&ctl->next_full[slot], use & 1, ctl)) {
-            *(volatile int*)&ctl->abort_flag = 1;
-            if (p.status && atomicCAS(p.status, 0, 1) == 0) { p.status[1] = 50; p.status[2] = (int)ord; p.status[3] = (int)blockIdx.x; }
-            ok = false;
-            return false;
-        }
-        const bool more = clc_answer(smem_u32(&ctl->next[slot]), block);
+        if (!ctl_wait(&ctl.next_full[slot], use & 1, ctl, gave_up, 50)) return false;
+        const bool more = clc_answer(smem_u32(&ctl.next[slot]), block);
         if (reader) {
             fence_proxy_async_smem();                   // the answer is read before the next one is written there
             __syncwarp();
-            if ((threadIdx.x & 31) == 0) mbar_arrive(smem_u32(&ctl->next_empty[slot]));
+            if ((threadIdx.x & 31) == 0) mbar_arrive(smem_u32(&ctl.next_empty[slot]));
         }
         if (!more) return false;
     }
@@ -216,7 +223,7 @@ __device__ __forceinline__ bool next_item(const AttnParams& p, SharedCtl* ctl, u
 template <int D, bool SOFTCAP, int GATE, int WALK>
 __global__ void __launch_bounds__(AttnCfg<D, GATE>::THREADS, 1)
 focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                  const __grid_constant__ CUtensorMap tm_v, const AttnParams p) {
+                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ AttnParams p) {
     using C = AttnCfg<D, GATE>;
     constexpr int NQ = C::NQ;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -267,7 +274,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         for (int x = 0; x < C::NINFO; ++x) {
             mbar_init(smem_u32(&ctl.info_full[x]), 1);
-            mbar_init(smem_u32(&ctl.info_empty[x]), C::THREADS / 32 - 3);
+            mbar_init(smem_u32(&ctl.info_empty[x]), C::TILE_READERS);
         }
         for (int x = 0; x < 2; ++x) {
             mbar_init(smem_u32(&ctl.next_full[x]), 1);
@@ -281,7 +288,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         ctl.abort_flag = 0;
         ctl.asked = 0;
-        ctl.limit_ns = p.wait_limit_ns;
+        ctl.limit_ns = (uint32_t)(p.wait_limit_ns < 4000000000ull ? p.wait_limit_ns : 4000000000ull);
         fence_mbar_init();
     }
     if (warp == 1) {
@@ -300,22 +307,21 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
             prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
-            long long nload = 0;
+            uint32_t nload = 0;
             uint32_t ninfo = 0;             // tiles handed on
             int it = 0;                     // items processed (items without key tiles are skipped by every role)
-            bool ok = true;
+            int bad = 0;                    // where a wait gave up
             // ask for the item after number `ord`, when all of that one's loads are on their way
             auto ask_next = [&](uint32_t ord) {
                 const uint32_t slot = ord & 1, use = ord >> 1;
-                if (use > 0 && !ctl_wait(&ctl.next_empty[slot], (use - 1) & 1, &ctl)) { report_timeout(p, &ctl, 51, (int)ord); ok = false; return; }
+                if (use > 0 && !ctl_wait(&ctl.next_empty[slot], (use - 1) & 1, ctl, bad, 51)) return;
                 mbar_arrive_expect_tx(smem_u32(&ctl.next_full[slot]), 16);
                 clc_try_cancel(smem_u32(&ctl.next[slot]), smem_u32(&ctl.next_full[slot]));
                 ctl.asked = ord + 1;
             };
-            Item t;
-            for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, false, t, ok); ++ord) {
-                const int A = t.A, hq = t.hq, b = t.bb, h = t.h, hk = h / p.G;
-                const int item = t.A;
+            Item t = {};
+            for (uint32_t ord = 0; !bad && next_item<WALK>(p, ctl, ord, false, t, bad); ++ord) {
+                const int A = t.A, hq = t.hq, b = t.bb, h = t.h, hk = p.by_G.div(h);
                 TileWalk<WALK> walk;
                 walk.init(p, hq, A * NQ, NQ);
                 int cls_at = -1;
@@ -325,7 +331,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     const int kb = walk.next();
                     if constexpr (WALK != WALK_DENSE) {
                         const uint32_t slot = ninfo % C::NINFO, use = ninfo / C::NINFO;
-                        if (use > 0 && !ctl_wait(&ctl.info_empty[slot], (use - 1) & 1, &ctl)) { report_timeout(p, &ctl, 12, item); ok = false; return -1; }
+                        if (use > 0 && !ctl_wait(&ctl.info_empty[slot], (use - 1) & 1, ctl, bad, 12)) return -1;
                         ++ninfo;
                         const uint32_t bar = smem_u32(&ctl.info_full[slot]);
                         info[slot].kb = kb;
@@ -352,62 +358,54 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     return kb;
                 };
                 int kb = next_tile();
-                if (!ok) break;
+                if (bad) break;
                 if (kb < 0) { ask_next(ord); continue; }
-                if (it > 0 && !ctl_wait(&ctl.q_empty, (it - 1) & 1, &ctl)) { report_timeout(p, &ctl, 10, item); break; }
+                if (it > 0 && !ctl_wait(&ctl.q_empty, (it - 1) & 1, ctl, bad, 10)) break;
                 mbar_arrive_expect_tx(smem_u32(&ctl.q_full), NQ * C::TILE_BYTES);
                 // in the sorted layout the copies are indexed [head of the batch][sorted slot]
                 const int qh = WALK == WALK_SORTED ? hq : h, qb = WALK == WALK_SORTED ? 0 : b;
                 const int kh = WALK == WALK_SORTED ? b * p.Hkv + hk : hk;
-                for (int x = 0; x < NQ; ++x)
-                    for (int c = 0; c < C::SUBT; ++c)
-                        tma_load_4d(sq + x * C::TILE_BYTES + c * C::SUB_BYTES, &tm_q, smem_u32(&ctl.q_full), c * 64,
-                                    (A * NQ + x) * 128, qh, qb);
-                // one K or V tile into the next stage(s) of the ring
+#pragma unroll 1
+                for (int c = 0; c < NQ * C::SUBT; ++c)
+                    tma_load_4d(sq + c * C::SUB_BYTES, &tm_q, smem_u32(&ctl.q_full), (c % C::SUBT) * 64, (A * NQ + c / C::SUBT) * 128, qh, qb);
+                // one K or V tile into the next stage(s) of the ring: K tiles as all keys x D / PARTS dimensions, V tiles as
+                // 128 / PARTS keys x all dimensions, in boxes of 64 columns
                 auto load_tile = [&](bool is_v, int tile) {
-                    for (int part = 0; part < C::PARTS; ++part) {
-                        if (nload == p.stall_at) { ++nload; continue; }      // diagnostic: this stage is never filled
-                        const int slot = (int)(nload % C::NSTAGE);
-                        const long long use = nload / C::NSTAGE;
-                        if (use > 0 && !ctl_wait(&ctl.kv_empty[slot], (uint32_t)((use - 1) & 1), &ctl)) {
-                            report_timeout(p, &ctl, 11, item);
-                            ok = false;
-                            return;
-                        }
+                    const CUtensorMap* const tm = is_v ? &tm_v : &tm_k;
+                    const int boxes = is_v ? C::SUBT : C::SUBT / C::PARTS;
+                    const uint32_t box_bytes = is_v ? C::SUB_BYTES / C::PARTS : C::SUB_BYTES;
+#pragma unroll 1
+                    for (int part = 0; part < C::PARTS; ++part, ++nload) {
+                        if ((long long)nload == p.stall_at) continue;      // diagnostic: this stage is never filled
+                        const uint32_t slot = nload % C::NSTAGE, use = nload / C::NSTAGE;
+                        if (use > 0 && !ctl_wait(&ctl.kv_empty[slot], (use - 1) & 1, ctl, bad, 11)) return;
                         const uint32_t bar = smem_u32(&ctl.kv_full[slot]);
-                        const uint32_t dst = skv + slot * C::STAGE_BYTES;
+                        const int row = tile * 128 + (is_v ? part * (128 / C::PARTS) : 0), col = is_v ? 0 : part * boxes * 64;
                         mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
-                        if (is_v) {     // 128 / PARTS keys x all dimensions: one box of 64 columns x 128 / PARTS rows per sub-tile
-                            for (int c = 0; c < C::SUBT; ++c)
-                                tma_load_4d(dst + c * (C::SUB_BYTES / C::PARTS), &tm_v, bar, c * 64, tile * 128 + part * (128 / C::PARTS),
-                                            kh, qb);
-                        } else {        // all keys x D / PARTS dimensions
-                            for (int c = 0; c < C::SUBT / C::PARTS; ++c)
-                                tma_load_4d(dst + c * C::SUB_BYTES, &tm_k, bar, (part * (C::SUBT / C::PARTS) + c) * 64, tile * 128, kh, qb);
-                        }
-                        ++nload;
+#pragma unroll
+                        for (int c = 0; c < boxes; ++c)
+                            tma_load_4d(skv + slot * C::STAGE_BYTES + c * box_bytes, tm, bar, col + c * 64, row, kh, qb);
                     }
                 };
-                if constexpr (C::K_AHEAD) {
-                    // load order K(0), then per tile K(next), V(current): the K of the next tile is needed first (its
-                    // S is issued before the current P V) and so travels ahead of the V it shares the ring with
-                    load_tile(false, kb);
-                    while (ok && kb >= 0) {
-                        const int nxt = next_tile();
-                        if (nxt >= 0) load_tile(false, nxt);
-                        if (ok) load_tile(true, kb);
-                        kb = nxt;
+                // Step j: the K of tile j and the V of tile j - 1, in the order in which the MMA warp takes them: with two query tiles
+                // V(current) is consumed and released before K(next); with one the S of the next tile is issued before the current P V
+                int kb_v = -1;
+                for (;;) {
+#pragma unroll
+                    for (int second = 0; second < 2; ++second) {
+                        if (bad) break;
+                        const bool is_v = (NQ == 2) != (second != 0);
+                        const int tile = is_v ? kb_v : kb;
+                        if (tile >= 0) load_tile(is_v, tile);
                     }
-                } else {
-                    // two query tiles: V(current) is consumed and released before K(next), so it goes first
-                    for (; ok && kb >= 0; kb = next_tile()) {
-                        load_tile(false, kb);
-                        if (ok) load_tile(true, kb);
-                    }
+                    if (bad || kb < 0) break;
+                    kb_v = kb;
+                    kb = next_tile();
                 }
-                if (ok) ask_next(ord);
+                if (!bad) ask_next(ord);
                 ++it;
             }
+            if (bad) give_up(p, &ctl, bad, t.A);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -417,37 +415,39 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         {
             constexpr uint32_t IDESC_S = idesc_bf16(128, 128, 0, 0);
             constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
-            long long nuse = 0;             // K/V stages consumed so far
-            uint32_t np[2] = {0, 0};        // P tiles consumed per S/P buffer
+            uint32_t nuse = 0;              // K/V stages consumed so far
+            uint32_t np = 0;                // two query tiles: key tiles whose P has been consumed
             uint32_t ninfo = 0;             // tiles taken from the ring
-            uint32_t gs = 0, gp = 0;        // NQ == 1: S tiles issued / P tiles consumed (buffer = count & 1)
+            uint32_t gs = 0, gp = 0;        // one query tile: S tiles issued / P tiles consumed (buffer = count & 1)
+            uint32_t ngt[2] = {0, 0};       // soft gate: G tiles per query tile
+            uint32_t ngk = 0;               // ... key operands taken
             int it = 0;
-            bool ok = true;
-            const uint64_t qdesc0 = smem_desc_sw128(sq, 16, 1024);
-            const uint64_t kvdesc0 = smem_desc_sw128(skv, 16, 1024);             // K tiles: K-major
-            const uint64_t vdesc0 = smem_desc_sw128(skv, C::SUB_BYTES / C::PARTS, 1024);     // V tiles: MN-major, 64-column chunks
-            // S[buf] = Q_x K^T
-            auto issue_s = [&](int x, int buf, int kslot) {
-                if (elect_one()) {
-                    const uint32_t d = tmem + (buf ? C::COL_S1 : C::COL_S0);
-                    const uint64_t ad = qdesc0 + (uint64_t)((x * C::TILE_BYTES) >> 4);
+            int bad = 0;                    // where a wait gave up
+            // lower halves of the operand descriptors (the upper ones are the same throughout)
+            const uint32_t qdesc0 = (uint32_t)smem_desc_sw128(sq, 16, 1024);
+            const uint32_t kdesc0 = (uint32_t)smem_desc_sw128(skv, 16, 1024);             // K tiles: K-major
+            const uint32_t vdesc0 = (uint32_t)smem_desc_sw128(skv, C::SUB_BYTES / C::PARTS, 1024);     // V tiles: MN-major, 64-column chunks
+            // S_x (+)= `steps` 16-deep steps of Q_x K^T from the first on, K from `kd` on
+            auto s_steps = [&](uint32_t d, uint32_t qd, uint32_t kd, int steps, bool more) {
 #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) {
-                        const uint64_t off = (uint64_t)(((ks / 4) * C::SUB_BYTES + (ks % 4) * 32) >> 4);
-                        umma_ss(d, ad + off, kvdesc0 + (uint64_t)((kslot * C::STAGE_BYTES) >> 4) + off, IDESC_S, ks > 0);
-                    }
+                for (int ks = 0; ks < steps; ++ks) {
+                    const uint32_t off = (ks >> 2) * (C::SUB_BYTES >> 4) + (ks & 3) * 2;
+                    umma_ss_lo(d, qd + off, kd + off, IDESC_S, more || ks > 0);
                 }
             };
-            // two query tiles, soft gate: G_x = g_q g_k^T into the place of S_x, if the pair of tiles holds a distant pair; returns
-            // when the softmax warps have it in registers
-            uint32_t ngt[2] = {0, 0};       // G tiles per query tile
-            uint32_t ngk = 0;               // key operands taken
-            auto issue_gate = [&](int x, int a0, int kb, int item) -> bool {
+            // O (+)= 16-key steps of P V
+            auto o_steps = [&](uint32_t d, uint32_t a, uint32_t vd, int steps, bool more) {
+#pragma unroll
+                for (int ks = 0; ks < steps; ++ks) umma_ts_lo(d, a + ks * 8, vd + ks * 128, IDESC_O, more || ks > 0);
+            };
+            // soft gate: G_x = g_q g_k^T into the place of S_x, if the pair of tiles holds a distant pair; returns when the softmax
+            // warps have it in registers
+            auto issue_gate = [&](int x, int a0, int kb) -> bool {
                 if constexpr (C::GATE_MMA) {
                     const bool g0 = gate_tile(p, a0, kb), g1 = gate_tile(p, a0 + 1, kb);
                     if (!(x ? g1 : g0)) return true;       // (a gated tile 0 without a gated tile 1 gives the key operand back itself)
                     const uint32_t buf = ngk & 1;
-                    if (!ctl_wait(&gctl.gk_full[buf], (ngk >> 1) & 1, &ctl)) { report_timeout(p, &ctl, 53, item); return false; }
+                    if (!ctl_wait(&gctl.gk_full[buf], (ngk >> 1) & 1, ctl, bad, 53)) return false;
                     tc_fence_after();
                     if (elect_one()) {
                         using Steps = GateSteps<C::GATE_CH>;
@@ -461,87 +461,56 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     }
                     __syncwarp();
                     if (x == 1 || !g1) ++ngk;
-                    if (!ctl_wait(&gctl.g_taken[x], ngt[x] & 1, &ctl)) { report_timeout(p, &ctl, 54, item); return false; }
-                    ++ngt[x];
+                    const uint32_t par = (x ? ngt[1]++ : ngt[0]++) & 1;
+                    if (!ctl_wait(&gctl.g_taken[x], par, ctl, bad, 54)) return false;
                     tc_fence_after();
                 }
                 return true;
             };
-            // O_x (+)= P[buf] V
-            auto issue_o = [&](int x, int buf, int vslot, bool first) {
-                if (elect_one()) {
-                    const uint32_t d = tmem + (x ? C::COL_O1 : C::COL_O0);
-                    const uint32_t a = tmem + (buf ? C::COL_S1 : C::COL_S0);
-                    const uint64_t bd = vdesc0 + (uint64_t)((vslot * C::STAGE_BYTES) >> 4);
-                    // split rows: the P of column half h sits at columns 64 h .. 64 h + 31
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        umma_ts(d, a + (C::NSPLIT == 2 ? (ks / 4) * 64 + (ks % 4) * 8 : ks * 8), bd + (uint64_t)((ks * 2048) >> 4),
-                                IDESC_O, (!first) || ks > 0);
-                }
-            };
             auto commit = [&](uint64_t* bar) {
                 if (elect_one()) umma_commit(smem_u32(bar));
             };
-            // a ring stage goes back to the producer once the MMAs issued so far have completed
-            auto release_tile = [&](int slot) { commit(&ctl.kv_empty[slot]); };
             // wait for the next tile of the ring
-            auto wait_kv = [&](int& slot, int where, int item) -> bool {
+            auto wait_kv = [&](int& slot, int where) -> bool {
                 slot = (int)(nuse % C::NSTAGE);
-                if (!ctl_wait(&ctl.kv_full[slot], (uint32_t)((nuse / C::NSTAGE) & 1), &ctl)) {
-                    report_timeout(p, &ctl, where, item);
-                    return false;
-                }
+                if (!ctl_wait(&ctl.kv_full[slot], (nuse / C::NSTAGE) & 1, ctl, bad, where)) return false;
                 ++nuse;
                 return true;
             };
             // One query tile: S[buf] = Q K^T and O (+)= P[buf] V stage by stage -- wait for the stage, issue the MMAs that
             // read it, hand it back.  The stages are taken in the ring's order: K(next) before V(current).
-            auto s_tile = [&](int buf, int where, int item) -> bool {
+            auto s_tile = [&](int buf) -> bool {
                 constexpr int KS = D / 16 / C::PARTS;            // k-steps per stage
-                const uint32_t d = tmem + (buf ? C::COL_S1 : C::COL_S0);
+#pragma unroll
                 for (int part = 0; part < C::PARTS; ++part) {
                     int slot;
-                    if (!wait_kv(slot, where, item)) return false;
+                    if (!wait_kv(slot, 21)) return false;
                     tc_fence_after();
                     if (elect_one()) {
-#pragma unroll
-                        for (int k2 = 0; k2 < KS; ++k2) {
-                            const int ks = part * KS + k2;
-                            const uint64_t qoff = (uint64_t)(((ks / 4) * C::SUB_BYTES + (ks % 4) * 32) >> 4);
-                            const uint64_t koff = (uint64_t)((slot * C::STAGE_BYTES + (k2 / 4) * C::SUB_BYTES + (k2 % 4) * 32) >> 4);
-                            umma_ss(d, qdesc0 + qoff, kvdesc0 + koff, IDESC_S, ks > 0);
-                        }
+                        s_steps(tmem + (buf ? C::COL_S1 : C::COL_S0), qdesc0 + part * (KS / 4) * (C::SUB_BYTES >> 4), kdesc0 + slot * (C::STAGE_BYTES >> 4), KS, part > 0);
+                        umma_commit(smem_u32(&ctl.kv_empty[slot]));
+                        if (part == C::PARTS - 1) umma_commit(smem_u32(&ctl.s_full[buf]));
                     }
-                    release_tile(slot);
-                }
-                commit(&ctl.s_full[buf]);
-                return true;
-            };
-            auto o_tile = [&](int buf, bool first, int where, int item) -> bool {
-                constexpr int KS = 8 / C::PARTS;
-                const uint32_t d = tmem + C::COL_O0;
-                const uint32_t a = tmem + (buf ? C::COL_S1 : C::COL_S0);
-                for (int part = 0; part < C::PARTS; ++part) {
-                    int slot;
-                    if (!wait_kv(slot, where, item)) return false;
-                    tc_fence_after();
-                    if (elect_one()) {
-#pragma unroll
-                        for (int k2 = 0; k2 < KS; ++k2) {
-                            const int ks = part * KS + k2;
-                            umma_ts(d, a + (C::NSPLIT == 2 ? (ks / 4) * 64 + (ks % 4) * 8 : ks * 8),
-                                    vdesc0 + (uint64_t)((slot * C::STAGE_BYTES + k2 * 2048) >> 4), IDESC_O, (!first) || ks > 0);
-                        }
-                    }
-                    release_tile(slot);
                 }
                 return true;
             };
-            Item t;
-            for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, true, t, ok); ++ord) {
+            auto o_tile = [&](int buf, bool first) -> bool {
+#pragma unroll
+                for (int part = 0; part < C::PARTS; ++part) {
+                    int slot;
+                    if (!wait_kv(slot, 22)) return false;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        // split rows: the P of column half h sits at columns 64 h .. 64 h + 31
+                        o_steps(tmem + C::COL_O0, tmem + (buf ? C::COL_S1 : C::COL_S0) + part * 64, vdesc0 + slot * (C::STAGE_BYTES >> 4), 8 / C::PARTS, !first || part > 0);
+                        umma_commit(smem_u32(&ctl.kv_empty[slot]));
+                    }
+                }
+                return true;
+            };
+            Item t = {};
+            for (uint32_t ord = 0; !bad && next_item<WALK>(p, ctl, ord, true, t, bad); ++ord) {
                 const int A = t.A, hq = t.hq;
-                const int item = t.A;
                 TileWalk<WALK> walk;
                 if constexpr (WALK == WALK_DENSE) walk.init(p, hq, A * NQ, NQ);
                 auto next_tile = [&]() -> int {
@@ -549,7 +518,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         return walk.next();
                     } else {
                         const uint32_t slot = ninfo % C::NINFO;
-                        if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, &ctl)) { report_timeout(p, &ctl, 27, item); ok = false; return -1; }
+                        if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, ctl, bad, 27)) return -1;
                         const int kb = info[slot].kb;
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctl.info_empty[slot]));
@@ -557,86 +526,75 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         return kb;
                     }
                 };
-                int cur = next_tile();
-                if (!ok) break;
-                if (cur < 0) continue;
-                if (!ctl_wait(&ctl.q_full, it & 1, &ctl)) { report_timeout(p, &ctl, 20, item); break; }
-                if constexpr (C::GATE_MMA) {
-                    if (!ctl_wait(&gctl.gq_full, it & 1, &ctl)) { report_timeout(p, &ctl, 29, item); break; }
-                }
-                if constexpr (NQ == 2) {
-                    int slot;
-                    if (!wait_kv(slot, 21, item)) break;
-                    tc_fence_after();
-                    if (!issue_gate(0, A * NQ, cur, item)) break;
-                    issue_s(0, 0, slot); commit(&ctl.s_full[0]);
-                    if (!issue_gate(1, A * NQ, cur, item)) break;
-                    issue_s(1, 1, slot); commit(&ctl.s_full[1]);
-                    release_tile(slot);
-                } else {
-                    if (!s_tile(gs & 1, 21, item)) break;
-                    ++gs;
-                }
-                bool first = true;
-                while (cur >= 0) {
-                    const int nxt = next_tile();
-                    if (!ok) break;
-                    int vslot = 0, kslot = 0;
-                    if constexpr (NQ == 2) {
-                        // the ring carries V(current) ahead of K(next) here (see the producer)
-                        if (!wait_kv(vslot, 22, item)) { ok = false; break; }
-                        if (nxt >= 0) {
-                            if (!wait_kv(kslot, 23, item)) { ok = false; break; }
+                // Steps of the item: step j issues the P V of tile j - 1 and the S of tile j, so the first has no P V and the last no S.
+                // Two query tiles: P V_0, S_0, P V_1, S_1, so that one tile's softmax runs during the other's MMAs.  One query tile: S of
+                // the next tile goes to the other buffer before the P V.
+                bool have_p = false, first = true;
+                for (;;) {
+                    const int kb = next_tile();
+                    if (bad) break;
+                    if (kb < 0 && !have_p) break;          // an item without key tiles
+                    if (!have_p) {
+                        if (!ctl_wait(&ctl.q_full, it & 1, ctl, bad, 20)) break;
+                        if constexpr (C::GATE_MMA) {
+                            if (!ctl_wait(&gctl.gq_full, it & 1, ctl, bad, 29)) break;
                         }
                     }
-                    if (nxt < 0) {                         // every S (and G) of this item has been issued
-                        commit(&ctl.q_empty);
-                        if constexpr (C::GATE_MMA) commit(&gctl.gq_empty);
-                    }
                     if constexpr (NQ == 2) {
-                        // query tile 0
-                        if (!ctl_wait(&ctl.p_full[0], np[0] & 1, &ctl)) { report_timeout(p, &ctl, 24, item); ok = false; break; }
-                        ++np[0];
-                        tc_fence_after();
-                        issue_o(0, 0, vslot, first);
-                        if (nxt >= 0) {
-                            if (!issue_gate(0, A * NQ, nxt, item)) { ok = false; break; }
-                            issue_s(0, 0, kslot); commit(&ctl.s_full[0]);
-                        } else {
-                            commit(&ctl.o_full[0]);
+                        // the ring carries V(current) ahead of K(next) (see the producer)
+                        int vslot = 0, kslot = 0;
+                        if (have_p && !wait_kv(vslot, 22)) break;
+                        if (kb >= 0) {
+                            if (!wait_kv(kslot, 23)) break;
+                        } else {                           // every S (and G) of this item has been issued
+                            commit(&ctl.q_empty);
+                            if constexpr (C::GATE_MMA) commit(&gctl.gq_empty);
                         }
-                        // query tile 1
-                        if (!ctl_wait(&ctl.p_full[1], np[1] & 1, &ctl)) { report_timeout(p, &ctl, 25, item); ok = false; break; }
-                        ++np[1];
-                        tc_fence_after();
-                        issue_o(1, 1, vslot, first);
-                        release_tile(vslot);
-                        if (nxt >= 0) {
-                            if (!issue_gate(1, A * NQ, nxt, item)) { ok = false; break; }
-                            issue_s(1, 1, kslot); commit(&ctl.s_full[1]);
-                            release_tile(kslot);
-                        } else {
-                            commit(&ctl.o_full[1]);
+#pragma unroll
+                        for (int x = 0; x < 2; ++x) {
+                            if (have_p && !ctl_wait(&ctl.p_full[x], np & 1, ctl, bad, 24 + x)) break;
+                            tc_fence_after();
+                            const uint32_t t_s = tmem + (x ? C::COL_S1 : C::COL_S0);
+                            if (have_p && elect_one()) {
+                                o_steps(tmem + (x ? C::COL_O1 : C::COL_O0), t_s, vdesc0 + vslot * (C::STAGE_BYTES >> 4), 8, !first);
+                                if (x == 1) umma_commit(smem_u32(&ctl.kv_empty[vslot]));
+                                if (kb < 0) umma_commit(smem_u32(&ctl.o_full[x]));
+                            }
+                            __syncwarp();
+                            if (kb < 0) continue;
+                            if (!issue_gate(x, A * NQ, kb)) break;
+                            if (elect_one()) {
+                                s_steps(t_s, qdesc0 + x * (C::TILE_BYTES >> 4), kdesc0 + kslot * (C::STAGE_BYTES >> 4), D / 16, false);
+                                umma_commit(smem_u32(&ctl.s_full[x]));
+                                if (x == 1) umma_commit(smem_u32(&ctl.kv_empty[kslot]));
+                            }
+                            __syncwarp();
                         }
+                        if (bad) break;
+                        if (have_p) { ++np; first = false; }
                     } else {
-                        // S of the next tile goes to the other buffer before this tile's PV is issued
-                        if (nxt >= 0) {
-                            if (!s_tile(gs & 1, 23, item)) { ok = false; break; }
+                        if (kb >= 0) {
+                            if (!s_tile(gs & 1)) break;
                             ++gs;
+                        } else {
+                            commit(&ctl.q_empty);
                         }
-                        const int buf = gp & 1;
-                        if (!ctl_wait(&ctl.p_full[buf], (gp >> 1) & 1, &ctl)) { report_timeout(p, &ctl, 26, item); ok = false; break; }
-                        ++gp;
-                        tc_fence_after();
-                        if (!o_tile(buf, first, 22, item)) { ok = false; break; }
-                        commit(&ctl.pv_done);
-                        if (nxt < 0) commit(&ctl.o_full[0]);
+                        if (have_p) {
+                            const int buf = gp & 1;
+                            if (!ctl_wait(&ctl.p_full[buf], (gp >> 1) & 1, ctl, bad, 26)) break;
+                            ++gp;
+                            tc_fence_after();
+                            if (!o_tile(buf, first)) break;
+                            commit(&ctl.pv_done);
+                            if (kb < 0) commit(&ctl.o_full[0]);
+                            first = false;
+                        }
                     }
-                    first = false;
-                    cur = nxt;
+                    if (kb < 0) { ++it; break; }
+                    have_p = true;
                 }
-                ++it;
             }
+            if (bad && lane == 0) give_up(p, &ctl, bad, t.A);
         }
         __syncwarp();
     } else if (C::GATE_MMA && warp < 4) {
@@ -646,16 +604,16 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         unsigned char* const gk = gq + 2 * C::GQ_BYTES;
         uint32_t ngk = 0;
         int it = 0;
-        bool ok = true;
-        Item t;
-        for (uint32_t ord = 0; ok && next_item<WALK>(p, &ctl, ord, true, t, ok); ++ord) {
-            const int a0 = t.A * NQ, item = t.A;
+        int bad = 0;                        // where a wait gave up
+        Item t = {};
+        for (uint32_t ord = 0; !bad && next_item<WALK>(p, ctl, ord, true, t, bad); ++ord) {
+            const int a0 = t.A * NQ;
             TileWalk<WALK_DENSE> walk;
             walk.init(p, t.hq, a0, NQ);
             int kb = walk.next();
             if (kb < 0) continue;
             const float* gseq = p.gate_g + (size_t)t.bb * p.n * p.gate_ld;
-            if (it > 0 && !ctl_wait(&gctl.gq_empty, (it - 1) & 1, &ctl)) { report_timeout(p, &ctl, 55, item); break; }
+            if (it > 0 && !ctl_wait(&gctl.gq_empty, (it - 1) & 1, ctl, bad, 55)) break;
 #pragma unroll 1
             for (int r = t64; r < 256; r += 64) {
                 const int i = a0 * 128 + r;
@@ -667,7 +625,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             for (; kb >= 0; kb = walk.next()) {
                 if (!gate_tile(p, a0, kb) && !gate_tile(p, a0 + 1, kb)) continue;
                 const uint32_t buf = ngk & 1, use = ngk >> 1;
-                if (use > 0 && !ctl_wait(&gctl.gk_empty[buf], (use - 1) & 1, &ctl)) { report_timeout(p, &ctl, 56, item); ok = false; break; }
+                if (use > 0 && !ctl_wait(&gctl.gk_empty[buf], (use - 1) & 1, ctl, bad, 56)) break;
                 ++ngk;
 #pragma unroll 1
                 for (int r = t64; r < 128; r += 64) {
@@ -680,6 +638,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
             ++it;
         }
+        if (bad && lane == 0) give_up(p, &ctl, bad, t.A);
         __syncwarp();
     } else if (warp >= 4) {
         // ------------------------------------------------------------------ softmax + epilogue
@@ -699,28 +658,122 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         uint32_t ninfo = 0;                                  // tiles taken from the ring
         uint32_t ng = 0;                                     // soft gate: tiles whose key assignments this warpgroup has staged
         int it = 0;
-        bool ok = true;
-        // An item's row position and mask are loaded while the item before it ends, so that its first tile need not wait for
-        // them (three dependent reads of L2 in the sorted order): its order entry before the wait for the last P V, the mask
-        // word before the output is written.
+        int bad = 0;                                         // where a wait gave up
+        // Each turn finds the next item, writes the one before out and then goes through the tiles.  An item's row position and mask
+        // are loaded while the item before it ends, so that its first tile need not wait for them (three dependent reads of L2 in
+        // the sorted order): its order entry before the wait for the last P V, the mask word before the output is written.
         Item t = {};
-        int i_row = -1;
-        uint32_t m_row = 0;
-        auto load_row = [&]() {
-            const int r = (t.A * NQ + x) * 128 + row_in_tile;
-            i_row = r;
-            // the row's position in the sequence: its index, or in the sorted layout the position its slot holds (-1: padding)
-            if constexpr (WALK == WALK_SORTED) i_row = dep_load(p.perm_q + (size_t)t.hq * p.nqp + r);
-        };
-        auto load_mask = [&]() {
-            if constexpr (WALK != WALK_DENSE) m_row = (i_row >= 0 && i_row < p.n) ? dep_load(p.mq + (size_t)t.hq * p.n + i_row) : 0u;
-        };
-        bool have = next_item<WALK>(p, &ctl, 0, true, t, ok);
-        if (have) { load_row(); load_mask(); }
-        for (uint32_t ord = 0; ok && have; ++ord) {
-            const int A = t.A, hq = t.hq, bb = t.bb, h = t.h;
-            const int item = t.A;
-            const int hk = bb * p.Hkv + h / p.G;
+        int i = -1;                                          // the row's position in the sequence
+        bool valid = false;
+        float m_used = -INFINITY, l = 0.f;
+        bool finish = false;                                 // an item whose tiles are through
+        for (uint32_t ord = 0;; ++ord) {
+            Item t_next = {};
+            const bool have = next_item<WALK>(p, ctl, ord, true, t_next, bad);
+            if (bad) break;
+            int i_next = -1;
+            uint32_t mi = 0;
+            if (have) {
+                // its index, or in the sorted layout the position its slot holds (-1: padding)
+                i_next = (t_next.A * NQ + x) * 128 + row_in_tile;
+                if constexpr (WALK == WALK_SORTED) i_next = dep_load(p.perm_q + (size_t)t_next.hq * p.nqp + i_next);
+            }
+            auto load_mask = [&]() {
+                if constexpr (WALK != WALK_DENSE) mi = (i_next >= 0 && i_next < p.n) ? dep_load(p.mq + (size_t)t_next.hq * p.n + i_next) : 0u;
+            };
+            if (finish) {
+                // ---- epilogue: O / l -> bf16 -> global, lse.  With a partial result to join (window pass of the split layout) the
+                // row's logsumexp there is read now, before a thread that shares the row can write the joint one.
+                const size_t row = (size_t)t.hq * p.n + (size_t)i;
+                float lse_other = -INFINITY;
+                if (WALK == WALK_TOKEN && p.join && valid) lse_other = p.lse[row];
+                if constexpr (NSPLIT == 2) {
+                    // the two halves add their row sums: two exchanges, the leading bf16 part of the sum and its remainder
+                    float other = 0.f, rest = l;
+                    bool xok = true;
+                    for (int piece = 0; piece < 2 && xok; ++piece) {
+                        const int par = (int)(nx & 1);
+                        const __nv_bfloat16 mine = __float2bfloat16_rn(rest);
+                        rest -= __bfloat162float(mine);
+                        xval(par, half, row_in_tile) = mine;
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctl.xchg[warp & 3]));
+                        xok = ctl_wait(&ctl.xchg[warp & 3], (uint32_t)par, ctl, bad, 38);
+                        other += __bfloat162float(xval(par, half ^ 1, row_in_tile));
+                        ++nx;
+                    }
+                    if (!xok) break;
+                    l += other;
+                }
+                if (!ctl_wait(&ctl.o_full[x], it & 1, ctl, bad, 40 + x)) break;
+                tc_fence_after();
+                load_mask();
+                const float inv_l = l > 0.f ? 1.f / l : 0.f;        // a row without any pair (possible in a partial pass): zeros, lse = -inf
+                float own = inv_l, w_other = 0.f, lse_row = (m_used + lg2_approx(l)) * LN2;
+                if (WALK == WALK_TOKEN && p.join) {
+                    // the two partial results cover disjoint sets of pairs and join through their logsumexps (Appendix D)
+                    const float m = fmaxf(lse_other, lse_row);
+                    const float wo = m == -INFINITY ? 0.f : __expf(lse_other - m), wl = m == -INFINITY ? 0.f : __expf(lse_row - m);
+                    const float tot = wo + wl, inv = tot > 0.f ? 1.f / tot : 0.f;
+                    own = inv_l * wl * inv;
+                    w_other = wo * inv;
+                    lse_row = tot > 0.f ? m + __logf(tot) : -INFINITY;
+                }
+                __nv_bfloat16* orow = p.o + (size_t)t.bb * p.o_sb + (size_t)t.h * p.o_sh + (size_t)(valid ? i : 0) * p.o_sn +
+                                      half * (D / 2);
+#pragma unroll 1
+                for (int c = 0; c < D / 16 / NSPLIT; ++c) {
+                    uint32_t ov[16];
+                    tmem_ld16(t_o + c * 16, ov);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * own);
+                    const size_t at = row * D + half * (D / 2) + c * 16;
+                    if constexpr (WALK == WALK_TOKEN) {
+                        if (w_other > 0.f) {               // (a partial result without any pair has unspecified contents)
+#pragma unroll
+                            for (int e = 0; e < 16; e += 4) {
+                                const float4 v4 = *reinterpret_cast<const float4*>(p.join + at + e);
+                                ov[e] = __float_as_uint(fmaf(v4.x, w_other, __uint_as_float(ov[e])));
+                                ov[e + 1] = __float_as_uint(fmaf(v4.y, w_other, __uint_as_float(ov[e + 1])));
+                                ov[e + 2] = __float_as_uint(fmaf(v4.z, w_other, __uint_as_float(ov[e + 2])));
+                                ov[e + 3] = __float_as_uint(fmaf(v4.w, w_other, __uint_as_float(ov[e + 3])));
+                            }
+                        }
+                    }
+                    if (!valid) continue;
+                    if (WALK == WALK_SORTED && p.o32) {
+#pragma unroll
+                        for (int e = 0; e < 16; e += 8) {
+                            uint32_t w[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) w[j] = ov[e + j];
+                            st_global_v8(p.o32 + at + e, w);
+                        }
+                    } else {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) w[j] = pack_bf16x2(__uint_as_float(ov[2 * j]), __uint_as_float(ov[2 * j + 1]));
+                        if (p.o_wide) {
+                            st_global_v8(orow + c * 16, w);
+                        } else {
+                            *reinterpret_cast<uint4*>(orow + c * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+                            *reinterpret_cast<uint4*>(orow + c * 16 + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+                        }
+                    }
+                }
+                if (valid && half == 0) p.lse[row] = lse_row;
+                tc_fence_before();
+                ++it;
+            } else {
+                load_mask();
+            }
+            if (!have) break;
+            t = t_next;
+            i = i_next;
+            valid = i >= 0 && i < p.n;
+            const int A = t.A, hq = t.hq, bb = t.bb;
+            const int hk = bb * p.Hkv + p.by_G.div(t.h);
             const int a = A * NQ + x;
             TileWalk<WALK> walk;
             if constexpr (WALK == WALK_DENSE) walk.init(p, hq, A * NQ, NQ);
@@ -730,7 +783,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     return walk.next();
                 } else {
                     const uint32_t slot = ninfo % C::NINFO;
-                    if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, &ctl)) { report_timeout(p, &ctl, 39, item); ok = false; return -1; }
+                    if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, ctl, bad, 39)) return -1;
                     tile = info + slot;
                     return tile->kb;
                 }
@@ -742,26 +795,16 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     ++ninfo;
                 }
             };
-            int kb = next_tile();
-            if (!ok) break;
-            if (kb < 0) {
-                tile_read();
-                have = next_item<WALK>(p, &ctl, ord + 1, true, t, ok);
-                if (have) { load_row(); load_mask(); }
-                continue;
-            }
-            const int i = i_row;
             int wmin = 0, wmax = 0;
             if constexpr (WALK == WALK_SORTED) {
                 wmin = __reduce_min_sync(0xffffffffu, i < 0 ? 0x7fffffff : i);
                 wmax = __reduce_max_sync(0xffffffffu, i);
             }
-            const bool valid = i >= 0 && i < p.n;
-            uint32_t mi = m_row;
             if (WALK == WALK_TOKEN) mi &= 0xffffffffu >> (32 - p.K);
             const int dfar = a * 128 - p.w;
             const int f_x = (WALK == WALK_TOKEN && dfar > 0) ? dfar >> 7 : 0;   // tiles b < f_x are far for this query tile
-            float m_used = -INFINITY, l = 0.f;
+            m_used = -INFINITY;
+            l = 0.f;
             bool first = true;
             // soft gate: this row's assignment times lambda / 2 (sigmoid(x) = 1/2 + 1/2 tanh(x / 2))
             constexpr bool GATE_ALU = GATE != 0 && !C::GATE_MMA;  // one query tile: the inner products are taken here
@@ -782,15 +825,18 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     }
                 }
             }
-            for (; kb >= 0; kb = next_tile()) {
+#pragma unroll 1
+            for (;;) {
+                const int kb = next_tile();
+                if (kb < 0) break;
                 TileMask tm;
                 if constexpr (WALK == WALK_SORTED) {
                     const bool share = (mi & tile->cls) != 0u;
                     build_tile_mask_sorted(tm, p.w, reinterpret_cast<const int32_t*>(tile->data), share, valid ? i : -1, wmin, wmax, !p.share_only);
-                    if (p.gbits_s && !tm.all_masked)
+                    if (p.gbits_s)
                         exclude_lower_groups(tm, p.gbits_s + ((size_t)hk * (p.nkp / 128) + kb) * p.K * 4, mi & ((1u << tile->pad[0]) - 1u), p.K);
                 } else if constexpr (WALK == WALK_DENSE) {
-                    build_tile_mask_dense(tm, p, a, kb, i);
+                    build_tile_mask_dense(tm, a, kb, i);
                 } else {
                     build_tile_mask(tm, p, a, kb, i, mi, f_x, tile->data);
                 }
@@ -805,7 +851,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 const bool tile_gated = C::GATE_MMA && gate_tile(p, a, kb);
                 if constexpr (GATE_ALU) {
                     // the same decision in all four warps of the warpgroup: does the tile hold a distant pair at all
-                    const bool tile_gated = !tm.all_masked && (a * 128 + 127 - p.w > gj0);
+                    const bool tile_gated = a * 128 + 127 - p.w > gj0;
                     if (tile_gated) {
                         unsigned char* gw = gate_sm + (wg * 2 + (ng & 1)) * C::GATE_BUF_BYTES;
                         const int col = (warp & 3) * 32 + lane;
@@ -818,7 +864,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctl.gbar[wg]));
-                        if (!ctl_wait(&ctl.gbar[wg], ng & 1, &ctl)) { report_timeout(p, &ctl, 37, item); ok = false; break; }
+                        if (!ctl_wait(&ctl.gbar[wg], ng & 1, ctl, bad, 37)) break;
                         ++ng;
                         gb = gw;
                         gated = __any_sync(0xffffffffu, valid && ifar > gj0);
@@ -828,7 +874,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 uint32_t sr[NC];
                 if constexpr (C::GATE_MMA) {
                     if (tile_gated) {
-                        if (!ctl_wait(&gctl.g_full[x], ng & 1, &ctl)) { report_timeout(p, &ctl, 37, item); ok = false; break; }
+                        if (!ctl_wait(&gctl.g_full[x], ng & 1, ctl, bad, 37)) break;
                         ++ng;
                         tc_fence_after();
                         const uint32_t t_g = tmem + lane_base + (x ? C::COL_S1 : C::COL_S0);
@@ -850,278 +896,183 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 // ---- wait for S
                 const int buf = NQ == 2 ? x : (int)(ns & 1);
                 const uint32_t par = NQ == 2 ? (ns & 1) : ((ns >> 1) & 1);
-                if (!ctl_wait(&ctl.s_full[buf], par, &ctl)) { report_timeout(p, &ctl, 30 + x, item); ok = false; break; }
+                if (!ctl_wait(&ctl.s_full[buf], par, ctl, bad, 30 + x)) break;
                 // this thread's NC S columns; its packed P columns overwrite the first half of them
                 const uint32_t t_s = tmem + lane_base + (buf ? C::COL_S1 : C::COL_S0) + half * NC;
                 tc_fence_after();
                 uint32_t pk[NC / 2];
-                if (tm.all_masked) {
+                if (tile_gated) {                    // the factors are in place of the scores
 #pragma unroll
-                    for (int c = 0; c < NC / 2; ++c) pk[c] = 0u;
-                } else {
-                    if (tile_gated) {                    // the factors are in place of the scores
+                    for (int c = 0; c < NC / 16; ++c) {      // 16 at a time beside the 128 factors: 32 took 944 us for 8192 tokens, 16 862
+                        uint32_t sv[16];
+                        tmem_ld16(t_s + c * 16, sv);
+                        tmem_wait_ld();
 #pragma unroll
-                        for (int c = 0; c < NC / 16; ++c) {      // 16 at a time beside the 128 factors: 32 took 944 us for 8192 tokens, 16 862 (D = 128 spills 236 bytes all the same)
-                            uint32_t sv[16];
-                            tmem_ld16(t_s + c * 16, sv);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int e = 0; e < 16; e += 2) {
-                                const float2 f = __fmul2_rn(make_float2(__uint_as_float(sr[c * 16 + e]), __uint_as_float(sr[c * 16 + e + 1])),
-                                                            make_float2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])));
-                                sr[c * 16 + e] = __float_as_uint(f.x);
-                                sr[c * 16 + e + 1] = __float_as_uint(f.y);
-                            }
+                        for (int e = 0; e < 16; e += 2) {
+                            const float2 f = __fmul2_rn(make_float2(__uint_as_float(sr[c * 16 + e]), __uint_as_float(sr[c * 16 + e + 1])),
+                                                        make_float2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])));
+                            sr[c * 16 + e] = __float_as_uint(f.x);
+                            sr[c * 16 + e + 1] = __float_as_uint(f.y);
                         }
-                    } else
+                    }
+                } else
 #pragma unroll
-                    for (int c = 0; c < NC / 32; ++c) {
-                        tmem_ld32(t_s + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
-                        if constexpr (GATE_ALU) {        // chunk by chunk: 32 scores, then their factors
-                            tmem_wait_ld();
-                            if (gated) {
-                                const bool wide = p.gate_ld == 8;
-                                const int nfar = ifar - gj0 < 0 ? 0 : (ifar - gj0 > NC ? NC : ifar - gj0);   // columns < nfar are distant
+                for (int c = 0; c < NC / 32; ++c) {
+                    tmem_ld32(t_s + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[c * 32]));
+                    if constexpr (GATE_ALU) {        // chunk by chunk: 32 scores, then their factors
+                        tmem_wait_ld();
+                        if (gated) {
+                            const bool wide = p.gate_ld == 8;
+                            const int nfar = ifar - gj0 < 0 ? 0 : (ifar - gj0 > NC ? NC : ifar - gj0);   // columns < nfar are distant
 #pragma unroll
-                                for (int e0 = 0; e0 < 32; e0 += 4) {        // four columns in flight
-                                    float arg[4];
-                                    if constexpr (GATE == 1) {
-                                        float4 k0[4], k1[4];
+                            for (int e0 = 0; e0 < 32; e0 += 4) {        // four columns in flight
+                                float arg[4];
+                                if constexpr (GATE == 1) {
+                                    float4 k0[4], k1[4];
 #pragma unroll
-                                        for (int u = 0; u < 4; ++u) {
-                                            const float4* kp = reinterpret_cast<const float4*>(gb + (c * 32 + e0 + u) * 32);
-                                            k0[u] = kp[0];
-                                            k1[u] = wide ? kp[1] : make_float4(0.f, 0.f, 0.f, 0.f);
-                                        }
-#pragma unroll
-                                        for (int u = 0; u < 4; ++u) {
-                                            float2 acc = __fmul2_rn(make_float2(gi[0], gi[1]), make_float2(k0[u].x, k0[u].y));
-                                            acc = __ffma2_rn(make_float2(gi[2], gi[3]), make_float2(k0[u].z, k0[u].w), acc);
-                                            if (wide) {
-                                                float2 acb = __fmul2_rn(make_float2(gi[4], gi[5]), make_float2(k1[u].x, k1[u].y));
-                                                acb = __ffma2_rn(make_float2(gi[6], gi[7]), make_float2(k1[u].z, k1[u].w), acb);
-                                                acc = __fadd2_rn(acc, acb);
-                                            }
-                                            arg[u] = acc.x + acc.y;
-                                        }
-                                    } else {
-                                        // longer assignments: piece by piece, two sums per column
-                                        float2 acc[4], acb[4];
-#pragma unroll
-                                        for (int u = 0; u < 4; ++u) acc[u] = acb[u] = make_float2(0.f, 0.f);
-#pragma unroll
-                                        for (int f = 0; f < GQ; ++f) {
-                                            float4 kf[4];
-#pragma unroll
-                                            for (int u = 0; u < 4; ++u)
-                                                kf[u] = reinterpret_cast<const float4*>(gb + (c * 32 + e0 + u) * C::GATE_ROW_BYTES)[f];
-#pragma unroll
-                                            for (int u = 0; u < 4; ++u) {
-                                                acc[u] = __ffma2_rn(make_float2(gi[4 * f], gi[4 * f + 1]), make_float2(kf[u].x, kf[u].y), acc[u]);
-                                                acb[u] = __ffma2_rn(make_float2(gi[4 * f + 2], gi[4 * f + 3]), make_float2(kf[u].z, kf[u].w), acb[u]);
-                                            }
-                                        }
-#pragma unroll
-                                        for (int u = 0; u < 4; ++u) arg[u] = (acc[u].x + acc[u].y) + (acb[u].x + acb[u].y);
+                                    for (int u = 0; u < 4; ++u) {
+                                        const float4* kp = reinterpret_cast<const float4*>(gb + (c * 32 + e0 + u) * 32);
+                                        k0[u] = kp[0];
+                                        k1[u] = wide ? kp[1] : make_float4(0.f, 0.f, 0.f, 0.f);
                                     }
 #pragma unroll
                                     for (int u = 0; u < 4; ++u) {
-                                        const float gate = fmaf(tanh_approx(arg[u]), 0.5f, 0.5f);
-                                        const float sv = __uint_as_float(sr[c * 32 + e0 + u]);
-                                        sr[c * 32 + e0 + u] = __float_as_uint(c * 32 + e0 + u < nfar ? sv * gate : sv);
+                                        float2 acc = __fmul2_rn(make_float2(gi[0], gi[1]), make_float2(k0[u].x, k0[u].y));
+                                        acc = __ffma2_rn(make_float2(gi[2], gi[3]), make_float2(k0[u].z, k0[u].w), acc);
+                                        if (wide) {
+                                            float2 acb = __fmul2_rn(make_float2(gi[4], gi[5]), make_float2(k1[u].x, k1[u].y));
+                                            acb = __ffma2_rn(make_float2(gi[6], gi[7]), make_float2(k1[u].z, k1[u].w), acb);
+                                            acc = __fadd2_rn(acc, acb);
+                                        }
+                                        arg[u] = acc.x + acc.y;
                                     }
+                                } else {
+                                    // longer assignments: piece by piece, two sums per column
+                                    float2 acc[4], acb[4];
+#pragma unroll
+                                    for (int u = 0; u < 4; ++u) acc[u] = acb[u] = make_float2(0.f, 0.f);
+#pragma unroll
+                                    for (int f = 0; f < GQ; ++f) {
+                                        float4 kf[4];
+#pragma unroll
+                                        for (int u = 0; u < 4; ++u)
+                                            kf[u] = reinterpret_cast<const float4*>(gb + (c * 32 + e0 + u) * C::GATE_ROW_BYTES)[f];
+#pragma unroll
+                                        for (int u = 0; u < 4; ++u) {
+                                            acc[u] = __ffma2_rn(make_float2(gi[4 * f], gi[4 * f + 1]), make_float2(kf[u].x, kf[u].y), acc[u]);
+                                            acb[u] = __ffma2_rn(make_float2(gi[4 * f + 2], gi[4 * f + 3]), make_float2(kf[u].z, kf[u].w), acb[u]);
+                                        }
+                                    }
+#pragma unroll
+                                    for (int u = 0; u < 4; ++u) arg[u] = (acc[u].x + acc[u].y) + (acb[u].x + acb[u].y);
+                                }
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    const float gate = fmaf(tanh_approx(arg[u]), 0.5f, 0.5f);
+                                    const float sv = __uint_as_float(sr[c * 32 + e0 + u]);
+                                    sr[c * 32 + e0 + u] = __float_as_uint(c * 32 + e0 + u < nfar ? sv * gate : sv);
                                 }
                             }
                         }
                     }
-                    tmem_wait_ld();
-                    if (SOFTCAP) {
-#pragma unroll
-                        for (int c = 0; c < NC; ++c) sr[c] = __float_as_uint(tanh_approx(__uint_as_float(sr[c]) * cap_in));
-                    }
-                    if (tm.masked) {
-#pragma unroll
-                        for (int c = 0; c < NC; ++c)
-                            sr[c] = ((tm.kw[(NSPLIT == 2 ? half * 2 : 0) + (c >> 5)] >> (c & 31)) & 1u) ? sr[c] : 0xff800000u;      // -inf
-                    }
-                    // ---- row maximum of the tile: four independent chains of three-input maxima
-                    float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
-#pragma unroll
-                    for (int c = 0; c < NC; c += 8) {
-                        mx0 = max3(mx0, __uint_as_float(sr[c]), __uint_as_float(sr[c + 1]));
-                        mx1 = max3(mx1, __uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3]));
-                        mx2 = max3(mx2, __uint_as_float(sr[c + 4]), __uint_as_float(sr[c + 5]));
-                        mx3 = max3(mx3, __uint_as_float(sr[c + 6]), __uint_as_float(sr[c + 7]));
-                    }
-                    float mraw = max3(mx0, mx1, fmaxf(mx2, mx3));
-                    if constexpr (NSPLIT == 2) {
-                        // the two threads of a row exchange the maxima of their halves and then take the same decisions
-                        const int par = (int)(nx & 1);
-                        const __nv_bfloat16 mine = __float2bfloat16_rn(mraw);
-                        xval(par, half, row_in_tile) = mine;
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&ctl.xchg[warp & 3]));
-                        if (!ctl_wait(&ctl.xchg[warp & 3], (uint32_t)par, &ctl)) { report_timeout(p, &ctl, 36, item); ok = false; }
-                        mraw = fmaxf(__bfloat162float(mine), __bfloat162float(xval(par, half ^ 1, row_in_tile)));
-                        ++nx;
-                    }
-                    const float mt = mraw * sl2;                     // log2 units (sl2 > 0; -inf stays -inf)
-                    // ---- lazy maximum: raise the reference only when it lags by more than the threshold
-                    float factor = 1.f;
-                    bool raise = false;
-                    if (m_used == -INFINITY) {
-                        m_used = mt;                                 // nothing accumulated yet for this row
-                    } else if (mt > m_used + RESCALE_THRESHOLD) {
-                        factor = ex2_approx(m_used - mt);
-                        m_used = mt;
-                        raise = true;
-                    }
-                    if (__any_sync(0xffffffffu, raise) && !first) {
-                        // O may only be touched once the previous PV of this query tile has completed.  With two
-                        // query tiles its commit precedes s_full; with double-buffered S it has its own barrier.
-                        bool pv_ok = true;
-                        if constexpr (NQ == 1) pv_ok = ctl_wait(&ctl.pv_done, (ns - 1) & 1, &ctl);
-                        if (!pv_ok) { report_timeout(p, &ctl, 35, item); ok = false; }
-                        tc_fence_after();
-#pragma unroll 1
-                        for (int c = 0; c < D / 16 / NSPLIT; ++c) {      // this thread's part of the O row
-                            uint32_t ov[16];
-                            tmem_ld16(t_o + c * 16, ov);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * factor);
-                            tmem_st16(t_o + c * 16, ov);
-                        }
-                    }
-                    l *= factor;
-                    const float msub = m_used == -INFINITY ? 0.f : m_used;
-                    // ---- probabilities: packed fp32 pairs; part of the exponentials on the FMA/ALU pipes
-                    const float2 sl2v = make_float2(sl2, sl2), nmv = make_float2(-msub, -msub);
-                    float2 acc[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[e] = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int c = 0; c < NC; c += 8) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 xv = __ffma2_rn(make_float2(__uint_as_float(sr[c + 2 * e]),
-                                                                     __uint_as_float(sr[c + 2 * e + 1])), sl2v, nmv);
-                            float2 pr;
-                            if (e >= 4 - EX2_POLY_PER_8 / 2) {
-                                pr = ex2_poly2(xv);
-                            } else {
-                                pr.x = ex2_approx(xv.x);
-                                pr.y = ex2_approx(xv.y);
-                            }
-                            acc[e] = __fadd2_rn(acc[e], pr);
-                            pk[(c >> 1) + e] = pack_bf16x2(pr.x, pr.y);
-                        }
-                    }
-                    l += (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y) + ((acc[2].x + acc[2].y) + (acc[3].x + acc[3].y));
                 }
+                tmem_wait_ld();
+                if (SOFTCAP) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) sr[c] = __float_as_uint(tanh_approx(__uint_as_float(sr[c]) * cap_in));
+                }
+                if (tm.masked) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c)
+                        sr[c] = ((tm.kw[(NSPLIT == 2 ? half * 2 : 0) + (c >> 5)] >> (c & 31)) & 1u) ? sr[c] : 0xff800000u;      // -inf
+                }
+                // ---- row maximum of the tile: four independent chains of three-input maxima
+                float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+#pragma unroll
+                for (int c = 0; c < NC; c += 8) {
+                    mx0 = max3(mx0, __uint_as_float(sr[c]), __uint_as_float(sr[c + 1]));
+                    mx1 = max3(mx1, __uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3]));
+                    mx2 = max3(mx2, __uint_as_float(sr[c + 4]), __uint_as_float(sr[c + 5]));
+                    mx3 = max3(mx3, __uint_as_float(sr[c + 6]), __uint_as_float(sr[c + 7]));
+                }
+                float mraw = max3(mx0, mx1, fmaxf(mx2, mx3));
+                if constexpr (NSPLIT == 2) {
+                    // the two threads of a row exchange the maxima of their halves and then take the same decisions
+                    const int par = (int)(nx & 1);
+                    const __nv_bfloat16 mine = __float2bfloat16_rn(mraw);
+                    xval(par, half, row_in_tile) = mine;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl.xchg[warp & 3]));
+                    ctl_wait(&ctl.xchg[warp & 3], (uint32_t)par, ctl, bad, 36);
+                    mraw = fmaxf(__bfloat162float(mine), __bfloat162float(xval(par, half ^ 1, row_in_tile)));
+                    ++nx;
+                }
+                const float mt = mraw * sl2;                     // log2 units (sl2 > 0; -inf stays -inf)
+                // ---- lazy maximum: raise the reference only when it lags by more than the threshold
+                float factor = 1.f;
+                bool raise = false;
+                if (m_used == -INFINITY) {
+                    m_used = mt;                                 // nothing accumulated yet for this row
+                } else if (mt > m_used + RESCALE_THRESHOLD) {
+                    factor = ex2_approx(m_used - mt);
+                    m_used = mt;
+                    raise = true;
+                }
+                l *= factor;
+                const float msub = m_used == -INFINITY ? 0.f : m_used;
+                // ---- probabilities: packed fp32 pairs; part of the exponentials on the FMA/ALU pipes
+                const float2 sl2v = make_float2(sl2, sl2), nmv = make_float2(-msub, -msub);
+                float2 acc[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[e] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < NC; c += 8) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 xv = __ffma2_rn(make_float2(__uint_as_float(sr[c + 2 * e]),
+                                                                 __uint_as_float(sr[c + 2 * e + 1])), sl2v, nmv);
+                        float2 pr;
+                        if (e >= 4 - EX2_POLY_PER_8 / 2) {
+                            pr = ex2_poly2(xv);
+                        } else {
+                            pr.x = ex2_approx(xv.x);
+                            pr.y = ex2_approx(xv.y);
+                        }
+                        acc[e] = __fadd2_rn(acc[e], pr);
+                        pk[(c >> 1) + e] = pack_bf16x2(pr.x, pr.y);
+                    }
+                }
+                l += (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y) + ((acc[2].x + acc[2].y) + (acc[3].x + acc[3].y));
 #pragma unroll
                 for (int c = 0; c < NC / 64; ++c) tmem_st32(t_s + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[c * 32]));
+                // (here, where no scores are held any more: before the exponentials the registers of this block slow the others down)
+                if (__any_sync(0xffffffffu, raise) && !first) {
+                    // O may only be touched once the previous PV of this query tile has completed.  With two
+                    // query tiles its commit precedes s_full; with double-buffered S it has its own barrier.
+                    if constexpr (NQ == 1) ctl_wait(&ctl.pv_done, (ns - 1) & 1, ctl, bad, 35);
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int c = 0; c < D / 16 / NSPLIT; ++c) {      // this thread's part of the O row
+                        uint32_t ov[16];
+                        tmem_ld16(t_o + c * 16, ov);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * factor);
+                        tmem_st16(t_o + c * 16, ov);
+                    }
+                }
                 tmem_wait_st();
                 tc_fence_before();
                 mbar_arrive(smem_u32(&ctl.p_full[buf]));
                 ++ns;
                 first = false;
-                if (!ok) break;
+                if (bad) break;
             }
-            if (!ok) break;
+            if (bad) break;
             tile_read();                                 // the end of the item
-            have = next_item<WALK>(p, &ctl, ord + 1, true, t, ok);
-            if (!ok) break;
-            if (have) load_row();
-            // ---- epilogue: O / l -> bf16 -> global, lse.  With a partial result to join (window pass of the split layout) the
-            // row's logsumexp there is read now, before a thread that shares the row can write the joint one.
-            float lse_other = -INFINITY;
-            if (WALK == WALK_TOKEN && p.join && valid) lse_other = p.lse[(size_t)hq * p.n + i];
-            if constexpr (NSPLIT == 2) {
-                // the two halves add their row sums: two exchanges, the leading bf16 part of the sum and its remainder
-                float other = 0.f, rest = l;
-                bool xok = true;
-                for (int piece = 0; piece < 2 && xok; ++piece) {
-                    const int par = (int)(nx & 1);
-                    const __nv_bfloat16 mine = __float2bfloat16_rn(rest);
-                    rest -= __bfloat162float(mine);
-                    xval(par, half, row_in_tile) = mine;
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&ctl.xchg[warp & 3]));
-                    xok = ctl_wait(&ctl.xchg[warp & 3], (uint32_t)par, &ctl);
-                    other += __bfloat162float(xval(par, half ^ 1, row_in_tile));
-                    ++nx;
-                }
-                if (!xok) { report_timeout(p, &ctl, 38, item); break; }
-                l += other;
-            }
-            if (!ctl_wait(&ctl.o_full[x], it & 1, &ctl)) { report_timeout(p, &ctl, 40 + x, item); break; }
-            tc_fence_after();
-            if (have) load_mask();
-            const float inv_l = l > 0.f ? 1.f / l : 0.f;        // a row without any pair (possible in a partial pass): zeros, lse = -inf
-            float own = inv_l, w_other = 0.f, lse_row = (m_used + lg2_approx(l)) * LN2;
-            if (WALK == WALK_TOKEN && p.join) {
-                // the two partial results cover disjoint sets of pairs and join through their logsumexps (Appendix D)
-                const float m = fmaxf(lse_other, lse_row);
-                const float wo = m == -INFINITY ? 0.f : __expf(lse_other - m), wl = m == -INFINITY ? 0.f : __expf(lse_row - m);
-                const float tot = wo + wl, inv = tot > 0.f ? 1.f / tot : 0.f;
-                own = inv_l * wl * inv;
-                w_other = wo * inv;
-                lse_row = tot > 0.f ? m + __logf(tot) : -INFINITY;
-            }
-            __nv_bfloat16* orow = p.o + (size_t)bb * p.o_sb + (size_t)h * p.o_sh + (size_t)(valid ? i : 0) * p.o_sn +
-                                  half * (D / 2);
-#pragma unroll 1
-            for (int c = 0; c < D / 32 / NSPLIT; ++c) {
-                uint32_t ov[32];
-                tmem_ld32(t_o + c * 32, ov);
-                tmem_wait_ld();
-                float add[32];
-                if constexpr (WALK == WALK_TOKEN) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) add[e] = 0.f;
-                    if (w_other > 0.f) {               // (a partial result without any pair has unspecified contents)
-                        const float* jrow = p.join + ((size_t)hq * p.n + (size_t)i) * D + half * (D / 2) + c * 32;
-#pragma unroll
-                        for (int e = 0; e < 32; e += 4) {
-                            const float4 v4 = *reinterpret_cast<const float4*>(jrow + e);
-                            add[e] = v4.x * w_other; add[e + 1] = v4.y * w_other; add[e + 2] = v4.z * w_other; add[e + 3] = v4.w * w_other;
-                        }
-                    }
-                }
-                auto out = [&](int e) {
-                    const float v = __uint_as_float(ov[e]);
-                    if constexpr (WALK == WALK_TOKEN) return fmaf(v, own, add[e]);
-                    else return v * own;
-                };
-                if (valid && p.o32) {
-                    float* o32row = p.o32 + ((size_t)hq * p.n + (size_t)i) * D + half * (D / 2) + c * 32;
-#pragma unroll
-                    for (int e = 0; e < 32; e += 8) {
-                        uint32_t w[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) w[j] = __float_as_uint(out(e + j));
-                        st_global_v8(o32row + e, w);
-                    }
-                } else if (valid) {
-#pragma unroll
-                    for (int e = 0; e < 32; e += 16) {
-                        uint32_t w[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) w[j] = pack_bf16x2(out(e + 2 * j), out(e + 2 * j + 1));
-                        if (p.o_wide) {
-                            st_global_v8(orow + c * 32 + e, w);
-                        } else {
-                            *reinterpret_cast<uint4*>(orow + c * 32 + e) = make_uint4(w[0], w[1], w[2], w[3]);
-                            *reinterpret_cast<uint4*>(orow + c * 32 + e + 8) = make_uint4(w[4], w[5], w[6], w[7]);
-                        }
-                    }
-                }
-            }
-            if (valid && half == 0) p.lse[(size_t)hq * p.n + i] = lse_row;
-            tc_fence_before();
-            ++it;
+            finish = !first;
         }
+        if (bad && lane == 0) give_up(p, &ctl, bad, t.A);
     }
     // ---------------------------------------------------------------------- teardown
     tc_fence_before();
@@ -1188,6 +1139,7 @@ static int launch_attn_t(const AttnArgs& a, cudaStream_t st) {
     p.lse = a.lse;
     p.status = a.dev_status;
     p.nitems = (long long)a.s.batch * a.s.Hq * p.nqb;
+    p.by_heads = Divisor(p.B * p.Hq); p.by_group = Divisor(p.nqb * p.G); p.by_G = Divisor(p.G); p.by_Hkv = Divisor(p.Hkv); p.by_Hq = Divisor(p.Hq);
     p.nqp = a.L.nqp; p.nkp = a.L.nkp; p.nqblk = a.L.nqp / 256;
     p.ipb = 2 / C::NQ;
     p.perm_q = sorted ? reinterpret_cast<const int32_t*>(a.ws + a.L.perm_q) : nullptr;
