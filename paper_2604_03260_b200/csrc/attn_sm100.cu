@@ -92,6 +92,13 @@ struct AttnCfg {
     // Ring order of the tiles.  With one query tile the S of the next key tile is issued before the current P V, so
     // K(next) travels ahead of V(current); with two query tiles V(current) is consumed and released first.
     static constexpr bool K_AHEAD = NQ == 1;
+    // Two query tiles, no gate: P is handed over in two parts, 96 columns and 32, so that most of P V runs while the last exponentials
+    // are taken and what lies between the last of them and the next S is a quarter of P V and that S.  From P to the next S
+    // 1250 -> 1000 cycles; 32 heads x 16384 tokens, dense: 1706 -> 1632 us, x 8192 in token order 530 -> 513, x 32768 class-sorted
+    // 6.41 -> 6.24 ms; in halves 1654, 520 and 6.29.  With the gate nothing is gained (707 -> 706 us at 8192 tokens, 268 -> 275 at
+    // D = 64): what is waited for there is G.
+    static constexpr bool SPLIT_P = NQ == 2 && GATE == 0;
+    static constexpr int P_FIRST = 96;
     static constexpr uint32_t COL_S0 = 0, COL_S1 = 128, COL_O0 = 256, COL_O1 = 256 + D;
     // With a single query tile two threads share a row: each of the two softmax warpgroups owns one 64-column
     // half of every key tile (its S columns, its P columns, its part of the row sum) and one half of the O row.
@@ -105,6 +112,7 @@ struct AttnCfg {
 struct SharedCtl {
     uint64_t q_full, q_empty;
     uint64_t s_full[2], p_full[2], o_full[2];
+    uint64_t p_rest[2];               // the second part of P (SPLIT_P)
     uint64_t pv_done;
     uint64_t xchg[4];                 // split rows, per 32-row quadrant: both column halves have published a per-row value
     uint64_t gbar[2];                 // soft gate, one query tile, per softmax warpgroup: the key assignments are in shared memory
@@ -266,6 +274,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         for (int x = 0; x < 2; ++x) {
             mbar_init(smem_u32(&ctl.s_full[x]), 1);
             mbar_init(smem_u32(&ctl.p_full[x]), 128 * C::NSPLIT);
+            mbar_init(smem_u32(&ctl.p_rest[x]), 128);
             mbar_init(smem_u32(&ctl.o_full[x]), 1);
         }
         for (int s = 0; s < C::NSTAGE; ++s) {
@@ -555,8 +564,18 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             if (have_p && !ctl_wait(&ctl.p_full[x], np & 1, ctl, bad, 24 + x)) break;
                             tc_fence_after();
                             const uint32_t t_s = tmem + (x ? C::COL_S1 : C::COL_S0);
+                            const uint32_t t_o = tmem + (x ? C::COL_O1 : C::COL_O0), vd = vdesc0 + vslot * (C::STAGE_BYTES >> 4);
+                            constexpr int STEPS1 = C::SPLIT_P ? C::P_FIRST / 16 : 0;      // of the 8 steps of P V
+                            if constexpr (C::SPLIT_P) {
+                                if (have_p) {
+                                    if (elect_one()) o_steps(t_o, t_s, vd, STEPS1, !first);
+                                    __syncwarp();
+                                    if (!ctl_wait(&ctl.p_rest[x], np & 1, ctl, bad, 44 + x)) break;
+                                    tc_fence_after();
+                                }
+                            }
                             if (have_p && elect_one()) {
-                                o_steps(tmem + (x ? C::COL_O1 : C::COL_O0), t_s, vdesc0 + vslot * (C::STAGE_BYTES >> 4), 8, !first);
+                                o_steps(t_o, t_s + STEPS1 * 8, vd + STEPS1 * 128, 8 - STEPS1, !first || C::SPLIT_P);
                                 if (x == 1) umma_commit(smem_u32(&ctl.kv_empty[vslot]));
                                 if (kb < 0) umma_commit(smem_u32(&ctl.o_full[x]));
                             }
@@ -1025,6 +1044,28 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 float2 acc[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[e] = make_float2(0.f, 0.f);
+                // The rows of O are brought to a raised reference just before P is handed over (before the exponentials, with all scores
+                // held, the registers of this block slow the others down), which the P V waits for.
+                auto hand_over = [&](uint64_t* bar, bool rescale) {
+                    if (rescale && __any_sync(0xffffffffu, raise) && !first) {
+                        // O may only be touched once the previous PV of this query tile has completed.  With two
+                        // query tiles its commit precedes s_full; with double-buffered S it has its own barrier.
+                        if constexpr (NQ == 1) ctl_wait(&ctl.pv_done, (ns - 1) & 1, ctl, bad, 35);
+                        tc_fence_after();
+#pragma unroll 1
+                        for (int c = 0; c < D / 16 / NSPLIT; ++c) {      // this thread's part of the O row
+                            uint32_t ov[16];
+                            tmem_ld16(t_o + c * 16, ov);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * factor);
+                            tmem_st16(t_o + c * 16, ov);
+                        }
+                    }
+                    tmem_wait_st();
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(bar));
+                };
 #pragma unroll
                 for (int c = 0; c < NC; c += 8) {
 #pragma unroll
@@ -1041,29 +1082,24 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         acc[e] = __fadd2_rn(acc[e], pr);
                         pk[(c >> 1) + e] = pack_bf16x2(pr.x, pr.y);
                     }
-                }
-                l += (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y) + ((acc[2].x + acc[2].y) + (acc[3].x + acc[3].y));
-#pragma unroll
-                for (int c = 0; c < NC / 64; ++c) tmem_st32(t_s + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[c * 32]));
-                // (here, where no scores are held any more: before the exponentials the registers of this block slow the others down)
-                if (__any_sync(0xffffffffu, raise) && !first) {
-                    // O may only be touched once the previous PV of this query tile has completed.  With two
-                    // query tiles its commit precedes s_full; with double-buffered S it has its own barrier.
-                    if constexpr (NQ == 1) ctl_wait(&ctl.pv_done, (ns - 1) & 1, ctl, bad, 35);
-                    tc_fence_after();
-#pragma unroll 1
-                    for (int c = 0; c < D / 16 / NSPLIT; ++c) {      // this thread's part of the O row
-                        uint32_t ov[16];
-                        tmem_ld16(t_o + c * 16, ov);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * factor);
-                        tmem_st16(t_o + c * 16, ov);
+                    if constexpr (C::SPLIT_P) {
+                        static_assert(C::P_FIRST == 96, "the stores below");
+                        if (c + 8 == C::P_FIRST) {
+                            tmem_st32(t_s, *reinterpret_cast<uint32_t(*)[32]>(&pk[0]));
+                            tmem_st16(t_s + 32, *reinterpret_cast<uint32_t(*)[16]>(&pk[32]));
+                            hand_over(&ctl.p_full[buf], true);
+                        }
                     }
                 }
-                tmem_wait_st();
-                tc_fence_before();
-                mbar_arrive(smem_u32(&ctl.p_full[buf]));
+                if constexpr (C::SPLIT_P) {
+                    tmem_st16(t_s + 48, *reinterpret_cast<uint32_t(*)[16]>(&pk[48]));
+                    hand_over(&ctl.p_rest[buf], false);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < NC / 64; ++c) tmem_st32(t_s + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[c * 32]));
+                    hand_over(&ctl.p_full[buf], true);
+                }
+                l += (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y) + ((acc[2].x + acc[2].y) + (acc[3].x + acc[3].y));
                 ++ns;
                 first = false;
                 if (bad) break;
