@@ -1,5 +1,5 @@
-"""ctypes binding of libfocus_b200.so: same names as the C ABI (include/focus.h), argument
-marshalling only.  torch supplies device memory and the current stream; every step of the path
+"""Binding of libfocus_b200.so: same names as the C ABI (include/focus.h), argument marshalling only, through ctypes; the
+calls of a decode step and of a short prompt take the same arguments through csrc/marshal.cpp.  torch supplies device memory and the current stream; every step of the path
 runs inside the library's CUDA kernels.  There is no CPU fallback: loading fails loudly when the
 library has not been built (``python -m paper_2604_03260_b200.build``)."""
 from __future__ import annotations
@@ -52,10 +52,11 @@ class FocusError(RuntimeError):
 
 
 _lib = None
+_marshal = None         # csrc/marshal.cpp
 
 
 def lib():
-    global _lib
+    global _lib, _marshal
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2604_03260_b200.build` "
@@ -112,7 +113,12 @@ def lib():
         L.focus_selftest_stalled_wait.argtypes = [SP, focus_tensor, focus_tensor, focus_tensor, focus_tensor, vp, C.c_uint64, vp, vp]
         L.focus_selftest_stalled_exchange.restype = C.c_int
         L.focus_selftest_stalled_exchange.argtypes = [SP, vp, f32, i32, vp, sz, C.c_int64, i32, vp, vp]
-        _lib = L
+        try:
+            from . import _marshal as m
+        except ImportError as e:
+            raise ImportError(f"{e}: build it with `python -m paper_2604_03260_b200.build`") from e
+        m.init(focus_shape)
+        _marshal, _lib = m, L
     return _lib
 
 
@@ -121,9 +127,16 @@ def _check(rc):
         raise FocusError(rc, lib().focus_last_error().decode())
 
 
-# A short call (a decode step, a prompt of a thousand tokens) takes the GPU no longer than Python takes to marshal its
-# arguments, so these stay plain: addresses and stream handles as integers, one look at a tensor's strides, the current
-# stream's handle without a Stream object around it (3.2 us per call of a step whose GPU work is 17).
+def _short():
+    """The calls whose GPU work is as short as their marshalling.  They answer with a status, or None when an argument is not of
+    the usual kind; it then goes the way of the other entry points."""
+    if _marshal is None:
+        lib()
+    return _marshal
+
+
+# Addresses and stream handles as integers, one look at a tensor's strides, the current stream's handle without a Stream object
+# around it.
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
@@ -163,16 +176,21 @@ def focus_version() -> int:
 
 
 def focus_assign(shape, x, H, centroids, masks_out, near_ties=None, near_tie_eps=1e-5, stream=None):
-    _check(lib().focus_assign(C.byref(shape), tensor_arg(x), H, _p(centroids), _p(masks_out), _p(near_ties),
-                              near_tie_eps, _stream(stream)))
+    rc = _short().assign(shape, x, H, centroids, masks_out, near_ties, near_tie_eps, stream)
+    if rc is None:
+        rc = lib().focus_assign(C.byref(shape), tensor_arg(x), H, _p(centroids), _p(masks_out), _p(near_ties), near_tie_eps, _stream(stream))
+    _check(rc)
 
 
 def focus_assign_hidden(shape, h, Wg, Cg, bias, folded, mq_out, mk_out, near_ties=None, near_tie_eps=1e-5, stream=None):
     """h bf16 [batch, n, d_model] (or [n, d_model]); Wg fp32 [d_model, d_g]; Cg fp32 [K, d_g]; folded fp32 [K, d_model] scratch"""
-    assert h.is_cuda and h.dtype == torch.bfloat16 and h.stride(-1) == 1
-    sb, sn = (h.stride(0), h.stride(1)) if h.dim() == 3 else (h.stride(0) * h.shape[0], h.stride(0))
-    _check(lib().focus_assign_hidden(C.byref(shape), _p(h), sb, sn, h.shape[-1], Wg.shape[1], _p(Wg), _p(Cg), _p(bias),
-                                     _p(folded), _p(mq_out), _p(mk_out), _p(near_ties), near_tie_eps, _stream(stream)))
+    rc = _short().assign_hidden(shape, h, Wg, Cg, bias, folded, mq_out, mk_out, near_ties, near_tie_eps, stream)
+    if rc is None:
+        assert h.is_cuda and h.dtype == torch.bfloat16 and h.stride(-1) == 1
+        sb, sn = (h.stride(0), h.stride(1)) if h.dim() == 3 else (h.stride(0) * h.shape[0], h.stride(0))
+        rc = lib().focus_assign_hidden(C.byref(shape), _p(h), sb, sn, h.shape[-1], Wg.shape[1], _p(Wg), _p(Cg), _p(bias),
+                                       _p(folded), _p(mq_out), _p(mk_out), _p(near_ties), near_tie_eps, _stream(stream))
+    _check(rc)
 
 
 def focus_tiles_layout_of(shape, layout) -> focus_tiles_layout:
@@ -186,13 +204,18 @@ def focus_tiles_workspace_bytes(shape, layout) -> int:
 
 
 def focus_build_tiles(shape, mq, mk, layout, ws, stream=None):
-    _check(lib().focus_build_tiles(C.byref(shape), _p(mq), _p(mk), layout, _p(ws), ws.numel() * ws.element_size(),
-                                   _stream(stream)))
+    rc = _short().build_tiles(shape, mq, mk, layout, ws, stream)
+    if rc is None:
+        rc = lib().focus_build_tiles(C.byref(shape), _p(mq), _p(mk), layout, _p(ws), ws.numel() * ws.element_size(), _stream(stream))
+    _check(rc)
 
 
 def focus_attn_fwd(shape, q, k, v, mq, mk, tiles_ws, layout, o, lse, dev_status=None, stream=None):
-    _check(lib().focus_attn_fwd(C.byref(shape), tensor_arg(q), tensor_arg(k), tensor_arg(v), _p(mq), _p(mk),
-                                _p(tiles_ws), layout, tensor_arg(o), _p(lse), _p(dev_status), _stream(stream)))
+    rc = _short().attn_fwd(shape, q, k, v, mq, mk, tiles_ws, layout, o, lse, dev_status, stream)
+    if rc is None:
+        rc = lib().focus_attn_fwd(C.byref(shape), tensor_arg(q), tensor_arg(k), tensor_arg(v), _p(mq), _p(mk),
+                                  _p(tiles_ws), layout, tensor_arg(o), _p(lse), _p(dev_status), _stream(stream))
+    _check(rc)
 
 
 def focus_decode_workspace_bytes(shape) -> int:
@@ -207,8 +230,11 @@ def focus_decode_step(shape, q, k, v, mq_new, mk, o, lse, ws, stream=None):
         if len(st) == 2:
             return focus_tensor(t.data_ptr(), st[0] * t.shape[0], st[0], t.shape[-1])
         return focus_tensor(t.data_ptr(), st[0], st[1], t.shape[-1])
-    _check(lib().focus_decode_step(C.byref(shape), vec_arg(q), tensor_arg(k), tensor_arg(v), _p(mq_new), _p(mk), vec_arg(o),
-                                   _p(lse), _p(ws), ws.numel() * ws.element_size(), _stream(stream)))
+    rc = _short().decode_step(shape, q, k, v, mq_new, mk, o, lse, ws, stream)
+    if rc is None:
+        rc = lib().focus_decode_step(C.byref(shape), vec_arg(q), tensor_arg(k), tensor_arg(v), _p(mq_new), _p(mk), vec_arg(o),
+                                     _p(lse), _p(ws), ws.numel() * ws.element_size(), _stream(stream))
+    _check(rc)
 
 
 def focus_soft_ld(K) -> int:

@@ -1,4 +1,4 @@
-"""In-tree build of libfocus_b200.so (nvcc, sm_100a only).  ``python -m paper_2604_03260_b200.build``."""
+"""In-tree build of libfocus_b200.so (nvcc, sm_100a only) and of the module in front of it (g++).  ``python -m paper_2604_03260_b200.build``."""
 from __future__ import annotations
 
 import os
@@ -9,6 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfocus_b200.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 SOURCES = ["api.cu", "assign.cu", "assign_hidden.cu", "sinkhorn.cu", "decode.cu", "tiles.cu", "tiles_sorted.cu", "attn_sm100.cu", "selftest.cu",
            "tma_host.cu", "noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -27,6 +28,19 @@ def _stale(target: str, deps) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _marshal_cmd(out: str) -> list:
+    """csrc/marshal.cpp: a Python module that reads torch tensors and calls the library"""
+    import sysconfig
+
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
+    return (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+             "-I", os.path.join(ROOT, "include"), "-I", os.path.join(t, "include"), "-I", os.path.join(t, "include", "torch", "csrc", "api", "include"),
+             "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "marshal.cpp"), "-o", out,
+             "-L", HERE, "-l:libfocus_b200.so", "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -57,6 +71,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + ".tmp%d" % os.getpid()
         subprocess.check_call([_nvcc(), "-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
+    if force or _stale(MARSHAL, [os.path.join(CSRC, "marshal.cpp"), os.path.join(ROOT, "include", "focus.h")]):
+        tmp = MARSHAL + ".tmp%d" % os.getpid()
+        subprocess.check_call(_marshal_cmd(tmp))
+        os.replace(tmp, MARSHAL)
     return LIB
 
 

@@ -1,0 +1,84 @@
+"""The short calls through csrc/marshal.cpp and through ctypes: the same results, the same errors."""
+import pytest
+import torch
+
+from paper_2604_03260_b200 import binding as fb
+from paper_2604_03260_b200 import inputs as fi
+
+pytestmark = pytest.mark.gpu
+
+
+class NotRead:
+    """in the place of the module: no argument is of the usual kind"""
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+class Sub(torch.Tensor):
+    pass
+
+
+def run(wl, wrap, batch, stream=None, eps=1e-5):
+    """assign -> build_tiles -> attn_fwd, a decode step, and the router, with tensors passed through `wrap`"""
+    dev = "cuda"
+    shape = fb.make_shape(wl.Hq, wl.Hkv, wl.n, wl.D, wl.K, wl.topk, wl.window, batch=batch)
+    Q, K, V, C = fi.make_inputs(wl, dev)
+    if batch > 1:
+        Q, K, V = (torch.stack([x] + [x.flip(1)] * (batch - 1)) for x in (Q, K, V))
+    K = torch.cat([K, K], dim=-2)[..., :wl.n, :]                # head stride other than n * D
+    mq, mk = (torch.zeros((batch * h, wl.n), dtype=torch.int32, device=dev) for h in (wl.Hq, wl.Hkv))
+    near = torch.zeros(1, dtype=torch.int64, device=dev)
+    fb.focus_assign(shape, wrap(Q), wl.Hq, wrap(C), wrap(mq), wrap(near), eps, stream)
+    fb.focus_assign(shape, wrap(K), wl.Hkv, C, mk, stream=stream)
+    ws = fb.alloc_workspace(shape, 0)
+    fb.focus_build_tiles(shape, wrap(mq), mk, 0, wrap(ws), stream)
+    O, lse, status = torch.zeros_like(Q), torch.zeros((batch * wl.Hq, wl.n), device=dev), torch.zeros(4, dtype=torch.int32, device=dev)
+    fb.focus_attn_fwd(shape, wrap(Q), wrap(K), wrap(V), mq, mk, ws, 0, wrap(O), lse, status, stream)
+    q1 = Q[..., -1, :]
+    o1, l1 = torch.zeros(q1.shape, dtype=torch.bfloat16, device=dev), torch.zeros(batch * wl.Hq, device=dev)
+    wd = torch.zeros(fb.focus_decode_workspace_bytes(shape), dtype=torch.uint8, device=dev)
+    fb.focus_decode_step(shape, wrap(q1), K, V, mq[:, -1].contiguous(), mk, wrap(o1), l1, wd, stream)
+    h = torch.sin(torch.arange(batch * wl.n * 64, device=dev)).to(torch.bfloat16).view(batch, wl.n, 64)
+    h = h[0] if batch == 1 else h
+    Wg, Cg = (torch.cos(torch.arange(m * 16, device=dev)).float().view(m, 16) for m in (64, wl.K))
+    f, hq, hk = torch.zeros((wl.K, 64), device=dev), torch.zeros_like(mq), torch.zeros_like(mk)
+    fb.focus_assign_hidden(shape, wrap(h), Wg, Cg, None, f, hq, hk, stream=stream)
+    torch.cuda.synchronize()
+    return mq, mk, near, O, lse, status, o1, l1, f, hq, hk
+
+
+@pytest.mark.parametrize("batch", [1, 3])
+def test_same_results_both_ways(monkeypatch, batch):
+    wl = fi.Workload("marshal", 4, 2, 64, 300, 4, 2, 32, seed=3)
+    got = run(wl, lambda t: t, batch)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    others = [run(wl, lambda t: t, batch, stream=torch.cuda.current_stream()), run(wl, lambda t: t.as_subclass(Sub), batch)]
+    with torch.cuda.stream(side):
+        others.append(run(wl, lambda t: t, batch))
+    monkeypatch.setattr(fb, "_marshal", NotRead())
+    others.append(run(wl, lambda t: t, batch))
+    for other in others:
+        for a, b in zip(got, other):
+            assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("direct", [True, False])
+def test_same_errors_both_ways(monkeypatch, direct):
+    if not direct:
+        monkeypatch.setattr(fb, "_marshal", NotRead())
+    wl = fi.Workload("marshal", 4, 2, 64, 40, 4, 2, 32, seed=3)
+    shape = fb.shape_of(wl)
+    Q, K, V, C = fi.make_inputs(wl, "cuda")
+    m = torch.zeros((4, 40), dtype=torch.int32, device="cuda")
+    for bad in (Q.float(), Q.cpu(), Q.transpose(1, 2), Q[0]):
+        with pytest.raises(AssertionError):
+            fb.focus_assign(shape, bad, 4, C, m)
+    with pytest.raises(fb.FocusError, match="focus status"):
+        fb.focus_assign(fb.make_shape(4, 2, 40, 63, 4, 2, 32), Q, 4, C, m)
+    with pytest.raises(fb.FocusError):
+        fb.focus_build_tiles(shape, m, m, 0, torch.zeros(16, dtype=torch.uint8, device="cuda"))
+    with pytest.raises((AttributeError, TypeError)):
+        fb.focus_attn_fwd(shape, Q, K, 7, None, None, None, 0, torch.empty_like(Q), m)
+    fb.focus_assign(shape, Q, 4, C, m, None, 0)                  # a whole number for a float
+    torch.cuda.synchronize()
