@@ -132,9 +132,10 @@ struct GateCtl {
     uint64_t g_full[2], g_taken[2];   // G of a query tile is in tensor memory / in the softmax warps' registers
 };
 
-// Bounded wait that also gives up when another role of the CTA has given up.  `gave_up` becomes `where`; the role reports it once, at
-// its end (give_up).  Few instructions, for there are some thirty places (the note on code size above); the try in front of the loop is
-// worth its own (D = 256, 16384 tokens dense: 1580 us without it, 1537 so).
+// Bounded wait that also gives up when another role of the CTA has given up.  `gave_up` becomes `where`; the role reports it at its
+// end (give_up), every lane that gave up, for the lanes of a warp may not all have.  Few instructions, for there are some thirty
+// places (the note on code size above); the try in front of the loop is worth its own (D = 256, 16384 tokens dense: 1580 us without
+// it, 1537 so).
 __device__ __forceinline__ bool ctl_wait(uint64_t* bar, uint32_t parity, SharedCtl& ctl, int& gave_up, int where) {
     if (mbar_try_wait(smem_u32(bar), parity)) return true;          // (a try lasts until the phase completes, or about a millisecond)
     uint32_t t0 = 0;
@@ -403,7 +404,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
                     for (int second = 0; second < 2; ++second) {
                         if (bad) break;
-                        const bool is_v = (NQ == 2) != (second != 0);
+                        const bool is_v = C::K_AHEAD == (second != 0);
                         const int tile = is_v ? kb_v : kb;
                         if (tile >= 0) load_tile(is_v, tile);
                     }
@@ -613,7 +614,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     have_p = true;
                 }
             }
-            if (bad && lane == 0) give_up(p, &ctl, bad, t.A);
+            if (bad) give_up(p, &ctl, bad, t.A);
         }
         __syncwarp();
     } else if (C::GATE_MMA && warp < 4) {
@@ -657,7 +658,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
             ++it;
         }
-        if (bad && lane == 0) give_up(p, &ctl, bad, t.A);
+        if (bad) give_up(p, &ctl, bad, t.A);
         __syncwarp();
     } else if (warp >= 4) {
         // ------------------------------------------------------------------ softmax + epilogue
@@ -1108,7 +1109,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             tile_read();                                 // the end of the item
             finish = !first;
         }
-        if (bad && lane == 0) give_up(p, &ctl, bad, t.A);
+        if (bad) give_up(p, &ctl, bad, t.A);
     }
     // ---------------------------------------------------------------------- teardown
     tc_fence_before();
