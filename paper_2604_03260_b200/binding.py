@@ -9,6 +9,8 @@ import os
 
 import torch
 
+from . import build as _build
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libfocus_b200.so")
 
@@ -114,12 +116,20 @@ def lib():
         L.focus_selftest_stalled_exchange.restype = C.c_int
         L.focus_selftest_stalled_exchange.argtypes = [SP, vp, f32, i32, vp, sz, C.c_int64, i32, vp, vp]
         try:
-            from . import _marshal as m
+            m = _load_marshal()
         except ImportError as e:
             raise ImportError(f"{e}: build it with `python -m paper_2604_03260_b200.build`") from e
-        m.init(focus_shape)
         _marshal, _lib = m, L
     return _lib
+
+
+def _load_marshal():
+    """csrc/marshal.cpp, if it was built for this torch and this Python: it knows the layout of their objects"""
+    from . import _marshal as m
+    if getattr(m, "built_for", None) != _build.marshal_abi():
+        raise ImportError(f"{m.__file__} was built for another torch or Python ({getattr(m, 'built_for', None)}, here {_build.marshal_abi()})")
+    m.init(focus_shape)
+    return m
 
 
 def _check(rc):

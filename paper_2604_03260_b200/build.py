@@ -4,12 +4,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfocus_b200.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))     # (other interpreters do not look for that name)
 SOURCES = ["api.cu", "assign.cu", "assign_hidden.cu", "sinkhorn.cu", "decode.cu", "tiles.cu", "tiles_sorted.cu", "attn_sm100.cu", "selftest.cu",
            "tma_host.cu", "noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -30,17 +31,34 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def marshal_abi() -> str:
+    """What the module depends on beside its source: it reads torch's tensor objects by their layout."""
+    import torch
+    return f"{torch.__version__} {torch.version.git_version} {sysconfig.get_config_var('SOABI')}"
+
+
 def _marshal_cmd(out: str) -> list:
     """csrc/marshal.cpp: a Python module that reads torch tensors and calls the library"""
-    import sysconfig
-
     import torch
     t = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
     return (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+             f'-DFOCUS_BUILT_FOR="{marshal_abi()}"',
              "-I", os.path.join(ROOT, "include"), "-I", os.path.join(t, "include"), "-I", os.path.join(t, "include", "torch", "csrc", "api", "include"),
              "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "marshal.cpp"), "-o", out,
              "-L", HERE, "-l:libfocus_b200.so", "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])
+
+
+def _marshal_stamp() -> str:
+    return os.path.join(HERE, "_build", "marshal.cmd")
+
+
+def marshal_stale() -> bool:
+    """the module is missing, older than its sources, or made by another command (another torch or Python among them)"""
+    if _stale(MARSHAL, [os.path.join(CSRC, "marshal.cpp"), os.path.join(ROOT, "include", "focus.h")]) or not os.path.exists(_marshal_stamp()):
+        return True
+    with open(_marshal_stamp()) as f:
+        return f.read() != "\n".join(_marshal_cmd(MARSHAL))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -71,10 +89,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + ".tmp%d" % os.getpid()
         subprocess.check_call([_nvcc(), "-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
-    if force or _stale(MARSHAL, [os.path.join(CSRC, "marshal.cpp"), os.path.join(ROOT, "include", "focus.h")]):
+    if force or marshal_stale():
         tmp = MARSHAL + ".tmp%d" % os.getpid()
         subprocess.check_call(_marshal_cmd(tmp))
         os.replace(tmp, MARSHAL)
+        with open(_marshal_stamp(), "w") as f:
+            f.write("\n".join(_marshal_cmd(MARSHAL)))
     return LIB
 
 

@@ -214,4 +214,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", "short calls of binding
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__marshal() {
+    PyObject* m = PyModule_Create(&module);
+    // the torch and the Python whose objects the code above reads; binding.py compares before it passes it any
+    if (m && PyModule_AddStringConstant(m, "built_for", FOCUS_BUILT_FOR)) Py_CLEAR(m);
+    return m;
+}

@@ -1,0 +1,60 @@
+"""The module in front of the library (csrc/marshal.cpp) reads torch's objects by their layout: it is used only with the torch and the
+Python that it was built for, and built again when they change.  CPU."""
+import sys
+import types
+
+import pytest
+
+import paper_2604_03260_b200 as package
+from paper_2604_03260_b200 import binding as fb
+from paper_2604_03260_b200 import build
+
+
+@pytest.fixture
+def put(monkeypatch):
+    """put(m): the next load of the binding finds `m` in the place of the module (None: no module)"""
+    fb.lib()                                    # (what is put back afterwards is the loaded state)
+    def put(m):
+        monkeypatch.setattr(fb, "_lib", None)
+        monkeypatch.setattr(fb, "_marshal", None)
+        monkeypatch.delattr(package, "_marshal", raising=False)
+        monkeypatch.setitem(sys.modules, package.__name__ + "._marshal", m)
+    return put
+
+
+def module(built_for):
+    """stands for a module built for `built_for`; records what it is given"""
+    m = types.ModuleType(package.__name__ + "._marshal")
+    m.__file__, m.given = "elsewhere", []
+    m.init = lambda *args: m.given.append(args)
+    if built_for is not None:
+        m.built_for = built_for
+    return m
+
+
+def test_the_module_beside_the_library_is_the_one_in_use():
+    fb.lib()
+    assert fb._marshal.__file__ == build.MARSHAL and fb._marshal.built_for == build.marshal_abi()
+    assert not build.marshal_stale()
+
+
+@pytest.mark.parametrize("built_for", [None, "2.0.0 0123abcd cpython-310-x86_64-linux-gnu"])
+def test_a_module_of_another_torch_is_given_nothing(put, built_for):
+    m = module(built_for)
+    put(m)
+    with pytest.raises(ImportError, match="another torch or Python"):
+        fb.lib()
+    assert m.given == []
+
+
+@pytest.mark.parametrize("change", ["torch", "python", "flags"])
+def test_the_module_is_built_again_after(monkeypatch, change):
+    import torch
+    cmd = build._marshal_cmd
+    if change == "torch":
+        monkeypatch.setattr(torch, "__version__", "99.0")
+    elif change == "python":
+        monkeypatch.setattr(build.sysconfig, "get_config_var", lambda name: "another")
+    else:
+        monkeypatch.setattr(build, "_marshal_cmd", lambda out: cmd(out) + ["-DX"])
+    assert build.marshal_stale()
