@@ -1,11 +1,12 @@
 """Binding of libfocus_b200.so: same names as the C ABI (include/focus.h), argument marshalling only, through ctypes; the
-calls of a decode step and of a short prompt take the same arguments through csrc/marshal.cpp.  torch supplies device memory and the current stream; every step of the path
-runs inside the library's CUDA kernels.  There is no CPU fallback: loading fails loudly when the
-library has not been built (``python -m paper_2604_03260_b200.build``)."""
+calls of a decode step and of a short prompt take the same arguments through csrc/marshal.cpp where that is built for this torch.
+torch supplies device memory and the current stream; every step of the path runs inside the library's CUDA kernels.  There is no CPU
+fallback: loading fails loudly when the library has not been built (``python -m paper_2604_03260_b200.build``)."""
 from __future__ import annotations
 
 import ctypes as C
 import os
+import warnings
 
 import torch
 
@@ -115,19 +116,27 @@ def lib():
         L.focus_selftest_stalled_wait.argtypes = [SP, focus_tensor, focus_tensor, focus_tensor, focus_tensor, vp, C.c_uint64, vp, vp]
         L.focus_selftest_stalled_exchange.restype = C.c_int
         L.focus_selftest_stalled_exchange.argtypes = [SP, vp, f32, i32, vp, sz, C.c_int64, i32, vp, vp]
-        try:
-            m = _load_marshal()
-        except ImportError as e:
-            raise ImportError(f"{e}: build it with `python -m paper_2604_03260_b200.build`") from e
-        _marshal, _lib = m, L
+        _marshal, _lib = _load_marshal(), L
     return _lib
+
+
+class _Ctypes:
+    """in the place of csrc/marshal.cpp where that cannot be loaded: knows no argument, so that every call goes through ctypes"""
+    @staticmethod
+    def assign(*args):
+        return None
+    assign_hidden = build_tiles = attn_fwd = decode_step = assign
 
 
 def _load_marshal():
     """csrc/marshal.cpp, if it was built for this torch and this Python: it knows the layout of their objects"""
-    from . import _marshal as m
-    if getattr(m, "built_for", None) != _build.marshal_abi():
-        raise ImportError(f"{m.__file__} was built for another torch or Python ({getattr(m, 'built_for', None)}, here {_build.marshal_abi()})")
+    try:
+        from . import _marshal as m
+        if getattr(m, "built_for", None) != _build.marshal_abi():
+            raise ImportError(f"{m.__file__} was built for another torch or Python ({getattr(m, 'built_for', None)}, here {_build.marshal_abi()})")
+    except ImportError as e:
+        warnings.warn(f"{e}: short calls take some 10 us longer through ctypes; `python -m paper_2604_03260_b200.build` builds the module", RuntimeWarning)
+        return _Ctypes
     m.init(focus_shape)
     return m
 

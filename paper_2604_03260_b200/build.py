@@ -61,6 +61,23 @@ def marshal_stale() -> bool:
         return f.read() != "\n".join(_marshal_cmd(MARSHAL))
 
 
+def build_marshal(force: bool = False) -> bool:
+    """The module, where torch's headers and g++ are to hand; without it the binding makes the same calls through ctypes."""
+    try:
+        if force or marshal_stale():
+            tmp = MARSHAL + ".tmp%d" % os.getpid()
+            subprocess.check_call(_marshal_cmd(tmp))
+            os.replace(tmp, MARSHAL)
+            with open(_marshal_stamp(), "w") as f:
+                f.write("\n".join(_marshal_cmd(MARSHAL)))
+        return True
+    except (ImportError, OSError, subprocess.CalledProcessError) as e:
+        print(f"csrc/marshal.cpp not built, calls go through ctypes: {e}", file=sys.stderr)
+        if os.path.exists(MARSHAL):             # of an older source or another torch
+            os.remove(MARSHAL)
+        return False
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     headers.append(os.path.join(ROOT, "include", "focus.h"))
@@ -89,12 +106,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + ".tmp%d" % os.getpid()
         subprocess.check_call([_nvcc(), "-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
-    if force or marshal_stale():
-        tmp = MARSHAL + ".tmp%d" % os.getpid()
-        subprocess.check_call(_marshal_cmd(tmp))
-        os.replace(tmp, MARSHAL)
-        with open(_marshal_stamp(), "w") as f:
-            f.write("\n".join(_marshal_cmd(MARSHAL)))
+    build_marshal(force)
     return LIB
 
 

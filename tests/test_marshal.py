@@ -1,9 +1,10 @@
 """The module in front of the library (csrc/marshal.cpp) reads torch's objects by their layout: it is used only with the torch and the
-Python that it was built for, and built again when they change.  CPU."""
+Python that it was built for, built again when they change, and done without where it cannot be had.  CPU."""
 import sys
 import types
 
 import pytest
+import torch
 
 import paper_2604_03260_b200 as package
 from paper_2604_03260_b200 import binding as fb
@@ -41,14 +42,40 @@ def test_the_module_beside_the_library_is_the_one_in_use():
 def test_a_module_of_another_torch_is_given_nothing(put, built_for):
     m = module(built_for)
     put(m)
-    with pytest.raises(ImportError, match="another torch or Python"):
+    with pytest.warns(RuntimeWarning, match="another torch or Python"):
         fb.lib()
-    assert m.given == []
+    assert m.given == [] and fb._marshal is not m
+
+
+def test_without_the_module_every_call_goes_through_ctypes(put):
+    put(None)
+    with pytest.warns(RuntimeWarning, match="through ctypes"):
+        assert fb.focus_version() >= 100
+    s = fb.make_shape(8, 4, 1000, 128, 4, 2, 16)
+    assert fb.focus_tiles_workspace_bytes(s, 0) > 0
+    x, m = torch.zeros((8, 1000, 128), dtype=torch.bfloat16), torch.zeros((8, 1000), dtype=torch.int32)
+    with pytest.raises(AssertionError):                  # not on the GPU: refused by the binding, as ever
+        fb.focus_assign(s, x, 8, x, m)
+    with pytest.raises(AssertionError):
+        fb.focus_assign_hidden(s, x[0], x, x, None, x, m, m)
+    with pytest.raises(AssertionError):
+        fb.focus_attn_fwd(s, x, x, x, m, m, m, 0, x, m)
+    with pytest.raises(AssertionError):
+        fb.focus_decode_step(s, x[:, 0], x, x, m, m, x[:, 0], m, m)
+
+
+@pytest.mark.parametrize("cmd", [["false"], ["no-such-compiler"]])
+def test_a_module_that_cannot_be_built_leaves_the_library(monkeypatch, tmp_path, cmd):
+    old = tmp_path / "_marshal.so"
+    old.write_text("of another torch")
+    monkeypatch.setattr(build, "MARSHAL", str(old))
+    monkeypatch.setattr(build, "_marshal_stamp", lambda: str(tmp_path / "stamp"))
+    monkeypatch.setattr(build, "_marshal_cmd", lambda out: cmd)
+    assert not build.build_marshal() and not old.exists()
 
 
 @pytest.mark.parametrize("change", ["torch", "python", "flags"])
 def test_the_module_is_built_again_after(monkeypatch, tmp_path, change):
-    import torch
     cmd = build._marshal_cmd
     monkeypatch.setattr(build, "_stale", lambda target, deps: False)            # the sources are as they were
     monkeypatch.setattr(build, "_marshal_stamp", lambda: str(tmp_path / "stamp"))
