@@ -116,7 +116,7 @@ def lib():
         L.focus_selftest_stalled_wait.argtypes = [SP, focus_tensor, focus_tensor, focus_tensor, focus_tensor, vp, C.c_uint64, vp, vp]
         L.focus_selftest_stalled_exchange.restype = C.c_int
         L.focus_selftest_stalled_exchange.argtypes = [SP, vp, f32, i32, vp, sz, C.c_int64, i32, vp, vp]
-        _marshal, _lib = _load_marshal(), L
+        _marshal, _lib = _load_marshal(L), L
     return _lib
 
 
@@ -128,7 +128,7 @@ class _Ctypes:
     assign_hidden = build_tiles = attn_fwd = decode_step = assign
 
 
-def _load_marshal():
+def _load_marshal(L):
     """csrc/marshal.cpp, if it was built for this torch and this Python: it knows the layout of their objects"""
     try:
         from . import _marshal as m
@@ -137,7 +137,8 @@ def _load_marshal():
     except ImportError as e:
         warnings.warn(f"{e}: short calls take some 10 us longer through ctypes; `python -m paper_2604_03260_b200.build` builds the module", RuntimeWarning)
         return _Ctypes
-    m.init(focus_shape)
+    m.init(focus_shape, *(C.cast(f, C.c_void_p).value for f in (L.focus_assign, L.focus_assign_hidden, L.focus_build_tiles, L.focus_attn_fwd,
+                                                                L.focus_decode_step)))
     return m
 
 

@@ -38,7 +38,7 @@ def marshal_abi() -> str:
 
 
 def _marshal_cmd(out: str) -> list:
-    """csrc/marshal.cpp: a Python module that reads torch tensors and calls the library"""
+    """csrc/marshal.cpp: a Python module that reads torch tensors and calls the library (whose addresses it is given)"""
     import torch
     t = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
@@ -46,7 +46,7 @@ def _marshal_cmd(out: str) -> list:
              f'-DFOCUS_BUILT_FOR="{marshal_abi()}"',
              "-I", os.path.join(ROOT, "include"), "-I", os.path.join(t, "include"), "-I", os.path.join(t, "include", "torch", "csrc", "api", "include"),
              "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "marshal.cpp"), "-o", out,
-             "-L", HERE, "-l:libfocus_b200.so", "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])
+             "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-lc10", "-lc10_cuda"])
 
 
 def _marshal_stamp() -> str:

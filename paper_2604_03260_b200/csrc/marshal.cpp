@@ -19,6 +19,13 @@ namespace {
 
 PyObject* shape_type;                // binding.focus_shape
 
+// The entry points, from the library that binding.py has loaded: linked against, the loader might find another copy of it.
+decltype(&focus_assign) p_assign;
+decltype(&focus_assign_hidden) p_assign_hidden;
+decltype(&focus_build_tiles) p_build_tiles;
+decltype(&focus_attn_fwd) p_attn_fwd;
+decltype(&focus_decode_step) p_decode_step;
+
 struct Args {
     PyObject* const* a;
     bool known = true;               // every argument so far was of a kind that is read here
@@ -117,7 +124,7 @@ PyObject* assign(PyObject*, PyObject* const* args, Py_ssize_t n) {
         auto near = static_cast<unsigned long long*>(a.ptr(5));
         auto eps = a.number(6);
         auto st = a.stream(7);
-        return [=] { return focus_assign(s, x, H, c, m, near, eps, st); };
+        return [=] { return p_assign(s, x, H, c, m, near, eps, st); };
     });
 }
 
@@ -146,7 +153,7 @@ PyObject* assign_hidden(PyObject*, PyObject* const* args, Py_ssize_t n) {
         auto near = static_cast<unsigned long long*>(a.ptr(8));
         auto eps = a.number(9);
         auto st = a.stream(10);
-        return [=] { return focus_assign_hidden(s, h.ptr, h.stride_b, h.stride_n, d, dg, Wg, Cg, bias, folded, mq, mk, near, eps, st); };
+        return [=] { return p_assign_hidden(s, h.ptr, h.stride_b, h.stride_n, d, dg, Wg, Cg, bias, folded, mq, mk, near, eps, st); };
     });
 }
 
@@ -159,7 +166,7 @@ PyObject* build_tiles(PyObject*, PyObject* const* args, Py_ssize_t n) {
         auto ws = a.ptr(4);
         auto bytes = a.bytes(4);
         auto st = a.stream(5);
-        return [=] { return focus_build_tiles(s, mq, mk, layout, ws, bytes, st); };
+        return [=] { return p_build_tiles(s, mq, mk, layout, ws, bytes, st); };
     });
 }
 
@@ -175,7 +182,7 @@ PyObject* attn_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {
         auto lse = static_cast<float*>(a.ptr(9));
         auto status = static_cast<int32_t*>(a.ptr(10));
         auto st = a.stream(11);
-        return [=] { return focus_attn_fwd(s, q, k, v, mq, mk, ws, layout, o, lse, status, st); };
+        return [=] { return p_attn_fwd(s, q, k, v, mq, mk, ws, layout, o, lse, status, st); };
     });
 }
 
@@ -191,18 +198,30 @@ PyObject* decode_step(PyObject*, PyObject* const* args, Py_ssize_t n) {
         auto ws = a.ptr(8);
         auto bytes = a.bytes(8);
         auto st = a.stream(9);
-        return [=] { return focus_decode_step(s, q, k, v, mq, mk, o, lse, ws, bytes, st); };
+        return [=] { return p_decode_step(s, q, k, v, mq, mk, o, lse, ws, bytes, st); };
     });
 }
 
-PyObject* init(PyObject*, PyObject* type) {
-    Py_INCREF(type);
-    Py_XSETREF(shape_type, type);
+// init(type of a shape, addresses of the entry points in the order above)
+PyObject* init(PyObject*, PyObject* const* args, Py_ssize_t n) {
+    if (n != 6) return PyErr_Format(PyExc_TypeError, "%zd arguments, not 6", n);
+    void* at[5];
+    for (int i = 0; i < 5; ++i) {
+        at[i] = PyLong_AsVoidPtr(args[1 + i]);
+        if (!at[i]) return PyErr_Occurred() ? nullptr : PyErr_Format(PyExc_ValueError, "no address");
+    }
+    p_assign = reinterpret_cast<decltype(p_assign)>(at[0]);
+    p_assign_hidden = reinterpret_cast<decltype(p_assign_hidden)>(at[1]);
+    p_build_tiles = reinterpret_cast<decltype(p_build_tiles)>(at[2]);
+    p_attn_fwd = reinterpret_cast<decltype(p_attn_fwd)>(at[3]);
+    p_decode_step = reinterpret_cast<decltype(p_decode_step)>(at[4]);
+    Py_INCREF(args[0]);
+    Py_XSETREF(shape_type, args[0]);
     Py_RETURN_NONE;
 }
 
 PyMethodDef methods[] = {
-    {"init", init, METH_O, "the type of a shape"},
+    {"init", (PyCFunction)(void*)init, METH_FASTCALL, nullptr},
     {"assign", (PyCFunction)(void*)assign, METH_FASTCALL, nullptr},
     {"assign_hidden", (PyCFunction)(void*)assign_hidden, METH_FASTCALL, nullptr},
     {"build_tiles", (PyCFunction)(void*)build_tiles, METH_FASTCALL, nullptr},

@@ -1,4 +1,9 @@
 """The short calls through csrc/marshal.cpp and through ctypes: the same results, the same errors."""
+import os
+import shutil
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -82,3 +87,23 @@ def test_same_errors_both_ways(monkeypatch, direct):
         fb.focus_attn_fwd(shape, Q, K, 7, None, None, None, 0, torch.empty_like(Q), m)
     fb.focus_assign(shape, Q, 4, C, m, None, 0)                  # a whole number for a float
     torch.cuda.synchronize()
+
+
+def test_the_library_loaded_is_the_one_called(tmp_path):
+    """LIB_PATH names a copy of the library: the short calls go to it too, and their errors are found there"""
+    copy = tmp_path / "libfocus_b200.so"
+    shutil.copy(fb.LIB_PATH, copy)
+    code = f"""
+import torch
+from paper_2604_03260_b200 import binding as fb
+fb.LIB_PATH = {str(copy)!r}
+m = torch.zeros((4, 40), dtype=torch.int32, device="cuda")
+try:
+    fb.focus_build_tiles(fb.make_shape(4, 2, 40, 64, 4, 2, 32), m, m, 0, torch.zeros(16, dtype=torch.uint8, device="cuda"))
+except fb.FocusError as e:
+    assert len(str(e)) > len(f"focus status {{e.status}}: "), str(e)
+    assert fb._marshal is not fb._Ctypes
+    print("refused")
+"""
+    out = subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(fb.LIB_PATH)), capture_output=True, text=True)
+    assert out.stdout.strip() == "refused", out.stderr

@@ -1,5 +1,6 @@
 """The module in front of the library (csrc/marshal.cpp) reads torch's objects by their layout: it is used only with the torch and the
 Python that it was built for, built again when they change, and done without where it cannot be had.  CPU."""
+import subprocess
 import sys
 import types
 
@@ -89,3 +90,14 @@ def test_the_module_is_built_again_after(monkeypatch, tmp_path, change):
     else:
         monkeypatch.setattr(build, "_marshal_cmd", lambda out: cmd(out) + ["-DX"])
     assert build.marshal_stale()
+
+
+def test_the_module_calls_the_library_that_the_binding_loaded():
+    """not a copy that the loader finds for itself: none is linked, and the addresses come from the loaded one"""
+    fb.lib()
+    m = fb._marshal
+    needed = subprocess.run(["readelf", "-d", m.__file__], check=True, capture_output=True, text=True).stdout
+    assert "libtorch_python" in needed and "libfocus" not in needed
+    for bad in ((), (fb.focus_shape,), (fb.focus_shape, 1, 2, 3, 4), (fb.focus_shape, 1, 2, 3, 4, 0), (fb.focus_shape, 1, 2, 3, 4, "x")):
+        with pytest.raises((TypeError, ValueError)):
+            m.init(*bad)
