@@ -72,6 +72,16 @@ struct Divisor {
     }
 };
 
+// Place in a ring of N slots guarded by a full and an empty mbarrier each: the slot, and the parity of its use.  Whoever empties the ring
+// waits for `phase`, whoever fills it for `phase ^ 1` (which a fresh barrier passes).  Nothing counts up: a count of 32 bits comes round
+// after 2^32 key tiles of one CTA, where a ring of 3 or 5 slots would jump.
+template <int N> struct RingAt {
+    uint32_t slot = 0, phase = 0;
+    __host__ __device__ void next() {
+        if (++slot == N) { slot = 0; phase ^= 1; }
+    }
+};
+
 struct AttnParams {
     int B, Hq, Hkv, G, n, K;
     int w;                   // window, at most n: positions and differences of positions stay within 32 bits

@@ -317,8 +317,9 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
             prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
-            uint32_t nload = 0;
-            uint32_t ninfo = 0;             // tiles handed on
+            RingAt<C::NSTAGE> kv;
+            RingAt<C::NINFO> handed;        // tiles handed on
+            long long until_stall = p.stall_at;
             int it = 0;                     // items processed (items without key tiles are skipped by every role)
             int bad = 0;                    // where a wait gave up
             // ask for the item after number `ord`, when all of that one's loads are on their way
@@ -340,9 +341,9 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 auto next_tile = [&]() -> int {
                     const int kb = walk.next();
                     if constexpr (WALK != WALK_DENSE) {
-                        const uint32_t slot = ninfo % C::NINFO, use = ninfo / C::NINFO;
-                        if (use > 0 && !ctl_wait(&ctl.info_empty[slot], (use - 1) & 1, ctl, bad, 12)) return -1;
-                        ++ninfo;
+                        const uint32_t slot = handed.slot;
+                        if (!ctl_wait(&ctl.info_empty[slot], handed.phase ^ 1, ctl, bad, 12)) return -1;
+                        handed.next();
                         const uint32_t bar = smem_u32(&ctl.info_full[slot]);
                         info[slot].kb = kb;
                         if (kb < 0) {
@@ -385,16 +386,15 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     const int boxes = is_v ? C::SUBT : C::SUBT / C::PARTS;
                     const uint32_t box_bytes = is_v ? C::SUB_BYTES / C::PARTS : C::SUB_BYTES;
 #pragma unroll 1
-                    for (int part = 0; part < C::PARTS; ++part, ++nload) {
-                        if ((long long)nload == p.stall_at) continue;      // diagnostic: this stage is never filled
-                        const uint32_t slot = nload % C::NSTAGE, use = nload / C::NSTAGE;
-                        if (use > 0 && !ctl_wait(&ctl.kv_empty[slot], (use - 1) & 1, ctl, bad, 11)) return;
-                        const uint32_t bar = smem_u32(&ctl.kv_full[slot]);
+                    for (int part = 0; part < C::PARTS; ++part, kv.next()) {
+                        if (until_stall-- == 0) continue;                  // diagnostic: this stage is never filled
+                        if (!ctl_wait(&ctl.kv_empty[kv.slot], kv.phase ^ 1, ctl, bad, 11)) return;
+                        const uint32_t bar = smem_u32(&ctl.kv_full[kv.slot]);
                         const int row = tile * 128 + (is_v ? part * (128 / C::PARTS) : 0), col = is_v ? 0 : part * boxes * 64;
                         mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
 #pragma unroll
                         for (int c = 0; c < boxes; ++c)
-                            tma_load_4d(skv + slot * C::STAGE_BYTES + c * box_bytes, tm, bar, col + c * 64, row, kh, qb);
+                            tma_load_4d(skv + kv.slot * C::STAGE_BYTES + c * box_bytes, tm, bar, col + c * 64, row, kh, qb);
                     }
                 };
                 // Step j: the K of tile j and the V of tile j - 1, in the order in which the MMA warp takes them: with two query tiles
@@ -425,12 +425,12 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         {
             constexpr uint32_t IDESC_S = idesc_bf16(128, 128, 0, 0);
             constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
-            uint32_t nuse = 0;              // K/V stages consumed so far
+            RingAt<C::NSTAGE> kv;
             uint32_t np = 0;                // two query tiles: key tiles whose P has been consumed
-            uint32_t ninfo = 0;             // tiles taken from the ring
+            RingAt<C::NINFO> taken;         // tiles taken from the ring
             uint32_t gs = 0, gp = 0;        // one query tile: S tiles issued / P tiles consumed (buffer = count & 1)
             uint32_t ngt[2] = {0, 0};       // soft gate: G tiles per query tile
-            uint32_t ngk = 0;               // ... key operands taken
+            RingAt<2> gkey;                 // ... key operands taken
             int it = 0;
             int bad = 0;                    // where a wait gave up
             // lower halves of the operand descriptors (the upper ones are the same throughout)
@@ -456,8 +456,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if constexpr (C::GATE_MMA) {
                     const bool g0 = gate_tile(p, a0, kb), g1 = gate_tile(p, a0 + 1, kb);
                     if (!(x ? g1 : g0)) return true;       // (a gated tile 0 without a gated tile 1 gives the key operand back itself)
-                    const uint32_t buf = ngk & 1;
-                    if (!ctl_wait(&gctl.gk_full[buf], (ngk >> 1) & 1, ctl, bad, 53)) return false;
+                    const uint32_t buf = gkey.slot;
+                    if (!ctl_wait(&gctl.gk_full[buf], gkey.phase, ctl, bad, 53)) return false;
                     tc_fence_after();
                     if (elect_one()) {
                         using Steps = GateSteps<C::GATE_CH>;
@@ -470,7 +470,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         if (x == 1 || !g1) umma_commit(smem_u32(&gctl.gk_empty[buf]));
                     }
                     __syncwarp();
-                    if (x == 1 || !g1) ++ngk;
+                    if (x == 1 || !g1) gkey.next();
                     const uint32_t par = (x ? ngt[1]++ : ngt[0]++) & 1;
                     if (!ctl_wait(&gctl.g_taken[x], par, ctl, bad, 54)) return false;
                     tc_fence_after();
@@ -482,9 +482,9 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             };
             // wait for the next tile of the ring
             auto wait_kv = [&](int& slot, int where) -> bool {
-                slot = (int)(nuse % C::NSTAGE);
-                if (!ctl_wait(&ctl.kv_full[slot], (nuse / C::NSTAGE) & 1, ctl, bad, where)) return false;
-                ++nuse;
+                slot = (int)kv.slot;
+                if (!ctl_wait(&ctl.kv_full[slot], kv.phase, ctl, bad, where)) return false;
+                kv.next();
                 return true;
             };
             // One query tile: S[buf] = Q K^T and O (+)= P[buf] V stage by stage -- wait for the stage, issue the MMAs that
@@ -527,12 +527,12 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     if constexpr (WALK == WALK_DENSE) {
                         return walk.next();
                     } else {
-                        const uint32_t slot = ninfo % C::NINFO;
-                        if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, ctl, bad, 27)) return -1;
+                        const uint32_t slot = taken.slot;
+                        if (!ctl_wait(&ctl.info_full[slot], taken.phase, ctl, bad, 27)) return -1;
                         const int kb = info[slot].kb;
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctl.info_empty[slot]));
-                        ++ninfo;
+                        taken.next();
                         return kb;
                     }
                 };
@@ -622,7 +622,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         const int t64 = threadIdx.x - 64;
         unsigned char* const gq = smem_raw + C::OFF_GATE;
         unsigned char* const gk = gq + 2 * C::GQ_BYTES;
-        uint32_t ngk = 0;
+        RingAt<2> gkey;
         int it = 0;
         int bad = 0;                        // where a wait gave up
         Item t = {};
@@ -644,9 +644,9 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             if (lane == 0) mbar_arrive(smem_u32(&gctl.gq_full));
             for (; kb >= 0; kb = walk.next()) {
                 if (!gate_tile(p, a0, kb) && !gate_tile(p, a0 + 1, kb)) continue;
-                const uint32_t buf = ngk & 1, use = ngk >> 1;
-                if (use > 0 && !ctl_wait(&gctl.gk_empty[buf], (use - 1) & 1, ctl, bad, 56)) break;
-                ++ngk;
+                const uint32_t buf = gkey.slot;
+                if (!ctl_wait(&gctl.gk_empty[buf], gkey.phase ^ 1, ctl, bad, 56)) break;
+                gkey.next();
 #pragma unroll 1
                 for (int r = t64; r < 128; r += 64) {
                     const int j = kb * 128 + r;
@@ -675,7 +675,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         const float sl2 = SOFTCAP ? p.softcap * LOG2E : p.scale * LOG2E;
         const float cap_in = SOFTCAP ? p.scale / p.softcap : 0.f;
         uint32_t ns = 0;                                     // S tiles consumed by this warpgroup
-        uint32_t ninfo = 0;                                  // tiles taken from the ring
+        RingAt<C::NINFO> taken;                              // tiles taken from the ring
         uint32_t ng = 0;                                     // soft gate: tiles whose key assignments this warpgroup has staged
         int it = 0;
         int bad = 0;                                         // where a wait gave up
@@ -802,17 +802,16 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if constexpr (WALK == WALK_DENSE) {
                     return walk.next();
                 } else {
-                    const uint32_t slot = ninfo % C::NINFO;
-                    if (!ctl_wait(&ctl.info_full[slot], (ninfo / C::NINFO) & 1, ctl, bad, 39)) return -1;
-                    tile = info + slot;
+                    if (!ctl_wait(&ctl.info_full[taken.slot], taken.phase, ctl, bad, 39)) return -1;
+                    tile = info + taken.slot;
                     return tile->kb;
                 }
             };
             auto tile_read = [&]() {                     // the warp is through with what the ring says of the tile
                 if constexpr (WALK != WALK_DENSE) {
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&ctl.info_empty[ninfo % C::NINFO]));
-                    ++ninfo;
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl.info_empty[taken.slot]));
+                    taken.next();
                 }
             };
             int wmin = 0, wmax = 0;
