@@ -391,7 +391,7 @@ FOCUS_API int focus_selftest_umma(int32_t D, const void* a, const void* b, const
  * that gave up, [2] = work item, [3] = CTA; the other roles of the CTA notice, nothing traps or hangs, tensor memory
  * is released and the kernel returns.  O and lse are left incomplete.  The device and the context stay usable.
  *   shape, q, k, v, o, lse   as for focus_attn_fwd (n >= 512; masks are not used)
- *   wait_limit_ns            1000 ... 4000000000; the bound is checked at a granularity of about 0.1 s
+ *   wait_limit_ns            1000 ... 4000000000; the bound is checked at a granularity of about 1 ms
  *   dev_status               device int32[4], zeroed by the caller, required
  */
 FOCUS_API int focus_selftest_stalled_wait(const focus_shape* shape, focus_tensor q, focus_tensor k, focus_tensor v,

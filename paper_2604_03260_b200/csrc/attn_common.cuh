@@ -82,6 +82,12 @@ template <int N> struct RingAt {
     }
 };
 
+// The clock of the bounded waits: nanoseconds in units of 1024, 32 bits of them.  They come round after 73 minutes; the low word of the
+// nanoseconds does after 4.3 s, so that a wait of 4 s whose block was not on the SM from its end until then began anew.
+__host__ __device__ inline uint32_t wait_ticks(unsigned long long ns) { return (uint32_t)(ns >> 10); }
+__host__ __device__ inline uint32_t wait_limit(unsigned long long ns) { return wait_ticks(ns) + 2; }       // (a wait's ends are rounded: never early)
+__host__ __device__ inline bool wait_over(uint32_t since, uint32_t now, uint32_t limit) { return now - since > limit; }
+
 struct AttnParams {
     int B, Hq, Hkv, G, n, K;
     int w;                   // window, at most n: positions and differences of positions stay within 32 bits

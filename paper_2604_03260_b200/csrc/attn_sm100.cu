@@ -119,7 +119,7 @@ struct SharedCtl {
     uint64_t kv_full[8], kv_empty[8];
     uint64_t info_full[4], info_empty[4];         // tile ring: handed on, read by TILE_READERS warps
     uint64_t next_full[2], next_empty[2];         // the answers below: arrived, read by the MMA warp and every softmax warp
-    uint32_t limit_ns;                // how long a wait may last before the role gives up
+    uint32_t limit;                   // how long a wait may last before the role gives up (wait_limit)
     uint32_t tmem_base;
     int abort_flag;
     uint32_t asked;                   // how many answers the TMA thread has asked for
@@ -142,9 +142,9 @@ __device__ __forceinline__ bool ctl_wait(uint64_t* bar, uint32_t parity, SharedC
 #pragma unroll 1
     for (;;) {
         if (mbar_try_wait(smem_u32(bar), parity)) return true;
-        const uint32_t now = globaltimer_lo() | 1u;
+        const uint32_t now = wait_ticks(globaltimer_ns()) | 1u;
         if (t0 == 0) t0 = now;
-        if (*(volatile int*)&ctl.abort_flag || now - t0 > ctl.limit_ns) break;
+        if (*(volatile int*)&ctl.abort_flag || wait_over(t0, now, ctl.limit)) break;
     }
     gave_up = where;
     return false;
@@ -298,7 +298,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         ctl.abort_flag = 0;
         ctl.asked = 0;
-        ctl.limit_ns = (uint32_t)(p.wait_limit_ns < 4000000000ull ? p.wait_limit_ns : 4000000000ull);
+        ctl.limit = wait_limit(p.wait_limit_ns);
         fence_mbar_init();
     }
     if (warp == 1) {

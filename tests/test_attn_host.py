@@ -29,9 +29,22 @@ template <int N> static void ring() {
     check(sizeof(at) == 8, "a slot and a phase", N, sizeof(at));
 }
 
+// a wait of up to 4 s that is looked at again only `late` after its end has ended, whenever it began and however late that is
+static void wait() {
+    for (unsigned long long limit : {1000ull, 2000000ull, 1000000000ull, 4000000000ull})
+        for (unsigned long long begin : {0ull, 1ull, 4294967295ull, (1ull << 42) - 1000, 1764859000123456789ull}) {
+            const uint32_t t0 = wait_ticks(begin) | 1u, l = wait_limit(limit);
+            for (unsigned long long late : {4096ull, 1000000ull, 294967296ull, 295000000ull, 300000000ull, 1000000000ull, 4294967296ull, 600000000000ull})
+                check(wait_over(t0, wait_ticks(begin + limit + late) | 1u, l), "a wait that has ended", (long long)limit, (long long)late);
+            for (int part = 0; part <= 100; ++part)
+                check(!wait_over(t0, wait_ticks(begin + limit / 100 * part) | 1u, l), "a wait that has not ended", (long long)limit, part);
+        }
+}
+
 int main(int, char** argv) {
     switch (std::atoi(argv[1])) {
         case 0: ring<2>(); ring<3>(); ring<4>(); ring<5>(); ring<6>(); ring<8>(); break;
+        case 1: wait(); break;
         default: return 2;
     }
 }
@@ -52,3 +65,8 @@ def test_places_in_a_ring_never_run_out(program):
     assert out.returncode == 0, out.stdout
     text = open(os.path.join(build.CSRC, "attn_sm100.cu")).read()
     assert "RingAt<C::NSTAGE>" in text and "% C::NSTAGE" not in text and "% C::NINFO" not in text
+
+
+def test_a_wait_that_was_not_looked_at_for_long_has_ended(program):
+    out = program(1)
+    assert out.returncode == 0, out.stdout
