@@ -388,8 +388,9 @@ FOCUS_API int focus_selftest_umma(int32_t D, const void* a, const void* b, const
  * mode with one stage of its K/V ring deliberately left unfilled, so that the role waiting for that stage runs into
  * its time limit.  Every wait inside the attention kernels is bounded (4 s in focus_attn_fwd); this entry point sets
  * the bound to `wait_limit_ns` and shows the exit taken when it expires: dev_status[0] = 1, [1] = code of the wait
- * that gave up, [2] = work item, [3] = CTA; the other roles of the CTA notice, nothing traps or hangs, tensor memory
- * is released and the kernel returns.  O and lse are left incomplete.  The device and the context stay usable.
+ * that gave up, [2] = query block at work (for codes 50 and 51, the queue of items: the item's number in the CTA),
+ * [3] = CTA; the other roles of the CTA notice, nothing traps or hangs, tensor memory is released and the kernel
+ * returns.  O and lse are left incomplete.  The device and the context stay usable.
  *   shape, q, k, v, o, lse   as for focus_attn_fwd (n >= 512; masks are not used)
  *   wait_limit_ns            1000 ... 4000000000; the bound is checked at a granularity of about 1 ms
  *   dev_status               device int32[4], zeroed by the caller, required

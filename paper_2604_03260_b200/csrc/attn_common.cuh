@@ -88,6 +88,13 @@ __host__ __device__ inline uint32_t wait_ticks(unsigned long long ns) { return (
 __host__ __device__ inline uint32_t wait_limit(unsigned long long ns) { return wait_ticks(ns) + 2; }       // (a wait's ends are rounded: never early)
 __host__ __device__ inline bool wait_over(uint32_t since, uint32_t now, uint32_t limit) { return now - since > limit; }
 
+// codes of the waits of the item queue: for the CTA's next item, for room to ask for one
+constexpr int WAIT_NEXT_ITEM = 50, WAIT_NEXT_ROOM = 51;
+// status word 2 of a wait that gave up: the query block at work, or the number in the CTA of the item waited for (50) or asking (51)
+__host__ __device__ inline int stalled_work(int where, int query_block, uint32_t ord) {
+    return where == WAIT_NEXT_ITEM || where == WAIT_NEXT_ROOM ? (int)ord : query_block;
+}
+
 struct AttnParams {
     int B, Hq, Hkv, G, n, K;
     int w;                   // window, at most n: positions and differences of positions stay within 32 bits

@@ -150,11 +150,11 @@ __device__ __forceinline__ bool ctl_wait(uint64_t* bar, uint32_t parity, SharedC
     return false;
 }
 
-__device__ __forceinline__ void give_up(const AttnParams& p, SharedCtl* ctl, int where, int item) {
+__device__ __forceinline__ void give_up(const AttnParams& p, SharedCtl* ctl, int where, int query_block, uint32_t ord) {
     *(volatile int*)&ctl->abort_flag = 1;
     if (p.status && atomicCAS(p.status, 0, 1) == 0) {
         p.status[1] = where;
-        p.status[2] = item;
+        p.status[2] = stalled_work(where, query_block, ord);
         p.status[3] = (int)blockIdx.x;
     }
 }
@@ -216,7 +216,7 @@ __device__ __forceinline__ bool next_item(const AttnParams& p, SharedCtl& ctl, u
     uint32_t block = blockIdx.x;
     if (ord > 0) {
         const uint32_t slot = (ord - 1) & 1, use = (ord - 1) >> 1;
-        if (!ctl_wait(&ctl.next_full[slot], use & 1, ctl, gave_up, 50)) return false;
+        if (!ctl_wait(&ctl.next_full[slot], use & 1, ctl, gave_up, WAIT_NEXT_ITEM)) return false;
         const bool more = clc_answer(smem_u32(&ctl.next[slot]), block);
         if (reader) {
             fence_proxy_async_smem();                   // the answer is read before the next one is written there
@@ -325,13 +325,14 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             // ask for the item after number `ord`, when all of that one's loads are on their way
             auto ask_next = [&](uint32_t ord) {
                 const uint32_t slot = ord & 1, use = ord >> 1;
-                if (use > 0 && !ctl_wait(&ctl.next_empty[slot], (use - 1) & 1, ctl, bad, 51)) return;
+                if (use > 0 && !ctl_wait(&ctl.next_empty[slot], (use - 1) & 1, ctl, bad, WAIT_NEXT_ROOM)) return;
                 mbar_arrive_expect_tx(smem_u32(&ctl.next_full[slot]), 16);
                 clc_try_cancel(smem_u32(&ctl.next[slot]), smem_u32(&ctl.next_full[slot]));
                 ctl.asked = ord + 1;
             };
             Item t = {};
-            for (uint32_t ord = 0; !bad && next_item<WALK>(p, ctl, ord, false, t, bad); ++ord) {
+            uint32_t ord = 0;
+            for (; !bad && next_item<WALK>(p, ctl, ord, false, t, bad); ++ord) {
                 const int A = t.A, hq = t.hq, b = t.bb, h = t.h, hk = p.by_G.div(h);
                 TileWalk<WALK> walk;
                 walk.init(p, hq, A * NQ, NQ);
@@ -370,7 +371,11 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 };
                 int kb = next_tile();
                 if (bad) break;
-                if (kb < 0) { ask_next(ord); continue; }
+                if (kb < 0) {
+                    ask_next(ord);
+                    if (bad) break;
+                    continue;
+                }
                 if (it > 0 && !ctl_wait(&ctl.q_empty, (it - 1) & 1, ctl, bad, 10)) break;
                 mbar_arrive_expect_tx(smem_u32(&ctl.q_full), NQ * C::TILE_BYTES);
                 // in the sorted layout the copies are indexed [head of the batch][sorted slot]
@@ -413,9 +418,10 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     kb = next_tile();
                 }
                 if (!bad) ask_next(ord);
+                if (bad) break;
                 ++it;
             }
-            if (bad) give_up(p, &ctl, bad, t.A);
+            if (bad) give_up(p, &ctl, bad, t.A, ord);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -519,7 +525,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 return true;
             };
             Item t = {};
-            for (uint32_t ord = 0; !bad && next_item<WALK>(p, ctl, ord, true, t, bad); ++ord) {
+            uint32_t ord = 0;
+            for (; !bad && next_item<WALK>(p, ctl, ord, true, t, bad); ++ord) {
                 const int A = t.A, hq = t.hq;
                 TileWalk<WALK> walk;
                 if constexpr (WALK == WALK_DENSE) walk.init(p, hq, A * NQ, NQ);
@@ -614,7 +621,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     have_p = true;
                 }
             }
-            if (bad) give_up(p, &ctl, bad, t.A);
+            if (bad) give_up(p, &ctl, bad, t.A, ord);
         }
         __syncwarp();
     } else if (C::GATE_MMA && warp < 4) {
@@ -626,7 +633,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         int it = 0;
         int bad = 0;                        // where a wait gave up
         Item t = {};
-        for (uint32_t ord = 0; !bad && next_item<WALK>(p, ctl, ord, true, t, bad); ++ord) {
+        uint32_t ord = 0;
+        for (; !bad && next_item<WALK>(p, ctl, ord, true, t, bad); ++ord) {
             const int a0 = t.A * NQ;
             TileWalk<WALK_DENSE> walk;
             walk.init(p, t.hq, a0, NQ);
@@ -658,7 +666,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
             ++it;
         }
-        if (bad) give_up(p, &ctl, bad, t.A);
+        if (bad) give_up(p, &ctl, bad, t.A, ord);
         __syncwarp();
     } else if (warp >= 4) {
         // ------------------------------------------------------------------ softmax + epilogue
@@ -687,7 +695,8 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         bool valid = false;
         float m_used = -INFINITY, l = 0.f;
         bool finish = false;                                 // an item whose tiles are through
-        for (uint32_t ord = 0;; ++ord) {
+        uint32_t ord = 0;
+        for (;; ++ord) {
             Item t_next = {};
             const bool have = next_item<WALK>(p, ctl, ord, true, t_next, bad);
             if (bad) break;
@@ -1108,7 +1117,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             tile_read();                                 // the end of the item
             finish = !first;
         }
-        if (bad) give_up(p, &ctl, bad, t.A);
+        if (bad) give_up(p, &ctl, bad, t.A, ord);
     }
     // ---------------------------------------------------------------------- teardown
     tc_fence_before();

@@ -41,10 +41,17 @@ static void wait() {
         }
 }
 
+// the waits of the item queue say which item of the CTA, all others the query block at work
+static void status() {
+    for (int where = 1; where < 100; ++where)
+        check(stalled_work(where, 7, 3) == (where == 50 || where == 51 ? 3 : 7), "status word 2", where, stalled_work(where, 7, 3));
+}
+
 int main(int, char** argv) {
     switch (std::atoi(argv[1])) {
         case 0: ring<2>(); ring<3>(); ring<4>(); ring<5>(); ring<6>(); ring<8>(); break;
         case 1: wait(); break;
+        case 2: status(); break;
         default: return 2;
     }
 }
@@ -70,3 +77,10 @@ def test_places_in_a_ring_never_run_out(program):
 def test_a_wait_that_was_not_looked_at_for_long_has_ended(program):
     out = program(1)
     assert out.returncode == 0, out.stdout
+
+
+def test_a_wait_of_the_item_queue_names_the_item(program):
+    out = program(2)
+    assert out.returncode == 0, out.stdout
+    text = open(os.path.join(build.CSRC, "attn_sm100.cu")).read()
+    assert text.count("give_up(p, &ctl, bad, t.A, ord)") == 4               # every role: TMA, MMA, gate operands, softmax
