@@ -13,14 +13,43 @@ from paper_2604_03260_b200 import inputs as fi
 pytestmark = pytest.mark.gpu
 
 
-class NotRead:
-    """in the place of the module: no argument is of the usual kind"""
+class Calls:
+    """In the place of the module: counts how often it was asked and how often it answered.  Without `behind`, no argument is of the
+    usual kind."""
+    def __init__(self, behind=None):
+        self.asked = self.answered = 0
+        self.behind = behind
+
     def __getattr__(self, name):
-        return lambda *args: None
+        def call(*args):
+            self.asked += 1
+            rc = getattr(self.behind, name)(*args) if self.behind else None
+            self.answered += rc is not None
+            return rc
+        return call
+
+
+@pytest.fixture
+def through(monkeypatch):
+    """through(direct) -> Calls: from here on the calls go through the module (with `direct`), or through ctypes"""
+    fb.lib()                         # before the patch: loading puts the module in its place
+    module = fb._marshal
+    assert module is not fb._Ctypes
+    put = []
+
+    def through(direct):
+        put.append(Calls(module if direct else None))
+        monkeypatch.setattr(fb, "_marshal", put[-1])
+        return put[-1]
+    yield through
+    assert not put or fb._marshal is put[-1]
 
 
 class Sub(torch.Tensor):
     pass
+
+
+CALLS = 6                            # of run()
 
 
 def run(wl, wrap, batch, stream=None, eps=1e-5):
@@ -53,25 +82,31 @@ def run(wl, wrap, batch, stream=None, eps=1e-5):
 
 
 @pytest.mark.parametrize("batch", [1, 3])
-def test_same_results_both_ways(monkeypatch, batch):
+def test_same_results_both_ways(through, batch):
     wl = fi.Workload("marshal", 4, 2, 64, 300, 4, 2, 32, seed=3)
+    calls = through(True)
     got = run(wl, lambda t: t, batch)
+    assert calls.asked == calls.answered == CALLS
     side = torch.cuda.Stream()
     side.wait_stream(torch.cuda.current_stream())
-    others = [run(wl, lambda t: t, batch, stream=torch.cuda.current_stream()), run(wl, lambda t: t.as_subclass(Sub), batch)]
+    others = [run(wl, lambda t: t, batch, stream=torch.cuda.current_stream())]
+    assert calls.asked == 2 * CALLS and calls.answered == CALLS                 # a stream object: through ctypes
+    others.append(run(wl, lambda t: t.as_subclass(Sub), batch))
+    assert calls.asked == 3 * CALLS and calls.answered == CALLS                 # a tensor subclass: too
     with torch.cuda.stream(side):
         others.append(run(wl, lambda t: t, batch))
-    monkeypatch.setattr(fb, "_marshal", NotRead())
+    assert calls.asked == 4 * CALLS and calls.answered == 2 * CALLS
+    calls = through(False)
     others.append(run(wl, lambda t: t, batch))
+    assert calls.asked == CALLS and calls.answered == 0
     for other in others:
         for a, b in zip(got, other):
             assert torch.equal(a, b)
 
 
 @pytest.mark.parametrize("direct", [True, False])
-def test_same_errors_both_ways(monkeypatch, direct):
-    if not direct:
-        monkeypatch.setattr(fb, "_marshal", NotRead())
+def test_same_errors_both_ways(through, direct):
+    through(direct)
     wl = fi.Workload("marshal", 4, 2, 64, 40, 4, 2, 32, seed=3)
     shape = fb.shape_of(wl)
     Q, K, V, C = fi.make_inputs(wl, "cuda")
@@ -87,6 +122,57 @@ def test_same_errors_both_ways(monkeypatch, direct):
         fb.focus_attn_fwd(shape, Q, K, 7, None, None, None, 0, torch.empty_like(Q), m)
     fb.focus_assign(shape, Q, 4, C, m, None, 0)                  # a whole number for a float
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("direct", [True, False])
+def test_same_errors_of_a_decode_step_and_of_the_router(through, direct):
+    calls = through(direct)
+    wl = fi.Workload("marshal", 4, 2, 64, 40, 4, 2, 32, seed=3)
+    shape = fb.shape_of(wl)
+    Q, K, V, C = fi.make_inputs(wl, "cuda")
+    mq, mk = torch.zeros(4, dtype=torch.int32, device="cuda"), torch.zeros((2, 40), dtype=torch.int32, device="cuda")
+    q, o, lse = Q[:, 0].contiguous(), torch.zeros((4, 64), dtype=torch.bfloat16, device="cuda"), torch.zeros(4, device="cuda")
+    ws = torch.zeros(fb.focus_decode_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    step = lambda q=q, k=K, o=o, ws=ws: fb.focus_decode_step(shape, q, k, V, mq, mk, o, lse, ws)
+    for bad in (q.float(), q.cpu(), torch.zeros((4, 128), dtype=torch.bfloat16, device="cuda")[:, ::2]):
+        with pytest.raises(AssertionError):
+            step(q=bad)
+        with pytest.raises(AssertionError):
+            step(o=bad)
+    with pytest.raises(IndexError):
+        step(q=q[0])                                             # [D]
+    with pytest.raises(AssertionError):
+        step(k=K[0])                                             # [n, D]
+    with pytest.raises(fb.FocusError):
+        step(ws=ws[:16])
+    with pytest.raises(AttributeError):
+        step(ws=None)
+    h = torch.zeros((40, 128), dtype=torch.bfloat16, device="cuda")
+    Wg, Cg, f = torch.zeros((64, 16), device="cuda"), torch.zeros((4, 16), device="cuda"), torch.zeros((4, 64), device="cuda")
+    hq, hk = torch.zeros((4, 40), dtype=torch.int32, device="cuda"), torch.zeros((2, 40), dtype=torch.int32, device="cuda")
+    route = lambda h=h[:, :64].contiguous(), Wg=Wg: fb.focus_assign_hidden(shape, h, Wg, Cg, None, f, hq, hk)
+    for bad in (h[:, ::2], h[:, :64].float(), h[:, :64].cpu()):  # the first: a stride along d_model
+        with pytest.raises(AssertionError):
+            route(h=bad)
+    with pytest.raises(IndexError):
+        route(Wg=Wg[0])
+    answered = calls.answered
+    step()
+    route()
+    torch.cuda.synchronize()
+    assert calls.answered == answered + (2 if direct else 0)
+
+
+@pytest.mark.parametrize("direct", [True, False])
+def test_a_tensor_without_storage_is_refused_both_ways(through, direct):
+    """under torch.func.vmap a tensor is of the usual class and says its strides, but has no address"""
+    calls = through(direct)
+    wl = fi.Workload("marshal", 4, 2, 64, 40, 4, 2, 32, seed=3)
+    Q, K, V, C = fi.make_inputs(wl, "cuda")
+    m = torch.zeros((4, 40), dtype=torch.int32, device="cuda")
+    with pytest.raises(RuntimeError):
+        torch.func.vmap(lambda q: fb.focus_assign(fb.shape_of(wl), q, 4, C, m))(torch.stack([Q, Q]))
+    assert calls.asked == 1 and calls.answered == 0
 
 
 def test_the_library_loaded_is_the_one_called(tmp_path):
