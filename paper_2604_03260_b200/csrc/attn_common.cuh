@@ -51,8 +51,9 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
     return r;
 }
 
-// Division of 0 <= n < 2^31 by d >= 1 as a multiplication: q = n (2^(31 + l) / d + 1) / 2^(31 + l) with 2^l >= d.  (The compiler's
-// own, for a divisor it does not know, is some 20 instructions.)
+// Division of 0 <= n < 2^31 by d >= 1 as a multiplication: q = n (2^(31 + l) / d + 1) / 2^(31 + l) with 2^l >= d (Granlund and
+// Montgomery, Division by Invariant Integers using Multiplication, 1994).  (The compiler's own, for a divisor it does not know, is
+// some 20 instructions.)
 struct Divisor {
     uint32_t d, m;
     int s;

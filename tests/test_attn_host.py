@@ -47,11 +47,27 @@ static void status() {
         check(stalled_work(where, 7, 3) == (where == 50 || where == 51 ? 3 : 7), "status word 2", where, stalled_work(where, 7, 3));
 }
 
+// quotients at both sides of every step near the ends of the range and in it
+static void divisor() {
+    const long long top = 0x7fffffffll;
+    auto one = [&](long long d) {
+        if (d < 1 || d > top) return;
+        const Divisor by((int)d);
+        for (long long q : {0ll, 1ll, 2ll, 1000ll, top / d / 2, top / d - 1, top / d})
+            for (long long n : {q * d - 1, q * d, q * d + 1, top - q})
+                if (n >= 0 && n <= top) check(by.div((int)n) == n / d, "quotient", n, d);
+    };
+    for (long long d = 1; d < 20000; ++d) one(d);
+    for (int l = 14; l <= 31; ++l)
+        for (long long e = -40; e <= 40; ++e) { one((1ll << l) + e); one((1ll << l) / 3 + e); one((1ll << l) / 5 * 3 + e); }
+}
+
 int main(int, char** argv) {
     switch (std::atoi(argv[1])) {
         case 0: ring<2>(); ring<3>(); ring<4>(); ring<5>(); ring<6>(); ring<8>(); break;
         case 1: wait(); break;
         case 2: status(); break;
+        case 3: divisor(); break;
         default: return 2;
     }
 }
@@ -84,3 +100,8 @@ def test_a_wait_of_the_item_queue_names_the_item(program):
     assert out.returncode == 0, out.stdout
     text = open(os.path.join(build.CSRC, "attn_sm100.cu")).read()
     assert text.count("give_up(p, &ctl, bad, t.A, ord)") == 4               # every role: TMA, MMA, gate operands, softmax
+
+
+def test_division_by_a_launch_parameter(program):
+    out = program(3)
+    assert out.returncode == 0, out.stdout
