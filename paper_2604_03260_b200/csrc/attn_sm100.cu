@@ -16,23 +16,25 @@
 //
 // Head dimension 256 does not leave room in TMEM for two query tiles (O alone is 256 columns), so
 // there an item is a single 128-row query tile, S is double-buffered over consecutive key tiles
-// and one warpgroup does the softmax while the MMAs of the neighbouring tiles run.
+// and the two softmax warpgroups share every row, a thread to each half of the key tile's columns.
 //
 // Training-time soft gate, two query tiles: the factor of a distant pair is a function of g_i . g_j, and those products are
 // an MMA as well.  For a pair of tiles that holds distant pairs G_x = g_q g_k^T goes to the place of S_x first, the softmax
 // warps take it into registers and work out the 128 factors while S_x = Q_x K^T is computed over it; warps 2 and 3 write
 // the operands (assignments split into bf16 terms).  Per key tile that leaves the softmax warps a tanh, a fused
 // multiply-add and half a packed multiplication per pair, in place of K / 2 packed multiply-adds on 2 K / 4 shared-memory
-// reads: 8192 tokens, K = 8, 32/8 heads: 1290 -> 862 us; 32768: 20.7 -> 13.5 ms.  At D = 256 tensor memory and the ring
-// leave one query tile, whose softmax warps evaluate the products themselves.
+// reads: 8192 tokens, K = 8, 32/8 heads: 1290 -> 862 us (742 with the shorter code below); 32768: 20.7 -> 13.5 ms.  At D = 256
+// tensor memory and the ring leave one query tile, whose softmax warps evaluate the products themselves.
 //
-// Code size: 45 to 82 KB a kernel, from 65 to 118.  The roles run side by side and each streams through its own code once per
-// tile, so what is executed per tile should fit the instruction caches, and code that is rarely executed should not lie in
-// between: waits and their reports inlined at full length, loops the compiler unrolled by itself and divisions by launch
-// parameters were half of it.  Loops with short trip counts therefore say `unroll 1`, except the issue of a tile's MMAs, whose
-// descriptors must be there when the tensor pipe is (rolled up: 1228 -> 1714 cycles from P to the next S).  12 heads x 16384
-// tokens at D = 64 in dense mode: 614 -> 547 us; 65536 tokens at D = 256 class-sorted: 13.1 -> 12.0 ms; 32 heads x 8192 in token
-// order: 551 -> 530 us, gated: 794 -> 707.
+// Code size: 46 to 82 KB a kernel, from 65 to 118 (0.59 to 0.82 of what each was).  The roles run side by side and each streams
+// through its own code once per tile: waits and their reports inlined at full length, loops the compiler unrolled by itself and
+// divisions by launch parameters were instructions to issue and registers to hold, and lay between what is executed per tile.  Loops
+// with short trip counts therefore say `unroll 1`, except the issue of a tile's MMAs, whose descriptors must be there when the tensor
+// pipe is (rolled up: 1228 -> 1714 cycles from P to the next S).  Together with the epilogue in pieces of 16 columns and the lower
+// halves of descriptors: 12 heads x 16384 tokens at D = 64 in dense mode: 614 -> 547 us; 65536 tokens at D = 256 class-sorted: 13.1 ->
+// 12.0 ms; 32 heads x 8192 in token order: 551 -> 530 us, gated: 794 -> 707.  By the counters (8192 tokens, token order and gated, the
+// hand-over of P in two parts included): 7 and 6 % fewer instructions, which waited for memory and tensor memory 0.95 -> 0.77 and
+// 3.5 -> 2.9 cycles each; the wait for instructions was never large (0.32 -> 0.26 and 0.42 -> 0.40).
 //
 // Which key tiles are visited, and in which order of items:
 //   dense mode      every tile up to the diagonal
@@ -931,7 +933,7 @@ focus_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 uint32_t pk[NC / 2];
                 if (tile_gated) {                    // the factors are in place of the scores
 #pragma unroll
-                    for (int c = 0; c < NC / 16; ++c) {      // 16 at a time beside the 128 factors: 32 took 944 us for 8192 tokens, 16 862
+                    for (int c = 0; c < NC / 16; ++c) {      // 16 at a time beside the 128 factors (8192 tokens: 742 us, 802 with 32)
                         uint32_t sv[16];
                         tmem_ld16(t_s + c * 16, sv);
                         tmem_wait_ld();
