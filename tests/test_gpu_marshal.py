@@ -13,43 +13,21 @@ from paper_2604_03260_b200 import inputs as fi
 pytestmark = pytest.mark.gpu
 
 
-class Calls:
-    """In the place of the module: counts how often it was asked and how often it answered.  Without `behind`, no argument is of the
-    usual kind."""
-    def __init__(self, behind=None):
-        self.asked = self.answered = 0
-        self.behind = behind
-
+class NotRead:
+    """in the place of the module: no argument is of the usual kind"""
     def __getattr__(self, name):
-        def call(*args):
-            self.asked += 1
-            rc = getattr(self.behind, name)(*args) if self.behind else None
-            self.answered += rc is not None
-            return rc
-        return call
+        return lambda *args: None
 
 
-@pytest.fixture
-def through(monkeypatch):
-    """through(direct) -> Calls: from here on the calls go through the module (with `direct`), or through ctypes"""
-    fb.lib()                         # before the patch: loading puts the module in its place
-    module = fb._marshal
-    assert module is not fb._Ctypes
-    put = []
-
-    def through(direct):
-        put.append(Calls(module if direct else None))
-        monkeypatch.setattr(fb, "_marshal", put[-1])
-        return put[-1]
-    yield through
-    assert not put or fb._marshal is put[-1]
+@pytest.fixture(autouse=True)
+def loaded():
+    """Loading puts the module in its place: before a test puts another there, and so that it is put back afterwards."""
+    fb.lib()
+    assert fb._marshal is not fb._Ctypes
 
 
 class Sub(torch.Tensor):
     pass
-
-
-CALLS = 6                            # of run()
 
 
 def run(wl, wrap, batch, stream=None, eps=1e-5):
@@ -82,31 +60,25 @@ def run(wl, wrap, batch, stream=None, eps=1e-5):
 
 
 @pytest.mark.parametrize("batch", [1, 3])
-def test_same_results_both_ways(through, batch):
+def test_same_results_both_ways(monkeypatch, batch):
     wl = fi.Workload("marshal", 4, 2, 64, 300, 4, 2, 32, seed=3)
-    calls = through(True)
     got = run(wl, lambda t: t, batch)
-    assert calls.asked == calls.answered == CALLS
     side = torch.cuda.Stream()
     side.wait_stream(torch.cuda.current_stream())
-    others = [run(wl, lambda t: t, batch, stream=torch.cuda.current_stream())]
-    assert calls.asked == 2 * CALLS and calls.answered == CALLS                 # a stream object: through ctypes
-    others.append(run(wl, lambda t: t.as_subclass(Sub), batch))
-    assert calls.asked == 3 * CALLS and calls.answered == CALLS                 # a tensor subclass: too
+    others = [run(wl, lambda t: t, batch, stream=torch.cuda.current_stream()), run(wl, lambda t: t.as_subclass(Sub), batch)]
     with torch.cuda.stream(side):
         others.append(run(wl, lambda t: t, batch))
-    assert calls.asked == 4 * CALLS and calls.answered == 2 * CALLS
-    calls = through(False)
+    monkeypatch.setattr(fb, "_marshal", NotRead())
     others.append(run(wl, lambda t: t, batch))
-    assert calls.asked == CALLS and calls.answered == 0
     for other in others:
         for a, b in zip(got, other):
             assert torch.equal(a, b)
 
 
 @pytest.mark.parametrize("direct", [True, False])
-def test_same_errors_both_ways(through, direct):
-    through(direct)
+def test_same_errors_both_ways(monkeypatch, direct):
+    if not direct:
+        monkeypatch.setattr(fb, "_marshal", NotRead())
     wl = fi.Workload("marshal", 4, 2, 64, 40, 4, 2, 32, seed=3)
     shape = fb.shape_of(wl)
     Q, K, V, C = fi.make_inputs(wl, "cuda")
@@ -122,6 +94,50 @@ def test_same_errors_both_ways(through, direct):
         fb.focus_attn_fwd(shape, Q, K, 7, None, None, None, 0, torch.empty_like(Q), m)
     fb.focus_assign(shape, Q, 4, C, m, None, 0)                  # a whole number for a float
     torch.cuda.synchronize()
+
+
+class Calls:
+    """In the place of the module: counts how often it was asked and how often it answered.  Without `behind`, no argument is of the
+    usual kind."""
+    def __init__(self, behind=None):
+        self.asked = self.answered = 0
+        self.behind = behind
+
+    def __getattr__(self, name):
+        def call(*args):
+            self.asked += 1
+            rc = getattr(self.behind, name)(*args) if self.behind else None
+            self.answered += rc is not None
+            return rc
+        return call
+
+
+@pytest.fixture
+def through(monkeypatch):
+    """through(direct) -> Calls: from here on the calls go through the module (with `direct`), or through ctypes"""
+    module, put = fb._marshal, []
+
+    def through(direct):
+        put.append(Calls(module if direct else None))
+        monkeypatch.setattr(fb, "_marshal", put[-1])
+        return put[-1]
+    yield through
+    assert fb._marshal is put[-1]
+
+
+def test_which_way_a_call_took(through):
+    wl = fi.Workload("marshal", 4, 2, 64, 300, 4, 2, 32, seed=3)
+    same, sub = lambda t: t, lambda t: t.as_subclass(Sub)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    for direct, wrap, stream, current, answered in (
+            (True, same, None, None, 6), (True, same, None, side, 6),
+            (True, same, torch.cuda.current_stream(), None, 0), (True, sub, None, None, 0),    # a stream object, a tensor subclass: through ctypes
+            (False, same, None, None, 0)):
+        calls = through(direct)
+        with torch.cuda.stream(current):
+            run(wl, wrap, 1, stream=stream)
+        assert calls.asked == 6 and calls.answered == answered
 
 
 @pytest.mark.parametrize("direct", [True, False])
