@@ -1,9 +1,11 @@
 // The short calls of binding.py without ctypes: tensors to addresses and strides, the current stream, the call.
 //
 // A decode step or a prompt of a thousand tokens takes the GPU 15 to 30 us, and marshalling the arguments of its three or four
-// calls through ctypes took the host as long: 8 us a focus_assign and 16 a focus_decode_step on a slow core.  A decode step over 2049
-// keys in a row of them: 33.0 -> 21.4 us (30.6 -> 19.4 on a faster host); from the call until the GPU is done, with the GPU idle before: 45.5 ->
-// 34.3, and a prompt of 1024 tokens in buffers not used before 65 -> 48.  The functions take what binding.py's take.  They answer None when an argument is none that they know how to read (a tensor
+// calls through ctypes took the host as long: 8 us a focus_assign and 16 a focus_decode_step on a slow core.  A decode step over
+// 2049 keys in a row of them: 33.0 -> 21.4 us (30.6 -> 19.4 on a faster host); from the call until the GPU is done, with the GPU
+// idle before: 45.5 -> 34.3, and a prompt of 1024 tokens in buffers not used before 65 -> 48.
+//
+// The functions take what binding.py's take.  They answer None when an argument is none that they know how to read (a tensor
 // subclass, a shape that is no focus_shape, ...), before anything has been enqueued; binding.py then goes through ctypes as for
 // its other entry points.
 #include <Python.h>
